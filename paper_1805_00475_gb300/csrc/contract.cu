@@ -959,12 +959,13 @@ struct tnc_batch_s {
          off_results = 0, off_limbs = 0, off_arena = 0, total = 0;
   size_t desc_bytes = 0;
   uint32_t n_forms = 0;
+  uint32_t n_heavy = 0;      // formulas contracted by whole clusters (the first of the order)
   uint64_t total_out = 0;
   std::vector<uint64_t> res_off;
   uint64_t max_arena = 0;    // entries
   uint64_t max_blob = 0;     // bytes of the largest descriptor blob
   uint64_t slot_entries = 0;  // global arena slot of one CTA (entries)
-  uint32_t slots = 0;         // CTAs any launch shape can have
+  uint32_t slots = 0;         // arena slots: CTAs (clusters, if every formula is heavy) any launch shape can have
   // launch configuration (autotuned)
   int threads = 128;
   int cta_cap = 0;           // CTAs per SM cap (0: as many as fit)
@@ -984,13 +985,44 @@ namespace {
 
 constexpr size_t kSmemMax = 227 * 1024;
 
-// CTAs of batch_kernel<RG, N30> per SM for (threads, dynamic shared memory),
+// Batch formulas contracted by whole clusters: those with more than
+// kHeavyShare of the batch's work (multiply-adds and entries) per resident CTA
+// (four per SM; per formula where there are fewer), and more than kHeavyMin;
+// none unless the largest exceeds kHeavyTop, below which a cluster's barriers
+// cost what its CTAs gain.  Measured on 2048 cubic VC formulas with n = 60
+// (4 residues; three seeds): no clusters 498-709 us, shares of 0.5 / 0.7 / 1 /
+// 1.4 / 2: 430 / 365 / 328 / 370 / 520 us; on 700 with n = 64: 850, 416, 331,
+// 280 us for none / 0.7 / 1 / 1.4; on 777 uneven 1-in-3 formulas (2 residues):
+// 1330-3130 us without, 226-545 us with.  20 formulas with n = 48, all below
+// kHeavyTop: 28-41 us without, 40-48 us with.
+constexpr uint32_t kClusterCtas = 8;
+constexpr double kHeavyShare = 1.2, kHeavyMin = 16384.0, kHeavyTop = 131072.0;
+
+// Launch configuration of clusters of `ctas` CTAs.
+struct ClusterLaunch {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at[1];
+  ClusterLaunch(unsigned grid, unsigned threads, size_t smem, cudaStream_t st, unsigned ctas) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ctas;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+  }
+  ClusterLaunch(const ClusterLaunch&) = delete;
+};
+
+// CTAs of batch_kernel<RG, N30, MODE> per SM for (threads, dynamic shared memory),
 // capped at `cap` (0: no cap).  The L1 / shared-memory split is then set to
 // the smallest shared-memory share that holds those CTAs, so that the rest of
 // the SM's 256 KiB serves as L1 for the formulas' global arenas.
-template <int RG, bool N30>
-int occupancy(int threads, size_t smem, int cap, int* blocks) {
-  auto k = tnc_dev::batch_kernel<RG, N30>;
+template <int RG, bool N30, int MODE>
+int occupancy(int threads, size_t smem, int cap, int* blocks, int* clusters) {
+  auto k = tnc_dev::batch_kernel<RG, N30, MODE>;
   // the limit is a property of the kernel, shared by every batch in the
   // process: set it to the device's maximum, not to this batch's need (a batch
   // configured later with smaller descriptors would otherwise make an earlier
@@ -1020,6 +1052,10 @@ int occupancy(int threads, size_t smem, int cap, int* blocks) {
     if (occ2 < occ) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
   }
   *blocks = occ;
+  if (MODE != tnc_dev::kBatchCtas && occ > 0) {
+    const ClusterLaunch cl(kClusterCtas * (unsigned)sm_count(), (unsigned)threads, smem, nullptr, kClusterCtas);
+    CUDA_TRY(cudaOccupancyMaxActiveClusters(clusters, k, &cl.cfg));
+  }
   return TNC_OK;
 }
 
@@ -1028,14 +1064,28 @@ int batch_configure(tnc_batch_t* b, int threads, size_t smem, int cap) {
   const int sms = sm_count();
   std::vector<int> grid;
   for (size_t gi = 0; gi < b->a.groups.rg.size(); gi++) {
-    int occ = 0;
+    int occ = 0, clusters = 0;
     const bool n30 = b->a.group((int)gi).near30 != 0;
     int rc = dispatch_rg(b->a.groups.rg[gi], [&](auto rgc) -> int {
-      return n30 ? occupancy<decltype(rgc)::value, true>(threads, b->max_blob + smem, cap, &occ)
-                 : occupancy<decltype(rgc)::value, false>(threads, b->max_blob + smem, cap, &occ);
+      constexpr int RG = decltype(rgc)::value;
+      const size_t sm = b->max_blob + smem;
+      if (b->n_heavy)
+        return n30 ? occupancy<RG, true, tnc_dev::kBatchClusters>(threads, sm, cap, &occ, &clusters)
+                   : occupancy<RG, false, tnc_dev::kBatchClusters>(threads, sm, cap, &occ, &clusters);
+      return n30 ? occupancy<RG, true, tnc_dev::kBatchCtas>(threads, sm, cap, &occ, &clusters)
+                 : occupancy<RG, false, tnc_dev::kBatchCtas>(threads, sm, cap, &occ, &clusters);
     });
     if (rc) return rc;
     if (occ <= 0) return set_error(TNC_ERR_TOO_LARGE, "batch kernel does not fit on an SM");
+    if (b->n_heavy) {  // clusters resident at once, as many as there is work for
+      const int n_light = (int)(b->n_forms - b->n_heavy), cs = (int)kClusterCtas;
+      int nc = std::min(clusters, std::max(1, sms * occ / cs));
+      nc = std::min(nc, std::max((int)b->n_heavy, (n_light + cs - 1) / cs));
+      nc = std::min(nc, (int)b->slots / (n_light ? cs : 1));
+      if (clusters <= 0 || nc <= 0) return set_error(TNC_ERR_TOO_LARGE, "no cluster of the batch kernel fits");
+      grid.push_back(nc * cs);
+      continue;
+    }
     grid.push_back(std::max(1, std::min<int>(std::min<int>(sms * occ, (int)b->n_forms), (int)b->slots)));
   }
   b->threads = threads;
@@ -1059,10 +1109,183 @@ size_t blob_put(std::vector<char>& blob, const void* src, size_t bytes) {
   return at;
 }
 
+// One formula's descriptor blob (the sections that batch_kernel copies to
+// shared memory) and the fields of its BForm that do not depend on the batch,
+// for `threads` threads sharing the formula.
+int pack_form(const tnc_plan_t* p, uint32_t threads, std::vector<char>& blob, BForm& f) {
+  if (p->tree.nodes.empty()) return set_error(TNC_ERR_INVALID, "batch formula with an empty network");
+  if (p->cost.max_rank > 24 || !p->low.lvl_fits)
+    return set_error(TNC_ERR_TOO_LARGE, "batch formulas must have plan rank <= 24");
+  const Lowered& lw = p->low;
+  if (lw.lvl_arena_entries >= (1ull << 32)) return set_error(TNC_ERR_TOO_LARGE, "formula arena above 2^32 entries");
+  if (lw.lvl_steps.size() >= 65535) return set_error(TNC_ERR_TOO_LARGE, "more than 65534 steps in one formula");
+  std::memset(&f, 0, sizeof(f));
+  blob.clear();
+  // per level: the share of one of the formula's `threads` lanes (at least
+  // 16 products), and per step the lane split sh of its long shared sums: an
+  // entry of a step is split over 2^sh lanes so that no lane sums much more
+  // than that share
+  const uint32_t nlev = lw.lvl_start.empty() ? 0 : (uint32_t)lw.lvl_start.size() - 1;
+  std::vector<uint32_t> lvl_log_t(nlev, 4), step_sh(lw.lvl_steps.size(), 0);
+  for (uint32_t l = 0; l < nlev; l++) {
+    uint64_t work = 0;
+    for (uint32_t si = lw.lvl_start[l]; si < lw.lvl_start[l + 1]; si++)
+      work += 1ull << (lw.lvl_steps[si].c + lw.lvl_steps[si].k);
+    uint32_t log_t = 4;
+    while (log_t < 24 && (1ull << log_t) * threads < work) log_t++;
+    lvl_log_t[l] = log_t;
+    for (uint32_t si = lw.lvl_start[l]; si < lw.lvl_start[l + 1]; si++) {
+      const StepDesc& d = lw.lvl_steps[si];
+      uint32_t sh = 0;
+      while (sh < 5 && sh < d.k && d.k - sh > log_t) sh++;
+      step_sh[si] = sh;
+    }
+  }
+  // steps, runs and address deltas.  A lane group of a whole-warp block
+  // advances its entry by 2^g (g = 5 - sh): delta[t - g] = w[t] -
+  // sum_{g <= j < t} w[j] for the operand weights w[j] of output bit j.
+  std::vector<BStep> steps;
+  std::vector<uint16_t> runs;
+  std::vector<int32_t> dls;  // pairs (A, B)
+  for (size_t si = 0; si < lw.lvl_steps.size(); si++) {
+    const StepDesc& d = lw.lvl_steps[si];
+    BStep bs;
+    std::memset(&bs, 0, sizeof(bs));
+    bs.a_off = (uint32_t)d.a_off;
+    bs.b_off = (uint32_t)d.b_off;
+    bs.c_off = (uint32_t)d.c_off;
+    bs.c = d.c;
+    bs.k = d.k;
+    bs.ka = d.ka;
+    bs.kb = d.kb;
+    if (runs.size() >= 65535 || dls.size() / 2 >= 65535)
+      return set_error(TNC_ERR_TOO_LARGE, "formula descriptors beyond 2^16 runs or deltas");
+    bs.run0 = (uint16_t)runs.size();
+    int64_t wA[32] = {0}, wB[32] = {0};
+    if (d.nra != TNC_BITMAP) {
+      for (int r = 0; r < d.nra; r++) {
+        const TncRun& x = d.map.runs.ra[r];
+        runs.push_back(pack_run(x.src, x.dst, x.len));
+        for (int q = 0; q < x.len; q++) wA[x.src + q] = 1ll << (x.dst + q);
+      }
+      for (int r = 0; r < d.nrb; r++) {
+        const TncRun& x = d.map.runs.rb[r];
+        runs.push_back(pack_run(x.src, x.dst, x.len));
+        for (int q = 0; q < x.len; q++) wB[x.src + q] = 1ll << (x.dst + q);
+      }
+      bs.nra = d.nra;
+      bs.nrb = d.nrb;
+    } else {
+      for (int side = 0; side < 2; side++)
+        for (int j = 0; j < d.c; j++)
+          if ((d.map.bit[j] >> 7) == side) {
+            runs.push_back(pack_run(j, d.map.bit[j] & 63, 1));
+            (side ? bs.nrb : bs.nra)++;
+            (side ? wB : wA)[j] = 1ll << (d.map.bit[j] & 63);
+          }
+    }
+    const uint32_t g = 5 - step_sh[si];
+    bs.g = (uint8_t)g;
+    bs.dl0 = (uint16_t)(dls.size() / 2);
+    for (uint32_t t = g; t < d.c; t++) {
+      int64_t sa = 0, sb = 0;
+      for (uint32_t j = g; j < t; j++) {
+        sa += wA[j];
+        sb += wB[j];
+      }
+      dls.push_back((int32_t)(wA[t] - sa));
+      dls.push_back((int32_t)(wB[t] - sb));
+    }
+    steps.push_back(bs);
+  }
+  // segments per level: steps whose entries take 32+ lanes get whole-warp
+  // blocks of V entries per lane group (V such that a lane's work is about
+  // half the level's share, at most 4); the others share packed segments
+  // lane by lane.  Segments are ordered by cost, longest first.
+  std::vector<Seg> segs;
+  std::vector<uint32_t> items, lvl{0};
+  for (uint32_t l = 0; l < nlev; l++) {
+    const uint32_t log_t = lvl_log_t[l];
+    struct Group {
+      uint32_t si, o, sh, cost;
+    };
+    std::vector<Group> small;
+    std::vector<std::pair<uint32_t, Seg>> lsegs;  // (cost, segment)
+    for (uint32_t si = lw.lvl_start[l]; si < lw.lvl_start[l + 1]; si++) {
+      const StepDesc& d = lw.lvl_steps[si];
+      const uint32_t sh = step_sh[si];
+      const uint32_t cost = 1u << (d.k - sh);
+      const uint32_t nout = 1u << d.c;
+      if ((nout << sh) < 32) {
+        for (uint32_t o = 0; o < nout; o++) small.push_back(Group{si, o, sh, cost});
+        continue;
+      }
+      const uint32_t G = 32u >> sh;
+      uint32_t V = 1;
+      while (V < 4 && 2 * V * G <= nout && (2 * V) * cost <= (1u << (log_t - 1))) V *= 2;
+      for (uint32_t o0 = 0; o0 < nout; o0 += G * V)
+        lsegs.push_back({cost * V, Seg{o0, (uint16_t)si, (uint8_t)V, (uint8_t)sh}});
+    }
+    // widest groups first: each group then starts at a multiple of its size
+    // and never crosses a 32-lane boundary
+    std::stable_sort(small.begin(), small.end(), [](const Group& x, const Group& y) {
+      return x.sh != y.sh ? x.sh > y.sh : x.cost > y.cost;
+    });
+    for (size_t g = 0; g < small.size();) {
+      const uint32_t first = (uint32_t)items.size();
+      uint32_t lanes = 0, cost = 0;
+      const uint8_t sh0 = (uint8_t)small[g].sh;
+      while (g < small.size() && lanes + (1u << small[g].sh) <= 32) {
+        const Group& q = small[g];
+        for (uint32_t j = 0; j < (1u << q.sh); j++) items.push_back(q.si | q.o << 16 | j << 21 | q.sh << 26);
+        lanes += 1u << q.sh;
+        cost = std::max(cost, q.cost);
+        g++;
+      }
+      lsegs.push_back({cost, Seg{first, tnc_dev::kPacked, (uint8_t)lanes, sh0}});
+    }
+    std::stable_sort(lsegs.begin(), lsegs.end(),
+                     [](const std::pair<uint32_t, Seg>& x, const std::pair<uint32_t, Seg>& y) {
+                       return x.first > y.first;
+                     });
+    for (const auto& x : lsegs) segs.push_back(x.second);
+    lvl.push_back((uint32_t)segs.size());
+  }
+  // the blob
+  blob_put(blob, steps.data(), steps.size() * sizeof(BStep));
+  f.segs_at = (uint32_t)blob_put(blob, segs.data(), segs.size() * sizeof(Seg));
+  f.items_at = (uint32_t)blob_put(blob, items.data(), items.size() * sizeof(uint32_t));
+  f.runs_at = (uint32_t)blob_put(blob, runs.data(), runs.size() * sizeof(uint16_t));
+  f.dl_at = (uint32_t)blob_put(blob, dls.data(), dls.size() * sizeof(int32_t));
+  f.lvl_at = (uint32_t)blob_put(blob, lvl.data(), lvl.size() * sizeof(uint32_t));
+  blob.resize((blob.size() + 15) / 16 * 16);
+  f.blob_n = (uint32_t)(blob.size() / 16);
+  f.nlev = nlev;
+  f.nleaf = (uint32_t)lw.leaves.size();
+  f.n_open = (uint32_t)p->net.open_vars.size();
+  f.n_out = 1u << f.n_open;
+  f.root_off = (uint32_t)(lw.lvl_steps.empty() ? lw.lvl_leaf_off[p->tree.root] : lw.lvl_root_off);
+  f.arena = (uint32_t)lw.lvl_arena_entries;
+  return TNC_OK;
+}
+
+// The leaves of a formula, their weight tables starting at table0.
+void pack_leaves(const Lowered& lw, uint32_t table0, std::vector<BLeaf>& leaves) {
+  for (size_t l = 0; l < lw.leaves.size(); l++) {
+    BLeaf bl;
+    std::memset(&bl, 0, sizeof(bl));
+    bl.off = (uint32_t)lw.lvl_leaf_off[l];
+    bl.table_off = lw.leaves[l].table_off + table0;
+    bl.kind = lw.leaves[l].kind;
+    bl.rank = lw.leaves[l].rank;
+    leaves.push_back(bl);
+  }
+}
+
 int batch_pack(tnc_batch_t* b) {
   const uint32_t n = b->n_forms;
   std::vector<BForm> forms(n);
-  std::vector<char> blobs;  // all formulas' blobs, each 16-byte aligned
+  std::vector<char> blobs, blob;  // all formulas' blobs, each 16-byte aligned
   std::vector<BLeaf> leaves;
   std::vector<uint32_t> tables;
   std::vector<uint8_t> perms;
@@ -1070,196 +1293,49 @@ int batch_pack(tnc_batch_t* b) {
   uint64_t out = 0;
   b->max_arena = 8;
   b->max_blob = 16;
+  // largest formulas first (longest-processing-time order)
+  std::vector<uint32_t> order(n);
+  for (uint32_t i = 0; i < n; i++) order[i] = i;
+  auto cost = [&](uint32_t i) { return b->plans[i]->cost.macs + b->plans[i]->cost.entries; };
+  std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) { return cost(x) > cost(y); });
+  double total = 0;
+  for (uint32_t i = 0; i < n; i++) total += cost(i);
+  // heavy formulas, contracted by whole clusters (batch_kernel)
+  const uint32_t ctas = 4u * (uint32_t)sm_count();  // resident at once
+  const double share = n <= ctas / kClusterCtas / 2 ? 0.0 : total / std::min(n, ctas);
+  while (cost(order[0]) > kHeavyTop && b->n_heavy < n &&
+         cost(order[b->n_heavy]) > std::max(kHeavyShare * share, kHeavyMin))
+    b->n_heavy++;
+  std::vector<uint32_t> threads(n, 256);
+  for (uint32_t i = 0; i < b->n_heavy; i++) threads[order[i]] = 256 * kClusterCtas;
   for (uint32_t i = 0; i < n; i++) {
     const tnc_plan_t* p = b->plans[i];
-    if (p->tree.nodes.empty()) return set_error(TNC_ERR_INVALID, "batch formula with an empty network");
-    if (p->cost.max_rank > 24 || !p->low.lvl_fits)
-      return set_error(TNC_ERR_TOO_LARGE, "batch formulas must have plan rank <= 24");
     const Lowered& lw = p->low;
-    if (lw.lvl_arena_entries >= (1ull << 32)) return set_error(TNC_ERR_TOO_LARGE, "formula arena above 2^32 entries");
-    if (lw.lvl_steps.size() >= 65535) return set_error(TNC_ERR_TOO_LARGE, "more than 65534 steps in one formula");
-    // per level: the share of one lane of a 256-thread CTA (at least 16
-    // products), and per step the lane split sh of its long shared sums: an
-    // entry of a step is split over 2^sh lanes so that no lane sums much more
-    // than that share
-    const uint32_t nlev = lw.lvl_start.empty() ? 0 : (uint32_t)lw.lvl_start.size() - 1;
-    std::vector<uint32_t> lvl_log_t(nlev, 4), step_sh(lw.lvl_steps.size(), 0);
-    for (uint32_t l = 0; l < nlev; l++) {
-      uint64_t work = 0;
-      for (uint32_t si = lw.lvl_start[l]; si < lw.lvl_start[l + 1]; si++)
-        work += 1ull << (lw.lvl_steps[si].c + lw.lvl_steps[si].k);
-      uint32_t log_t = 4;
-      while (log_t < 24 && (1ull << log_t) * 256 < work) log_t++;
-      lvl_log_t[l] = log_t;
-      for (uint32_t si = lw.lvl_start[l]; si < lw.lvl_start[l + 1]; si++) {
-        const StepDesc& d = lw.lvl_steps[si];
-        uint32_t sh = 0;
-        while (sh < 5 && sh < d.k && d.k - sh > log_t) sh++;
-        step_sh[si] = sh;
-      }
-    }
-    // steps, runs and address deltas.  A lane group of a whole-warp block
-    // advances its entry by 2^g (g = 5 - sh): delta[t - g] = w[t] -
-    // sum_{g <= j < t} w[j] for the operand weights w[j] of output bit j.
-    std::vector<BStep> steps;
-    std::vector<uint16_t> runs;
-    std::vector<int32_t> dls;  // pairs (A, B)
-    for (size_t si = 0; si < lw.lvl_steps.size(); si++) {
-      const StepDesc& d = lw.lvl_steps[si];
-      BStep bs;
-      std::memset(&bs, 0, sizeof(bs));
-      bs.a_off = (uint32_t)d.a_off;
-      bs.b_off = (uint32_t)d.b_off;
-      bs.c_off = (uint32_t)d.c_off;
-      bs.c = d.c;
-      bs.k = d.k;
-      bs.ka = d.ka;
-      bs.kb = d.kb;
-      if (runs.size() >= 65535 || dls.size() / 2 >= 65535)
-        return set_error(TNC_ERR_TOO_LARGE, "formula descriptors beyond 2^16 runs or deltas");
-      bs.run0 = (uint16_t)runs.size();
-      int64_t wA[32] = {0}, wB[32] = {0};
-      if (d.nra != TNC_BITMAP) {
-        for (int r = 0; r < d.nra; r++) {
-          const TncRun& x = d.map.runs.ra[r];
-          runs.push_back(pack_run(x.src, x.dst, x.len));
-          for (int q = 0; q < x.len; q++) wA[x.src + q] = 1ll << (x.dst + q);
-        }
-        for (int r = 0; r < d.nrb; r++) {
-          const TncRun& x = d.map.runs.rb[r];
-          runs.push_back(pack_run(x.src, x.dst, x.len));
-          for (int q = 0; q < x.len; q++) wB[x.src + q] = 1ll << (x.dst + q);
-        }
-        bs.nra = d.nra;
-        bs.nrb = d.nrb;
-      } else {
-        for (int side = 0; side < 2; side++)
-          for (int j = 0; j < d.c; j++)
-            if ((d.map.bit[j] >> 7) == side) {
-              runs.push_back(pack_run(j, d.map.bit[j] & 63, 1));
-              (side ? bs.nrb : bs.nra)++;
-              (side ? wB : wA)[j] = 1ll << (d.map.bit[j] & 63);
-            }
-      }
-      const uint32_t g = 5 - step_sh[si];
-      bs.g = (uint8_t)g;
-      bs.dl0 = (uint16_t)(dls.size() / 2);
-      for (uint32_t t = g; t < d.c; t++) {
-        int64_t sa = 0, sb = 0;
-        for (uint32_t j = g; j < t; j++) {
-          sa += wA[j];
-          sb += wB[j];
-        }
-        dls.push_back((int32_t)(wA[t] - sa));
-        dls.push_back((int32_t)(wB[t] - sb));
-      }
-      steps.push_back(bs);
-    }
-    // segments per level: steps whose entries take 32+ lanes get whole-warp
-    // blocks of V entries per lane group (V such that a lane's work is about
-    // half the level's share, at most 4); the others share packed segments
-    // lane by lane.  Segments are ordered by cost, longest first.
-    std::vector<Seg> segs;
-    std::vector<uint32_t> items, lvl{0};
-    for (uint32_t l = 0; l < nlev; l++) {
-      const uint32_t log_t = lvl_log_t[l];
-      struct Group {
-        uint32_t si, o, sh, cost;
-      };
-      std::vector<Group> small;
-      std::vector<std::pair<uint32_t, Seg>> lsegs;  // (cost, segment)
-      for (uint32_t si = lw.lvl_start[l]; si < lw.lvl_start[l + 1]; si++) {
-        const StepDesc& d = lw.lvl_steps[si];
-        const uint32_t sh = step_sh[si];
-        const uint32_t cost = 1u << (d.k - sh);
-        const uint32_t nout = 1u << d.c;
-        if ((nout << sh) < 32) {
-          for (uint32_t o = 0; o < nout; o++) small.push_back(Group{si, o, sh, cost});
-          continue;
-        }
-        const uint32_t G = 32u >> sh;
-        uint32_t V = 1;
-        while (V < 4 && 2 * V * G <= nout && (2 * V) * cost <= (1u << (log_t - 1))) V *= 2;
-        for (uint32_t o0 = 0; o0 < nout; o0 += G * V)
-          lsegs.push_back({cost * V, Seg{o0, (uint16_t)si, (uint8_t)V, (uint8_t)sh}});
-      }
-      // widest groups first: each group then starts at a multiple of its size
-      // and never crosses a 32-lane boundary
-      std::stable_sort(small.begin(), small.end(), [](const Group& x, const Group& y) {
-        return x.sh != y.sh ? x.sh > y.sh : x.cost > y.cost;
-      });
-      for (size_t g = 0; g < small.size();) {
-        const uint32_t first = (uint32_t)items.size();
-        uint32_t lanes = 0, cost = 0;
-        const uint8_t sh0 = (uint8_t)small[g].sh;
-        while (g < small.size() && lanes + (1u << small[g].sh) <= 32) {
-          const Group& q = small[g];
-          for (uint32_t j = 0; j < (1u << q.sh); j++) items.push_back(q.si | q.o << 16 | j << 21 | q.sh << 26);
-          lanes += 1u << q.sh;
-          cost = std::max(cost, q.cost);
-          g++;
-        }
-        lsegs.push_back({cost, Seg{first, tnc_dev::kPacked, (uint8_t)lanes, sh0}});
-      }
-      std::stable_sort(lsegs.begin(), lsegs.end(),
-                       [](const std::pair<uint32_t, Seg>& x, const std::pair<uint32_t, Seg>& y) {
-                         return x.first > y.first;
-                       });
-      for (const auto& x : lsegs) segs.push_back(x.second);
-      lvl.push_back((uint32_t)segs.size());
-    }
-    // the blob
-    std::vector<char> blob;
-    blob_put(blob, steps.data(), steps.size() * sizeof(BStep));
     BForm& f = forms[i];
-    std::memset(&f, 0, sizeof(f));
-    f.segs_at = (uint32_t)blob_put(blob, segs.data(), segs.size() * sizeof(Seg));
-    f.items_at = (uint32_t)blob_put(blob, items.data(), items.size() * sizeof(uint32_t));
-    f.runs_at = (uint32_t)blob_put(blob, runs.data(), runs.size() * sizeof(uint16_t));
-    f.dl_at = (uint32_t)blob_put(blob, dls.data(), dls.size() * sizeof(int32_t));
-    f.lvl_at = (uint32_t)blob_put(blob, lvl.data(), lvl.size() * sizeof(uint32_t));
-    blob.resize((blob.size() + 15) / 16 * 16);
+    const int rc = pack_form(p, threads[i], blob, f);
+    if (rc) return rc;
     f.blob = (uint32_t)(blobs.size() / 16);
-    f.blob_n = (uint32_t)(blob.size() / 16);
     blobs.insert(blobs.end(), blob.begin(), blob.end());
     b->max_blob = std::max<uint64_t>(b->max_blob, blob.size());
-    f.nlev = nlev;
     f.leaf0 = (uint32_t)leaves.size();
-    f.nleaf = (uint32_t)lw.leaves.size();
     f.res_off = (uint32_t)out;
-    f.n_open = (uint32_t)p->net.open_vars.size();
-    f.n_out = 1u << f.n_open;
     f.perm_off = (uint32_t)perms.size();
-    f.root_off = (uint32_t)(lw.lvl_steps.empty() ? lw.lvl_leaf_off[p->tree.root] : lw.lvl_root_off);
-    f.arena = (uint32_t)lw.lvl_arena_entries;
-
     b->res_off[i] = out;
     out += f.n_out;
-    const uint32_t toff = (uint32_t)tables.size();
-    for (size_t l = 0; l < lw.leaves.size(); l++) {
-      BLeaf bl;
-      std::memset(&bl, 0, sizeof(bl));
-      bl.off = (uint32_t)lw.lvl_leaf_off[l];
-      bl.table_off = lw.leaves[l].table_off + toff;
-      bl.kind = lw.leaves[l].kind;
-      bl.rank = lw.leaves[l].rank;
-      leaves.push_back(bl);
-    }
+    pack_leaves(lw, (uint32_t)tables.size(), leaves);
     tables.insert(tables.end(), lw.leaf_tables.begin(), lw.leaf_tables.end());
     perms.insert(perms.end(), lw.root_perm.begin(), lw.root_perm.end());
     b->max_arena = std::max<uint64_t>(b->max_arena, lw.lvl_arena_entries);
   }
   if (blobs.size() / 16 >= (1ull << 32)) return set_error(TNC_ERR_TOO_LARGE, "batch descriptors above 64 GiB");
   b->total_out = out;
-  // one global arena slot per CTA: at most 32 CTAs per SM in any launch shape
+  // global arena slots: one per CTA, at most 32 CTAs per SM in any launch
+  // shape (one per cluster where all formulas are heavy)
   b->slot_entries = (b->max_arena + 7) / 8 * 8;
-  b->slots = (uint32_t)std::min<uint64_t>(n, (uint64_t)sm_count() * 32u);
-  // largest formulas first (longest-processing-time order)
-  std::vector<uint32_t> order(n);
-  for (uint32_t i = 0; i < n; i++) order[i] = i;
-  std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) {
-    return b->plans[x]->cost.macs + b->plans[x]->cost.entries > b->plans[y]->cost.macs + b->plans[y]->cost.entries;
-  });
+  const uint32_t n_light = n - b->n_heavy;
+  uint64_t units = n;
+  if (b->n_heavy && n_light) units = (uint64_t)kClusterCtas * std::max(b->n_heavy, (n_light + kClusterCtas - 1) / kClusterCtas);
+  b->slots = (uint32_t)std::min<uint64_t>(units, (uint64_t)sm_count() * 32u);
   const int rg_max = b->a.groups.rg.empty() ? 1 : b->a.groups.rg[0];
   // workspace layout
   size_t o = 0;
@@ -1318,14 +1394,25 @@ int batch_enqueue(tnc_batch_t* b, void* dev_ws, cudaStream_t st) {
     args.smem_cap = (uint32_t)(b->smem_bytes / (rg * sizeof(uint32_t)));
     args.R = b->a.R;
     args.col = b->a.groups.col[gi];
+    args.n_heavy = b->n_heavy;
+    args.cluster_slots = b->n_heavy == b->n_forms;
     const ModGroup mg = b->a.group((int)gi);
     const int grid = b->grid[gi];
     const size_t smem = b->max_blob + b->smem_bytes;
     const int threads = b->threads;
     int rc = dispatch_rg(rg, [&](auto rgc) -> int {
       constexpr int RG = decltype(rgc)::value;
-      if (mg.near30) tnc_dev::batch_kernel<RG, true><<<grid, threads, smem, st>>>(args, mg);
-      else tnc_dev::batch_kernel<RG, false><<<grid, threads, smem, st>>>(args, mg);
+      if (b->n_heavy) {
+        const ClusterLaunch cl((unsigned)grid, (unsigned)threads, smem, st, kClusterCtas);
+        CUDA_TRY(cudaLaunchKernelEx(
+            &cl.cfg,
+            mg.near30 ? tnc_dev::batch_kernel<RG, true, tnc_dev::kBatchClusters>
+                      : tnc_dev::batch_kernel<RG, false, tnc_dev::kBatchClusters>,
+            args, mg, b->a.crt));
+        return TNC_OK;
+      }
+      if (mg.near30) tnc_dev::batch_kernel<RG, true><<<grid, threads, smem, st>>>(args, mg, b->a.crt);
+      else tnc_dev::batch_kernel<RG, false><<<grid, threads, smem, st>>>(args, mg, b->a.crt);
       CUDA_TRY(cudaGetLastError());
       return TNC_OK;
     });

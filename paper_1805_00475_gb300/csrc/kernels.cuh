@@ -507,38 +507,41 @@ struct CrtConsts {
   int n_limbs;                    // <= kCrtMaxLimbs
 };
 
-__global__ void crt_kernel(const uint32_t* __restrict__ residues, uint64_t n_entries, CrtConsts cc,
-                           uint32_t* __restrict__ limbs) {
-  for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n_entries;
-       e += (uint64_t)gridDim.x * blockDim.x) {
-    uint32_t v[kCrtMaxResidues];
-    const uint32_t* r = residues + e * cc.R;
-    for (int i = 0; i < cc.R; i++) {
-      const uint32_t p = cc.p[i];
-      const uint64_t mu = cc.mu[i];
-      uint32_t ri = r[i] % p;
-      if (i == 0) {
-        v[0] = ri;
-        continue;
-      }
-      uint32_t t = mod_reduce(v[i - 1], p, mu);
-      for (int j = i - 2; j >= 0; j--) t = mod_reduce((uint64_t)t * cc.p[j] + v[j], p, mu);
-      const uint32_t diff = ri >= t ? ri - t : ri + (p - t);
-      v[i] = mod_reduce((uint64_t)diff * cc.inv[i], p, mu);
+// Residues r[0..R) of one entry to its n_limbs limbs.
+__device__ __noinline__ void crt_entry(const uint32_t* r, const CrtConsts& cc, uint32_t* limbs) {
+  uint32_t v[kCrtMaxResidues];
+  for (int i = 0; i < cc.R; i++) {
+    const uint32_t p = cc.p[i];
+    const uint64_t mu = cc.mu[i];
+    uint32_t ri = r[i] % p;
+    if (i == 0) {
+      v[0] = ri;
+      continue;
     }
-    uint32_t x[kCrtMaxLimbs];
-    for (int l = 0; l < kCrtMaxLimbs; l++) x[l] = 0;
-    x[0] = v[cc.R - 1];
-    for (int i = cc.R - 2; i >= 0; i--) {
-      uint64_t carry = v[i];
-      for (int l = 0; l < cc.n_limbs; l++) {
-        const uint64_t t = (uint64_t)x[l] * cc.p[i] + carry;
-        x[l] = (uint32_t)t;
-        carry = t >> 32;
-      }
-    }
-    for (int l = 0; l < cc.n_limbs; l++) limbs[e * cc.n_limbs + l] = x[l];
+    uint32_t t = mod_reduce(v[i - 1], p, mu);
+    for (int j = i - 2; j >= 0; j--) t = mod_reduce((uint64_t)t * cc.p[j] + v[j], p, mu);
+    const uint32_t diff = ri >= t ? ri - t : ri + (p - t);
+    v[i] = mod_reduce((uint64_t)diff * cc.inv[i], p, mu);
   }
+  uint32_t x[kCrtMaxLimbs];
+  for (int l = 0; l < kCrtMaxLimbs; l++) x[l] = 0;
+  x[0] = v[cc.R - 1];
+  for (int i = cc.R - 2; i >= 0; i--) {
+    uint64_t carry = v[i];
+    for (int l = 0; l < cc.n_limbs; l++) {
+      const uint64_t t = (uint64_t)x[l] * cc.p[i] + carry;
+      x[l] = (uint32_t)t;
+      carry = t >> 32;
+    }
+  }
+  for (int l = 0; l < cc.n_limbs; l++) limbs[l] = x[l];
+}
+
+__global__ void crt_kernel(const uint32_t* __restrict__ residues, uint64_t n_entries,
+                           const __grid_constant__ CrtConsts cc, uint32_t* __restrict__ limbs) {
+  for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n_entries;
+       e += (uint64_t)gridDim.x * blockDim.x)
+    crt_entry(residues + e * cc.R, cc, limbs + e * cc.n_limbs);
 }
 
 // ------------------------------------------------------- persistent batch
@@ -677,7 +680,27 @@ struct BatchArgs {
   uint32_t smem_cap;      // entries of dynamic shared memory available for an arena
   int R;
   int col;                // first residue column of this group
+  // cluster launches only
+  uint32_t n_heavy;       // the first n_heavy formulas of `order` are contracted by whole clusters
+  uint32_t cluster_slots; // arena slots are per cluster (there are no other formulas), not per CTA
+  uint32_t* limbs;        // not NULL: this launch also runs the CRT (one formula, the last residue group)
 };
+
+// Every thread of the CTAs of a cluster, with the memory ordering of a
+// __syncthreads over all of them (global memory included).
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_ctas() {
+  uint32_t n;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
+  return n;
+}
+__device__ __forceinline__ uint32_t cluster_cta() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
 
 __device__ __forceinline__ uint32_t map_runs(uint32_t o, const uint16_t* runs, int n) {
   uint32_t a = 0;
@@ -697,22 +720,64 @@ __device__ __forceinline__ uint32_t map_runs(uint32_t o, const uint16_t* runs, i
 // slot of global memory, reused by each formula the CTA takes, so that the
 // live arenas (CTAs x slot) stay in L2 instead of every formula's arena being
 // written back to DRAM.
-template <int RG, bool N30 = false>
-__global__ void __launch_bounds__(256) batch_kernel(BatchArgs a, ModGroup mg) {
+//
+// CLUSTER: the grid is made of clusters.  The batch's heaviest formulas (the
+// first n_heavy) are contracted first, each by all CTAs of one cluster: the
+// segments of a level are shared out over the warps of the cluster, the
+// barrier between levels is the cluster's, the tensors live in the slot of the
+// cluster's first CTA (formula t goes to cluster t, then back and forth).  A
+// formula that takes longer alone than the batch's average CTA would
+// otherwise be what the launch ends with.  Then every CTA takes formulas from
+// the queue as above.
+enum BatchMode { kBatchCtas, kBatchClusters, kBatchSolo };  // kBatchSolo: one formula, one cluster, and its CRT
+template <int RG, bool N30 = false, int MODE = kBatchCtas>
+__global__ void __launch_bounds__(256, MODE == kBatchCtas ? 0 : (RG == 4 && !N30 ? 3 : 4))
+    batch_kernel(BatchArgs a, ModGroup mg, const __grid_constant__ CrtConsts cc) {
+  constexpr bool CLUSTER = MODE != kBatchCtas;
   extern __shared__ uint4 smem_raw[];
   __shared__ uint32_t task;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31;
   uint4* blob = smem_raw;
   uint32_t* sarena = reinterpret_cast<uint32_t*>(smem_raw + (a.blob_cap >> 4));
+  bool coop = CLUSTER;       // contracting the heavy formulas, cluster by cluster
+  uint32_t round = 0;
   for (;;) {
-    if (threadIdx.x == 0) task = atomicAdd(a.queue, 1u);
-    __syncthreads();
-    const uint32_t t = task;
-    if (t >= a.n_forms) break;
+    uint32_t t;
+    if (CLUSTER && coop) {
+      const uint32_t nc = gridDim.x / cluster_ctas(), c = blockIdx.x / cluster_ctas();
+      t = round * nc + ((round & 1u) ? nc - 1u - c : c);
+      round++;
+      if (t >= a.n_heavy) {
+        if (a.n_heavy == a.n_forms) break;
+        coop = false;
+        continue;
+      }
+    } else {
+      if (threadIdx.x == 0) task = atomicAdd(a.queue, 1u);
+      __syncthreads();
+      t = task;
+      if (CLUSTER) t += a.n_heavy;
+      if (t >= a.n_forms) break;
+    }
+    // the threads and warps that share this formula
+    uint32_t tid = threadIdx.x, nthreads = blockDim.x;
+    if (CLUSTER && coop) {
+      tid += cluster_cta() * blockDim.x;
+      nthreads *= cluster_ctas();
+    }
+    const uint32_t warp = tid >> 5, nwarps = nthreads >> 5;
     const BForm f = a.forms[a.order[t]];
     for (uint32_t i = threadIdx.x; i < f.blob_n; i += blockDim.x) blob[i] = a.blobs[f.blob + i];
-    uint32_t* arena = f.arena <= a.smem_cap ? sarena : a.garena + (uint64_t)blockIdx.x * a.slot_entries * RG;
-    for (uint32_t l = threadIdx.x; l < f.nleaf; l += blockDim.x) {
+    uint32_t* arena = a.garena;
+    if (CLUSTER && coop)
+      arena += (uint64_t)(a.cluster_slots ? blockIdx.x / cluster_ctas() : blockIdx.x - cluster_cta()) * a.slot_entries * RG;
+    else
+      arena = f.arena <= a.smem_cap ? sarena : arena + (uint64_t)blockIdx.x * a.slot_entries * RG;
+    auto barrier = [&] {
+      if (CLUSTER && coop) cluster_barrier();
+      else __syncthreads();
+    };
+    for (uint32_t l = tid; l < f.nleaf; l += nthreads) {
       const BLeaf ld = a.leaves[f.leaf0 + l];
       uint32_t* dst = arena + (uint64_t)ld.off * RG;
       const uint32_t n = 1u << ld.rank;
@@ -723,7 +788,7 @@ __global__ void __launch_bounds__(256) batch_kernel(BatchArgs a, ModGroup mg) {
         store_entry<RG>(dst + (uint64_t)idx * RG, v);
       }
     }
-    __syncthreads();
+    barrier();
     const char* bb = reinterpret_cast<const char*>(blob);
     const BStep* steps = reinterpret_cast<const BStep*>(bb);
     const Seg* segs = reinterpret_cast<const Seg*>(bb + f.segs_at);
@@ -798,16 +863,19 @@ __global__ void __launch_bounds__(256) batch_kernel(BatchArgs a, ModGroup mg) {
         }
         if (active && slice == 0) store_entry<RG>(arena + ((uint64_t)d.c_off + o) * RG, out);
       }
-      __syncthreads();
+      barrier();
     }
-    for (uint32_t J = threadIdx.x; J < f.n_out; J += blockDim.x) {
+    for (uint32_t J = tid; J < f.n_out; J += nthreads) {
       uint32_t ad = 0;
       for (uint32_t j = 0; j < f.n_open; j++) ad |= ((J >> a.perms[f.perm_off + j]) & 1u) << j;
 #pragma unroll
       for (int r = 0; r < RG; r++)
         a.results[((uint64_t)f.res_off + J) * a.R + a.col + r] = arena[((uint64_t)f.root_off + ad) * RG + r];
     }
-    __syncthreads();
+    barrier();
+    if (MODE == kBatchSolo && a.limbs)
+      for (uint32_t J = tid; J < f.n_out; J += nthreads)
+        crt_entry(a.results + (uint64_t)J * a.R, cc, a.limbs + (uint64_t)J * cc.n_limbs);
   }
 }
 
