@@ -431,6 +431,307 @@ int fill_count(tnc_count* out, uint64_t n_out, const Arith& a, const uint32_t* r
   return TNC_OK;
 }
 
+// ---------------------------------------------------- packed descriptors
+
+using tnc_dev::BForm;
+using tnc_dev::BLeaf;
+using tnc_dev::BStep;
+using tnc_dev::Seg;
+
+// Launch configuration of clusters of `ctas` CTAs.
+struct ClusterLaunch {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at[1];
+  ClusterLaunch(unsigned grid, unsigned threads, size_t smem, cudaStream_t st, unsigned ctas) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ctas;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+  }
+  ClusterLaunch(const ClusterLaunch&) = delete;
+};
+
+uint16_t pack_run(int src, int dst, int len) { return (uint16_t)(src | (dst << 5) | (len << 10)); }
+
+// Appends `bytes` at a 16-byte boundary of the blob; returns the offset.
+size_t blob_put(std::vector<char>& blob, const void* src, size_t bytes) {
+  const size_t at = (blob.size() + 15) / 16 * 16;
+  blob.resize(at + bytes);
+  if (bytes) std::memcpy(blob.data() + at, src, bytes);
+  return at;
+}
+
+// One formula's descriptor blob (the sections that batch_kernel copies to
+// shared memory) and the fields of its BForm that do not depend on the batch,
+// for `threads` threads sharing the formula.
+int pack_form(const tnc_plan_t* p, uint32_t threads, std::vector<char>& blob, BForm& f) {
+  if (p->tree.nodes.empty()) return set_error(TNC_ERR_INVALID, "batch formula with an empty network");
+  if (p->cost.max_rank > 24 || !p->low.lvl_fits)
+    return set_error(TNC_ERR_TOO_LARGE, "batch formulas must have plan rank <= 24");
+  const Lowered& lw = p->low;
+  if (lw.lvl_arena_entries >= (1ull << 32)) return set_error(TNC_ERR_TOO_LARGE, "formula arena above 2^32 entries");
+  if (lw.lvl_steps.size() >= 65535) return set_error(TNC_ERR_TOO_LARGE, "more than 65534 steps in one formula");
+  std::memset(&f, 0, sizeof(f));
+  blob.clear();
+  // per level: the share of one of the formula's `threads` lanes (at least
+  // 16 products), and per step the lane split sh of its long shared sums: an
+  // entry of a step is split over 2^sh lanes so that no lane sums much more
+  // than that share
+  const uint32_t nlev = lw.lvl_start.empty() ? 0 : (uint32_t)lw.lvl_start.size() - 1;
+  std::vector<uint32_t> lvl_log_t(nlev, 4), step_sh(lw.lvl_steps.size(), 0);
+  for (uint32_t l = 0; l < nlev; l++) {
+    uint64_t work = 0;
+    for (uint32_t si = lw.lvl_start[l]; si < lw.lvl_start[l + 1]; si++)
+      work += 1ull << (lw.lvl_steps[si].c + lw.lvl_steps[si].k);
+    uint32_t log_t = 4;
+    while (log_t < 24 && (1ull << log_t) * threads < work) log_t++;
+    lvl_log_t[l] = log_t;
+    for (uint32_t si = lw.lvl_start[l]; si < lw.lvl_start[l + 1]; si++) {
+      const StepDesc& d = lw.lvl_steps[si];
+      uint32_t sh = 0;
+      while (sh < 5 && sh < d.k && d.k - sh > log_t) sh++;
+      step_sh[si] = sh;
+    }
+  }
+  // steps, runs and address deltas.  A lane group of a whole-warp block
+  // advances its entry by 2^g (g = 5 - sh): delta[t - g] = w[t] -
+  // sum_{g <= j < t} w[j] for the operand weights w[j] of output bit j.
+  std::vector<BStep> steps;
+  std::vector<uint16_t> runs;
+  std::vector<int32_t> dls;  // pairs (A, B)
+  for (size_t si = 0; si < lw.lvl_steps.size(); si++) {
+    const StepDesc& d = lw.lvl_steps[si];
+    BStep bs;
+    std::memset(&bs, 0, sizeof(bs));
+    bs.a_off = (uint32_t)d.a_off;
+    bs.b_off = (uint32_t)d.b_off;
+    bs.c_off = (uint32_t)d.c_off;
+    bs.c = d.c;
+    bs.k = d.k;
+    bs.ka = d.ka;
+    bs.kb = d.kb;
+    if (runs.size() >= 65535 || dls.size() / 2 >= 65535)
+      return set_error(TNC_ERR_TOO_LARGE, "formula descriptors beyond 2^16 runs or deltas");
+    bs.run0 = (uint16_t)runs.size();
+    int64_t wA[32] = {0}, wB[32] = {0};
+    if (d.nra != TNC_BITMAP) {
+      for (int r = 0; r < d.nra; r++) {
+        const TncRun& x = d.map.runs.ra[r];
+        runs.push_back(pack_run(x.src, x.dst, x.len));
+        for (int q = 0; q < x.len; q++) wA[x.src + q] = 1ll << (x.dst + q);
+      }
+      for (int r = 0; r < d.nrb; r++) {
+        const TncRun& x = d.map.runs.rb[r];
+        runs.push_back(pack_run(x.src, x.dst, x.len));
+        for (int q = 0; q < x.len; q++) wB[x.src + q] = 1ll << (x.dst + q);
+      }
+      bs.nra = d.nra;
+      bs.nrb = d.nrb;
+    } else {
+      for (int side = 0; side < 2; side++)
+        for (int j = 0; j < d.c; j++)
+          if ((d.map.bit[j] >> 7) == side) {
+            runs.push_back(pack_run(j, d.map.bit[j] & 63, 1));
+            (side ? bs.nrb : bs.nra)++;
+            (side ? wB : wA)[j] = 1ll << (d.map.bit[j] & 63);
+          }
+    }
+    const uint32_t g = 5 - step_sh[si];
+    bs.g = (uint8_t)g;
+    bs.dl0 = (uint16_t)(dls.size() / 2);
+    for (uint32_t t = g; t < d.c; t++) {
+      int64_t sa = 0, sb = 0;
+      for (uint32_t j = g; j < t; j++) {
+        sa += wA[j];
+        sb += wB[j];
+      }
+      dls.push_back((int32_t)(wA[t] - sa));
+      dls.push_back((int32_t)(wB[t] - sb));
+    }
+    steps.push_back(bs);
+  }
+  // segments per level: steps whose entries take 32+ lanes get whole-warp
+  // blocks of V entries per lane group (V such that a lane's work is about
+  // half the level's share, at most 4); the others share packed segments
+  // lane by lane.  Segments are ordered by cost, longest first.
+  std::vector<Seg> segs;
+  std::vector<uint32_t> items, lvl{0};
+  for (uint32_t l = 0; l < nlev; l++) {
+    const uint32_t log_t = lvl_log_t[l];
+    struct Group {
+      uint32_t si, o, sh, cost;
+    };
+    std::vector<Group> small;
+    std::vector<std::pair<uint32_t, Seg>> lsegs;  // (cost, segment)
+    for (uint32_t si = lw.lvl_start[l]; si < lw.lvl_start[l + 1]; si++) {
+      const StepDesc& d = lw.lvl_steps[si];
+      const uint32_t sh = step_sh[si];
+      const uint32_t cost = 1u << (d.k - sh);
+      const uint32_t nout = 1u << d.c;
+      if ((nout << sh) < 32) {
+        for (uint32_t o = 0; o < nout; o++) small.push_back(Group{si, o, sh, cost});
+        continue;
+      }
+      const uint32_t G = 32u >> sh;
+      uint32_t V = 1;
+      while (V < 4 && 2 * V * G <= nout && (2 * V) * cost <= (1u << (log_t - 1))) V *= 2;
+      for (uint32_t o0 = 0; o0 < nout; o0 += G * V)
+        lsegs.push_back({cost * V, Seg{o0, (uint16_t)si, (uint8_t)V, (uint8_t)sh}});
+    }
+    // widest groups first: each group then starts at a multiple of its size
+    // and never crosses a 32-lane boundary
+    std::stable_sort(small.begin(), small.end(), [](const Group& x, const Group& y) {
+      return x.sh != y.sh ? x.sh > y.sh : x.cost > y.cost;
+    });
+    for (size_t g = 0; g < small.size();) {
+      const uint32_t first = (uint32_t)items.size();
+      uint32_t lanes = 0, cost = 0;
+      const uint8_t sh0 = (uint8_t)small[g].sh;
+      while (g < small.size() && lanes + (1u << small[g].sh) <= 32) {
+        const Group& q = small[g];
+        for (uint32_t j = 0; j < (1u << q.sh); j++) items.push_back(q.si | q.o << 16 | j << 21 | q.sh << 26);
+        lanes += 1u << q.sh;
+        cost = std::max(cost, q.cost);
+        g++;
+      }
+      lsegs.push_back({cost, Seg{first, tnc_dev::kPacked, (uint8_t)lanes, sh0}});
+    }
+    std::stable_sort(lsegs.begin(), lsegs.end(),
+                     [](const std::pair<uint32_t, Seg>& x, const std::pair<uint32_t, Seg>& y) {
+                       return x.first > y.first;
+                     });
+    for (const auto& x : lsegs) segs.push_back(x.second);
+    lvl.push_back((uint32_t)segs.size());
+  }
+  // the blob
+  blob_put(blob, steps.data(), steps.size() * sizeof(BStep));
+  f.segs_at = (uint32_t)blob_put(blob, segs.data(), segs.size() * sizeof(Seg));
+  f.items_at = (uint32_t)blob_put(blob, items.data(), items.size() * sizeof(uint32_t));
+  f.runs_at = (uint32_t)blob_put(blob, runs.data(), runs.size() * sizeof(uint16_t));
+  f.dl_at = (uint32_t)blob_put(blob, dls.data(), dls.size() * sizeof(int32_t));
+  f.lvl_at = (uint32_t)blob_put(blob, lvl.data(), lvl.size() * sizeof(uint32_t));
+  blob.resize((blob.size() + 15) / 16 * 16);
+  f.blob_n = (uint32_t)(blob.size() / 16);
+  f.nlev = nlev;
+  f.nleaf = (uint32_t)lw.leaves.size();
+  f.n_open = (uint32_t)p->net.open_vars.size();
+  f.n_out = 1u << f.n_open;
+  f.root_off = (uint32_t)(lw.lvl_steps.empty() ? lw.lvl_leaf_off[p->tree.root] : lw.lvl_root_off);
+  f.arena = (uint32_t)lw.lvl_arena_entries;
+  return TNC_OK;
+}
+
+// The leaves of a formula, their weight tables starting at table0.
+void pack_leaves(const Lowered& lw, uint32_t table0, std::vector<BLeaf>& leaves) {
+  for (size_t l = 0; l < lw.leaves.size(); l++) {
+    BLeaf bl;
+    std::memset(&bl, 0, sizeof(bl));
+    bl.off = (uint32_t)lw.lvl_leaf_off[l];
+    bl.table_off = lw.leaves[l].table_off + table0;
+    bl.kind = lw.leaves[l].kind;
+    bl.rank = lw.leaves[l].rank;
+    leaves.push_back(bl);
+  }
+}
+
+// ---------------------------------------------------------------- one launch
+//
+// A small formula on TNC_PATH_INT64 runs as one launch per residue group: one
+// cluster contracts it level by level (batch_kernel's heavy-formula form, leaf
+// fill and result extraction included) and the last group's launch also runs
+// the CRT; descriptors go up in one copy, results come down in one.  The
+// launches of contract_group take 3 to 6 us per tree level whatever the
+// level's work, and its copies of pageable memory about 10 us each.
+// Up to kSoloMax multiply-adds and entries per residue (contract_group behind
+// its launches uses all SMs; same box, both ways, 4 residues: 2^12.6 205 ->
+// 134 us, 2^15.8 244 -> 135, 2^19.7 256 -> 158, 2^21.9 254 -> 262, 2^24.4
+// 328 -> 522), on clusters of 16 CTAs from kSoloWide on (2^19.7: 158 us
+// against 180 on 8; 2^15: no difference).
+constexpr double kSoloMax = 4e6, kSoloWide = 3e4;
+
+}  // namespace
+
+namespace tnc {
+struct SoloPack {
+  bool ok = false;
+  uint32_t ctas = 1;
+  std::vector<char> bytes;  // forms, blob, leaves, tables, perms, order: copied to the workspace as they are
+  size_t off_blob = 0, off_leaves = 0, off_tables = 0, off_perms = 0, off_order = 0;
+  size_t blob_bytes = 0;
+};
+}  // namespace tnc
+
+namespace {
+
+void make_solo(const tnc_plan_t* p, SoloPack& s) {
+  const double cost = p->cost.macs + p->cost.entries;
+  if (p->tree.nodes.empty() || cost > kSoloMax || p->cost.max_rank > 24 || !p->low.lvl_fits) return;
+  s.ctas = cost < kSoloWide ? 8 : 16;
+  std::vector<char> blob;
+  BForm f;
+  if (pack_form(p, 256 * s.ctas, blob, f) != TNC_OK) {  // (descriptor limits: the general path takes it)
+    clear_error();
+    return;
+  }
+  std::vector<BLeaf> leaves;
+  pack_leaves(p->low, 0, leaves);
+  const uint32_t first = 0;
+  s.blob_bytes = blob.size();
+  blob_put(s.bytes, &f, sizeof(f));
+  s.off_blob = blob_put(s.bytes, blob.data(), blob.size());
+  s.off_leaves = blob_put(s.bytes, leaves.data(), leaves.size() * sizeof(BLeaf));
+  s.off_tables = blob_put(s.bytes, p->low.leaf_tables.data(), p->low.leaf_tables.size() * sizeof(uint32_t));
+  s.off_perms = blob_put(s.bytes, p->low.root_perm.data(), p->low.root_perm.size());
+  s.off_order = blob_put(s.bytes, &first, sizeof(first));
+  s.ok = blob.size() <= 160 * 1024;
+}
+
+// Enqueues the one-launch contraction (descriptors up, a launch per residue
+// group); results and limbs are left in their workspace sections.
+int solo_enqueue(const SoloPack& s, const SeqLayout& L, const Arith& a, char* ws, cudaStream_t st) {
+  CUDA_TRY(cudaMemcpyAsync(ws, s.bytes.data(), s.bytes.size(), cudaMemcpyHostToDevice, st));
+  g_h2d_bytes += s.bytes.size();
+  for (size_t gi = 0; gi < a.groups.rg.size(); gi++) {
+    tnc_dev::BatchArgs args{};
+    args.forms = (const BForm*)ws;
+    args.blobs = (const uint4*)(ws + s.off_blob);
+    args.leaves = (const BLeaf*)(ws + s.off_leaves);
+    args.tables = (const uint32_t*)(ws + s.off_tables);
+    args.perms = (const uint8_t*)(ws + s.off_perms);
+    args.order = (const uint32_t*)(ws + s.off_order);
+    args.n_forms = args.n_heavy = args.cluster_slots = 1;
+    args.results = (uint32_t*)(ws + L.off_results);
+    args.garena = (uint32_t*)(ws + L.off_arena);
+    args.blob_cap = (uint32_t)s.blob_bytes;
+    args.R = a.R;
+    args.col = a.groups.col[gi];
+    args.limbs = gi + 1 == a.groups.rg.size() ? (uint32_t*)(ws + L.off_limbs) : nullptr;
+    const ModGroup mg = a.group((int)gi);
+    int rc = dispatch_rg(a.groups.rg[gi], [&](auto rgc) -> int {
+      constexpr int RG = decltype(rgc)::value;
+      auto k = mg.near30 ? tnc_dev::batch_kernel<RG, true, tnc_dev::kBatchSolo>
+                         : tnc_dev::batch_kernel<RG, false, tnc_dev::kBatchSolo>;
+      if (s.blob_bytes > 48 * 1024 - 64)
+        CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
+      if (s.ctas > 8) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      const ClusterLaunch cl(s.ctas, 256, s.blob_bytes, st, s.ctas);
+      CUDA_TRY(cudaLaunchKernelEx(&cl.cfg, k, args, mg, a.crt));
+      return TNC_OK;
+    });
+    if (rc) return rc;
+    g_launches.leaf_fill++;
+    g_launches.level++;
+    g_launches.extract++;
+  }
+  g_launches.crt++;
+  return TNC_OK;
+}
+
 }  // namespace
 
 extern "C" size_t tnc_workspace_bytes(const tnc_plan_t* plan, int32_t n_residues) {
@@ -536,6 +837,25 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
   if (((uintptr_t)dev_ws) % kAlign) return set_error(TNC_ERR_INVALID, "workspace must be 256-byte aligned");
   if (inject_hit(TNC_INJECT_LAUNCH)) return set_error(TNC_ERR_CUDA, "injected failure (TNC_INJECT_LAUNCH)");
   char* ws = (char*)dev_ws;
+  if (nw == 1 && !sum_into && opts->path == TNC_PATH_INT64 && !g_time_dense) {
+    std::call_once(work[0]->solo_once, [&] {
+      auto s = std::make_shared<SoloPack>();
+      make_solo(work[0], *s);
+      work[0]->solo = std::move(s);
+    });
+    const SoloPack& s = *work[0]->solo;
+    if (s.ok && s.bytes.size() <= L.off_results) {  // (the descriptor sections and scratch before the results)
+      rc = solo_enqueue(s, L, a, ws, st);
+      if (rc) return rc;
+      std::vector<uint32_t> h((L.off_limbs - L.off_results) / 4 + L.n_out * a.crt.n_limbs);
+      CUDA_TRY(cudaMemcpyAsync(h.data(), ws + L.off_results, h.size() * 4, cudaMemcpyDeviceToHost, st));
+      g_d2h_bytes += h.size() * 4;
+      CUDA_TRY(cudaStreamSynchronize(st));
+      if (inject_hit(TNC_INJECT_TIMEOUT)) return set_error(TNC_ERR_TIMEOUT, "a tensor-core step timed out waiting for its MMAs");
+      return fill_count(&outs[work_idx[0]], L.n_out, a, h.data(), h.data() + (L.off_limbs - L.off_results) / 4,
+                        result_flags(work[0], a));
+    }
+  }
   // Every plan runs level by level (the tree-level schedule of the lowering);
   // offsets are shifted to the plan's part of the group's arena, tables and
   // results.
@@ -944,11 +1264,6 @@ extern "C" int tnc_contract_many(const tnc_plan_t* const* plans, int32_t n, cons
 
 // ======================================================================= batch
 
-using tnc_dev::BForm;
-using tnc_dev::BLeaf;
-using tnc_dev::BStep;
-using tnc_dev::Seg;
-
 struct tnc_batch_s {
   std::vector<const tnc_plan_t*> plans;
   Arith a;
@@ -997,24 +1312,6 @@ constexpr size_t kSmemMax = 227 * 1024;
 // kHeavyTop: 28-41 us without, 40-48 us with.
 constexpr uint32_t kClusterCtas = 8;
 constexpr double kHeavyShare = 1.2, kHeavyMin = 16384.0, kHeavyTop = 131072.0;
-
-// Launch configuration of clusters of `ctas` CTAs.
-struct ClusterLaunch {
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute at[1];
-  ClusterLaunch(unsigned grid, unsigned threads, size_t smem, cudaStream_t st, unsigned ctas) {
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = ctas;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-  }
-  ClusterLaunch(const ClusterLaunch&) = delete;
-};
 
 // CTAs of batch_kernel<RG, N30, MODE> per SM for (threads, dynamic shared memory),
 // capped at `cap` (0: no cap).  The L1 / shared-memory split is then set to
@@ -1097,189 +1394,6 @@ int batch_configure(tnc_batch_t* b, int threads, size_t smem, int cap) {
     b->gexec = nullptr;
   }
   return TNC_OK;
-}
-
-uint16_t pack_run(int src, int dst, int len) { return (uint16_t)(src | (dst << 5) | (len << 10)); }
-
-// Appends `bytes` at a 16-byte boundary of the blob; returns the offset.
-size_t blob_put(std::vector<char>& blob, const void* src, size_t bytes) {
-  const size_t at = (blob.size() + 15) / 16 * 16;
-  blob.resize(at + bytes);
-  if (bytes) std::memcpy(blob.data() + at, src, bytes);
-  return at;
-}
-
-// One formula's descriptor blob (the sections that batch_kernel copies to
-// shared memory) and the fields of its BForm that do not depend on the batch,
-// for `threads` threads sharing the formula.
-int pack_form(const tnc_plan_t* p, uint32_t threads, std::vector<char>& blob, BForm& f) {
-  if (p->tree.nodes.empty()) return set_error(TNC_ERR_INVALID, "batch formula with an empty network");
-  if (p->cost.max_rank > 24 || !p->low.lvl_fits)
-    return set_error(TNC_ERR_TOO_LARGE, "batch formulas must have plan rank <= 24");
-  const Lowered& lw = p->low;
-  if (lw.lvl_arena_entries >= (1ull << 32)) return set_error(TNC_ERR_TOO_LARGE, "formula arena above 2^32 entries");
-  if (lw.lvl_steps.size() >= 65535) return set_error(TNC_ERR_TOO_LARGE, "more than 65534 steps in one formula");
-  std::memset(&f, 0, sizeof(f));
-  blob.clear();
-  // per level: the share of one of the formula's `threads` lanes (at least
-  // 16 products), and per step the lane split sh of its long shared sums: an
-  // entry of a step is split over 2^sh lanes so that no lane sums much more
-  // than that share
-  const uint32_t nlev = lw.lvl_start.empty() ? 0 : (uint32_t)lw.lvl_start.size() - 1;
-  std::vector<uint32_t> lvl_log_t(nlev, 4), step_sh(lw.lvl_steps.size(), 0);
-  for (uint32_t l = 0; l < nlev; l++) {
-    uint64_t work = 0;
-    for (uint32_t si = lw.lvl_start[l]; si < lw.lvl_start[l + 1]; si++)
-      work += 1ull << (lw.lvl_steps[si].c + lw.lvl_steps[si].k);
-    uint32_t log_t = 4;
-    while (log_t < 24 && (1ull << log_t) * threads < work) log_t++;
-    lvl_log_t[l] = log_t;
-    for (uint32_t si = lw.lvl_start[l]; si < lw.lvl_start[l + 1]; si++) {
-      const StepDesc& d = lw.lvl_steps[si];
-      uint32_t sh = 0;
-      while (sh < 5 && sh < d.k && d.k - sh > log_t) sh++;
-      step_sh[si] = sh;
-    }
-  }
-  // steps, runs and address deltas.  A lane group of a whole-warp block
-  // advances its entry by 2^g (g = 5 - sh): delta[t - g] = w[t] -
-  // sum_{g <= j < t} w[j] for the operand weights w[j] of output bit j.
-  std::vector<BStep> steps;
-  std::vector<uint16_t> runs;
-  std::vector<int32_t> dls;  // pairs (A, B)
-  for (size_t si = 0; si < lw.lvl_steps.size(); si++) {
-    const StepDesc& d = lw.lvl_steps[si];
-    BStep bs;
-    std::memset(&bs, 0, sizeof(bs));
-    bs.a_off = (uint32_t)d.a_off;
-    bs.b_off = (uint32_t)d.b_off;
-    bs.c_off = (uint32_t)d.c_off;
-    bs.c = d.c;
-    bs.k = d.k;
-    bs.ka = d.ka;
-    bs.kb = d.kb;
-    if (runs.size() >= 65535 || dls.size() / 2 >= 65535)
-      return set_error(TNC_ERR_TOO_LARGE, "formula descriptors beyond 2^16 runs or deltas");
-    bs.run0 = (uint16_t)runs.size();
-    int64_t wA[32] = {0}, wB[32] = {0};
-    if (d.nra != TNC_BITMAP) {
-      for (int r = 0; r < d.nra; r++) {
-        const TncRun& x = d.map.runs.ra[r];
-        runs.push_back(pack_run(x.src, x.dst, x.len));
-        for (int q = 0; q < x.len; q++) wA[x.src + q] = 1ll << (x.dst + q);
-      }
-      for (int r = 0; r < d.nrb; r++) {
-        const TncRun& x = d.map.runs.rb[r];
-        runs.push_back(pack_run(x.src, x.dst, x.len));
-        for (int q = 0; q < x.len; q++) wB[x.src + q] = 1ll << (x.dst + q);
-      }
-      bs.nra = d.nra;
-      bs.nrb = d.nrb;
-    } else {
-      for (int side = 0; side < 2; side++)
-        for (int j = 0; j < d.c; j++)
-          if ((d.map.bit[j] >> 7) == side) {
-            runs.push_back(pack_run(j, d.map.bit[j] & 63, 1));
-            (side ? bs.nrb : bs.nra)++;
-            (side ? wB : wA)[j] = 1ll << (d.map.bit[j] & 63);
-          }
-    }
-    const uint32_t g = 5 - step_sh[si];
-    bs.g = (uint8_t)g;
-    bs.dl0 = (uint16_t)(dls.size() / 2);
-    for (uint32_t t = g; t < d.c; t++) {
-      int64_t sa = 0, sb = 0;
-      for (uint32_t j = g; j < t; j++) {
-        sa += wA[j];
-        sb += wB[j];
-      }
-      dls.push_back((int32_t)(wA[t] - sa));
-      dls.push_back((int32_t)(wB[t] - sb));
-    }
-    steps.push_back(bs);
-  }
-  // segments per level: steps whose entries take 32+ lanes get whole-warp
-  // blocks of V entries per lane group (V such that a lane's work is about
-  // half the level's share, at most 4); the others share packed segments
-  // lane by lane.  Segments are ordered by cost, longest first.
-  std::vector<Seg> segs;
-  std::vector<uint32_t> items, lvl{0};
-  for (uint32_t l = 0; l < nlev; l++) {
-    const uint32_t log_t = lvl_log_t[l];
-    struct Group {
-      uint32_t si, o, sh, cost;
-    };
-    std::vector<Group> small;
-    std::vector<std::pair<uint32_t, Seg>> lsegs;  // (cost, segment)
-    for (uint32_t si = lw.lvl_start[l]; si < lw.lvl_start[l + 1]; si++) {
-      const StepDesc& d = lw.lvl_steps[si];
-      const uint32_t sh = step_sh[si];
-      const uint32_t cost = 1u << (d.k - sh);
-      const uint32_t nout = 1u << d.c;
-      if ((nout << sh) < 32) {
-        for (uint32_t o = 0; o < nout; o++) small.push_back(Group{si, o, sh, cost});
-        continue;
-      }
-      const uint32_t G = 32u >> sh;
-      uint32_t V = 1;
-      while (V < 4 && 2 * V * G <= nout && (2 * V) * cost <= (1u << (log_t - 1))) V *= 2;
-      for (uint32_t o0 = 0; o0 < nout; o0 += G * V)
-        lsegs.push_back({cost * V, Seg{o0, (uint16_t)si, (uint8_t)V, (uint8_t)sh}});
-    }
-    // widest groups first: each group then starts at a multiple of its size
-    // and never crosses a 32-lane boundary
-    std::stable_sort(small.begin(), small.end(), [](const Group& x, const Group& y) {
-      return x.sh != y.sh ? x.sh > y.sh : x.cost > y.cost;
-    });
-    for (size_t g = 0; g < small.size();) {
-      const uint32_t first = (uint32_t)items.size();
-      uint32_t lanes = 0, cost = 0;
-      const uint8_t sh0 = (uint8_t)small[g].sh;
-      while (g < small.size() && lanes + (1u << small[g].sh) <= 32) {
-        const Group& q = small[g];
-        for (uint32_t j = 0; j < (1u << q.sh); j++) items.push_back(q.si | q.o << 16 | j << 21 | q.sh << 26);
-        lanes += 1u << q.sh;
-        cost = std::max(cost, q.cost);
-        g++;
-      }
-      lsegs.push_back({cost, Seg{first, tnc_dev::kPacked, (uint8_t)lanes, sh0}});
-    }
-    std::stable_sort(lsegs.begin(), lsegs.end(),
-                     [](const std::pair<uint32_t, Seg>& x, const std::pair<uint32_t, Seg>& y) {
-                       return x.first > y.first;
-                     });
-    for (const auto& x : lsegs) segs.push_back(x.second);
-    lvl.push_back((uint32_t)segs.size());
-  }
-  // the blob
-  blob_put(blob, steps.data(), steps.size() * sizeof(BStep));
-  f.segs_at = (uint32_t)blob_put(blob, segs.data(), segs.size() * sizeof(Seg));
-  f.items_at = (uint32_t)blob_put(blob, items.data(), items.size() * sizeof(uint32_t));
-  f.runs_at = (uint32_t)blob_put(blob, runs.data(), runs.size() * sizeof(uint16_t));
-  f.dl_at = (uint32_t)blob_put(blob, dls.data(), dls.size() * sizeof(int32_t));
-  f.lvl_at = (uint32_t)blob_put(blob, lvl.data(), lvl.size() * sizeof(uint32_t));
-  blob.resize((blob.size() + 15) / 16 * 16);
-  f.blob_n = (uint32_t)(blob.size() / 16);
-  f.nlev = nlev;
-  f.nleaf = (uint32_t)lw.leaves.size();
-  f.n_open = (uint32_t)p->net.open_vars.size();
-  f.n_out = 1u << f.n_open;
-  f.root_off = (uint32_t)(lw.lvl_steps.empty() ? lw.lvl_leaf_off[p->tree.root] : lw.lvl_root_off);
-  f.arena = (uint32_t)lw.lvl_arena_entries;
-  return TNC_OK;
-}
-
-// The leaves of a formula, their weight tables starting at table0.
-void pack_leaves(const Lowered& lw, uint32_t table0, std::vector<BLeaf>& leaves) {
-  for (size_t l = 0; l < lw.leaves.size(); l++) {
-    BLeaf bl;
-    std::memset(&bl, 0, sizeof(bl));
-    bl.off = (uint32_t)lw.lvl_leaf_off[l];
-    bl.table_off = lw.leaves[l].table_off + table0;
-    bl.kind = lw.leaves[l].kind;
-    bl.rank = lw.leaves[l].rank;
-    leaves.push_back(bl);
-  }
 }
 
 int batch_pack(tnc_batch_t* b) {

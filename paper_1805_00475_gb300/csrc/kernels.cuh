@@ -731,7 +731,7 @@ __device__ __forceinline__ uint32_t map_runs(uint32_t o, const uint16_t* runs, i
 // the queue as above.
 enum BatchMode { kBatchCtas, kBatchClusters, kBatchSolo };  // kBatchSolo: one formula, one cluster, and its CRT
 template <int RG, bool N30 = false, int MODE = kBatchCtas>
-__global__ void __launch_bounds__(256, MODE == kBatchCtas ? 0 : (RG == 4 && !N30 ? 3 : 4))
+__global__ void __launch_bounds__(256, MODE == kBatchCtas ? 0 : (MODE == kBatchSolo ? 1 : (RG == 4 && !N30 ? 3 : 4)))
     batch_kernel(BatchArgs a, ModGroup mg, const __grid_constant__ CrtConsts cc) {
   constexpr bool CLUSTER = MODE != kBatchCtas;
   extern __shared__ uint4 smem_raw[];

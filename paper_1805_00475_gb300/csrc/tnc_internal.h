@@ -2,6 +2,8 @@
 #pragma once
 
 #include <cstdint>
+#include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -95,12 +97,19 @@ struct tnc_network_s {
   tnc::Network net;
 };
 
+namespace tnc {
+struct SoloPack;  // contract.cu
+}
+
 struct tnc_plan_s {
   tnc::Network net;  // own copy: a plan outlives its network handle
   tnc::Tree tree;
   tnc::TreeCost cost;
   tnc::Lowered low;
   tnc_plan_stats stats{};
+  // descriptors of the one-launch contraction, packed by the first call that uses them
+  mutable std::once_flag solo_once;
+  mutable std::shared_ptr<const tnc::SoloPack> solo;
 };
 
 namespace tnc {

@@ -51,3 +51,30 @@ def test_batch_with_heavy_formulas(sizes, R, wide):
         got = b.download(ws)
         for n, r in zip(sizes, got):
             assert r.residues.tolist() == want[n].residues.tolist() and r.counts == want[n].counts, (n, shape)
+
+
+def _solo_forms():
+    open_vc = I.cubic_vertex_cover(30, 3)
+    open_vc.open_vars = [7, 0, 12, 29, 4]
+    return {"one_variable": I.Formula(1, [], []), "worked_example": I.worked_example(),
+            "1in3_n20": I.one_in_three(20, 12, 3), "open_vc_n30": open_vc, "vc_n44": I.cubic_vertex_cover(44, 0),
+            "vc_n60": I.cubic_vertex_cover(60, 0), "vc_n90": I.cubic_vertex_cover(90, 1)}
+
+
+@pytest.mark.parametrize("R,wide", [(1, False), (2, True), (3, False), (4, False), (5, True), (16, False)])
+@pytest.mark.parametrize("name", list(_solo_forms()))
+def test_one_launch_contraction(name, R, wide):
+    """Small formulas run in one launch per residue group; the allocation-free
+    entry point runs the same plan step by step."""
+    f = _solo_forms()[name]
+    p = tnc.plan_formula(f, heuristic="best")
+    primes = WIDE[:R] if wide else None
+    want = tnc.contract_noalloc(p, n_residues=R, primes=primes)
+    for _ in range(2):
+        r = tnc.contract(p, n_residues=R, primes=primes)
+        lc = tnc.last_launch_counts()
+        groups = bin(R % 4).count("1") + R // 4
+        assert lc["level"] == groups and lc["crt"] == 1 and lc["grid_step"] == lc["splitk"] == lc["outer"] == 0
+        assert r.residues.tolist() == want.residues.tolist() and r.counts == want.counts and r.flags == want.flags
+    if f.n_vars <= 60:
+        assert r.residues.tolist() == oracle.residues(oracle.count(f), r.primes)
