@@ -116,7 +116,8 @@ int make_arith(const tnc_contract_opts* o, Arith& a) {
   if (o->n_residues < 1 || o->n_residues > max_r)
     return set_error(TNC_ERR_INVALID, p8 ? "n_residues must be in [1, 53]" : "n_residues must be in [1, 16]");
   a.R = o->n_residues;
-  if (o->primes) {
+  a.primes = p8 ? default_primes_p8(a.R) : default_primes(a.R);
+  if (o->primes && !std::equal(a.primes.begin(), a.primes.end(), o->primes)) {  // (the default ones need no test)
     a.primes.assign(o->primes, o->primes + a.R);
     for (int i = 0; i < a.R; i++) {
       uint32_t p = a.primes[i];
@@ -126,8 +127,6 @@ int make_arith(const tnc_contract_opts* o, Arith& a) {
       for (int j = 0; j < i; j++)
         if (a.primes[j] == p) return set_error(TNC_ERR_INVALID, "primes must be distinct");
     }
-  } else {
-    a.primes = p8 ? default_primes_p8(a.R) : default_primes(a.R);
   }
   a.crt = CrtConsts{};
   a.crt.R = a.R;

@@ -19,9 +19,8 @@ const char* last_error_cstr() { return g_err.c_str(); }
 
 // ---------------------------------------------------------------- primes
 
-static uint64_t mulmod64(uint64_t a, uint64_t b, uint64_t m) {
-  return (uint64_t)((unsigned __int128)a * b % m);
-}
+// (operands below m < 2^32: the product fits 64 bits)
+static uint64_t mulmod64(uint64_t a, uint64_t b, uint64_t m) { return a * b % m; }
 static uint64_t powmod64(uint64_t a, uint64_t e, uint64_t m) {
   uint64_t r = 1 % m;
   a %= m;
@@ -63,18 +62,24 @@ bool is_prime_u32(uint32_t n) {
   return true;
 }
 
-std::vector<uint32_t> default_primes(int n) {
+// The n largest primes up to the odd number `from`.
+static std::vector<uint32_t> primes_down(uint32_t from, int n) {
   std::vector<uint32_t> out;
-  for (uint32_t x = kDefaultPrimeBound - 1; (int)out.size() < n && x > 2; x -= 2)
+  for (uint32_t x = from; (int)out.size() < n && x > 2; x -= 2)
     if (is_prime_u32(x)) out.push_back(x);
   return out;
 }
 
+// The default primes are constants, found once (16 of them took 40 us, on
+// every call that named no primes); n beyond the tables gets what there is.
+std::vector<uint32_t> default_primes(int n) {
+  static const std::vector<uint32_t> all = primes_down(kDefaultPrimeBound - 1, 64);
+  return std::vector<uint32_t>(all.begin(), all.begin() + std::min<size_t>(all.size(), (size_t)std::max(n, 0)));
+}
+
 std::vector<uint32_t> default_primes_p8(int n) {
-  std::vector<uint32_t> out;
-  for (uint32_t x = kP8PrimeMax; (int)out.size() < n && x > 2; x -= 2)
-    if (is_prime_u32(x)) out.push_back(x);
-  return out;
+  static const std::vector<uint32_t> all = primes_down(kP8PrimeMax, kP8MaxResidues);
+  return std::vector<uint32_t>(all.begin(), all.begin() + std::min<size_t>(all.size(), (size_t)std::max(n, 0)));
 }
 
 // ---------------------------------------------------------------- network

@@ -477,7 +477,10 @@ def _workspace(nbytes: int, ws=None):
 
 def workspace_bytes(p: Plan, n_residues: int, path: str = "int64", primes=None) -> int:
     """tnc_workspace_bytes_opts for the path (tnc_workspace_bytes on int64 / tc)."""
-    o, _ = _opts(n_residues, primes, path)
+    return _plan_bytes(p, _opts(n_residues, primes, path)[0])
+
+
+def _plan_bytes(p: Plan, o: _ContractOpts) -> int:
     nb = int(lib().tnc_workspace_bytes_opts(p.h, ctypes.byref(o)))
     if nb == 0:
         raise TncError(-1, lib().tnc_last_error().decode() or "invalid contract options")
@@ -487,7 +490,7 @@ def workspace_bytes(p: Plan, n_residues: int, path: str = "int64", primes=None) 
 def contract(p: Plan, n_residues: int = 4, primes=None, workspace=None, stream=None, path: str = "int64") -> Count:
     """Contract one plan on the GPU (tnc_contract); returns exact counts."""
     o, pr = _opts(n_residues, primes, path)
-    nb = workspace_bytes(p, n_residues, path, primes)
+    nb = _plan_bytes(p, o)
     ws = _workspace(nb, workspace)
     c, res, limbs = _count_buffers(1 << p.n_open, n_residues)
     _check(lib().tnc_contract(p.h, ctypes.byref(o), ctypes.c_void_p(ws.data_ptr()), nb, _stream_ptr(stream),
