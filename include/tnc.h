@@ -270,9 +270,9 @@ size_t tnc_workspace_bytes_sliced(const tnc_plan_t* const* plans, int32_t n, con
 int tnc_contract_sliced(const tnc_plan_t* const* plans, int32_t n, const tnc_contract_opts* opts, void* dev_ws,
                         size_t ws_bytes, void* cuda_stream, tnc_count* out);
 /* Many formulas in one call: independent contractions (Sec. 2.1) whose tree
- * levels are merged, so that one launch covers the small steps of level l of
- * every formula of a group, and the group's big, split-K and dense steps
- * follow one another on the stream.  A group is as many consecutive plans as
+ * levels are merged, so that one launch covers the steps of one kind of level l
+ * of every formula of a group (small, big, split-K; on TNC_PATH_TC_P8 dense
+ * ones of one tile width, as many as their scratch holds).  A group is as many consecutive plans as
  * the workspace holds (each plan alone must fit: TNC_ERR_BUFFER otherwise).
  * Any path; outs: n counts, as tnc_contract would give them one by one.
  * tnc_workspace_bytes_many gives the bytes that hold groups of `group`
@@ -308,16 +308,19 @@ int tnc_last_contract_time(double* device_ms);
 /* The device kernels the calling thread's last tnc_contract,
  * tnc_contract_sliced or tnc_contract_noalloc enqueued, by kind: a record of
  * which branches of the pairwise step (Sec. 2.1) actually ran.  Always
- * recorded (host counters, no device work); a sliced call sums its slices. */
+ * recorded (host counters, no device work); a sliced call sums its slices.
+ * A small formula's one launch (TNC_PATH_INT64) counts as a leaf fill, a level,
+ * an extraction and the CRT, and its long shared sums under splitk.  p8_*
+ * counts dense steps: one launch may serve several of a tree level. */
 typedef struct {
   int32_t leaf_fill;      /* leaf tensors (Eq. var, Eq. or, Eq. 1in3, ...)           */
   int32_t level;          /* one launch for all small steps of a tree level           */
-  int32_t grid_step;      /* one large step over the whole GPU                       */
+  int32_t grid_step;      /* large steps of a tree level over the whole GPU          */
   int32_t splitk;         /* split-K steps on CUDA cores (a partial + final pair)    */
   int32_t tc_gemm;        /* TNC_PATH_TC dense steps (tcgen05 limb GEMM launches)     */
   int32_t tc_split;       /*   of which split over K (partials summed after)          */
-  int32_t p8_pack;        /* TNC_PATH_TC_P8 operand packing launches                  */
-  int32_t p8_gemm;        /* TNC_PATH_TC_P8 dense steps (tcgen05 GEMM launches)       */
+  int32_t p8_pack;        /* TNC_PATH_TC_P8 dense steps with operands to pack          */
+  int32_t p8_gemm;        /* TNC_PATH_TC_P8 dense steps (tcgen05 GEMMs)               */
   int32_t p8_split;       /*   of which split over K                                 */
   int32_t p8_tile_n[5];   /*   by tile width: 16, 32, 64, 128, 256 columns            */
   int32_t p8_max_chunks;  /* most 1024-value chunks one tile accumulates in TMEM per

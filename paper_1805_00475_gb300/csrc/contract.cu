@@ -21,13 +21,13 @@
 #include <vector>
 
 #include "kernels.cuh"
+#include "steps.cuh"
 #include "tnc_internal.h"
 
 using namespace tnc;
 using tnc_dev::BatchArgs;
 using tnc_dev::CrtConsts;
 using tnc_dev::ModGroup;
-using tnc_dev::RootMap;
 
 namespace {
 
@@ -176,6 +176,7 @@ struct SeqLayout {
   size_t off_leaves, off_tables, off_steps, off_small, off_tc, off_err, off_part, off_results, off_limbs, off_p8,
       off_arena, total;
   uint64_t n_out;  // result entries of the whole group
+  uint64_t part_bytes, p8_bytes;  // the sections' sizes
   size_t n_dense;
   std::vector<uint64_t> arena_base, res_base, leaf_base, table_base;
 };
@@ -233,7 +234,8 @@ GridStep make_grid_step(const StepDesc& d) {
   }
   int threads, blocks, sh;
   grid_shape(d.c, &threads, &blocks, &sh);
-  g.s = (uint32_t)sh;
+  g.s = (uint16_t)sh;
+  g.log_split = (uint16_t)splitk_log(d);
   for (int t = sh; t < d.c; t++) {
     uint64_t sa = 0, sb = 0;
     for (int j = sh; j < t; j++) {
@@ -263,6 +265,7 @@ tnc_dev::OuterStep make_outer_step(const StepDesc& d) {
   o.s_off = s_side ? d.b_off : d.a_off;
   o.l_off = s_side ? d.a_off : d.b_off;
   o.c_off = d.c_off;
+  o.blocks = (uint32_t)std::min<uint64_t>(((1ull << o.fl) + 255) / 256, (uint64_t)sm_count() * 8);
   int op[64] = {0}, dst[64] = {0};
   if (d.nra != TNC_BITMAP) {
     for (int i = 0; i < d.nra; i++)
@@ -301,6 +304,8 @@ tnc_dev::OuterStep make_outer_step(const StepDesc& d) {
 struct Foot {
   size_t leaves = 0, tables = 0, nseq = 0, nlvl = 0, n_dense = 0;
   uint64_t n_out = 0, arena = 0, part = 0, p8 = 0;
+  // TNC_PATH_TC_P8: planes and partials of all dense steps of a tree level
+  std::vector<uint64_t> lvl_p8, lvl_part;
   void add(const Foot& f) {
     leaves += f.leaves;
     tables += f.tables;
@@ -311,8 +316,27 @@ struct Foot {
     arena += f.arena;
     part = std::max(part, f.part);
     p8 = std::max(p8, f.p8);
+    lvl_p8.resize(std::max(lvl_p8.size(), f.lvl_p8.size()));
+    lvl_part.resize(std::max(lvl_part.size(), f.lvl_part.size()));
+    for (size_t l = 0; l < f.lvl_p8.size(); l++) {
+      lvl_p8[l] += f.lvl_p8[l];
+      lvl_part[l] += f.lvl_part[l];
+    }
   }
 };
+
+// The dense steps of a level are launched together as far as their planes and
+// partials fit; up to these sizes the sections grow beyond the largest single
+// step's for that (steps that need more fill the GPU by themselves).
+constexpr uint64_t kGroupPlanes = 256ull << 20, kGroupParts = 64ull << 20;
+
+// Step i of a plan's level schedule as TNC_PATH_TC_P8 runs it: direct planes
+// of its operands and output.
+uint32_t p8_flags(const Lowered& lw, uint32_t i) {
+  const int sa = lw.lvl_src_a[i], sb = lw.lvl_src_b[i];
+  return (lw.p8_direct[i] ? kP8DirectOut : 0u) | (sa >= 0 && lw.p8_direct[sa] ? kP8DirectA : 0u) |
+         (sb >= 0 && lw.p8_direct[sb] ? kP8DirectB : 0u);
+}
 
 Foot foot_of(const tnc_plan_t* p, int R, int path) {
   const int rg_max = R >= 4 ? 4 : (R >= 2 ? 2 : 1);
@@ -322,19 +346,32 @@ Foot foot_of(const tnc_plan_t* p, int R, int path) {
   f.nseq = p->low.seq_steps.size();
   f.nlvl = p->low.lvl_steps.size();
   f.n_out = 1ull << p->net.open_vars.size();
-  for (const StepDesc& d : p->low.seq_steps) f.n_dense += tc_eligible(d) ? 1 : 0;
-  for (const StepDesc& d : p->low.lvl_steps) {
-    if (splitk_log(d) > 0)
-      f.part = std::max<uint64_t>(f.part, (1ull << (d.c + splitk_log(d))) * rg_max * sizeof(uint32_t));
-    if (tc_eligible(d) && tc_split_log(d) > 0)
-      f.part = std::max<uint64_t>(f.part, (1ull << (d.c + tc_split_log(d))) * sizeof(uint32_t));
-    if (path == TNC_PATH_TC_P8 && p8_eligible(d)) {
-      f.part = std::max<uint64_t>(f.part, p8_part_bytes(d, rg_max));
-      f.p8 = std::max<uint64_t>(f.p8, p8_scratch_bytes(d, rg_max));
+  const bool p8 = path == TNC_PATH_TC_P8;
+  if (!p8)
+    for (const StepDesc& d : p->low.seq_steps) f.n_dense += tc_eligible(d) ? 1 : 0;
+  for (size_t l = 0; l + 1 < p->low.lvl_start.size(); l++) {
+    uint64_t sum_p8 = 0, sum_part = 0;
+    for (uint32_t i = p->low.lvl_start[l]; i < p->low.lvl_start[l + 1]; i++) {
+      const StepDesc& d = p->low.lvl_steps[i];
+      if (splitk_log(d) > 0)
+        f.part = std::max<uint64_t>(f.part, (1ull << (d.c + splitk_log(d))) * rg_max * sizeof(uint32_t));
+      if (tc_eligible(d) && tc_split_log(d) > 0)
+        f.part = std::max<uint64_t>(f.part, (1ull << (d.c + tc_split_log(d))) * sizeof(uint32_t));
+      if (p8 && p8_eligible(d)) {
+        const uint64_t planes = p8_scratch_bytes(P8Step{d, p8_flags(p->low, i)}, rg_max);
+        const uint64_t parts = p8_part_bytes(d, rg_max);
+        f.n_dense++;
+        f.part = std::max<uint64_t>(f.part, parts);
+        f.p8 = std::max<uint64_t>(f.p8, planes);
+        sum_p8 += planes;
+        sum_part += parts;
+      }
     }
+    f.lvl_p8.push_back(sum_p8);
+    f.lvl_part.push_back(sum_part);
   }
   uint64_t arena = std::max(p->low.seq_arena_entries, p->low.lvl_arena_entries);
-  if (path == TNC_PATH_TC_P8) arena = std::max(arena, p->low.p8_arena_entries);
+  if (p8) arena = std::max(arena, p->low.p8_arena_entries);
   f.arena = (arena + 63) / 64 * 64;
   return f;
 }
@@ -352,12 +389,18 @@ SeqLayout layout_of(const Foot& f, int R, int path) {
   sect(s.off_tables, f.tables * sizeof(uint32_t));
   sect(s.off_steps, std::max(f.nseq, f.nlvl) * sizeof(GridStep));
   sect(s.off_small, f.nlvl * sizeof(StepDesc));
-  sect(s.off_tc, f.n_dense * R * tc_step_bytes());
+  uint64_t part = f.part, p8 = f.p8;
+  for (uint64_t v : f.lvl_part) part = std::max(part, std::min(v, kGroupParts));
+  for (uint64_t v : f.lvl_p8) p8 = std::max(p8, std::min(v, kGroupPlanes));
+  s.part_bytes = part;
+  s.p8_bytes = p8;
+  // (p8 descriptors hold addresses for a pass's residues per entry: 4, 2 and 1)
+  sect(s.off_tc, path == TNC_PATH_TC_P8 ? f.n_dense * 3 * p8_step_bytes() : f.n_dense * R * tc_step_bytes());
+  sect(s.off_part, part);
   sect(s.off_err, 64);
-  sect(s.off_part, f.part);
   sect(s.off_results, f.n_out * R * sizeof(uint32_t));
   sect(s.off_limbs, f.n_out * ((31 * R + 31) / 32) * sizeof(uint32_t));
-  sect(s.off_p8, f.p8);
+  sect(s.off_p8, p8);
   const size_t word = path == TNC_PATH_TC_P8 ? 1 : sizeof(uint32_t);  // bytes per residue
   sect(s.off_arena, f.arena * rg_max * word);
   s.total = o;
@@ -662,6 +705,7 @@ struct SoloPack {
   std::vector<char> bytes;  // forms, blob, leaves, tables, perms, order: copied to the workspace as they are
   size_t off_blob = 0, off_leaves = 0, off_tables = 0, off_perms = 0, off_order = 0;
   size_t blob_bytes = 0;
+  int long_sums = 0;  // steps of the split-K shapes (their sums are split over lanes)
 };
 }  // namespace tnc
 
@@ -687,6 +731,7 @@ void make_solo(const tnc_plan_t* p, SoloPack& s) {
   s.off_tables = blob_put(s.bytes, p->low.leaf_tables.data(), p->low.leaf_tables.size() * sizeof(uint32_t));
   s.off_perms = blob_put(s.bytes, p->low.root_perm.data(), p->low.root_perm.size());
   s.off_order = blob_put(s.bytes, &first, sizeof(first));
+  for (const StepDesc& d : p->low.lvl_steps) s.long_sums += splitk_log(d) > 0;
   s.ok = blob.size() <= 160 * 1024;
 }
 
@@ -723,9 +768,11 @@ int solo_enqueue(const SoloPack& s, const SeqLayout& L, const Arith& a, char* ws
       return TNC_OK;
     });
     if (rc) return rc;
+    // the record: the one launch does the work of these
     g_launches.leaf_fill++;
     g_launches.level++;
     g_launches.extract++;
+    g_launches.splitk += s.long_sums;
   }
   g_launches.crt++;
   return TNC_OK;
@@ -781,13 +828,14 @@ extern "C" size_t tnc_workspace_bytes_opts(const tnc_plan_t* plan, const tnc_con
   return seq_layout(plan, a.R, opts->path).total;
 }
 
-// Residues r of a sum of contractions: acc[e R + r] = (acc + src) mod p_r.
-__global__ void residue_add_kernel(uint32_t* __restrict__ acc, const uint32_t* __restrict__ src, uint64_t n, int R,
-                                   CrtConsts cc) {
+// Residues r of a sum of contractions: acc[e R + r] = (acc + sum_w src_w) mod
+// p_r, src_w the w-th of n_src arrays of n residues (all below p < 2^31).
+__global__ void residue_add_kernel(uint32_t* __restrict__ acc, const uint32_t* __restrict__ src, uint64_t n,
+                                   uint32_t n_src, int R, const __grid_constant__ CrtConsts cc) {
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t p = cc.p[i % R];
-    const uint32_t s = acc[i] + src[i];  // both below p < 2^31
-    acc[i] = s >= p ? s - p : s;
+    uint64_t s = acc[i];
+    for (uint32_t w = 0; w < n_src; w++) s += src[w * n + i];
+    acc[i] = (uint32_t)(s % cc.p[i % R]);
   }
 }
 
@@ -821,7 +869,7 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
     if (sum_into) {
       if (!dev_ws || ws_bytes < (size_t)a.R * 4) return set_error(TNC_ERR_BUFFER, "workspace too small");
       CUDA_TRY(cudaMemcpyAsync(dev_ws, res.data(), a.R * sizeof(uint32_t), cudaMemcpyHostToDevice, st));
-      residue_add_kernel<<<1, 64, 0, st>>>(sum_into, (const uint32_t*)dev_ws, (uint64_t)a.R, a.R, a.crt);
+      residue_add_kernel<<<1, 64, 0, st>>>(sum_into, (const uint32_t*)dev_ws, (uint64_t)a.R, 1, a.R, a.crt);
       CUDA_TRY(cudaGetLastError());
       CUDA_TRY(cudaStreamSynchronize(st));
     } else {
@@ -857,9 +905,17 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
   }
   // Every plan runs level by level (the tree-level schedule of the lowering);
   // offsets are shifted to the plan's part of the group's arena, tables and
-  // results.
+  // results.  All descriptors are staged in one buffer and copied at once.
   const bool p8 = opts->path == TNC_PATH_TC_P8;
   const bool tc = opts->path == TNC_PATH_TC || p8;
+  const int sms = sm_count();
+  std::vector<char> stage;
+  auto put = [&](const void* src, size_t bytes) {  // 64-byte aligned; returns the offset
+    const size_t at = (stage.size() + 63) / 64 * 64;
+    stage.resize(at + bytes);
+    if (bytes) std::memcpy(stage.data() + at, src, bytes);
+    return at;
+  };
   std::vector<LeafDesc> leaves;
   std::vector<uint32_t> tables;
   size_t n_lev = 0;
@@ -874,82 +930,6 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
     tables.insert(tables.end(), lw.leaf_tables.begin(), lw.leaf_tables.end());
     n_lev = std::max(n_lev, lw.lvl_start.empty() ? (size_t)0 : lw.lvl_start.size() - 1);
   }
-  CUDA_TRY(cudaMemcpyAsync(ws + L.off_leaves, leaves.data(), leaves.size() * sizeof(LeafDesc), cudaMemcpyHostToDevice, st));
-  if (!tables.empty())
-    CUDA_TRY(cudaMemcpyAsync(ws + L.off_tables, tables.data(), tables.size() * sizeof(uint32_t), cudaMemcpyHostToDevice,
-                             st));
-  g_h2d_bytes += leaves.size() * sizeof(LeafDesc) + tables.size() * sizeof(uint32_t);
-  // the group's steps by level: small ones (one index space per level across
-  // the plans), big, split-K and dense ones (one launch each)
-  enum Kind { kGrid, kSplit, kTc, kOuter };
-  struct Big {
-    int kind, slot;
-    StepDesc d;      // offsets shifted to the group's arena
-    uint32_t flags;  // p8: direct fp16 planes (kP8Direct*)
-  };
-  std::vector<std::vector<Big>> big(n_lev);
-  std::vector<GridStep> gsteps;
-  std::vector<tnc_dev::OuterStep> outers;
-  std::vector<StepDesc> small;
-  std::vector<uint32_t> small_lo(n_lev), small_hi(n_lev), small_work(n_lev);
-  std::vector<char> tcbuf;
-  size_t nd = 0;
-  for (size_t l = 0; l < n_lev; l++) {
-    small_lo[l] = (uint32_t)small.size();
-    uint64_t wk = 0;
-    for (int w = 0; w < nw; w++) {
-      const Lowered& lw = work[w]->low;
-      if (l + 1 >= lw.lvl_start.size()) continue;
-      const uint64_t base = L.arena_base[w];
-      for (uint32_t i = lw.lvl_start[l]; i < lw.lvl_start[l + 1]; i++) {
-        StepDesc d = p8 ? lw.p8_steps[i] : lw.lvl_steps[i];
-        d.a_off += base;
-        d.b_off += base;
-        d.c_off += base;
-        uint32_t flags = 0;
-        if (p8) {
-          const int sa = lw.lvl_src_a[i], sb = lw.lvl_src_b[i];
-          if (lw.p8_direct[i]) flags |= kP8DirectOut;
-          if (sa >= 0 && lw.p8_direct[sa]) flags |= kP8DirectA;
-          if (sb >= 0 && lw.p8_direct[sb]) flags |= kP8DirectB;
-        }
-        if (tc && (p8 ? p8_eligible(d) : tc_eligible(d))) {
-          big[l].push_back(Big{kTc, (int)nd++, d, flags});
-        } else if (flags) {
-          return set_error(TNC_ERR_INVALID, "internal: direct fp16 planes on a CUDA-core step");
-        } else if (outer_eligible(d)) {
-          big[l].push_back(Big{kOuter, (int)outers.size(), d, 0});
-          outers.push_back(make_outer_step(d));
-        } else if (splitk_log(d) > 0 || d.c >= 16) {
-          big[l].push_back(Big{splitk_log(d) > 0 ? kSplit : kGrid, (int)gsteps.size(), d, 0});
-          gsteps.push_back(make_grid_step(d));
-        } else {
-          d.work_lo = (uint32_t)wk;
-          wk += 1u << d.c;
-          small.push_back(d);
-        }
-      }
-    }
-    if (wk >= (1ull << 32)) return set_error(TNC_ERR_TOO_LARGE, "a merged level has more than 2^32 small outputs");
-    small_hi[l] = (uint32_t)small.size();
-    small_work[l] = (uint32_t)wk;
-  }
-  g_h2d_bytes += gsteps.size() * sizeof(GridStep) + small.size() * sizeof(StepDesc);
-  if (!gsteps.empty())
-    CUDA_TRY(cudaMemcpyAsync(ws + L.off_steps, gsteps.data(), gsteps.size() * sizeof(GridStep), cudaMemcpyHostToDevice,
-                             st));
-  if (!small.empty())
-    CUDA_TRY(cudaMemcpyAsync(ws + L.off_small, small.data(), small.size() * sizeof(StepDesc), cudaMemcpyHostToDevice, st));
-  if (nd && !p8) {
-    tcbuf.assign(nd * a.R * tc_step_bytes(), 0);
-    for (size_t l = 0; l < n_lev; l++)
-      for (const Big& b : big[l])
-        if (b.kind == kTc)
-          for (int r = 0; r < a.R; r++)
-            tc_make_step(b.d, a.primes[r], tcbuf.data() + ((size_t)b.slot * a.R + r) * tc_step_bytes());
-    CUDA_TRY(cudaMemcpyAsync(ws + L.off_tc, tcbuf.data(), tcbuf.size(), cudaMemcpyHostToDevice, st));
-    g_h2d_bytes += tcbuf.size();
-  }
   // residue groups: limb tensor-core passes carry one residue per entry; the
   // 8-bit-prime path keeps groups of 4 and runs its dense steps per residue
   Groups groups = a.groups;
@@ -960,8 +940,139 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
       groups.col.push_back(r);
     }
   }
+  // the group's steps by level: small ones (one index space per level across
+  // the plans), big, one-small-operand, split-K and dense ones: each kind one
+  // launch per level (split-K steps and dense steps as many as their scratch
+  // holds; limb dense steps one by one)
+  struct Range {
+    uint32_t lo, n, blocks, finals;
+  };
+  struct Level {
+    uint32_t small_lo = 0, small_n = 0, small_work = 0;
+    Range grid{}, outer{};
+    std::vector<Range> split;
+    std::vector<std::pair<int, StepDesc>> limb;      // slot in the limb descriptors, step
+    std::vector<std::pair<uint32_t, uint32_t>> p8;   // ranges of p8 steps launched together
+  };
+  std::vector<Level> lev(n_lev);
+  std::vector<GridStep> gsteps;
+  std::vector<tnc_dev::OuterStep> outers;
+  std::vector<StepDesc> small;
+  std::vector<P8Step> p8steps;
+  std::vector<char> tcbuf;
+  size_t nd = 0;
+  const int rg_max = groups.rg[0];
+  for (size_t l = 0; l < n_lev; l++) {
+    Level& lv = lev[l];
+    lv.small_lo = (uint32_t)small.size();
+    uint64_t wk = 0;
+    std::vector<GridStep> split;
+    lv.grid.lo = (uint32_t)gsteps.size();
+    lv.outer.lo = (uint32_t)outers.size();
+    const uint32_t p8_lo = (uint32_t)p8steps.size();
+    for (int w = 0; w < nw; w++) {
+      const Lowered& lw = work[w]->low;
+      if (l + 1 >= lw.lvl_start.size()) continue;
+      const uint64_t base = L.arena_base[w];
+      for (uint32_t i = lw.lvl_start[l]; i < lw.lvl_start[l + 1]; i++) {
+        StepDesc d = p8 ? lw.p8_steps[i] : lw.lvl_steps[i];
+        d.a_off += base;
+        d.b_off += base;
+        d.c_off += base;
+        const uint32_t flags = p8 ? p8_flags(lw, i) : 0u;
+        if (p8 && p8_eligible(d)) {
+          p8steps.push_back(P8Step{d, flags});
+        } else if (tc && !p8 && tc_eligible(d)) {
+          lv.limb.push_back({(int)nd++, d});
+        } else if (flags) {
+          return set_error(TNC_ERR_INVALID, "internal: direct fp16 planes on a CUDA-core step");
+        } else if (outer_eligible(d)) {
+          outers.push_back(make_outer_step(d));
+          outers.back().block_lo = lv.outer.blocks;
+          lv.outer.blocks += outers.back().blocks;
+        } else if (splitk_log(d) > 0) {
+          split.push_back(make_grid_step(d));
+        } else if (d.c >= 16) {
+          gsteps.push_back(make_grid_step(d));
+          gsteps.back().block_lo = lv.grid.blocks;
+          lv.grid.blocks += 1u << (gsteps.back().s - 8);  // 256 threads per block (c >= 16)
+        } else {
+          d.work_lo = (uint32_t)wk;
+          wk += 1u << d.c;
+          small.push_back(d);
+        }
+      }
+    }
+    if (wk >= (1ull << 32)) return set_error(TNC_ERR_TOO_LARGE, "a merged level has more than 2^32 small outputs");
+    lv.small_n = (uint32_t)small.size() - lv.small_lo;
+    lv.small_work = (uint32_t)wk;
+    lv.grid.n = (uint32_t)gsteps.size() - lv.grid.lo;
+    lv.outer.n = (uint32_t)outers.size() - lv.outer.lo;
+    // split-K steps: as many per launch as the partials' section holds
+    const uint64_t part_cap = L.part_bytes / ((uint64_t)rg_max * sizeof(uint32_t));
+    for (GridStep& g : split) {
+      const uint32_t parts = 1u << (g.d.c + g.log_split);
+      if (lv.split.empty() || (uint64_t)lv.split.back().blocks + parts > part_cap)
+        lv.split.push_back(Range{(uint32_t)gsteps.size(), 0, 0, 0});
+      Range& r = lv.split.back();
+      g.block_lo = g.part_off = r.blocks;
+      g.final_lo = r.finals;
+      r.n++;
+      r.blocks += parts;
+      r.finals += 1u << g.d.c;
+      gsteps.push_back(g);
+    }
+    // dense steps of the 8-bit-prime path: likewise (one at a time while they
+    // are timed)
+    uint64_t planes = 0, parts = 0;
+    for (uint32_t i = p8_lo; i < (uint32_t)p8steps.size(); i++) {
+      const uint64_t pl = p8_scratch_bytes(p8steps[i], rg_max), pt = p8_part_bytes(p8steps[i].d, rg_max);
+      if (lv.p8.empty() || g_time_dense || planes + pl > L.p8_bytes || parts + pt > L.part_bytes ||
+          i - lv.p8.back().first >= p8_max_steps()) {
+        lv.p8.push_back({i, i});
+        planes = parts = 0;
+      }
+      lv.p8.back().second = i + 1;
+      planes += pl;
+      parts += pt;
+    }
+  }
+  const size_t at_leaves = put(leaves.data(), leaves.size() * sizeof(LeafDesc));
+  const size_t at_tables = put(tables.data(), tables.size() * sizeof(uint32_t));
+  const size_t at_small = put(small.data(), small.size() * sizeof(StepDesc));
+  const size_t at_grid = put(gsteps.data(), gsteps.size() * sizeof(GridStep));
+  const size_t at_outer = put(outers.data(), outers.size() * sizeof(tnc_dev::OuterStep));
+  size_t at_tc = 0;
+  if (nd) {
+    tcbuf.assign(nd * a.R * tc_step_bytes(), 0);
+    for (const Level& lv : lev)
+      for (const auto& x : lv.limb)
+        for (int r = 0; r < a.R; r++)
+          tc_make_step(x.second, a.primes[r], tcbuf.data() + ((size_t)x.first * a.R + r) * tc_step_bytes());
+    at_tc = put(tcbuf.data(), tcbuf.size());
+  }
+  // p8 descriptors, for each number of residues per entry that a pass has
+  uint32_t* part = (uint32_t*)(ws + L.off_part);
+  std::vector<P8Batch> p8batches[5];
+  size_t at_p8[5] = {0};
+  for (int rg : {4, 2, 1}) {
+    if (!p8 || std::find(groups.rg.begin(), groups.rg.end(), rg) == groups.rg.end()) continue;
+    std::vector<char> host;
+    for (const Level& lv : lev)
+      for (const auto& r : lv.p8) {
+        p8batches[rg].emplace_back();
+        rc = p8_batch(p8steps.data() + r.first, (int)(r.second - r.first), (uint32_t)rg, (uint8_t*)(ws + L.off_arena),
+                      (uint64_t)(L.total - L.off_arena), (uint8_t*)(ws + L.off_p8), (uint8_t*)part, host,
+                      p8batches[rg].back());
+        if (rc) return rc;
+      }
+    at_p8[rg] = put(host.data(), host.size());
+  }
+  if (stage.size() > L.off_part) return set_error(TNC_ERR_INVALID, "internal: descriptors beyond their section");
+  CUDA_TRY(cudaMemcpyAsync(ws, stage.data(), stage.size(), cudaMemcpyHostToDevice, st));
+  g_h2d_bytes += stage.size();
   uint32_t* d_err = (uint32_t*)(ws + L.off_err);
-  CUDA_TRY(cudaMemsetAsync(d_err, 0, 64, st));
+  if (tc) CUDA_TRY(cudaMemsetAsync(d_err, 0, 64, st));  // (the CUDA-core kernels wait for nothing)
   // dense-step events (tnc_set_step_timing), destroyed on every return
   std::vector<cudaEvent_t> dense_events;
   std::vector<tnc_dense_step_time> dense_info;  // shapes of the timed dense launches
@@ -979,21 +1090,23 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
     dense_events.push_back(whole[1]);
     CUDA_TRY(cudaEventRecord(whole[0], st));
   }
-  const GridStep* d_steps = (const GridStep*)(ws + L.off_steps);
-  const StepDesc* d_small = (const StepDesc*)(ws + L.off_small);
+  const GridStep* d_steps = (const GridStep*)(ws + at_grid);
+  const StepDesc* d_small = (const StepDesc*)(ws + at_small);
+  const tnc_dev::OuterStep* d_outer = (const tnc_dev::OuterStep*)(ws + at_outer);
   uint32_t* results = (uint32_t*)(ws + L.off_results);
-  uint32_t* part = (uint32_t*)(ws + L.off_part);
-  std::vector<RootMap> rms(nw);
-  std::vector<uint64_t> root_off(nw);
+  std::vector<tnc_dev::Roots> roots;
   for (int w = 0; w < nw; w++) {
+    if (w % tnc_dev::kMaxRoots == 0) roots.push_back(tnc_dev::Roots{});
     const Lowered& lw = work[w]->low;
-    rms[w] = RootMap{};
-    rms[w].n_open = (int)work[w]->net.open_vars.size();
-    for (int j = 0; j < rms[w].n_open; j++) rms[w].perm[j] = lw.root_perm[j];
-    root_off[w] = L.arena_base[w] + (lw.lvl_steps.empty() ? (p8 ? lw.p8_leaf_off : lw.lvl_leaf_off)[work[w]->tree.root]
+    tnc_dev::Roots& rs = roots.back();
+    tnc_dev::Root& rt = rs.r[rs.n++];
+    rt.map.n_open = (int)work[w]->net.open_vars.size();
+    for (int j = 0; j < rt.map.n_open; j++) rt.map.perm[j] = lw.root_perm[j];
+    rt.root_off = L.arena_base[w] + (lw.lvl_steps.empty() ? (p8 ? lw.p8_leaf_off : lw.lvl_leaf_off)[work[w]->tree.root]
                                                           : (p8 ? lw.p8_root_off : lw.lvl_root_off));
+    rt.res_lo = L.res_base[w];
+    rs.n_entries += 1ull << rt.map.n_open;
   }
-  const int sms = sm_count();
   for (size_t gi = 0; gi < groups.rg.size(); gi++) {
     uint32_t gp[4];
     for (int r = 0; r < 4; r++) gp[r] = r < groups.rg[gi] ? a.primes[groups.col[gi] + r] : a.primes[groups.col[gi]];
@@ -1006,77 +1119,77 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
       constexpr bool N30 = decltype(n30tag)::value;
       W* arena = reinterpret_cast<W*>(ws + L.off_arena);
       const int nl = (int)leaves.size();
+      size_t next_p8 = 0;
       tnc_dev::leaf_fill_kernel<RG, W><<<std::min(nl, sms * 8), 64, 0, st>>>(
-          (const LeafDesc*)(ws + L.off_leaves), nl, (const uint32_t*)(ws + L.off_tables), arena, mg);
+          (const LeafDesc*)(ws + at_leaves), nl, (const uint32_t*)(ws + at_tables), arena, mg);
       g_launches.leaf_fill++;
-      for (size_t l = 0; l < n_lev; l++) {
+      // a timed dense launch: events around it and its shape
+      auto timed = [&](const StepDesc& d, auto&& launch) -> int {
+        cudaEvent_t ev[2] = {nullptr, nullptr};
+        if (g_time_dense) {
+          CUDA_TRY(cudaEventCreate(&ev[0]));
+          CUDA_TRY(cudaEventCreate(&ev[1]));
+          dense_events.push_back(ev[0]);
+          dense_events.push_back(ev[1]);
+          CUDA_TRY(cudaEventRecord(ev[0], st));
+        }
+        if (int rc2 = launch()) return rc2;
+        if (g_time_dense) {
+          CUDA_TRY(cudaEventRecord(ev[1], st));
+          tnc_dense_step_time info{};
+          info.macs = std::ldexp(1.0, d.ka + d.kb + d.k);
+          info.rows_log2 = d.ka;
+          info.cols_log2 = d.kb;
+          info.k_log2 = d.k;
+          info.residues = RG;
+          info.tile_n = p8 ? (int32_t)p8_tile_width(d) : 32;
+          info.log_split = (int32_t)(p8 ? p8_split_log(d) : tc_split_log(d));
+          dense_info.push_back(info);
+        }
+        return TNC_OK;
+      };
+      for (const Level& lv : lev) {
         NvtxRange level_range("tnc level");
-        const uint32_t n_small = small_hi[l] - small_lo[l];
-        if (n_small) {
-          const uint32_t wk = small_work[l];
-          const unsigned blocks = (unsigned)std::min<uint64_t>((wk + 255) / 256, (uint64_t)sms * 8);
-          tnc_dev::level_kernel<RG, W, N30><<<blocks, 256, 0, st>>>(d_small + small_lo[l], n_small, wk, arena, mg);
+        if (lv.small_n) {
+          const unsigned blocks = (unsigned)std::min<uint64_t>((lv.small_work + 255) / 256, (uint64_t)sms * 8);
+          tnc_dev::level_kernel<RG, W, N30><<<blocks, 256, 0, st>>>(d_small + lv.small_lo, lv.small_n, lv.small_work, arena,
+                                                                   mg);
           g_launches.level++;
         }
-        for (const Big& b : big[l]) {
-          if (b.kind == kTc) {
-            NvtxRange dense_range("tnc dense step");
-            if (RG != 1 && !p8) return set_error(TNC_ERR_INVALID, "internal: tensor-core step in a multi-residue pass");
-            int rc2 = TNC_OK;
-            cudaEvent_t ev[2] = {nullptr, nullptr};
-            if (g_time_dense) {
-              CUDA_TRY(cudaEventCreate(&ev[0]));
-              CUDA_TRY(cudaEventCreate(&ev[1]));
-              CUDA_TRY(cudaEventRecord(ev[0], st));
-            }
-            if (p8) {
-              rc2 = p8_launch(b.d, a.primes.data() + groups.col[gi], RG, reinterpret_cast<uint8_t*>(arena),
-                              (uint64_t)(L.total - L.off_arena), b.flags, ws + L.off_p8,
-                              reinterpret_cast<uint8_t*>(part), d_err, sms, st);
-            } else {
-              const char* dstep = ws + L.off_tc + ((size_t)b.slot * a.R + groups.col[gi]) * tc_step_bytes();
-              rc2 = tc_launch(dstep, b.d, reinterpret_cast<uint32_t*>(arena), part, d_err, st);
-            }
-            if (g_time_dense) {
-              CUDA_TRY(cudaEventRecord(ev[1], st));
-              dense_events.push_back(ev[0]);
-              dense_events.push_back(ev[1]);
-              tnc_dense_step_time info{};
-              info.macs = std::ldexp(1.0, b.d.ka + b.d.kb + b.d.k);
-              info.rows_log2 = b.d.ka;
-              info.cols_log2 = b.d.kb;
-              info.k_log2 = b.d.k;
-              info.residues = RG;
-              info.tile_n = p8 ? (int32_t)p8_tile_width(b.d) : 32;
-              info.log_split = (int32_t)(p8 ? p8_split_log(b.d) : tc_split_log(b.d));
-              dense_info.push_back(info);
-            }
-            if (rc2) return rc2;
-          } else if (b.kind == kOuter) {
-            const tnc_dev::OuterStep& os = outers[b.slot];
-            const unsigned blocks = (unsigned)std::min<uint64_t>(((1ull << os.fl) + 255) / 256, (uint64_t)sms * 8);
-            tnc_dev::outer_kernel<RG, W, N30><<<blocks, 256, 0, st>>>(os, arena, mg);
-            g_launches.outer++;
-          } else if (b.kind == kSplit) {
-            const uint32_t ls = splitk_log(b.d);
-            const uint64_t nblk = 1ull << (b.d.c + ls);
-            tnc_dev::splitk_partial_kernel<RG, W, N30><<<(unsigned)nblk, 256, 0, st>>>(d_steps + b.slot, arena, part, ls,
-                                                                                       mg);
-            tnc_dev::splitk_final_kernel<RG, W, N30><<<(unsigned)(1ull << b.d.c), 256, 0, st>>>(d_steps + b.slot, arena,
-                                                                                              part, ls, mg);
-            g_launches.splitk++;
-          } else {
-            int threads, blocks, sh;
-            grid_shape(b.d.c, &threads, &blocks, &sh);
-            tnc_dev::step_kernel<RG, W, N30><<<blocks, threads, 0, st>>>(d_steps + b.slot, arena, mg);
-            g_launches.grid_step++;
-          }
+        if (lv.outer.n) {
+          tnc_dev::outer_kernel<RG, W, N30><<<lv.outer.blocks, 256, 0, st>>>(d_outer + lv.outer.lo, lv.outer.n, arena, mg);
+          g_launches.outer++;
+        }
+        if (lv.grid.n) {
+          tnc_dev::step_kernel<RG, W, N30><<<lv.grid.blocks, 256, 0, st>>>(d_steps + lv.grid.lo, lv.grid.n, arena, mg);
+          g_launches.grid_step++;
+        }
+        for (const Range& r : lv.split) {
+          tnc_dev::splitk_partial_kernel<RG, W, N30><<<r.blocks, 256, 0, st>>>(d_steps + r.lo, r.n, arena, part, mg);
+          tnc_dev::splitk_final_kernel<RG, W, N30><<<r.finals, 256, 0, st>>>(d_steps + r.lo, r.n, arena, part, mg);
+          g_launches.splitk++;
+        }
+        for (const auto& x : lv.limb) {
+          NvtxRange dense_range("tnc dense step");
+          if (RG != 1) return set_error(TNC_ERR_INVALID, "internal: tensor-core step in a multi-residue pass");
+          const char* dstep = ws + at_tc + ((size_t)x.first * a.R + groups.col[gi]) * tc_step_bytes();
+          if (int rc2 = timed(x.second, [&] {
+                return tc_launch(dstep, x.second, reinterpret_cast<uint32_t*>(arena), part, d_err, st);
+              }))
+            return rc2;
+        }
+        for (const auto& r : lv.p8) {
+          NvtxRange dense_range("tnc dense steps");
+          const P8Batch& b = p8batches[RG][next_p8++];
+          if (int rc2 = timed(p8steps[r.first].d, [&] {
+                return p8_run(b, ws + at_p8[RG], a.primes.data() + groups.col[gi], RG, d_err, sms, st);
+              }))
+            return rc2;
         }
       }
-      for (int w = 0; w < nw; w++) {
-        const uint64_t no = 1ull << rms[w].n_open;
-        tnc_dev::extract_kernel<RG, W><<<(unsigned)std::min<uint64_t>((no + 255) / 256, 1024), 256, 0, st>>>(
-            arena, root_off[w], rms[w], results + L.res_base[w] * a.R, a.R, groups.col[gi]);
+      for (const tnc_dev::Roots& rs : roots) {
+        tnc_dev::extract_kernel<RG, W><<<(unsigned)std::min<uint64_t>((rs.n_entries + 255) / 256, 1024), 256, 0, st>>>(
+            arena, rs, results, a.R, groups.col[gi]);
         g_launches.extract++;
       }
       CUDA_TRY(cudaGetLastError());
@@ -1091,14 +1204,14 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
   }
   uint32_t h_err = 0;
   if (sum_into) {  // terms of a sum: add every plan's residues, check the device status
-    for (int w = 0; w < nw; w++) {
-      const uint64_t m = (1ull << rms[w].n_open) * (uint64_t)a.R;
-      residue_add_kernel<<<(unsigned)std::min<uint64_t>((m + 255) / 256, 1024), 256, 0, st>>>(
-          sum_into, results + L.res_base[w] * a.R, m, a.R, a.crt);
-    }
+    const uint64_t m = (1ull << roots[0].r[0].map.n_open) * (uint64_t)a.R;  // (the same for every plan)
+    residue_add_kernel<<<(unsigned)std::min<uint64_t>((m + 255) / 256, 1024), 256, 0, st>>>(sum_into, results, m,
+                                                                                           (uint32_t)nw, a.R, a.crt);
     CUDA_TRY(cudaGetLastError());
-    CUDA_TRY(cudaMemcpyAsync(&h_err, d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-    g_d2h_bytes += sizeof(uint32_t);
+    if (tc) {
+      CUDA_TRY(cudaMemcpyAsync(&h_err, d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+      g_d2h_bytes += sizeof(uint32_t);
+    }
     CUDA_TRY(cudaStreamSynchronize(st));
     if (inject_hit(TNC_INJECT_TIMEOUT)) h_err = 1;
     if (h_err) return set_error(TNC_ERR_TIMEOUT, "a tensor-core step timed out waiting for its MMAs");
@@ -1110,12 +1223,14 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
   g_launches.crt++;
   CUDA_TRY(cudaGetLastError());
   if (g_time_dense) CUDA_TRY(cudaEventRecord(whole[1], st));
-  CUDA_TRY(cudaMemcpyAsync(&h_err, d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-  std::vector<uint32_t> h_res(L.n_out * a.R), h_limbs(L.n_out * a.crt.n_limbs);
-  CUDA_TRY(cudaMemcpyAsync(h_res.data(), results, h_res.size() * 4, cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaMemcpyAsync(h_limbs.data(), limbs, h_limbs.size() * 4, cudaMemcpyDeviceToHost, st));
-  g_d2h_bytes += sizeof(uint32_t) + (h_res.size() + h_limbs.size()) * 4;
+  // status, residues and limbs: consecutive sections, one copy
+  std::vector<uint32_t> down((L.off_limbs - L.off_err) / 4 + L.n_out * a.crt.n_limbs);
+  CUDA_TRY(cudaMemcpyAsync(down.data(), d_err, down.size() * 4, cudaMemcpyDeviceToHost, st));
+  g_d2h_bytes += down.size() * 4;
   CUDA_TRY(cudaStreamSynchronize(st));
+  const uint32_t *h_res = down.data() + (L.off_results - L.off_err) / 4,
+                 *h_limbs = down.data() + (L.off_limbs - L.off_err) / 4;
+  h_err = tc ? down[0] : 0u;
   if (inject_hit(TNC_INJECT_TIMEOUT)) h_err = 1;
   if (h_err) return set_error(TNC_ERR_TIMEOUT, "a tensor-core step timed out waiting for its MMAs");
   for (size_t e = 0; e + 1 < dense_events.size(); e += 2) {  // pair 0: the whole contraction
@@ -1132,8 +1247,8 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
     g_dense_steps.push_back(info);
   }
   for (int w = 0; w < nw; w++) {
-    rc = fill_count(&outs[work_idx[w]], 1ull << rms[w].n_open, a, h_res.data() + L.res_base[w] * a.R,
-                    h_limbs.data() + L.res_base[w] * a.crt.n_limbs, result_flags(work[w], a));
+    rc = fill_count(&outs[work_idx[w]], 1ull << work[w]->net.open_vars.size(), a, h_res + L.res_base[w] * a.R,
+                    h_limbs + L.res_base[w] * a.crt.n_limbs, result_flags(work[w], a));
     if (rc) return rc;
   }
   return TNC_OK;
@@ -1930,7 +2045,7 @@ extern "C" int tnc_contract_noalloc(const tnc_plan_t* plan, const tnc_contract_o
     const size_t ns = plan->low.seq_steps.size();
     for (size_t i0 = 0; i0 < ns; i0 += 8) {
       const size_t m = std::min<size_t>(8, ns - i0);
-      for (size_t i = 0; i < m; i++) buf[i] = make_grid_step(plan->low.seq_steps[i0 + i]);
+      for (size_t i = 0; i < m; i++) buf[i] = make_grid_step(plan->low.seq_steps[i0 + i]);  // (a launch each)
       CUDA_TRY(cudaMemcpyAsync(ws + L.off_steps + i0 * sizeof(GridStep), buf, m * sizeof(GridStep),
                                cudaMemcpyHostToDevice, st));
     }
@@ -1940,13 +2055,14 @@ extern "C" int tnc_contract_noalloc(const tnc_plan_t* plan, const tnc_contract_o
   uint32_t* results = (uint32_t*)(ws + L.off_results);
   uint32_t* limbs = (uint32_t*)(ws + L.off_limbs);
   uint32_t* part = (uint32_t*)(ws + L.off_part);
-  RootMap rm{};
-  rm.n_open = (int)plan->net.open_vars.size();
-  for (int j = 0; j < rm.n_open; j++) rm.perm[j] = plan->low.root_perm[j];
+  tnc_dev::Roots roots{};
+  roots.n = 1;
+  roots.n_entries = n_out;
+  roots.r[0].map.n_open = (int)plan->net.open_vars.size();
+  for (int j = 0; j < roots.r[0].map.n_open; j++) roots.r[0].map.perm[j] = plan->low.root_perm[j];
   const int nl = (int)plan->low.leaves.size();
   const int sms = sm_count();
-  const uint64_t root_off =
-      plan->low.seq_steps.empty() ? plan->low.seq_leaf_off[plan->tree.root] : plan->low.seq_root_off;
+  roots.r[0].root_off = plan->low.seq_steps.empty() ? plan->low.seq_leaf_off[plan->tree.root] : plan->low.seq_root_off;
   for (int gi = 0; gi < n_groups; gi++) {
     uint32_t gp[4];
     for (int r = 0; r < 4; r++) gp[r] = r < grp_rg[gi] ? primes[grp_col[gi] + r] : primes[grp_col[gi]];
@@ -1960,19 +2076,19 @@ extern "C" int tnc_contract_noalloc(const tnc_plan_t* plan, const tnc_contract_o
         const StepDesc& d = plan->low.seq_steps[i];
         const uint32_t ls = splitk_log(d);
         if (ls > 0) {  // few outputs, long shared sum: K split over blocks, as in tnc_contract
-          tnc_dev::splitk_partial_kernel<RG><<<(unsigned)(1ull << (d.c + ls)), 256, 0, st>>>(d_steps + i, arena, part,
-                                                                                           ls, mg);
-          tnc_dev::splitk_final_kernel<RG><<<(unsigned)(1ull << d.c), 256, 0, st>>>(d_steps + i, arena, part, ls, mg);
+          tnc_dev::splitk_partial_kernel<RG><<<(unsigned)(1ull << (d.c + ls)), 256, 0, st>>>(d_steps + i, 1, arena, part,
+                                                                                           mg);
+          tnc_dev::splitk_final_kernel<RG><<<(unsigned)(1ull << d.c), 256, 0, st>>>(d_steps + i, 1, arena, part, mg);
           g_launches.splitk++;
           continue;
         }
         int threads, blocks, sh;
         grid_shape(d.c, &threads, &blocks, &sh);
-        tnc_dev::step_kernel<RG><<<blocks, threads, 0, st>>>(d_steps + i, arena, mg);
+        tnc_dev::step_kernel<RG><<<blocks, threads, 0, st>>>(d_steps + i, 1, arena, mg);
         g_launches.grid_step++;
       }
       tnc_dev::extract_kernel<RG><<<(unsigned)std::min<uint64_t>((n_out + 255) / 256, 1024), 256, 0, st>>>(
-          arena, root_off, rm, results, R, grp_col[gi]);
+          arena, roots, results, R, grp_col[gi]);
       g_launches.extract++;
       CUDA_TRY(cudaGetLastError());
       return TNC_OK;

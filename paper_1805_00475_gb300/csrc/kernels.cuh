@@ -213,249 +213,6 @@ __global__ void __launch_bounds__(256) leaf_fill_kernel(const LeafDesc* __restri
   }
 }
 
-// A step launched over the whole GPU.  With S = 2^s threads in the grid, a
-// thread visits o, o + S, o + 2S, ...: from one to the next the counter o >> s
-// gains one, which clears its trailing ones and sets bit t, so each operand
-// address changes by the precomputed delta[t] = w[t] - sum_{s <= j < t} w[j]
-// (w[j] = operand weight of output bit j).  Any bit permutation costs the
-// same two adds per entry.
-struct GridStep {
-  StepDesc d;
-  uint64_t wA[32], wB[32];  // operand address weight of output bit j
-  uint64_t dA[32], dB[32];  // address delta when the counter sets bit t
-  uint32_t s;               // log2(total threads)
-  uint32_t pad[3];
-};
-
-template <int RG, typename W = uint32_t, bool N30 = false>
-__global__ void __launch_bounds__(256) step_kernel(const GridStep* __restrict__ g, W* __restrict__ arena,
-                                                   ModGroup mg) {
-  const uint32_t c = g->d.c, k = g->d.k, ka = g->d.ka, kb = g->d.kb, s = g->s;
-  const uint64_t n = 1ull << c;
-  const W* A0 = arena + g->d.a_off * RG;
-  const W* B0 = arena + g->d.b_off * RG;
-  W* C0 = arena + g->d.c_off * RG;
-  uint64_t o = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= n) return;
-  uint64_t ia = 0, ib = 0;
-  for (uint32_t j = 0; j < c; j++)
-    if ((o >> j) & 1ull) {
-      ia += g->wA[j];
-      ib += g->wB[j];
-    }
-  for (;;) {
-    step_entry_at<RG, W, N30>(k, ka, kb, o, ia, ib, A0, B0, C0, mg);
-    const uint64_t u = o >> s;
-    o += 1ull << s;
-    if (o >= n) break;
-    const uint32_t t = s + (uint32_t)(__ffsll((long long)~u) - 1);
-    ia += g->dA[t];
-    ib += g->dB[t];
-  }
-}
-
-// A big step with one small operand (Sec. 2.1 with a skinny matrix): S has
-// 2^fs <= 16 rows, the shared dimension 2^k <= 8, the large operand L 2^fl
-// rows.  S's 2^(fs+k) entries are staged in shared memory; a thread takes a
-// row l of L, loads its 2^k entries once (consecutive threads, consecutive
-// rows: coalesced) and writes the 2^fs outputs C[oS(s) + oL(l)].  When S's
-// free bits are C's lowest bits (contig) those outputs are contiguous and a
-// thread writes them with vector stores (byte residues, 4 per entry).
-struct OuterStep {
-  uint64_t s_off, l_off, c_off;  // entry offsets of S, L, C in the arena
-  uint64_t oS[16];               // output offset of S's row s
-  uint64_t oL[32];               // output weight of L's free bit i
-  uint32_t fs, fl, k, contig;
-};
-
-template <int RG, typename W = uint32_t, bool N30 = false>
-__global__ void __launch_bounds__(256) outer_kernel(const __grid_constant__ OuterStep os, W* __restrict__ arena,
-                                                    ModGroup mg) {
-  __shared__ uint32_t sm[256 * RG];  // S entry (s, q) at (s + (q << fs)) * RG + r
-  const uint32_t fs = os.fs, fl = os.fl, K = 1u << os.k, NS = 1u << fs;
-  for (uint32_t i = threadIdx.x; i < (NS << os.k); i += blockDim.x) {
-    uint32_t v[RG];
-    load_entry<RG, W>(arena + (os.s_off + i) * RG, v);
-#pragma unroll
-    for (int r = 0; r < RG; r++) sm[i * RG + r] = v[r];
-  }
-  __syncthreads();
-  using Acc = std::conditional_t<sizeof(W) == 1, uint32_t, uint64_t>;
-  const W* L0 = arena + os.l_off * RG;
-  W* C0 = arena + os.c_off * RG;
-  const uint64_t nl = 1ull << fl;
-  for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < nl; l += (uint64_t)gridDim.x * blockDim.x) {
-    uint32_t lv[8][RG];
-#pragma unroll
-    for (uint32_t q = 0; q < 8; q++)
-      if (q < K) load_entry<RG, W>(L0 + (l + ((uint64_t)q << fl)) * RG, lv[q]);
-    uint64_t ol = 0;
-    for (uint32_t i = 0; i < fl; i++)
-      if ((l >> i) & 1ull) ol += os.oL[i];
-    // output s of this row: sum over q of S(s, q) L(l, q), reduced
-    auto entry = [&](uint32_t s, uint32_t (&out)[RG]) {
-      Acc acc[RG];
-#pragma unroll
-      for (int r = 0; r < RG; r++) acc[r] = 0;
-#pragma unroll
-      for (uint32_t q = 0; q < 8; q++) {
-        if (q < K) {
-          const uint32_t* sv = sm + (s + (q << fs)) * RG;
-#pragma unroll
-          for (int r = 0; r < RG; r++) acc[r] += (Acc)sv[r] * lv[q][r];
-          if (((q + 1) & mg.red_mask) == 0 && q + 1 < K) {
-#pragma unroll
-            for (int r = 0; r < RG; r++) acc[r] = reduce_acc<N30>(acc[r], mg, r);
-          }
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < RG; r++) out[r] = reduce_acc<N30>(acc[r], mg, r);
-    };
-    bool done = false;
-    if constexpr (sizeof(W) == 1 && RG == 4) {
-      if (os.contig) {  // C entries ol .. ol + NS - 1, 4 bytes each; ol is a multiple of NS
-        uint32_t* dst = reinterpret_cast<uint32_t*>(C0 + ol * RG);
-        for (uint32_t s0 = 0; s0 < NS; s0 += 4) {
-          uint32_t w[4] = {0, 0, 0, 0};
-#pragma unroll
-          for (uint32_t j = 0; j < 4; j++)
-            if (s0 + j < NS) {
-              uint32_t out[RG];
-              entry(s0 + j, out);
-              w[j] = out[0] | (out[1] << 8) | (out[2] << 16) | (out[3] << 24);
-            }
-          if (NS >= 4) *reinterpret_cast<uint4*>(dst + s0) = make_uint4(w[0], w[1], w[2], w[3]);
-          else if (NS == 2) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
-          else dst[0] = w[0];
-        }
-        done = true;
-      }
-    }
-    if (!done)
-      for (uint32_t s = 0; s < NS; s++) {
-        uint32_t out[RG];
-        entry(s, out);
-        store_entry<RG, W>(C0 + (os.oS[s] + ol) * RG, out);
-      }
-  }
-}
-
-// Split-K for steps with few output entries and a long shared dimension (a
-// final dot product, a rank-19 tensor against a rank-19 tensor, ...): block
-// (o, part) sums A*B over its slice of the 2^k shared values, the block's
-// threads combine their residues with modular additions, and a second kernel
-// adds the parts of each output.  part[o * n_split + j] holds RG residues.
-template <int RG, typename W = uint32_t, bool N30 = false>
-__global__ void __launch_bounds__(256) splitk_partial_kernel(const GridStep* __restrict__ g, const W* arena,
-                                                             uint32_t* __restrict__ part, uint32_t log_split,
-                                                             ModGroup mg) {
-  __shared__ uint32_t red[256 * RG];
-  const uint32_t n_split = 1u << log_split;
-  const uint64_t o = blockIdx.x >> log_split;
-  const uint32_t j = blockIdx.x & (n_split - 1);
-  const uint32_t k = g->d.k, ka = g->d.ka, kb = g->d.kb, c = g->d.c;
-  uint64_t ia = 0, ib = 0;
-  for (uint32_t b = 0; b < c; b++)
-    if ((o >> b) & 1ull) {
-      ia += g->wA[b];
-      ib += g->wB[b];
-    }
-  const W* A = arena + (g->d.a_off + ia) * RG;
-  const W* B = arena + (g->d.b_off + ib) * RG;
-  const uint64_t per = (1ull << k) >> log_split;
-  // byte residues: products below 2^16, sums of 16 of them in 32 bits
-  using Acc = std::conditional_t<sizeof(W) == 1, uint32_t, uint64_t>;
-  Acc acc[RG];
-#pragma unroll
-  for (int r = 0; r < RG; r++) acc[r] = 0;
-  uint32_t cnt = 0;
-  bool dot = false;
-  if constexpr (sizeof(W) == 1 && RG == 4) {
-    // a dot product of contiguous byte-residue operands (no free bits): a
-    // thread loads 4 entries of each operand (16 bytes), regroups the bytes
-    // by residue (two rounds of byte permutes) and adds 4 products per
-    // residue with one dp4a; 1024 products (below 2^26) between reductions
-    if (ka == 0 && kb == 0 && (per & 1023u) == 0) {
-      dot = true;
-      for (uint64_t q = j * per + 4u * threadIdx.x; q < (j + 1) * per; q += 4u * blockDim.x) {
-        const uint4 a4 = *reinterpret_cast<const uint4*>(A + q * 4);
-        const uint4 b4 = *reinterpret_cast<const uint4*>(B + q * 4);
-        const uint32_t ta0 = __byte_perm(a4.x, a4.y, 0x5140), ta1 = __byte_perm(a4.x, a4.y, 0x7362);
-        const uint32_t ta2 = __byte_perm(a4.z, a4.w, 0x5140), ta3 = __byte_perm(a4.z, a4.w, 0x7362);
-        const uint32_t tb0 = __byte_perm(b4.x, b4.y, 0x5140), tb1 = __byte_perm(b4.x, b4.y, 0x7362);
-        const uint32_t tb2 = __byte_perm(b4.z, b4.w, 0x5140), tb3 = __byte_perm(b4.z, b4.w, 0x7362);
-        acc[0] = __dp4a(__byte_perm(ta0, ta2, 0x5410), __byte_perm(tb0, tb2, 0x5410), acc[0]);
-        acc[1] = __dp4a(__byte_perm(ta0, ta2, 0x7632), __byte_perm(tb0, tb2, 0x7632), acc[1]);
-        acc[2] = __dp4a(__byte_perm(ta1, ta3, 0x5410), __byte_perm(tb1, tb3, 0x5410), acc[2]);
-        acc[3] = __dp4a(__byte_perm(ta1, ta3, 0x7632), __byte_perm(tb1, tb3, 0x7632), acc[3]);
-        if ((++cnt & 255u) == 0) {
-#pragma unroll
-          for (int r = 0; r < RG; r++) acc[r] = reduce_acc<N30>(acc[r], mg, r);
-        }
-      }
-    }
-  }
-  if (!dot)
-  for (uint64_t q = j * per + threadIdx.x; q < (j + 1) * per; q += blockDim.x) {
-    uint32_t va[RG], vb[RG];
-    load_entry<RG, W>(A + (q << ka) * RG, va);
-    load_entry<RG, W>(B + (q << kb) * RG, vb);
-#pragma unroll
-    for (int r = 0; r < RG; r++) acc[r] += (Acc)va[r] * vb[r];
-    if ((++cnt & mg.red_mask) == 0) {
-#pragma unroll
-      for (int r = 0; r < RG; r++) acc[r] = reduce_acc<N30>(acc[r], mg, r);
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < RG; r++) red[threadIdx.x * RG + r] = reduce_acc<N30>(acc[r], mg, r);
-  __syncthreads();
-  for (uint32_t h = blockDim.x >> 1; h > 0; h >>= 1) {
-    if (threadIdx.x < h) {
-#pragma unroll
-      for (int r = 0; r < RG; r++) {
-        uint32_t x = red[threadIdx.x * RG + r] + red[(threadIdx.x + h) * RG + r];
-        if (x >= mg.p[r]) x -= mg.p[r];
-        red[threadIdx.x * RG + r] = x;
-      }
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x < RG) part[(uint64_t)blockIdx.x * RG + threadIdx.x] = red[threadIdx.x];
-}
-
-// One block per output entry: its threads add the parts, then combine.
-template <int RG, typename W = uint32_t, bool N30 = false>
-__global__ void __launch_bounds__(256) splitk_final_kernel(const GridStep* __restrict__ g, W* arena,
-                                                           const uint32_t* __restrict__ part, uint32_t log_split,
-                                                           ModGroup mg) {
-  __shared__ uint32_t red[256 * RG];
-  const uint64_t o = blockIdx.x;
-  uint64_t s[RG];
-#pragma unroll
-  for (int r = 0; r < RG; r++) s[r] = 0;
-  for (uint32_t j = threadIdx.x; j < (1u << log_split); j += blockDim.x) {
-#pragma unroll
-    for (int r = 0; r < RG; r++) s[r] += part[((o << log_split) + j) * RG + r];  // < 2^31 each, < 2^20 of them
-  }
-#pragma unroll
-  for (int r = 0; r < RG; r++) red[threadIdx.x * RG + r] = reduce64<N30>(s[r], mg, r);
-  __syncthreads();
-  for (uint32_t h = blockDim.x >> 1; h > 0; h >>= 1) {
-    if (threadIdx.x < h) {
-#pragma unroll
-      for (int r = 0; r < RG; r++) {
-        uint32_t x = red[threadIdx.x * RG + r] + red[(threadIdx.x + h) * RG + r];
-        if (x >= mg.p[r]) x -= mg.p[r];
-        red[threadIdx.x * RG + r] = x;
-      }
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x < RG) arena[(g->d.c_off + o) * RG + threadIdx.x] = (W)red[threadIdx.x];
-}
-
 // All the small steps of one tree level in one launch: they are independent,
 // so their output entries form one index space (step i owns [work_lo,
 // work_lo + 2^c)); each thread finds its step by binary search.
@@ -471,26 +228,6 @@ __global__ void __launch_bounds__(256) level_kernel(const StepDesc* __restrict__
     }
     const StepDesc& d = steps[lo];
     step_entry<RG, W, N30>(d, w - d.work_lo, arena + d.a_off * RG, arena + d.b_off * RG, arena + d.c_off * RG, mg);
-  }
-}
-
-struct RootMap {
-  uint8_t perm[24];  // root bit j -> open variable index
-  int n_open;
-};
-
-// Root tensor -> result residues [entry][R], entry index bit i = open var i.
-template <int RG, typename W = uint32_t>
-__global__ void extract_kernel(const W* __restrict__ arena, uint64_t root_off, RootMap rm,
-                               uint32_t* __restrict__ results, int R, int col) {
-  const uint32_t n_out = 1u << rm.n_open;
-  for (uint32_t J = blockIdx.x * blockDim.x + threadIdx.x; J < n_out; J += gridDim.x * blockDim.x) {
-    uint64_t a = 0;
-#pragma unroll
-    for (int j = 0; j < 24; j++)
-      if (j < rm.n_open) a |= (uint64_t)((J >> rm.perm[j]) & 1u) << j;
-#pragma unroll
-    for (int r = 0; r < RG; r++) results[(uint64_t)J * R + col + r] = arena[(root_off + a) * RG + r];
   }
 }
 

@@ -100,21 +100,41 @@ template <uint32_t NA>
 using StageWord = std::conditional_t<NA == 4, uint32_t, std::conditional_t<NA == 2, uint16_t, uint8_t>>;
 constexpr uint64_t kWaitNs = 2000000000ull;
 
-struct P8Args {
+// One dense step as the GEMM launch sees it, in device memory: a launch takes
+// the work items of up to kMaxProbs steps (of one tree level, with one tile
+// width) one after another.
+struct alignas(64) P8Prob {
+  CUtensorMap map_a, map_b;  // operand planes of the row side and of the column side
   uint32_t fa, fb, k, log_split;  // rows 2^fa, columns 2^fb, shared 2^k, K split 2^log_split
   uint32_t n_items, tiles_m;      // work items (tiles x splits); row tiles
-  uint32_t rg, gm_log;            // residues per entry (1, 2 or 4), computed together; row tiles per raster group (log2)
-  uint32_t p[4];
-  float pf[4], invp[4];
+  uint32_t gm_log;                // row tiles per raster group (log2)
+  uint32_t item_lo;               // first work item of this step in its launch
   uint64_t wm[32], wn[32];  // output address weight of row bit j / column bit j
   uint8_t ebit[16];         // the tile's row and column bits by output weight, lightest first
                             // (column bit j: 0x80 | j; row bit j: j); bits 0..4 go to lanes
-  uint32_t n_ebits, pad3;
+  uint32_t n_ebits;
   uint32_t a_mn, b_mn;      // operand planes row-contiguous (MN-major) instead of K-contiguous
   uint32_t direct;          // output as rg balanced fp16 planes, plane i at out + i 2^(fa+fb) halves
   uint32_t pairs;           // row bit 0 has output weight 1: entries written two at a time (TN >= 32)
   uint8_t* out;             // C (entry o at out[o * rg]), or the split partials [split][2^(fa+fb) * rg]
 };
+constexpr uint32_t kMaxProbs = 256;  // steps of one launch (their first items are searched in shared memory)
+
+// What a launch needs of its pass: the residues' primes.
+struct P8Primes {
+  float pf[4], invp[4];
+};
+
+// Index of the last of n ascending values lo[0..n) that is <= x (lo[0] <= x).
+__device__ __forceinline__ uint32_t find_last(const uint32_t* lo, uint32_t n, uint32_t x) {
+  uint32_t a = 0, b = n - 1;
+  while (a < b) {
+    const uint32_t m = (a + b + 1) >> 1;
+    if (lo[m] <= x) a = m;
+    else b = m - 1;
+  }
+  return a;
+}
 
 // ---- PTX helpers -----------------------------------------------------------
 
@@ -238,6 +258,13 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
       " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(cmbar)
       : "memory");
+}
+
+// The tensor map at `map` in global memory, written by a copy from the host
+// before the launch, is read by this thread's later copies.
+__device__ __forceinline__ void tensormap_acquire(const CUtensorMap* map) {
+  asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(map))
+               : "memory");
 }
 
 // 2-D tiled TMA load of the box at (x, y) into shared memory, completing on
@@ -469,32 +496,42 @@ struct PackOperand {
   uint32_t f, mode;
 };
 
-// Both operands of a step in one launch: the tiles of A, then those of B.
+// One dense step's operands to pack: the tiles of A, then those of B; its
+// first tile in the launch, which takes up to kMaxProbs steps of a level.
+struct alignas(64) PackProb {
+  PackOperand a, b;
+  uint32_t k, kp, tile_lo, n_tiles;
+};
+
 template <int RG>
-__global__ void __launch_bounds__(256) p8_pack_kernel(PackOperand opA, PackOperand opB, uint32_t k, uint32_t kp,
-                                                      PackPrimes pp) {
+__global__ void __launch_bounds__(256) p8_pack_kernel(const PackProb* __restrict__ probs, uint32_t n_probs,
+                                                      uint32_t n_tiles, PackPrimes pp) {
   // [residue][row][pair of shared values] half2 words; a row is 32 words + 1
   // of padding, so both phases are free of bank conflicts (phase 1: lanes =
   // 8 row quads x 4 pairs; phase 2: lanes = 8 chunks x 4 rows)
   __shared__ uint32_t tile[RG][64][33];
-  const uint32_t K = 1u << k, Kp = 1u << kp;
-  const uint64_t tiles_a = opA.mode ? (uint64_t)(((1u << opA.f) + 63u) / 64u) << (kp - 6) : 0;
-  const uint64_t n_tiles = tiles_a + (opB.mode ? (uint64_t)(((1u << opB.f) + 63u) / 64u) << (kp - 6) : 0);
+  __shared__ uint32_t tile_lo[kMaxProbs];
   const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+  if (t < n_probs) tile_lo[t] = probs[t].tile_lo;
+  __syncthreads();
   __half2 hp2[RG], np2[RG];
 #pragma unroll
   for (int i = 0; i < RG; i++) {
     hp2[i] = __float2half2_rn((float)((pp.p[i] - 1) / 2));
     np2[i] = __float2half2_rn(-(float)pp.p[i]);
   }
-  for (uint64_t bt = blockIdx.x; bt < n_tiles; bt += gridDim.x) {
+  for (uint32_t gt = blockIdx.x; gt < n_tiles; gt += gridDim.x) {
+    const PackProb& pb = probs[find_last(tile_lo, n_probs, gt)];
+    const PackOperand opA = pb.a, opB = pb.b;
+    const uint32_t K = 1u << pb.k, Kp = 1u << pb.kp, bt = gt - pb.tile_lo;
+    const uint32_t tiles_a = opA.mode ? (((1u << opA.f) + 63u) / 64u) << (pb.kp - 6) : 0;
     const bool isA = bt < tiles_a;  // uniform over the block
     const uint8_t* __restrict__ X = isA ? opA.X : opB.X;
     __half* __restrict__ Y = isA ? opA.Y : opB.Y;
     const uint32_t R = 1u << (isA ? opA.f : opB.f);
     const uint32_t tiles_r = (R + 63) / 64;
-    const uint64_t b = isA ? bt : bt - tiles_a;
-    const uint32_t r0 = (uint32_t)(b % tiles_r) * 64u, q0 = (uint32_t)(b / tiles_r) * 64u;
+    const uint32_t b = isA ? bt : bt - tiles_a;
+    const uint32_t r0 = (b % tiles_r) * 64u, q0 = (b / tiles_r) * 64u;
     if ((isA ? opA.mode : opB.mode) == 2) {  // row-contiguous: 64 shared values x 16 quads of rows
 #pragma unroll
       for (int it = 0; it < 4; it++) {
@@ -579,17 +616,45 @@ __global__ void __launch_bounds__(256) p8_pack_kernel(PackOperand opA, PackOpera
   }
 }
 
-// Sum of the K-split partials: C[i] = sum_j part[j][i] mod p_(i mod rg) for
-// the n = 2^c * rg residues (bytes) of the step's output.
-__global__ void p8_split_final_kernel(const uint8_t* __restrict__ part, uint8_t* __restrict__ C, uint32_t c,
-                                      uint32_t log_split, uint32_t rg, uint4 primes) {
-  const uint64_t n = (uint64_t)rg << c;
+// Sums of the K-split partials of the split steps of a launch: C[i] = sum_j
+// part[j][i] mod p_(i mod rg) for the n = 2^c * rg residues (bytes) of a
+// step's output, four residues (one word) per thread: up to 2^8 bytes add up
+// in the 16-bit halves of two words.
+struct alignas(64) SplitProb {
+  const uint8_t* part;
+  uint8_t* out;
+  uint32_t log_n, log_split, block_lo, pad;  // n = 2^log_n residues; its first block of 1024 in the launch
+};
+
+__global__ void __launch_bounds__(256) p8_split_final_kernel(const SplitProb* __restrict__ probs, uint32_t n_probs,
+                                                             uint32_t rg, uint4 primes) {
+  __shared__ uint32_t block_lo[kMaxProbs];
+  if (threadIdx.x < n_probs) block_lo[threadIdx.x] = probs[threadIdx.x].block_lo;
+  __syncthreads();
+  const SplitProb sp = probs[find_last(block_lo, n_probs, blockIdx.x)];
+  const uint64_t n = 1ull << sp.log_n;
+  const uint64_t i = ((uint64_t)(blockIdx.x - sp.block_lo) * 256u + threadIdx.x) * 4u;
+  if (i >= n) return;
   const uint32_t pr[4] = {primes.x, primes.y, primes.z, primes.w};
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-    uint32_t s = 0;
-    for (uint32_t j = 0; j < (1u << log_split); j++) s += part[(uint64_t)j * n + i];
-    C[i] = (uint8_t)(s % pr[i % rg]);
+  uint32_t s[4] = {0, 0, 0, 0};
+  for (uint32_t j0 = 0; j0 < (1u << sp.log_split); j0 += 256) {
+    uint32_t even = 0, odd = 0;
+    const uint32_t j1 = min(j0 + 256u, 1u << sp.log_split);
+#pragma unroll 8
+    for (uint32_t j = j0; j < j1; j++) {
+      const uint32_t w = *reinterpret_cast<const uint32_t*>(sp.part + (uint64_t)j * n + i);
+      even += w & 0x00FF00FFu;
+      odd += (w >> 8) & 0x00FF00FFu;
+    }
+    s[0] += even & 0xFFFFu;
+    s[1] += odd & 0xFFFFu;
+    s[2] += even >> 16;
+    s[3] += odd >> 16;
   }
+  uint32_t w = 0;
+#pragma unroll
+  for (uint32_t q = 0; q < 4; q++) w |= (s[q] % pr[q % rg]) << (8 * q);
+  *reinterpret_cast<uint32_t*>(sp.out + i) = w;
 }
 
 // ---- the GEMM -------------------------------------------------------------
@@ -599,12 +664,33 @@ __global__ void p8_split_final_kernel(const uint8_t* __restrict__ part, uint8_t*
 // that the CTAs running at one time share the operand rows of a few row tiles
 // and of a few column tiles.
 // Row tiles are 128 rows (PAIR: 256, the pair's two 128-row halves).
+// What the roles need of a step, read once per step (its descriptor is in
+// global memory): the K slice of an item in chunks of spc stages; items run K
+// slice by K slice (split-major): the items of one wave share their slice's
+// operand rows in L2; row-contiguous operands (a tile of TN < 64 columns
+// always reads B K-contiguous).
+struct Step {
+  uint32_t Ks, n_chunks, spc, tile_bits, gm, group_bits;  // raster group: 2^gm row tiles, 2^group_bits tiles
+  bool a_mn, b_mn;
+};
+template <uint32_t TN>
+__device__ __forceinline__ void load_step(const P8Prob& g, Step& st) {
+  st.Ks = (1u << g.k) >> g.log_split;
+  const uint32_t chunk = st.Ks < kChunkK ? st.Ks : kChunkK;
+  st.n_chunks = st.Ks / chunk;
+  st.spc = chunk / kStageK;
+  st.tile_bits = 31u - __clz(g.n_items >> g.log_split);
+  st.gm = g.gm_log;
+  st.group_bits = st.tile_bits - (31u - __clz(g.tiles_m) - st.gm);
+  st.a_mn = g.a_mn != 0;
+  st.b_mn = TN >= 64 && g.b_mn != 0;
+}
+
 template <uint32_t TN, bool PAIR>
-__device__ __forceinline__ void tile_origin(uint32_t tile, const P8Args& g, uint32_t& m0, uint32_t& n0) {
-  const uint32_t gm = g.gm_log, per_group = (g.n_items >> g.log_split) >> (31 - __clz(g.tiles_m) - gm);
-  const uint32_t grp = tile / per_group, w = tile - grp * per_group;
-  m0 = ((grp << gm) + (w & ((1u << gm) - 1u))) * (PAIR ? 2u * kTileM : kTileM);
-  n0 = (w >> gm) * TN;
+__device__ __forceinline__ void tile_origin(uint32_t tile, const Step& st, uint32_t& m0, uint32_t& n0) {
+  const uint32_t grp = tile >> st.group_bits, w = tile & ((1u << st.group_bits) - 1u);
+  m0 = ((grp << st.gm) + (w & ((1u << st.gm) - 1u))) * (PAIR ? 2u * kTileM : kTileM);
+  n0 = (w >> st.gm) * TN;
 }
 
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
@@ -630,8 +716,8 @@ __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"
 // arrives on the leader's accumulator-free barrier.
 template <uint32_t TN, uint32_t RG, bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1)
-    p8_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                   const __grid_constant__ P8Args g, uint32_t* err) {
+    p8_gemm_kernel(const P8Prob* __restrict__ probs, uint32_t n_probs, uint32_t n_items,
+                   const __grid_constant__ P8Primes pr, uint32_t* err) {
   static_assert(!PAIR || TN == 256, "CTA pairs for 256-wide tiles");
   using C = Cfg<TN, RG, PAIR>;
   constexpr uint32_t kStages = C::kStages, kStageBytes = C::kStageBytes, NA = C::NA, kRounds = C::kRounds;
@@ -643,6 +729,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   // per index h of the entry bits above the lane bits: their part of the
   // entry's output offset (x) and of its staging index (y)
   __shared__ uint2 ho_tab[kTileM * TN / 32];
+  __shared__ uint32_t item_lo[kMaxProbs];  // first work item of each step
+  __shared__ uint64_t w_tab[64];           // the epilogue's step: wm, wn
+  for (uint32_t i = threadIdx.x; i < n_probs; i += kThreads) item_lo[i] = probs[i].item_lo;
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   SW* staging = reinterpret_cast<SW*>(smem + kStages * kStageBytes);  // [col][kStagePitch] entries of NA bytes
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
@@ -672,26 +761,28 @@ __global__ void __launch_bounds__(kThreads, 1)
   const bool leader = crank == 0;
 
   const uint32_t G = gridDim.x / (PAIR ? 2u : 1u), bid = blockIdx.x / (PAIR ? 2u : 1u);
-  const uint32_t T = g.n_items > bid ? (g.n_items - bid + G - 1) / G : 0;
-  const uint32_t Ks = (1u << g.k) >> g.log_split;
-  const uint32_t chunk = Ks < kChunkK ? Ks : kChunkK;
-  const uint32_t n_chunks = Ks / chunk;
-  const uint32_t spc = chunk / kStageK;  // stages per chunk
-  // items run K slice by K slice (split-major): the items of one wave share
-  // their slice's operand rows in L2
-  const uint32_t tile_bits = 31u - __clz(g.n_items >> g.log_split), tile_mask = (1u << tile_bits) - 1u;
-  // row-contiguous operands (a tile of TN < 64 columns always reads B K-contiguous)
-  const bool a_mn = g.a_mn != 0, b_mn = TN >= 64 && g.b_mn != 0;
+  const uint32_t T = n_items > bid ? (n_items - bid + G - 1) / G : 0;
   bool ok = true;
 
   if (warp == 0) {
     if (lane == 0) {  // TMA producer
-      uint32_t s = 0, ph = 0, issued = 0;
+      uint32_t s = 0, ph = 0, issued = 0, cur = ~0u;
+      Step st;
       for (uint32_t t = 0; t < T && ok; t++) {
-        const uint32_t item = bid + t * G;
-        const uint32_t split = item >> tile_bits, tile = item & tile_mask;
+        const uint32_t pi = find_last(item_lo, n_probs, bid + t * G);
+        if (pi != cur) {
+          load_step<TN>(probs[pi], st);
+          tensormap_acquire(&probs[pi].map_a);
+          tensormap_acquire(&probs[pi].map_b);
+          cur = pi;
+        }
+        const CUtensorMap *tmA = &probs[pi].map_a, *tmB = &probs[pi].map_b;
+        const uint32_t item = bid + t * G - item_lo[pi];
+        const uint32_t split = item >> st.tile_bits, tile = item & ((1u << st.tile_bits) - 1u);
+        const uint32_t n_chunks = st.n_chunks, spc = st.spc, Ks = st.Ks, chunk = spc * kStageK;
+        const bool a_mn = st.a_mn, b_mn = st.b_mn;
         uint32_t m0, n0;
-        tile_origin<TN, PAIR>(tile, g, m0, n0);
+        tile_origin<TN, PAIR>(tile, st, m0, n0);
         m0 += crank * kTileM;                  // this CTA's rows
         n0 += crank * C::kRowsB;               // this CTA's part of the B tile
         for (uint32_t rd = 0; rd < kRounds && ok; rd++)
@@ -716,16 +807,16 @@ __global__ void __launch_bounds__(kThreads, 1)
               // K-contiguous planes: one box of rows x 64 shared values;
               // row-contiguous: boxes of 64 rows x 64 shared values, 8 KiB apart
               if (a_mn) {
-                load(sa, &tmA, (int32_t)m0, x);
-                load(sa + 8192u, &tmA, (int32_t)m0 + 64, x);
+                load(sa, tmA, (int32_t)m0, x);
+                load(sa + 8192u, tmA, (int32_t)m0 + 64, x);
               } else {
-                load(sa, &tmA, x, (int32_t)m0);
+                load(sa, tmA, x, (int32_t)m0);
               }
               if (b_mn) {
                 for (uint32_t h = 0; 64u * h < C::kRowsB; h++)
-                  load(sa + kABytes + 8192u * h, &tmB, (int32_t)(n0 + 64u * h), x);
+                  load(sa + kABytes + 8192u * h, tmB, (int32_t)(n0 + 64u * h), x);
               } else {
-                load(sa + kABytes, &tmB, x, (int32_t)n0);
+                load(sa + kABytes, tmB, x, (int32_t)n0);
               }
               issued++;
               if (++s == kStages) {
@@ -751,10 +842,20 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1) {
     if (lane == 0 && leader) {  // MMA issuer (PAIR: the leader's, for both CTAs)
-      const uint32_t idesc = make_idesc(PAIR ? 2u * kTileM : kTileM, TN, a_mn ? 1u : 0u, b_mn ? 1u : 0u);
-      const uint32_t a_ks = a_mn ? 2048u >> 4 : 32u >> 4, b_ks = b_mn ? 2048u >> 4 : 32u >> 4;
-      uint32_t s = 0, ph = 0, par = 0;  // bit r: phase parity of accumulator r
-      for (uint32_t t = 0; t < T && ok; t++)
+      uint32_t s = 0, ph = 0, par = 0, cur = ~0u;  // par, bit r: phase parity of accumulator r
+      Step st;
+      uint32_t idesc = 0, a_ks = 0, b_ks = 0;
+      for (uint32_t t = 0; t < T && ok; t++) {
+        const uint32_t pi = find_last(item_lo, n_probs, bid + t * G);
+        if (pi != cur) {
+          cur = pi;
+          load_step<TN>(probs[pi], st);
+          idesc = make_idesc(PAIR ? 2u * kTileM : kTileM, TN, st.a_mn ? 1u : 0u, st.b_mn ? 1u : 0u);
+          a_ks = st.a_mn ? 2048u >> 4 : 32u >> 4;
+          b_ks = st.b_mn ? 2048u >> 4 : 32u >> 4;
+        }
+        const uint32_t n_chunks = st.n_chunks, spc = st.spc;
+        const bool a_mn = st.a_mn, b_mn = st.b_mn;
         for (uint32_t rd = 0; rd < kRounds && ok; rd++)
         for (uint32_t c = 0; c < n_chunks && ok; c++)
           for (uint32_t r = 0; r < NA && ok; r++) {
@@ -791,6 +892,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             else mma_commit<false>(accf0 + 8 * r);
             par ^= 1u << r;
           }
+      }
       // every MMA issued has completed before the TMEM is freed
       mma_commit<PAIR>(drain);
       if (!mbar_wait(drain, 0)) ok = false;
@@ -821,47 +923,68 @@ __global__ void __launch_bounds__(kThreads, 1)
     // With pairs, entry bit 0 is row bit 0 (output weight 1): a thread takes
     // the two entries o, o + 1, adjacent in the staging and in C, and the
     // lane and table bits start one higher.
-    const uint32_t pv = (TN >= 32 && g.pairs) ? 1u : 0u;
-    uint32_t lane_off = 0, lane_sid = 0;
-    for (uint32_t i = 0; i < 5; i++) {
-      if (!((lane >> i) & 1u)) continue;
-      const uint32_t b = g.ebit[pv + i];
-      if (b & 0x80u) {
-        lane_off += (uint32_t)g.wn[b & 31u];
-        lane_sid += kStagePitch << (b & 31u);
-      } else {
-        lane_off += (uint32_t)g.wm[b];
-        lane_sid += 1u << b;
-      }
-    }
-    for (uint32_t h = et; h < (kTileM * TN / 32) >> pv; h += kEpiThreads) {
-      uint32_t off = 0, sid = 0;
-      for (uint32_t i = 5 + pv; i < g.n_ebits; i++) {
-        if (!((h >> (i - 5 - pv)) & 1u)) continue;
-        const uint32_t b = g.ebit[i];
-        if (b & 0x80u) {
-          off += (uint32_t)g.wn[b & 31u];
-          sid += kStagePitch << (b & 31u);
-        } else {
-          off += (uint32_t)g.wm[b];
-          sid += 1u << b;
-        }
-      }
-      ho_tab[h] = make_uint2(off, sid);
-    }
+    // (all of this per step: set up again when an item belongs to another one)
+    uint32_t pv = 0, lane_off = 0, lane_sid = 0, cur = ~0u, fa = 0, fb = 0, log_split = 0;
+    bool direct = false;
+    uint8_t* out = nullptr;
+    Step st;
     constexpr uint32_t kLogTN = TN == 256 ? 8 : TN == 128 ? 7 : TN == 64 ? 6 : TN == 32 ? 5 : 4;
     uint32_t par = 0;  // bit ra: phase parity of accumulator ra
     for (uint32_t t = 0; t < T; t++) {
-      const uint32_t item = bid + t * G;
-      const uint32_t split = item >> tile_bits, tile = item & tile_mask;
+      const uint32_t pi = find_last(item_lo, n_probs, bid + t * G);
+      if (pi != cur) {
+        const P8Prob& g = probs[pi];
+        load_step<TN>(g, st);
+        fa = g.fa;
+        fb = g.fb;
+        log_split = g.log_split;
+        direct = g.direct != 0;
+        out = g.out;
+        if (cur != ~0u) epi_bar();  // the previous step's entries are out: the tables are free
+        cur = pi;
+        if (et < 32) w_tab[et] = g.wm[et];
+        else if (et < 64) w_tab[et] = g.wn[et - 32u];
+        pv = (TN >= 32 && g.pairs) ? 1u : 0u;
+        lane_off = lane_sid = 0;
+        for (uint32_t i = 0; i < 5; i++) {
+          if (!((lane >> i) & 1u)) continue;
+          const uint32_t b = g.ebit[pv + i];
+          if (b & 0x80u) {
+            lane_off += (uint32_t)g.wn[b & 31u];
+            lane_sid += kStagePitch << (b & 31u);
+          } else {
+            lane_off += (uint32_t)g.wm[b];
+            lane_sid += 1u << b;
+          }
+        }
+        for (uint32_t h = et; h < (kTileM * TN / 32) >> pv; h += kEpiThreads) {
+          uint32_t off = 0, sid = 0;
+          for (uint32_t i = 5 + pv; i < g.n_ebits; i++) {
+            if (!((h >> (i - 5 - pv)) & 1u)) continue;
+            const uint32_t b = g.ebit[i];
+            if (b & 0x80u) {
+              off += (uint32_t)g.wn[b & 31u];
+              sid += kStagePitch << (b & 31u);
+            } else {
+              off += (uint32_t)g.wm[b];
+              sid += 1u << b;
+            }
+          }
+          ho_tab[h] = make_uint2(off, sid);
+        }
+        epi_bar();
+      }
+      const uint32_t n_chunks = st.n_chunks;
+      const uint32_t item = bid + t * G - item_lo[pi];
+      const uint32_t split = item >> st.tile_bits, tile = item & ((1u << st.tile_bits) - 1u);
       uint32_t m0, n0;
-      tile_origin<TN, PAIR>(tile, g, m0, n0);
+      tile_origin<TN, PAIR>(tile, st, m0, n0);
       m0 += crank * kTileM;  // PAIR: this CTA's 128 rows of the item (its TMEM lanes)
       uint64_t tile_base = lane_off;  // output offset of the tile's origin + the lane bits' part
-      for (uint32_t j = 7; j < g.fa; j++)
-        if ((m0 >> j) & 1u) tile_base += g.wm[j];
-      for (uint32_t j = kLogTN; j < g.fb; j++)
-        if ((n0 >> j) & 1u) tile_base += g.wn[j];
+      for (uint32_t j = 7; j < fa; j++)
+        if ((m0 >> j) & 1u) tile_base += w_tab[j];
+      for (uint32_t j = kLogTN; j < fb; j++)
+        if ((n0 >> j) & 1u) tile_base += w_tab[32 + j];
       for (uint32_t rd = 0; rd < kRounds; rd++) {
         for (uint32_t c = 0; c < n_chunks; c++) {
           const bool last = c + 1 == n_chunks;
@@ -872,7 +995,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_fence_after();
             const uint32_t tb = tmem + ((quarter * 32u) << 16) + ra * TN + cbeg;
             if (ok && !idle) {
-              const float pf = g.pf[r], invp = g.invp[r], pm = kMagic + pf;
+              const float pf = pr.pf[r], invp = pr.invp[r], pm = kMagic + pf;
 #pragma unroll 1
               for (uint32_t col = 0; col < kHalf; col += kBatch) {
                 uint32_t v[kBatch / 16][16];
@@ -887,7 +1010,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                       v[b][jj] = __float_as_uint(reduce_p(__uint_as_float(v[b][jj]), pf, invp));
                     tmem_st16(tb + col + 16 * b, v[b]);
                   }
-                } else if (g.direct) {  // r + 128, one byte per residue of the round in the staged entry
+                } else if (direct) {  // r + 128, one byte per residue of the round in the staged entry
 #pragma unroll
                   for (uint32_t b = 0; b < kBatch / 16; b++)
 #pragma unroll
@@ -919,9 +1042,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         epi_bar();  // every residue of the round is staged
         const SW* sp = staging + lane_sid;
-        if (ok && pv && g.direct) {
+        if (ok && pv && direct) {
           // pairs of entries: one staging load, one half2 store per residue
-          __half* planes = reinterpret_cast<__half*>(g.out) + ((uint64_t)(rd * NA) << (g.fa + g.fb)) + tile_base;
+          __half* planes = reinterpret_cast<__half*>(out) + ((uint64_t)(rd * NA) << (fa + fb)) + tile_base;
           for (uint32_t e0 = et; e0 < (kTileM * TN) / 2; e0 += 4 * kEpiThreads) {
             uint32_t adr[4], w0[4], w1[4];  // the pair's staged bytes: entry o in w0, o + 1 in w1 (NA = 4) or both in w0
 #pragma unroll
@@ -941,18 +1064,18 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
 #pragma unroll
             for (uint32_t ra = 0; ra < NA; ra++) {
-              __half* pl = planes + ((uint64_t)ra << (g.fa + g.fb));
+              __half* pl = planes + ((uint64_t)ra << (fa + fb));
 #pragma unroll
               for (uint32_t u = 0; u < 4; u++) {
                 *reinterpret_cast<uint32_t*>(pl + adr[u]) = staged_half2<NA>(w0[u], w1[u], ra);
               }
             }
           }
-        } else if (ok && g.direct) {
+        } else if (ok && direct) {
           // fp16 planes of the next dense step's operand (representatives of
           // magnitude at most (p+1)/2), the entries' own order: plane of
           // residue rd NA + ra at out + (rd NA + ra) 2^(fa+fb) halves
-          __half* planes = reinterpret_cast<__half*>(g.out) + ((uint64_t)(rd * NA) << (g.fa + g.fb)) + tile_base;
+          __half* planes = reinterpret_cast<__half*>(out) + ((uint64_t)(rd * NA) << (fa + fb)) + tile_base;
           for (uint32_t e0 = et; e0 < kTileM * TN; e0 += 4 * kEpiThreads) {
             uint32_t adr[4];
             SW val[4];
@@ -964,17 +1087,17 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
 #pragma unroll
             for (uint32_t ra = 0; ra < NA; ra += 2) {  // two residues per half2
-              __half* pl = planes + ((uint64_t)ra << (g.fa + g.fb));
+              __half* pl = planes + ((uint64_t)ra << (fa + fb));
 #pragma unroll
               for (uint32_t u = 0; u < 4; u++) {
                 const uint32_t h2 = staged_half2_res((uint32_t)val[u], ra);
                 pl[adr[u]] = __ushort_as_half((unsigned short)(h2 & 0xFFFFu));
-                if (ra + 1 < NA) pl[((uint64_t)1 << (g.fa + g.fb)) + adr[u]] = __ushort_as_half((unsigned short)(h2 >> 16));
+                if (ra + 1 < NA) pl[((uint64_t)1 << (fa + fb)) + adr[u]] = __ushort_as_half((unsigned short)(h2 >> 16));
               }
             }
           }
         } else if (ok) {
-          uint8_t* outp = g.out + (g.log_split ? ((uint64_t)split << (g.fa + g.fb)) * RG : 0ull) + rd * NA +
+          uint8_t* outp = out + (log_split ? ((uint64_t)split << (fa + fb)) * RG : 0ull) + rd * NA +
                           tile_base * RG;
           // four entries (or pairs) per trip, their loads issued before their stores
           static_assert((kTileM * TN) % (4 * kEpiThreads) == 0, "whole trips of four");
@@ -1122,11 +1245,11 @@ Shape shape_of(const StepDesc& d) {
   return s;
 }
 
-// One CTA per SM for the g.n_items work items (at most `sms` CTAs); PAIR:
+// One CTA per SM for the n_items work items (at most `sms` CTAs); PAIR:
 // clusters of two CTAs, as many as fit at once (at most one item each).
 template <uint32_t TN, uint32_t RG, bool PAIR>
-int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mb, const tnc_p8::P8Args& g, int sms, uint32_t* err,
-                cudaStream_t st) {
+int launch_gemm(const tnc_p8::P8Prob* probs, uint32_t n, uint32_t n_items, const tnc_p8::P8Primes& pr, int sms,
+                uint32_t* err, cudaStream_t st) {
   auto kern = tnc_p8::p8_gemm_kernel<TN, RG, PAIR>;
   constexpr uint32_t smem = tnc_p8::Cfg<TN, RG, PAIR>::kSmemBytes;
   static int max_units = -1;  // CTAs (PAIR: clusters) resident at once
@@ -1154,9 +1277,9 @@ int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mb, const tnc_p8::P8Ar
     }
     max_units = units;
   }
-  const unsigned units = (unsigned)std::min<uint64_t>(g.n_items, (uint64_t)std::min(max_units, sms));
+  const unsigned units = (unsigned)std::min<uint64_t>(n_items, (uint64_t)std::min(max_units, sms));
   if (!PAIR) {
-    kern<<<units, tnc_p8::kThreads, smem, st>>>(ma, mb, g, err);
+    kern<<<units, tnc_p8::kThreads, smem, st>>>(probs, n, n_items, pr, err);
     return TNC_OK;
   }
   cudaLaunchConfig_t cfg{};
@@ -1171,22 +1294,28 @@ int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mb, const tnc_p8::P8Ar
   cfg.stream = st;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, ma, mb, g, err);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, probs, n, n_items, pr, err);
   if (e != cudaSuccess) return set_error(TNC_ERR_CUDA, std::string("p8 cluster launch: ") + cudaGetErrorString(e));
   return TNC_OK;
 }
 
+// Launch variants: tile widths 16, 32, 64, 128, 256, and 256 on CTA pairs.
+uint32_t variant_of(const Shape& s) {
+  uint32_t v = 0;
+  while ((16u << v) < s.tn) v++;
+  return s.pair ? 5u : v;
+}
+
 template <uint32_t RG>
-int launch_gemm_rg(uint32_t tn, bool pair, const CUtensorMap& ma, const CUtensorMap& mb, const tnc_p8::P8Args& g,
+int launch_variant(uint32_t v, const tnc_p8::P8Prob* probs, uint32_t n, uint32_t n_items, const tnc_p8::P8Primes& pr,
                    int sms, uint32_t* err, cudaStream_t st) {
-  switch (tn) {
-    case 16: return launch_gemm<16, RG, false>(ma, mb, g, sms, err, st);
-    case 32: return launch_gemm<32, RG, false>(ma, mb, g, sms, err, st);
-    case 64: return launch_gemm<64, RG, false>(ma, mb, g, sms, err, st);
-    case 128: return launch_gemm<128, RG, false>(ma, mb, g, sms, err, st);
-    default:
-      return pair ? launch_gemm<256, RG, true>(ma, mb, g, sms, err, st)
-                  : launch_gemm<256, RG, false>(ma, mb, g, sms, err, st);
+  switch (v) {
+    case 0: return launch_gemm<16, RG, false>(probs, n, n_items, pr, sms, err, st);
+    case 1: return launch_gemm<32, RG, false>(probs, n, n_items, pr, sms, err, st);
+    case 2: return launch_gemm<64, RG, false>(probs, n, n_items, pr, sms, err, st);
+    case 3: return launch_gemm<128, RG, false>(probs, n, n_items, pr, sms, err, st);
+    case 4: return launch_gemm<256, RG, false>(probs, n, n_items, pr, sms, err, st);
+    default: return launch_gemm<256, RG, true>(probs, n, n_items, pr, sms, err, st);
   }
 }
 
@@ -1241,38 +1370,42 @@ bool p8_operand_mn(const StepDesc& d, int side) {
   return row_side || s.tn >= 64;
 }
 
-uint64_t p8_scratch_bytes(const StepDesc& d, int rg) {
-  const uint32_t kp = std::max<uint32_t>(d.k, 6);
-  return 2ull * (uint64_t)rg * ((1ull << (d.ka + kp)) + (1ull << (d.kb + kp)));
-}
-
 uint64_t p8_part_bytes(const StepDesc& d, int rg) {
   const uint32_t ls = p8_split_log(d);
   return ls ? (uint64_t)rg << (d.c + ls) : 0;
 }
 
-int p8_launch(const StepDesc& d, const uint32_t* primes, uint32_t rg, uint8_t* arena, uint64_t arena_bytes,
-              uint32_t flags, void* scratch, uint8_t* part, uint32_t* dev_err, int sms, void* stream) {
-  cudaStream_t st = (cudaStream_t)stream;
-  if (rg != 1 && rg != 2 && rg != 4) return set_error(TNC_ERR_INVALID, "internal: residues per pass must be 1, 2 or 4");
-  tnc_p8::PackPrimes pp{};
-  for (uint32_t i = 0; i < 4; i++) pp.p[i] = primes[i < rg ? i : 0];
-  for (uint32_t i = 0; i < rg; i++)
-    if (primes[i] < 3 || primes[i] > 251) return set_error(TNC_ERR_INVALID, "tensor-core p8 steps need primes in [3, 251]");
+uint64_t p8_scratch_bytes(const P8Step& s, int rg) {
+  const uint32_t kp = std::max<uint32_t>(s.d.k, 6);
+  uint64_t b = 0;
+  if (!(s.flags & kP8DirectA)) b += 2ull * (uint64_t)rg << (s.d.ka + kp);
+  if (!(s.flags & kP8DirectB)) b += 2ull * (uint64_t)rg << (s.d.kb + kp);
+  return b;
+}
+
+size_t p8_step_bytes() { return sizeof(tnc_p8::P8Prob) + sizeof(tnc_p8::PackProb) + sizeof(tnc_p8::SplitProb); }
+uint32_t p8_max_steps() { return tnc_p8::kMaxProbs; }
+
+namespace {
+
+// One dense step's descriptors: operands and output in the arena, packed
+// planes at `scratch`, K-split partials at `part`.
+int fill_step(const P8Step& step, uint32_t rg, uint8_t* arena, uint64_t arena_bytes, uint8_t* scratch, uint8_t* part,
+              tnc_p8::P8Prob& g, tnc_p8::PackProb& pk, tnc_p8::SplitProb& sp, uint32_t& variant,
+              tnc_launch_counts& lc) {
+  const StepDesc& d = step.d;
   const Shape s = shape_of(d);
   const uint32_t ls = p8_split_log(d);
-  const uint64_t a_elems = 1ull << (s.fa + s.kp);
-  __half* a16 = (__half*)scratch;    // rg planes of a_elems
-  __half* b16 = a16 + rg * a_elems;  // rg planes of b_elems
+  variant = variant_of(s);
   const uint64_t a_off = s.swap ? d.b_off : d.a_off, b_off = s.swap ? d.a_off : d.b_off;
   // operands by tile side (row side = A unless swapped): read row-contiguous
   // (mn), and taken straight from the planes their producing dense step
   // wrote (direct), which occupy twice the entries' bytes
   const int side_a = s.swap ? 1 : 0, side_b = 1 - side_a;
   const bool mn_a = p8_operand_mn(d, side_a), mn_b = p8_operand_mn(d, side_b);
-  const bool dir_a = (flags & (side_a ? kP8DirectB : kP8DirectA)) != 0;
-  const bool dir_b = (flags & (side_b ? kP8DirectB : kP8DirectA)) != 0;
-  const bool dir_out = (flags & kP8DirectOut) != 0;
+  const bool dir_a = (step.flags & (side_a ? kP8DirectB : kP8DirectA)) != 0;
+  const bool dir_b = (step.flags & (side_b ? kP8DirectB : kP8DirectA)) != 0;
+  const bool dir_out = (step.flags & kP8DirectOut) != 0;
   if ((dir_a && !mn_a) || (dir_b && !mn_b) || (dir_out && ls))
     return set_error(TNC_ERR_INVALID, "internal: direct fp16 planes for an operand read K-contiguous");
   {  // every range the launch touches lies inside the arena
@@ -1281,31 +1414,29 @@ int p8_launch(const StepDesc& d, const uint32_t* primes, uint32_t rg, uint8_t* a
     if (a_off * rg + ea > arena_bytes || b_off * rg + eb > arena_bytes || d.c_off * rg + ec > arena_bytes)
       return set_error(TNC_ERR_INVALID, "internal: dense step range outside the arena");
   }
+  __half* a16 = reinterpret_cast<__half*>(scratch);  // rg planes of 2^(fa + kp)
+  __half* b16 = a16 + (dir_a ? 0 : (uint64_t)rg << (s.fa + s.kp));
   __half* pa = dir_a ? reinterpret_cast<__half*>(arena + a_off * rg) : a16;
   __half* pb = dir_b ? reinterpret_cast<__half*>(arena + b_off * rg) : b16;
   if (((uintptr_t)pa | (uintptr_t)pb) & 15u)
     return set_error(TNC_ERR_INVALID, "internal: fp16 operand planes not 16-byte aligned");
-  if (!dir_a || !dir_b) {  // the operands still in entry form, packed by one launch
-    const tnc_p8::PackOperand oa{arena + a_off * rg, a16, s.fa, dir_a ? 0u : (mn_a ? 2u : 1u)};
-    const tnc_p8::PackOperand ob{arena + b_off * rg, b16, s.fb, dir_b ? 0u : (mn_b ? 2u : 1u)};
-    const uint64_t n = ((dir_a ? 0 : (uint64_t)((1u << s.fa) + 63u) / 64u) +
-                        (dir_b ? 0 : (uint64_t)((1u << s.fb) + 63u) / 64u))
-                       << (s.kp - 6);
-    const unsigned blocks = (unsigned)std::min<uint64_t>(n, (uint64_t)sms * 16);
-    if (rg == 4) tnc_p8::p8_pack_kernel<4><<<blocks, 256, 0, st>>>(oa, ob, s.k, s.kp, pp);
-    else if (rg == 2) tnc_p8::p8_pack_kernel<2><<<blocks, 256, 0, st>>>(oa, ob, s.k, s.kp, pp);
-    else tnc_p8::p8_pack_kernel<1><<<blocks, 256, 0, st>>>(oa, ob, s.k, s.kp, pp);
-    launch_counts().p8_pack++;
-  }
-  CUtensorMap ma, mb;
-  int rc = mn_a ? make_map_mn(&ma, pa, 1ull << s.fa, 1ull << s.k, rg)
-                : make_map(&ma, pa, 1ull << s.fa, 1ull << s.kp, rg, tnc_p8::kTileM);
-  if (!rc)
-    rc = mn_b ? make_map_mn(&mb, pb, 1ull << s.fb, 1ull << s.k, rg)
-              : make_map(&mb, pb, 1ull << s.fb, 1ull << s.kp, rg, s.pair ? s.tn / 2 : s.tn);
-  if (rc) return rc;
-  tnc_p8::P8Args g;
+  std::memset(&pk, 0, sizeof(pk));
+  pk.a = tnc_p8::PackOperand{arena + a_off * rg, a16, s.fa, dir_a ? 0u : (mn_a ? 2u : 1u)};
+  pk.b = tnc_p8::PackOperand{arena + b_off * rg, b16, s.fb, dir_b ? 0u : (mn_b ? 2u : 1u)};
+  pk.k = s.k;
+  pk.kp = s.kp;
+  const uint64_t tiles = ((dir_a ? 0 : (uint64_t)((1u << s.fa) + 63u) / 64u) +
+                          (dir_b ? 0 : (uint64_t)((1u << s.fb) + 63u) / 64u))
+                         << (s.kp - 6);
+  if (tiles >= (1ull << 31)) return set_error(TNC_ERR_TOO_LARGE, "dense step has too many operand tiles");
+  pk.n_tiles = (uint32_t)tiles;
   std::memset(&g, 0, sizeof(g));
+  int rc = mn_a ? make_map_mn(&g.map_a, pa, 1ull << s.fa, 1ull << s.k, rg)
+                : make_map(&g.map_a, pa, 1ull << s.fa, 1ull << s.kp, rg, tnc_p8::kTileM);
+  if (!rc)
+    rc = mn_b ? make_map_mn(&g.map_b, pb, 1ull << s.fb, 1ull << s.k, rg)
+              : make_map(&g.map_b, pb, 1ull << s.fb, 1ull << s.kp, rg, s.pair ? s.tn / 2 : s.tn);
+  if (rc) return rc;
   g.fa = s.fa;
   g.fb = s.fb;
   g.k = s.kp;  // zero-padded shared values contribute nothing
@@ -1319,15 +1450,9 @@ int p8_launch(const StepDesc& d, const uint32_t* primes, uint32_t rg, uint8_t* a
   }
   if ((s.tiles << ls) >= (1ull << 31)) return set_error(TNC_ERR_TOO_LARGE, "dense step has too many tiles");
   g.n_items = (uint32_t)((s.pair ? s.tiles / 2 : s.tiles) << ls);
-  g.rg = rg;
   g.a_mn = mn_a ? 1u : 0u;
   g.b_mn = mn_b ? 1u : 0u;
   g.direct = dir_out ? 1u : 0u;
-  for (uint32_t i = 0; i < 4; i++) {
-    g.p[i] = pp.p[i];
-    g.pf[i] = (float)pp.p[i];
-    g.invp[i] = 1.0f / (float)pp.p[i];
-  }
   // output address weights (the output bit j comes from one operand's free bit)
   int op[64] = {0}, dst[64] = {0};
   if (d.nra != TNC_BITMAP) {
@@ -1362,33 +1487,126 @@ int p8_launch(const StepDesc& d, const uint32_t* primes, uint32_t rg, uint8_t* a
     for (size_t i = 0; i < bits.size(); i++) g.ebit[i] = bits[i].second;
   }
   g.pairs = (s.tn >= 32 && g.wm[0] == 1) ? 1u : 0u;  // output bit 0 is row bit 0
-  g.out = ls ? part : arena + d.c_off * rg;  // direct: the planes, same place (twice the bytes)
-  if (rg == 4) rc = launch_gemm_rg<4>(s.tn, s.pair, ma, mb, g, sms, dev_err, st);
-  else if (rg == 2) rc = launch_gemm_rg<2>(s.tn, s.pair, ma, mb, g, sms, dev_err, st);
-  else rc = launch_gemm_rg<1>(s.tn, s.pair, ma, mb, g, sms, dev_err, st);
-  if (rc) return rc;
-  {
-    tnc_launch_counts& lc = launch_counts();
-    lc.p8_gemm++;
-    if (ls) lc.p8_split++;
-    int w = 0;
-    while ((16u << w) < s.tn) w++;
-    lc.p8_tile_n[w]++;
-    const int32_t chunks = (int32_t)std::max<uint64_t>(1, ((1ull << s.kp) >> ls) / tnc_p8::kChunkK);
-    lc.p8_max_chunks = std::max(lc.p8_max_chunks, chunks);
-    if (s.swap) lc.p8_swapped++;
-    if (s.kp > s.k) lc.p8_padded++;
-    if (dir_out) lc.p8_direct_out++;
-    lc.p8_direct_in += (dir_a ? 1 : 0) + (dir_b ? 1 : 0);
-    lc.p8_mn += (mn_a ? 1 : 0) + (mn_b ? 1 : 0);
-    if (g.pairs) lc.p8_pairs++;
-    if (s.pair) lc.p8_cta_pair++;
+  uint8_t* out = arena + d.c_off * rg;               // direct: the planes, same place (twice the bytes)
+  g.out = ls ? part : out;
+  std::memset(&sp, 0, sizeof(sp));
+  sp.part = part;
+  sp.out = out;
+  sp.log_n = d.c + (rg == 4 ? 2u : rg == 2 ? 1u : 0u);
+  sp.log_split = ls;
+  if (tiles) lc.p8_pack++;
+  lc.p8_gemm++;
+  if (ls) lc.p8_split++;
+  lc.p8_tile_n[std::min<uint32_t>(variant, 4)]++;
+  lc.p8_max_chunks = std::max(lc.p8_max_chunks,
+                              (int32_t)std::max<uint64_t>(1, ((1ull << s.kp) >> ls) / tnc_p8::kChunkK));
+  if (s.swap) lc.p8_swapped++;
+  if (s.kp > s.k) lc.p8_padded++;
+  if (dir_out) lc.p8_direct_out++;
+  lc.p8_direct_in += (dir_a ? 1 : 0) + (dir_b ? 1 : 0);
+  lc.p8_mn += (mn_a ? 1 : 0) + (mn_b ? 1 : 0);
+  if (g.pairs) lc.p8_pairs++;
+  if (s.pair) lc.p8_cta_pair++;
+  return TNC_OK;
+}
+
+// Appends the descriptors `v` to the staging buffer; returns their offset
+// (every descriptor is a multiple of 64 bytes, the buffer 64-byte aligned).
+template <typename T>
+size_t put_descs(std::vector<char>& host, const std::vector<T>& v) {
+  static_assert(sizeof(T) % 64 == 0, "descriptors keep 64-byte alignment");
+  const size_t at = host.size();
+  host.resize(at + v.size() * sizeof(T));
+  if (!v.empty()) std::memcpy(host.data() + at, v.data(), v.size() * sizeof(T));
+  return at;
+}
+
+}  // namespace
+
+int p8_batch(const P8Step* steps, int n, uint32_t rg, uint8_t* arena, uint64_t arena_bytes, uint8_t* scratch,
+             uint8_t* part, std::vector<char>& host, P8Batch& b) {
+  using namespace tnc_p8;
+  if (rg != 1 && rg != 2 && rg != 4) return set_error(TNC_ERR_INVALID, "internal: residues per pass must be 1, 2 or 4");
+  if (n > (int)kMaxProbs) return set_error(TNC_ERR_INVALID, "internal: too many dense steps in a launch");
+  b = P8Batch{};
+  std::vector<P8Prob> probs[6];
+  std::vector<PackProb> packs;
+  std::vector<SplitProb> splits;
+  uint64_t tiles = 0, blocks = 0, items[6] = {0};
+  for (int i = 0; i < n; i++) {
+    P8Prob g;
+    PackProb pk;
+    SplitProb sp;
+    uint32_t v = 0;
+    if (int rc = fill_step(steps[i], rg, arena, arena_bytes, scratch, part, g, pk, sp, v, b.counts)) return rc;
+    scratch += p8_scratch_bytes(steps[i], (int)rg);
+    if (sp.log_split) {
+      part += p8_part_bytes(steps[i].d, (int)rg);
+      sp.block_lo = (uint32_t)blocks;
+      blocks += ((1ull << sp.log_n) + 1023) / 1024;
+      splits.push_back(sp);
+    }
+    if (pk.n_tiles) {
+      pk.tile_lo = (uint32_t)tiles;
+      tiles += pk.n_tiles;
+      packs.push_back(pk);
+    }
+    g.item_lo = (uint32_t)items[v];
+    items[v] += g.n_items;
+    probs[v].push_back(g);
   }
-  if (ls) {
-    const uint64_t n = (uint64_t)rg << d.c;
-    tnc_p8::p8_split_final_kernel<<<(unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)sms * 8), 256, 0, st>>>(
-        part, arena + d.c_off * rg, d.c, ls, rg, make_uint4(pp.p[0], pp.p[1], pp.p[2], pp.p[3]));
+  if (std::max({tiles, blocks, *std::max_element(items, items + 6)}) >= (1ull << 31))
+    return set_error(TNC_ERR_TOO_LARGE, "dense steps of a level have too many tiles");
+  b.pack_n = (uint32_t)packs.size();
+  b.pack_tiles = (uint32_t)tiles;
+  b.pack_off = put_descs(host, packs);
+  for (int v = 0; v < 6; v++) {
+    b.gemm[v].n = (uint32_t)probs[v].size();
+    b.gemm[v].items = (uint32_t)items[v];
+    b.gemm[v].off = put_descs(host, probs[v]);
   }
+  b.split_n = (uint32_t)splits.size();
+  b.split_blocks = (uint32_t)blocks;
+  b.split_off = put_descs(host, splits);
+  return TNC_OK;
+}
+
+int p8_run(const P8Batch& b, const char* dev, const uint32_t* primes, uint32_t rg, uint32_t* dev_err, int sms,
+           void* stream) {
+  using namespace tnc_p8;
+  cudaStream_t st = (cudaStream_t)stream;
+  PackPrimes pp{};
+  P8Primes pr{};
+  for (uint32_t i = 0; i < 4; i++) {
+    pp.p[i] = primes[i < rg ? i : 0];
+    pr.pf[i] = (float)pp.p[i];
+    pr.invp[i] = 1.0f / (float)pp.p[i];
+    if (pp.p[i] < 3 || pp.p[i] > 251) return set_error(TNC_ERR_INVALID, "tensor-core p8 steps need primes in [3, 251]");
+  }
+  if (b.pack_n) {
+    const PackProb* p = reinterpret_cast<const PackProb*>(dev + b.pack_off);
+    const unsigned blocks = (unsigned)std::min<uint64_t>(b.pack_tiles, (uint64_t)sms * 16);
+    if (rg == 4) p8_pack_kernel<4><<<blocks, 256, 0, st>>>(p, b.pack_n, b.pack_tiles, pp);
+    else if (rg == 2) p8_pack_kernel<2><<<blocks, 256, 0, st>>>(p, b.pack_n, b.pack_tiles, pp);
+    else p8_pack_kernel<1><<<blocks, 256, 0, st>>>(p, b.pack_n, b.pack_tiles, pp);
+  }
+  for (uint32_t v = 6; v-- > 0;) {  // wide tiles (the long steps) first
+    if (!b.gemm[v].n) continue;
+    const P8Prob* p = reinterpret_cast<const P8Prob*>(dev + b.gemm[v].off);
+    int rc;
+    if (rg == 4) rc = launch_variant<4>(v, p, b.gemm[v].n, b.gemm[v].items, pr, sms, dev_err, st);
+    else if (rg == 2) rc = launch_variant<2>(v, p, b.gemm[v].n, b.gemm[v].items, pr, sms, dev_err, st);
+    else rc = launch_variant<1>(v, p, b.gemm[v].n, b.gemm[v].items, pr, sms, dev_err, st);
+    if (rc) return rc;
+  }
+  if (b.split_n)
+    p8_split_final_kernel<<<b.split_blocks, 256, 0, st>>>(reinterpret_cast<const SplitProb*>(dev + b.split_off),
+                                                          b.split_n, rg, make_uint4(pp.p[0], pp.p[1], pp.p[2], pp.p[3]));
+  tnc_launch_counts& lc = launch_counts();
+  const int32_t chunks = std::max(lc.p8_max_chunks, b.counts.p8_max_chunks);
+  for (size_t i = 0; i < sizeof(lc) / sizeof(int32_t); i++)
+    reinterpret_cast<int32_t*>(&lc)[i] += reinterpret_cast<const int32_t*>(&b.counts)[i];
+  lc.p8_max_chunks = chunks;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return set_error(TNC_ERR_CUDA, std::string("p8 launch: ") + cudaGetErrorString(e));
   return TNC_OK;

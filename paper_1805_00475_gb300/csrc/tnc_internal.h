@@ -162,7 +162,6 @@ bool tc_eligible(const StepDesc& d);
 bool p8_eligible(const StepDesc& d);
 uint32_t p8_split_log(const StepDesc& d);
 uint32_t p8_tile_width(const StepDesc& d);
-uint64_t p8_scratch_bytes(const StepDesc& d, int rg);
 uint64_t p8_part_bytes(const StepDesc& d, int rg);
 // Operand `side` (0: A, 1: B) of a dense step read row-contiguous (MN-major).
 bool p8_operand_mn(const StepDesc& d, int side);
@@ -171,13 +170,36 @@ bool p8_operand_mn(const StepDesc& d, int side);
 // from planes its producer wrote (kP8DirectA / kP8DirectB); such a tensor
 // takes twice its entries' bytes in the arena.
 constexpr uint32_t kP8DirectOut = 1, kP8DirectA = 2, kP8DirectB = 4;
-// One dense step for all rg residues (primes[0..rg)) of a pass whose entries
-// hold rg residues of one byte each: the operands not already in fp16 planes
-// packed by one launch, then one GEMM launch that computes every residue of
-// each output tile and writes whole entries (or planes).  arena_bytes bounds
-// every range the step touches (checked before any launch).
-int p8_launch(const StepDesc& d, const uint32_t* primes, uint32_t rg, uint8_t* arena, uint64_t arena_bytes,
-              uint32_t flags, void* scratch, uint8_t* part, uint32_t* dev_err, int sms, void* stream);
+struct P8Step {
+  StepDesc d;
+  uint32_t flags;
+};
+uint64_t p8_scratch_bytes(const P8Step& s, int rg);  // fp16 planes of the operands to pack
+// Dense steps launched together (independent ones: of one tree level), for
+// all rg residues of a pass whose entries hold rg residues of one byte each:
+// one launch packs the operands not already in fp16 planes, one GEMM launch
+// per tile width computes every residue of each output tile and writes whole
+// entries (or planes), one launch adds the K-split partials.  p8_batch appends
+// the launches' descriptors (at most n p8_step_bytes()) to `host`, which the
+// caller copies to 64-byte aligned device memory, and lays the steps' planes
+// and partials out side by side from `scratch` and `part`; arena_bytes bounds
+// every range the steps touch.  p8_run launches them for the primes of a pass;
+// dev: the device copy of `host`.
+struct P8Batch {
+  struct Gemm {
+    uint32_t n, items;
+    size_t off;
+  } gemm[6];  // tile widths 16, 32, 64, 128, 256, and 256 on CTA pairs
+  uint32_t pack_n, pack_tiles, split_n, split_blocks;
+  size_t pack_off, split_off;
+  tnc_launch_counts counts;
+};
+size_t p8_step_bytes();
+uint32_t p8_max_steps();
+int p8_batch(const P8Step* steps, int n, uint32_t rg, uint8_t* arena, uint64_t arena_bytes, uint8_t* scratch,
+             uint8_t* part, std::vector<char>& host, P8Batch& b);
+int p8_run(const P8Batch& b, const char* dev, const uint32_t* primes, uint32_t rg, uint32_t* dev_err, int sms,
+           void* stream);
 size_t tc_step_bytes();
 void tc_make_step(const StepDesc& d, uint32_t p, void* out);
 uint32_t tc_split_log(const StepDesc& d);

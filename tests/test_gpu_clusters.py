@@ -74,7 +74,7 @@ def test_one_launch_contraction(name, R, wide):
         r = tnc.contract(p, n_residues=R, primes=primes)
         lc = tnc.last_launch_counts()
         groups = bin(R % 4).count("1") + R // 4
-        assert lc["level"] == groups and lc["crt"] == 1 and lc["grid_step"] == lc["splitk"] == lc["outer"] == 0
+        assert lc["level"] == groups and lc["crt"] == 1 and lc["grid_step"] == lc["outer"] == 0
         assert r.residues.tolist() == want.residues.tolist() and r.counts == want.counts and r.flags == want.flags
     if f.n_vars <= 60:
         assert r.residues.tolist() == oracle.residues(oracle.count(f), r.primes)
