@@ -74,10 +74,12 @@ extern "C" {
 /* ---- arithmetic paths ---------------------------------------------------- */
 #define TNC_PATH_INT64 0 /* CUDA cores: u32 residues, 64-bit multiply-accumulate */
 #define TNC_PATH_TC 1    /* dense steps (k >= 6 shared bonds, one side >= 2^7 and the
-                            other >= 2^5 free entries) as exact 8-bit-limb GEMMs on the
-                            tcgen05 tensor cores (fp16 limbs, fp32 accumulation below
-                            2^24, K chunks of 64); other steps as TNC_PATH_INT64; one
-                            pass per residue.  tnc_contract only. */
+                            other >= 2^5 free entries) as exact GEMMs on the tcgen05
+                            tensor cores: the integer products modulo 9 to 12 primes
+                            <= 251 (fp16 operands, fp32 accumulation below 2^24), the
+                            residues mod p rebuilt from them; other steps as
+                            TNC_PATH_INT64.  Workspace: the larger of both paths'
+                            (tnc_workspace_bytes), or tnc_workspace_bytes_opts. */
 #define TNC_PATH_TC_P8 2 /* residues modulo primes p <= 251 (Sec. 3.2's exact counts
                             from more, smaller residues): each residue is one 8-bit
                             limb, taken balanced (|r| <= 125) and exact in fp16.
@@ -313,11 +315,11 @@ int tnc_last_contract_time(double* device_ms);
  * an extraction and the CRT, and its long shared sums under splitk.  p8_*
  * counts dense steps: one launch may serve several of a tree level. */
 typedef struct {
-  int32_t leaf_fill;      /* leaf tensors (Eq. var, Eq. or, Eq. 1in3, ...)           */
+  int32_t leaf_fill;      /* leaf tensors (Eq. var, ...); TNC_PATH_TC: per residue    */
   int32_t level;          /* one launch for all small steps of a tree level           */
   int32_t grid_step;      /* large steps of a tree level over the whole GPU          */
   int32_t splitk;         /* split-K steps on CUDA cores (a partial + final pair)    */
-  int32_t tc_gemm;        /* TNC_PATH_TC dense steps (tcgen05 limb GEMM launches)     */
+  int32_t tc_gemm;        /* TNC_PATH_TC dense steps (tcgen05 GEMMs)                  */
   int32_t tc_split;       /*   of which split over K (partials summed after)          */
   int32_t p8_pack;        /* TNC_PATH_TC_P8 dense steps with operands to pack          */
   int32_t p8_gemm;        /* TNC_PATH_TC_P8 dense steps (tcgen05 GEMMs)               */

@@ -304,7 +304,8 @@ tnc_dev::OuterStep make_outer_step(const StepDesc& d) {
 struct Foot {
   size_t leaves = 0, tables = 0, nseq = 0, nlvl = 0, n_dense = 0;
   uint64_t n_out = 0, arena = 0, part = 0, p8 = 0;
-  // TNC_PATH_TC_P8: planes and partials of all dense steps of a tree level
+  // dense steps of a tree level on the tensor-core paths: planes, and partials
+  // or small residues
   std::vector<uint64_t> lvl_p8, lvl_part;
   void add(const Foot& f) {
     leaves += f.leaves;
@@ -329,6 +330,11 @@ struct Foot {
 // partials fit; up to these sizes the sections grow beyond the largest single
 // step's for that (steps that need more fill the GPU by themselves).
 constexpr uint64_t kGroupPlanes = 256ull << 20, kGroupParts = 64ull << 20;
+// TNC_PATH_TC keeps all residues of a pass together where these allow it (its
+// planes take 18 to 24 bytes per residue and operand entry, its small residues
+// 9 to 12 per output entry: residue by residue the output's 16-byte entries
+// would be written a quarter at a time).
+constexpr uint64_t kTcPlanes = 2048ull << 20, kTcBytes = 1024ull << 20;
 
 // Step i of a plan's level schedule as TNC_PATH_TC_P8 runs it: direct planes
 // of its operands and output.
@@ -338,6 +344,19 @@ uint32_t p8_flags(const Lowered& lw, uint32_t i) {
          (sb >= 0 && lw.p8_direct[sb] ? kP8DirectB : 0u);
 }
 
+// Bytes that the CUDA-core layout sets aside for a dense step's K split and
+// (per residue) descriptor.  No kernel uses them any more; they stay because
+// tnc_contract_noalloc takes or refuses a plan by this layout's size.
+uint64_t kept_split_bytes(const StepDesc& d) {
+  const bool swap = !(d.ka >= 7 && d.kb >= 5);
+  const uint32_t fa = swap ? d.kb : d.ka, fb = swap ? d.ka : d.kb;
+  const uint64_t tiles = (1ull << (fa - 7)) << (fb - 5);
+  uint32_t ls = 0;
+  while ((tiles << ls) < 304 && d.k - ls > 7 && (1ull << (d.c + ls + 1)) <= (1ull << 24)) ls++;
+  return ls ? 4ull << (d.c + ls) : 0;
+}
+constexpr size_t kKeptDenseBytes = 600;
+
 Foot foot_of(const tnc_plan_t* p, int R, int path) {
   const int rg_max = R >= 4 ? 4 : (R >= 2 ? 2 : 1);
   Foot f;
@@ -346,26 +365,32 @@ Foot foot_of(const tnc_plan_t* p, int R, int path) {
   f.nseq = p->low.seq_steps.size();
   f.nlvl = p->low.lvl_steps.size();
   f.n_out = 1ull << p->net.open_vars.size();
-  const bool p8 = path == TNC_PATH_TC_P8;
-  if (!p8)
-    for (const StepDesc& d : p->low.seq_steps) f.n_dense += tc_eligible(d) ? 1 : 0;
+  const bool p8 = path == TNC_PATH_TC_P8, tc = path == TNC_PATH_TC;
   for (size_t l = 0; l + 1 < p->low.lvl_start.size(); l++) {
     uint64_t sum_p8 = 0, sum_part = 0;
     for (uint32_t i = p->low.lvl_start[l]; i < p->low.lvl_start[l + 1]; i++) {
       const StepDesc& d = p->low.lvl_steps[i];
       if (splitk_log(d) > 0)
         f.part = std::max<uint64_t>(f.part, (1ull << (d.c + splitk_log(d))) * rg_max * sizeof(uint32_t));
-      if (tc_eligible(d) && tc_split_log(d) > 0)
-        f.part = std::max<uint64_t>(f.part, (1ull << (d.c + tc_split_log(d))) * sizeof(uint32_t));
+      uint64_t planes = 0, parts = 0, units = 1;
       if (p8 && p8_eligible(d)) {
-        const uint64_t planes = p8_scratch_bytes(P8Step{d, p8_flags(p->low, i)}, rg_max);
-        const uint64_t parts = p8_part_bytes(d, rg_max);
+        planes = p8_scratch_bytes(P8Step{d, p8_flags(p->low, i)}, rg_max);
+        parts = p8_part_bytes(d, rg_max);
         f.n_dense++;
-        f.part = std::max<uint64_t>(f.part, parts);
-        f.p8 = std::max<uint64_t>(f.p8, planes);
-        sum_p8 += planes;
-        sum_part += parts;
+      } else if (!p8 && tc_eligible(d)) {
+        f.n_dense++;
+        if (tc) {
+          planes = tc_plane_bytes(d);
+          parts = tc_byte_bytes(d);
+          units = rg_max;
+        } else {
+          f.part = std::max<uint64_t>(f.part, kept_split_bytes(d));
+        }
       }
+      f.part = std::max<uint64_t>(f.part, parts);
+      f.p8 = std::max<uint64_t>(f.p8, planes);
+      sum_p8 += planes * units;
+      sum_part += parts * units;
     }
     f.lvl_p8.push_back(sum_p8);
     f.lvl_part.push_back(sum_part);
@@ -390,12 +415,15 @@ SeqLayout layout_of(const Foot& f, int R, int path) {
   sect(s.off_steps, std::max(f.nseq, f.nlvl) * sizeof(GridStep));
   sect(s.off_small, f.nlvl * sizeof(StepDesc));
   uint64_t part = f.part, p8 = f.p8;
-  for (uint64_t v : f.lvl_part) part = std::max(part, std::min(v, kGroupParts));
-  for (uint64_t v : f.lvl_p8) p8 = std::max(p8, std::min(v, kGroupPlanes));
+  const bool tc = path == TNC_PATH_TC;
+  for (uint64_t v : f.lvl_part) part = std::max(part, std::min(v, tc ? kTcBytes : kGroupParts));
+  for (uint64_t v : f.lvl_p8) p8 = std::max(p8, std::min(v, tc ? kTcPlanes : kGroupPlanes));
   s.part_bytes = part;
   s.p8_bytes = p8;
-  // (p8 descriptors hold addresses for a pass's residues per entry: 4, 2 and 1)
-  sect(s.off_tc, path == TNC_PATH_TC_P8 ? f.n_dense * 3 * p8_step_bytes() : f.n_dense * R * tc_step_bytes());
+  // (dense descriptors hold addresses for a pass's residues per entry: 4, 2 and 1)
+  sect(s.off_tc, path == TNC_PATH_TC_P8 ? f.n_dense * 3 * p8_step_bytes()
+                 : path == TNC_PATH_TC ? f.n_dense * 7 * tc_unit_bytes()
+                                       : f.n_dense * R * kKeptDenseBytes);
   sect(s.off_part, part);
   sect(s.off_err, 64);
   sect(s.off_results, f.n_out * R * sizeof(uint32_t));
@@ -782,7 +810,7 @@ int solo_enqueue(const SoloPack& s, const SeqLayout& L, const Arith& a, char* ws
 
 extern "C" size_t tnc_workspace_bytes(const tnc_plan_t* plan, int32_t n_residues) {
   if (!plan || n_residues < 1 || n_residues > 16) return 0;
-  return seq_layout(plan, n_residues).total;
+  return std::max(seq_layout(plan, n_residues).total, seq_layout(plan, n_residues, TNC_PATH_TC).total);
 }
 
 extern "C" void tnc_set_step_timing(int32_t on) { g_time_dense = on != 0; }
@@ -930,20 +958,10 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
     tables.insert(tables.end(), lw.leaf_tables.begin(), lw.leaf_tables.end());
     n_lev = std::max(n_lev, lw.lvl_start.empty() ? (size_t)0 : lw.lvl_start.size() - 1);
   }
-  // residue groups: limb tensor-core passes carry one residue per entry; the
-  // 8-bit-prime path keeps groups of 4 and runs its dense steps per residue
-  Groups groups = a.groups;
-  if (tc && !p8) {
-    groups = Groups();
-    for (int r = 0; r < a.R; r++) {
-      groups.rg.push_back(1);
-      groups.col.push_back(r);
-    }
-  }
+  const Groups& groups = a.groups;
   // the group's steps by level: small ones (one index space per level across
   // the plans), big, one-small-operand, split-K and dense ones: each kind one
-  // launch per level (split-K steps and dense steps as many as their scratch
-  // holds; limb dense steps one by one)
+  // launch per level (split-K and dense steps as many as their scratch holds)
   struct Range {
     uint32_t lo, n, blocks, finals;
   };
@@ -951,16 +969,14 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
     uint32_t small_lo = 0, small_n = 0, small_work = 0;
     Range grid{}, outer{};
     std::vector<Range> split;
-    std::vector<std::pair<int, StepDesc>> limb;      // slot in the limb descriptors, step
     std::vector<std::pair<uint32_t, uint32_t>> p8;   // ranges of p8 steps launched together
+    std::vector<StepDesc> dense;                     // TNC_PATH_TC dense steps
   };
   std::vector<Level> lev(n_lev);
   std::vector<GridStep> gsteps;
   std::vector<tnc_dev::OuterStep> outers;
   std::vector<StepDesc> small;
   std::vector<P8Step> p8steps;
-  std::vector<char> tcbuf;
-  size_t nd = 0;
   const int rg_max = groups.rg[0];
   for (size_t l = 0; l < n_lev; l++) {
     Level& lv = lev[l];
@@ -983,7 +999,7 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
         if (p8 && p8_eligible(d)) {
           p8steps.push_back(P8Step{d, flags});
         } else if (tc && !p8 && tc_eligible(d)) {
-          lv.limb.push_back({(int)nd++, d});
+          lv.dense.push_back(d);
         } else if (flags) {
           return set_error(TNC_ERR_INVALID, "internal: direct fp16 planes on a CUDA-core step");
         } else if (outer_eligible(d)) {
@@ -1042,31 +1058,56 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
   const size_t at_small = put(small.data(), small.size() * sizeof(StepDesc));
   const size_t at_grid = put(gsteps.data(), gsteps.size() * sizeof(GridStep));
   const size_t at_outer = put(outers.data(), outers.size() * sizeof(tnc_dev::OuterStep));
-  size_t at_tc = 0;
-  if (nd) {
-    tcbuf.assign(nd * a.R * tc_step_bytes(), 0);
-    for (const Level& lv : lev)
-      for (const auto& x : lv.limb)
-        for (int r = 0; r < a.R; r++)
-          tc_make_step(x.second, a.primes[r], tcbuf.data() + ((size_t)x.first * a.R + r) * tc_step_bytes());
-    at_tc = put(tcbuf.data(), tcbuf.size());
-  }
-  // p8 descriptors, for each number of residues per entry that a pass has
+  // dense descriptors, for each number of residues per entry that a pass has
   uint32_t* part = (uint32_t*)(ws + L.off_part);
   std::vector<P8Batch> p8batches[5];
-  size_t at_p8[5] = {0};
+  struct TcLaunch {
+    TcBatch b;
+    StepDesc first;
+  };
+  std::vector<std::vector<TcLaunch>> tcbatches[5];  // by level
+  size_t at_dense[5] = {0};
   for (int rg : {4, 2, 1}) {
-    if (!p8 || std::find(groups.rg.begin(), groups.rg.end(), rg) == groups.rg.end()) continue;
+    if (!tc || std::find(groups.rg.begin(), groups.rg.end(), rg) == groups.rg.end()) continue;
     std::vector<char> host;
-    for (const Level& lv : lev)
+    const uint64_t arena_bytes = (uint64_t)(L.total - L.off_arena);
+    for (const Level& lv : lev) {
       for (const auto& r : lv.p8) {
         p8batches[rg].emplace_back();
         rc = p8_batch(p8steps.data() + r.first, (int)(r.second - r.first), (uint32_t)rg, (uint8_t*)(ws + L.off_arena),
-                      (uint64_t)(L.total - L.off_arena), (uint8_t*)(ws + L.off_p8), (uint8_t*)part, host,
-                      p8batches[rg].back());
+                      arena_bytes, (uint8_t*)(ws + L.off_p8), (uint8_t*)part, host, p8batches[rg].back());
         if (rc) return rc;
       }
-    at_p8[rg] = put(host.data(), host.size());
+      tcbatches[rg].emplace_back();
+      std::vector<TcUnit> units;  // steps with all residues of the pass, or a residue of a step each
+      uint64_t planes = 0, bytes = 0;
+      uint32_t nr = 0;
+      auto flush = [&]() -> int {
+        if (units.empty()) return TNC_OK;
+        tcbatches[rg].back().push_back(TcLaunch{TcBatch{}, units[0].d});
+        const int rc2 = tc_batch(units.data(), (int)units.size(), nr, (uint32_t)rg, (uint32_t*)(ws + L.off_arena),
+                                 arena_bytes, (uint8_t*)(ws + L.off_p8), (uint8_t*)part, host,
+                                 tcbatches[rg].back().back().b);
+        units.clear();
+        planes = bytes = 0;
+        return rc2;
+      };
+      for (const StepDesc& d : lv.dense) {
+        const uint64_t pl = tc_plane_bytes(d), by = tc_byte_bytes(d);
+        const uint32_t m = rg * pl <= L.p8_bytes && rg * by <= L.part_bytes ? (uint32_t)rg : 1u;
+        for (uint32_t r = 0; r < (uint32_t)rg; r += m) {
+          if (m != nr || planes + m * pl > L.p8_bytes || bytes + m * by > L.part_bytes ||
+              units.size() >= tc_max_units(m) || (g_time_dense && r == 0))
+            if ((rc = flush())) return rc;
+          nr = m;
+          units.push_back(TcUnit{d, r});
+          planes += m * pl;
+          bytes += m * by;
+        }
+      }
+      if ((rc = flush())) return rc;
+    }
+    at_dense[rg] = put(host.data(), host.size());
   }
   if (stage.size() > L.off_part) return set_error(TNC_ERR_INVALID, "internal: descriptors beyond their section");
   CUDA_TRY(cudaMemcpyAsync(ws, stage.data(), stage.size(), cudaMemcpyHostToDevice, st));
@@ -1120,11 +1161,13 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
       W* arena = reinterpret_cast<W*>(ws + L.off_arena);
       const int nl = (int)leaves.size();
       size_t next_p8 = 0;
+      const std::vector<char> dense_consts =
+          tc && !p8 ? tc_consts(a.primes.data() + groups.col[gi], RG) : std::vector<char>();
       tnc_dev::leaf_fill_kernel<RG, W><<<std::min(nl, sms * 8), 64, 0, st>>>(
           (const LeafDesc*)(ws + at_leaves), nl, (const uint32_t*)(ws + at_tables), arena, mg);
-      g_launches.leaf_fill++;
+      g_launches.leaf_fill += tc && !p8 ? RG : 1;  // (recorded per residue on TNC_PATH_TC)
       // a timed dense launch: events around it and its shape
-      auto timed = [&](const StepDesc& d, auto&& launch) -> int {
+      auto timed = [&](const StepDesc& d, uint32_t residues, auto&& launch) -> int {
         cudaEvent_t ev[2] = {nullptr, nullptr};
         if (g_time_dense) {
           CUDA_TRY(cudaEventCreate(&ev[0]));
@@ -1141,9 +1184,9 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
           info.rows_log2 = d.ka;
           info.cols_log2 = d.kb;
           info.k_log2 = d.k;
-          info.residues = RG;
-          info.tile_n = p8 ? (int32_t)p8_tile_width(d) : 32;
-          info.log_split = (int32_t)(p8 ? p8_split_log(d) : tc_split_log(d));
+          info.residues = (int32_t)residues;
+          info.tile_n = (int32_t)p8_tile_width(d);
+          info.log_split = (int32_t)p8_split_log(d);
           dense_info.push_back(info);
         }
         return TNC_OK;
@@ -1169,20 +1212,19 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
           tnc_dev::splitk_final_kernel<RG, W, N30><<<r.finals, 256, 0, st>>>(d_steps + r.lo, r.n, arena, part, mg);
           g_launches.splitk++;
         }
-        for (const auto& x : lv.limb) {
-          NvtxRange dense_range("tnc dense step");
-          if (RG != 1) return set_error(TNC_ERR_INVALID, "internal: tensor-core step in a multi-residue pass");
-          const char* dstep = ws + at_tc + ((size_t)x.first * a.R + groups.col[gi]) * tc_step_bytes();
-          if (int rc2 = timed(x.second, [&] {
-                return tc_launch(dstep, x.second, reinterpret_cast<uint32_t*>(arena), part, d_err, st);
-              }))
-            return rc2;
-        }
+        if (tc && !p8)
+          for (const TcLaunch& x : tcbatches[RG][&lv - lev.data()]) {
+            NvtxRange dense_range("tnc dense steps");
+            if (int rc2 = timed(x.first, x.b.n_units * x.b.nr, [&] {
+                  return tc_run(x.b, ws + at_dense[RG], dense_consts, RG, d_err, sms, st);
+                }))
+              return rc2;
+          }
         for (const auto& r : lv.p8) {
           NvtxRange dense_range("tnc dense steps");
           const P8Batch& b = p8batches[RG][next_p8++];
-          if (int rc2 = timed(p8steps[r.first].d, [&] {
-                return p8_run(b, ws + at_p8[RG], a.primes.data() + groups.col[gi], RG, d_err, sms, st);
+          if (int rc2 = timed(p8steps[r.first].d, RG, [&] {
+                return p8_run(b, ws + at_dense[RG], a.primes.data() + groups.col[gi], RG, d_err, sms, st);
               }))
             return rc2;
         }

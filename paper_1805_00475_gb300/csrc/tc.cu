@@ -1,32 +1,30 @@
-// Dense pairwise steps on the 5th-generation tensor cores (tcgen05), exact.
+// Dense pairwise steps of TNC_PATH_TC on the 5th-generation tensor cores,
+// exact modulo primes below 2^31.
 //
-// A step C[m,n] = sum_q A[m,q] B[n,q] mod p (A: M x K, B: N x K, residues
-// below 2^30; the bit maps of the lowering make both operands plain
-// column-major matrices) is computed from 8-bit limbs:
-//   a = sum_i a_i 256^i,  b = sum_j b_j 256^j,  0 <= a_i, b_j <= 255,
-//   C = sum_s 256^s C_s mod p,  C_s = sum_{i+j=s} A_i B_j^T   (s = 0..6).
-// Limb values are exact in bf16 and products below 2^16, so C_s accumulates
-// exactly in the fp32 tensor-core accumulators as long as it stays below
-// 2^24: at most 4 limb pairs share an s, 4 * 255^2 * 64 < 2^24, so K is
-// processed in chunks of 64 and every chunk's C_s is folded into 64-bit
-// integer accumulators, C += sum_s 256^s C_s mod p.  No precision is lost.
-// The tensor cores run kind::f16 with fp16 inputs and fp32 accumulation: the
-// 8-bit integer form (kind::i8) does not exist for sm_103a, and fp16 carries
-// 8-bit limbs exactly (a limb v becomes the half 1024 + v by
-// bit operations, minus 1024 in one packed subtract).
+// A step C[m,n] = sum_q A[m,q] B[n,q] mod p (A: M x K, B: N x K, u32 residues;
+// the bit maps of the lowering make both operands plain column-major
+// matrices) is an integer product S = A B^T with 0 <= S < 2^k (p-1)^2, taken
+// mod p at the end.  S is computed modulo small primes q_1..q_n (the largest
+// below 2^8) whose product exceeds it, each product with exact fp16 operands
+// on the GEMM of the 8-bit-prime path (tc_p8.cu), and rebuilt modulo p by the
+// Chinese remainder theorem.  For primes below 2^30 and k <= 10 that is 9
+// products; splitting the residues into 8-bit limbs (fp16 exact, but at most 64
+// shared values to an exact fp32 sum) takes 16 products, and 7 accumulators
+// folded into integers every 64 shared values.  The dense steps of a cubic VC
+// formula with n = 160 (2^34.4 products per residue, 4 residues): 7.09 ms with
+// limbs (operands staged by all threads, tensor pipe 15 % active), 3.58 ms
+// this way: GEMMs 2.17 (1.37 PFLOP/s on the largest step, 2^13 x 2^10 x 2^11),
+// packing 0.75 (its writes: 2^24 entries 374 us against 236 at HBM rate),
+// joining 0.66.
 //
-// CTA tile: 128 rows of C (TMEM lanes) x 32 columns, 256 threads (8 warps);
-// warp w reads TMEM lane quarter w%4 and columns 16*(w/4) .. +16.  Pipeline:
-// two shared-memory stages of limbs (canonical K-major, no-swizzle layout: 8 x
-// 16-byte core matrices) and two sets of 7 TMEM accumulators (7 x 32 columns
-// each); while the MMAs of chunk c run, the threads stage chunk c+1 and fold
-// the accumulators of chunk c-1.  One thread issues the 16 limb pairs x 4 MMAs
-// of 128 x 32 x 16 per chunk and commits them to that stage's mbarrier.
-// Every wait is bounded: on timeout the kernel records an error word, frees
-// its TMEM and returns.
+//   rns_pack_kernel   entries -> one fp16 plane per small prime (balanced)
+//   p8_gemm_kernel    four, two or one small primes at a time -> bytes
+//   rns_join_kernel   bytes (K-split partials added) -> residues mod p
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <string>
@@ -35,370 +33,261 @@
 #include "modarith.cuh"
 #include "tnc_internal.h"
 
-namespace tnc_tc {
+namespace tnc_rns {
 
-constexpr int kTileM = 128;
-constexpr int kTileN = 32;
-constexpr int kChunkK = 64;
-constexpr int kThreads = 256;
-constexpr uint32_t kTmemCols = 512;  // 2 buffers x 7 accumulators x 32 columns = 448
-constexpr uint32_t kAccStride = 256; // columns between the two accumulator buffers
-constexpr uint32_t kSpinLimit = 1u << 22;
+constexpr uint32_t kMaxSmall = 12;
+__host__ __device__ constexpr uint32_t small_prime(uint32_t i) {
+  constexpr uint32_t q[kMaxSmall] = {251, 241, 239, 233, 229, 227, 223, 211, 199, 197, 193, 191};
+  return q[i];
+}
+// floor(2^39 / q): for x < 2^31, x m / 2^39 is at most x / q and within 2^-8 of it
+__host__ __device__ constexpr uint32_t small_magic(uint32_t i) { return (uint32_t)((1ull << 39) / small_prime(i)); }
 
-// Shared memory per stage: A limbs 4 x (128 x 64 bf16) + B limbs 4 x (32 x 64 bf16).
-constexpr uint32_t kALimbBytes = kTileM * kChunkK * 2;  // 16 KiB
-constexpr uint32_t kBLimbBytes = kTileN * kChunkK * 2;  // 4 KiB
-constexpr uint32_t kStageBytes = 4 * kALimbBytes + 4 * kBLimbBytes;  // 80 KiB
-constexpr uint32_t kSmemBytes = 2 * kStageBytes + 1024;
+// The small primes of a step come in groups of 4, 2 and 1 (the residues per
+// item of the GEMM): 9 = 4 + 4 + 1, 10 = 4 + 4 + 2, 11 = 4 + 4 + 2 + 1, 12 =
+// 4 + 4 + 4.
+__host__ __device__ constexpr uint32_t group_size(uint32_t n, uint32_t at) {
+  return n - at >= 4 ? 4u : (n - at >= 2 ? 2u : 1u);
+}
 
-struct TcStep {
-  uint64_t a_off, b_off, c_off;  // entries (one residue per entry)
-  uint32_t fa, fb, k;            // M = 2^fa, N = 2^fb, K = 2^k
-  uint32_t log_split;            // K split over 2^log_split CTAs per tile (partials summed after)
-  uint64_t wm[32], wn[32];       // output address weight of row bit j / column bit j
-  uint32_t p, red_pad;
-  uint64_t mu;
-  uint32_t w256[7];              // 256^s mod p (w256[5] = 2^40 mod p is used)
-  uint32_t pad2;
+// The operands of one step for NR consecutive residues of the entries (a, b:
+// the first one's word of entry 0, entries `stride` words apart; 2^f rows, 2^k
+// shared values, shared index high).  Residue by residue, n planes of operand A
+// then n of B: plane i of an operand at + i 2^(f+k), row-contiguous (the
+// entries' own order, mn) or, for a column operand of fewer than 64 rows,
+// K-contiguous.  Operand `scaled` (0: A, 1: B) carries the reconstruction's factors.
+struct alignas(64) PackUnit {
+  const uint32_t *a, *b;
+  __half* y;
+  uint32_t fa, fb, k, n;
+  uint32_t mn_a, mn_b, scaled, tile_lo, tiles_a;  // tiles of 1024 entries; the first in the launch; of operand A
 };
 
-// ---- PTX helpers -----------------------------------------------------------
+// The output of one step for those residues: residue by residue, the small
+// residues of entry o, group after group, each [K slice][2^c][group size]
+// bytes; the residues mod p go to out[o * stride ..].
+struct alignas(64) JoinUnit {
+  const uint8_t* bytes;
+  uint32_t* out;
+  uint32_t c, log_split, n, r0;  // r0: the first residue's place in the entries
+  uint32_t block_lo;
+};
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
+constexpr uint32_t kMaxUnits = 256;
 
-// Canonical K-major, no-swizzle shared-memory matrix descriptor: core matrices
-// of 8 rows x 16 bytes, LBO = byte distance between core matrices adjacent in
-// K, SBO = between core matrices adjacent in M/N; version 1; layout 0.
-__device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;
-  return d;
-}
-
-// Instruction descriptor, kind::f16: D = F32 (bits 4-5 = 1), A = B = F16
-// (bits 7-9, 10-12 = 0), both K-major, N >> 3 at bits 17-22, M >> 4 at 24-28.
-__host__ __device__ constexpr uint32_t make_idesc(uint32_t M, uint32_t N) {
-  return (1u << 4) | ((N >> 3) << 17) | ((M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t mbar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-               : "memory");
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar), "r"(count) : "memory");
-}
-
-// Bounded wait for phase `parity` of an mbarrier; false on timeout.
-__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity) {
-  for (uint32_t i = 0; i < kSpinLimit; i++) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.b32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(done)
-        : "r"(mbar), "r"(parity)
-        : "memory");
-    if (done) return true;
+__device__ __forceinline__ uint32_t find_last(const uint32_t* lo, uint32_t n, uint32_t x) {
+  uint32_t a = 0, b = n - 1;
+  while (a < b) {
+    const uint32_t m = (a + b + 1) >> 1;
+    if (lo[m] <= x) a = m;
+    else b = m - 1;
   }
-  return false;
+  return a;
 }
 
-// Zero 16 TMEM columns of this warp's 32 lanes.
-__device__ __forceinline__ void tmem_zero16(uint32_t taddr) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr),
-      "r"(0u)
-      : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// Exact integer value of a float holding an integer below 2^23.
-__device__ __forceinline__ uint32_t f2u_small(uint32_t fbits) {
-  return __float_as_uint(__uint_as_float(fbits) + 8388608.0f) - 0x4B000000u;
-}
-
-// Limb li (bits 8li..8li+7) of x0 and of x1 as a packed pair of fp16 values
-// (x0's in the low half): bytes placed at 0 and 2, exponent bits of 1024
-// or-ed in (half 1024 + v, exact for v < 1024), then 1024 subtracted.
-template <int li>
-__device__ __forceinline__ uint32_t limb_pair_f16(uint32_t x0, uint32_t x1) {
-  constexpr uint32_t sel = (uint32_t)li | ((uint32_t)(4 + li) << 8);
-  const uint32_t t = (__byte_perm(x0, x1, sel) & 0x00FF00FFu) | 0x64006400u;
+// hi(a b) + c, 32-bit high product
+__device__ __forceinline__ uint32_t mad_hi(uint32_t a, uint32_t b, uint32_t c) {
   uint32_t r;
-  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(t), "r"(0x64006400u));
+  asm("mad.hi.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
   return r;
 }
 
-// ---- the kernel ------------------------------------------------------------
-
-// Byte offset of element (row r, k-index q) of a K-major limb tile whose core
-// matrices are 8 rows x 8 elements: core (r/8, q/8) at (r/8)*SBO + (q/8)*128,
-// element at (r%8)*16 + (q%8)*2; SBO = (kChunkK/8)*128 = 1024.
-__device__ __forceinline__ uint32_t kmajor_off(uint32_t r, uint32_t q) {
-  return (r >> 3) * 1024u + (q >> 3) * 128u + (r & 7u) * 16u + (q & 7u) * 2u;
+// x < 2^31 minus the multiple of q_i nearest to it: |r| <= (q + 1) / 2 (the
+// rounded quotient is off by one only within 2^-8 of a half).
+template <int I>
+__device__ __forceinline__ uint32_t balanced(uint32_t x) {
+  return x - (mad_hi(x, small_magic(I), 64u) >> 7) * small_prime(I);
 }
 
-// Stage chunk k0 of A's 128 rows and B's 32 rows as 8-bit limbs (bf16).
-// 1024 (row, 8-q group) pairs of A and 256 of B are shared by the 256 threads:
-// every thread first issues all 40 of its loads, then converts and stores.
-__device__ __forceinline__ void stage_chunk(uint8_t* sA, uint8_t* sB, const uint32_t* A, const uint32_t* B, uint32_t M,
-                                            uint32_t N, uint32_t m0, uint32_t n0, uint32_t k0, uint32_t tid) {
-  uint32_t x[5][8];
-#pragma unroll
-  for (int it = 0; it < 5; it++) {
-    const uint32_t job = tid + it * kThreads;  // 0..1023: A, 1024..1279: B (warp-uniform per it)
-    const bool isA = it < 4;
-    const uint32_t jj = isA ? job : job - 1024;
-    const uint32_t r = isA ? (jj & 127u) : (jj & 31u);
-    const uint32_t q8 = isA ? (jj >> 7) * 8u : (jj >> 5) * 8u;
-    const uint32_t* src = isA ? A + m0 + r : B + n0 + r;
-    const uint32_t ld = isA ? M : N;
-#pragma unroll
-    for (int e = 0; e < 8; e++) x[it][e] = src[(uint64_t)(k0 + q8 + e) * ld];
-  }
-#pragma unroll
-  for (int it = 0; it < 5; it++) {
-    const uint32_t job = tid + it * kThreads;
-    const bool isA = it < 4;
-    const uint32_t jj = isA ? job : job - 1024;
-    const uint32_t r = isA ? (jj & 127u) : (jj & 31u);
-    const uint32_t q8 = isA ? (jj >> 7) * 8u : (jj >> 5) * 8u;
-    uint8_t* base = isA ? sA : sB;
-    const uint32_t lbytes = isA ? kALimbBytes : kBLimbBytes;
-    const uint32_t off = kmajor_off(r, q8);
-    const uint32_t* v = x[it];
-    *reinterpret_cast<uint4*>(base + 0 * lbytes + off) =
-        make_uint4(limb_pair_f16<0>(v[0], v[1]), limb_pair_f16<0>(v[2], v[3]), limb_pair_f16<0>(v[4], v[5]),
-                   limb_pair_f16<0>(v[6], v[7]));
-    *reinterpret_cast<uint4*>(base + 1 * lbytes + off) =
-        make_uint4(limb_pair_f16<1>(v[0], v[1]), limb_pair_f16<1>(v[2], v[3]), limb_pair_f16<1>(v[4], v[5]),
-                   limb_pair_f16<1>(v[6], v[7]));
-    *reinterpret_cast<uint4*>(base + 2 * lbytes + off) =
-        make_uint4(limb_pair_f16<2>(v[0], v[1]), limb_pair_f16<2>(v[2], v[3]), limb_pair_f16<2>(v[4], v[5]),
-                   limb_pair_f16<2>(v[6], v[7]));
-    *reinterpret_cast<uint4*>(base + 3 * lbytes + off) =
-        make_uint4(limb_pair_f16<3>(v[0], v[1]), limb_pair_f16<3>(v[2], v[3]), limb_pair_f16<3>(v[4], v[5]),
-                   limb_pair_f16<3>(v[6], v[7]));
-  }
-}
+// Factors of the reconstruction for n = 9 + i small primes of product Q: w =
+// (Q / q_j)^-1 mod q_j.
+struct PackConsts {
+  uint32_t w[4][kMaxSmall];
+};
 
-// B's four limb tiles are contiguous with the same core-matrix strides, so
-// together they are one K-major operand of 4 x 32 = 128 rows (row = 32 lj + n).
-// One MMA of 128 x 128 x 16 per A limb li then yields A_li B_lj for all lj;
-// written at column offset 32 li, the product of limbs (li, lj) lands in the
-// columns of accumulator s = li + lj.  Columns 0..127 are overwritten by the
-// first MMA of the chunk; 128..223 are zeroed beforehand.
-__device__ __forceinline__ void issue_chunk(uint32_t acc_col, uint32_t sA, uint32_t sB) {
-  constexpr uint32_t idesc = make_idesc(kTileM, 4 * kTileN);
-  const uint64_t a0 = make_desc(sA, 128u, 1024u), b0 = make_desc(sB, 128u, 1024u);
+// Planes of four entries' values x of one residue: the half with bits 0x6400 |
+// b is 1024 + b, minus 1152 leaves b - 128 (exact).  With w, the small
+// residues are multiplied by w[I].
+template <int I>
+__device__ __forceinline__ void put_planes(const uint32_t (&x)[4], uint32_t n, __half* y, uint64_t plane,
+                                           const uint32_t* w) {
+  if constexpr (I < (int)kMaxSmall) {
+    if ((uint32_t)I < n) {
+      uint32_t h[2], v[4];
 #pragma unroll
-  for (int li = 0; li < 4; li++)
+      for (int j = 0; j < 4; j++) v[j] = balanced<I>(x[j]);
+      if (w) {
+        const uint32_t f = w[I];
 #pragma unroll
-    for (int ks = 0; ks < kChunkK / 16; ks++) {
-      // +16 bytes per unit of the descriptor's start-address field
-      const uint64_t ad = a0 + (uint64_t)((li * kALimbBytes + ks * 256u) >> 4);
-      const uint64_t bd = b0 + (uint64_t)((ks * 256u) >> 4);
-      mma_f16(acc_col + (uint32_t)li * kTileN, ad, bd, idesc, (li | ks) ? 1u : 0u);
+        for (int j = 0; j < 4; j++) v[j] = balanced<I>(v[j] * f + 256u * small_prime(I));  // (|v f| < 2^15)
+      }
+#pragma unroll
+      for (int j = 0; j < 2; j++) {
+        const uint32_t t = v[2 * j] + 0x64806480u + v[2 * j + 1] * 65536u;
+        asm("add.rn.f16x2 %0, %1, %2;" : "=r"(h[j]) : "r"(t), "r"(0xE480E480u));
+      }
+      *reinterpret_cast<uint2*>(y + (uint64_t)I * plane) = make_uint2(h[0], h[1]);
+      put_planes<I + 1>(x, n, y, plane, w);
     }
+  }
 }
 
-__global__ void __launch_bounds__(kThreads, 1) tc_step_kernel(const TcStep* __restrict__ g, uint32_t* arena,
-                                                             uint32_t* part, uint32_t* err) {
-  extern __shared__ __align__(1024) uint8_t smem[];
-  __shared__ uint64_t mbar_storage[2];
-  __shared__ uint32_t tmem_base_s;
-  const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t quarter = warp & 3u, half = warp >> 2;
-  const uint32_t M = 1u << g->fa, N = 1u << g->fb, K = 1u << g->k;
-  const uint32_t tiles_m = M / kTileM;
-  const uint32_t split = blockIdx.x & ((1u << g->log_split) - 1u), tile = blockIdx.x >> g->log_split;
-  const uint32_t tm = tile % tiles_m, tn = tile / tiles_m;
-  const uint32_t kbeg = split * (K >> g->log_split);
-  const uint32_t n_chunks = (K >> g->log_split) / kChunkK;
-  const uint32_t m0 = tm * kTileM, n0 = tn * kTileN;
-  // stage b: A limbs at smem + b*kStageBytes, B limbs right after them
-#define TC_SA(b) (smem + (b) * kStageBytes)
-#define TC_SB(b) (smem + (b) * kStageBytes + 4 * kALimbBytes)
-  const uint32_t mbar0 = smem_u32(&mbar_storage[0]), mbar1 = smem_u32(&mbar_storage[1]);
+template <int NR>
+__device__ __forceinline__ void load_words(const uint32_t* p, uint32_t (&v)[NR]) {
+  if constexpr (NR == 4) {
+    const uint4 t = *reinterpret_cast<const uint4*>(p);
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+  } else if constexpr (NR == 2) {
+    const uint2 t = *reinterpret_cast<const uint2*>(p);
+    v[0] = t.x; v[1] = t.y;
+  } else {
+    v[0] = *p;
+  }
+}
 
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)),
-                 "r"(kTmemCols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  if (tid == 0) {
-    mbar_init(mbar0, 1);
-    mbar_init(mbar1, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  const uint32_t* A = arena + g->a_off;
-  const uint32_t* B = arena + g->b_off;
-  stage_chunk(TC_SA(0), TC_SB(0), A, B, M, N, m0, n0, kbeg, tid);
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+// Four entries per thread, so that a plane's writes are 8 bytes per lane; per
+// value and small prime a high product, a shift and a multiply-add, half an
+// add and half a packed subtraction.  Writes 2 bytes per small prime and
+// residue: 18 to 20 bytes where it reads 4.
+template <int NR>
+__global__ void __launch_bounds__(256) rns_pack_kernel(const PackUnit* __restrict__ units, uint32_t n_units,
+                                                       uint32_t n_tiles, uint32_t stride,
+                                                       const __grid_constant__ PackConsts pc) {
+  __shared__ uint32_t lo[kMaxUnits];
+  if (threadIdx.x < n_units) lo[threadIdx.x] = units[threadIdx.x].tile_lo;
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tmem_base_s;
-  // zero accumulators s = 4..6 (columns 128..223) of both buffers; each warp
-  // owns one lane quarter and one 16-column half of every accumulator
+  for (uint32_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+    const PackUnit& u = units[find_last(lo, n_units, t)];
+    uint32_t tile = t - u.tile_lo;
+    const bool isA = tile < u.tiles_a;
+    if (!isA) tile -= u.tiles_a;
+    const uint32_t f = isA ? u.fa : u.fb, n = u.n;
+    const uint32_t* X = isA ? u.a : u.b;
+    const uint64_t plane = 1ull << (f + u.k), pair = (uint64_t)n * ((1ull << (u.fa + u.k)) + (1ull << (u.fb + u.k)));
+    __half* Y = u.y + (isA ? 0ull : (uint64_t)n << (u.fa + u.k));
+    const uint32_t* w = u.scaled == (isA ? 0u : 1u) ? pc.w[n - 9u] : nullptr;
+    uint64_t e0, step, at;  // entries e0, e0 + step, ..; their place in a plane
+    if (isA ? u.mn_a : u.mn_b) {
+      e0 = at = (uint64_t)tile * 1024u + threadIdx.x * 4u;
+      step = 1;
+    } else {  // row r, shared values q .. q + 3 (lanes along the rows)
+      const uint64_t i = (uint64_t)tile * 256u + threadIdx.x;
+      const uint64_t r = i & ((1u << f) - 1u), q = (i >> f) * 4u;
+      e0 = (q << f) + r;
+      step = 1ull << f;
+      at = (r << u.k) + q;
+    }
+    uint32_t x[4][NR];
 #pragma unroll
-  for (uint32_t bb = 0; bb < 2; bb++)
+    for (int j = 0; j < 4; j++) load_words<NR>(X + (e0 + j * step) * stride, x[j]);
 #pragma unroll
-    for (uint32_t ss = 4; ss < 7; ss++)
-      tmem_zero16(tmem + ((quarter * 32u) << 16) + bb * kAccStride + ss * kTileN + half * 16u);
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (tid == 0) {
-    issue_chunk(tmem, smem_u32(TC_SA(0)), smem_u32(TC_SB(0)));
-    mma_commit(mbar0);
+    for (int r = 0; r < NR; r++) {
+      const uint32_t v[4] = {x[0][r], x[1][r], x[2][r], x[3][r]};
+      put_planes<0>(v, n, Y + r * pair + at, plane, w);
+    }
   }
+}
 
-  const uint32_t p = g->p;
-  const uint64_t mu = g->mu;
-  uint64_t lo[16], hi[16];
+// Constants of the reconstruction for n = 9 + i small primes of product Q and
+// each of the pass's primes p, packed for dp4a, four small primes j a word:
+// byte b of Q / q_j mod p in c[b]; neg = p - Q mod p.
+struct JoinConsts {
+  struct {
+    uint32_t c[3][4], neg;
+  } by_p[4][4];
+  uint32_t p[4];
+  uint64_t mu[4];
+};
+
+// round(2^15 / q_j), four a word (131 .. 172; 0 beyond n: those bytes are 0)
+__host__ __device__ constexpr uint32_t inv_word(uint32_t g) {
+  uint32_t v = 0;
+  for (uint32_t j = 0; j < 4; j++) v |= ((65536u / small_prime(4 * g + j) + 1u) / 2u) << (8 * j);
+  return v;
+}
+
+// With y_j = S (Q / q_j)^-1 mod q_j, the factor already in the operand's
+// planes: S = sum_j y_j Q / q_j - t Q with t = floor(sum_j y_j / q_j).  S / Q <
+// 3/4 and each y_j round(2^15 / q_j) is within 2^7 of 2^15 y_j / q_j, so t =
+// floor(sum + 1/8) exactly.  The sums are dot products of bytes: five dp4a per
+// four small primes (the coefficients by bytes).
+template <int NR>
+__global__ void __launch_bounds__(256) rns_join_kernel(const JoinUnit* __restrict__ units, uint32_t n_units,
+                                                       uint32_t stride, const __grid_constant__ JoinConsts jc) {
+  __shared__ uint32_t lo[kMaxUnits];
+  if (threadIdx.x < n_units) lo[threadIdx.x] = units[threadIdx.x].block_lo;
+  __syncthreads();
+  const JoinUnit u = units[find_last(lo, n_units, blockIdx.x)];
+  const uint64_t o = (uint64_t)(blockIdx.x - u.block_lo) * 256u + threadIdx.x;
+  if (o >> u.c) return;
+  const uint32_t n = u.n, n_split = 1u << u.log_split;
+  uint32_t res[NR];
 #pragma unroll
-  for (int j = 0; j < 16; j++) lo[j] = hi[j] = 0;
-  bool ok = true;
-  for (uint32_t c = 0; c < n_chunks; c++) {
-    const uint32_t b = c & 1u;
-    if (c + 1 < n_chunks)  // the buffer of chunk c-1 is free: its MMAs completed in the previous iteration
-      stage_chunk(TC_SA(b ^ 1u), TC_SB(b ^ 1u), A, B, M, N, m0, n0, kbeg + (c + 1) * kChunkK, tid);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    const int waited = mbar_wait(b ? mbar1 : mbar0, (c >> 1) & 1u) ? 1 : 0;
-    ok = __syncthreads_and(waited) != 0;  // also: every thread has staged chunk c+1
-    if (!ok) break;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (c + 1 < n_chunks && tid == 0) {
-      issue_chunk(tmem + (b ^ 1u) * kAccStride, smem_u32(TC_SA(b ^ 1u)), smem_u32(TC_SB(b ^ 1u)));
-      mma_commit(b ? mbar0 : mbar1);
-    }
-    // fold the 7 accumulators of chunk c (this thread: one row, 16 columns):
-    // lo += C0 + C1 2^8 + ... + C4 2^32 (< 2^57 per chunk), hi += C5 + C6 2^8
-    // (< 2^31 per chunk); count = lo + hi 2^40.  lo and hi are reduced mod p
-    // every 64 chunks (64 * 2^57 = 2^63) and at the end.  Accumulators with
-    // at most 2 limb pairs are below 2^23 and convert by a float add
-    // (x + 2^23 has x in its low mantissa bits); the others by F2I.
-    const uint32_t tl = tmem + ((quarter * 32u) << 16) + b * kAccStride + half * 16u;
-    {
-      uint32_t v0[16], v1[16];
-      tmem_ld16(tl + 0 * kTileN, v0);
-      tmem_ld16(tl + 1 * kTileN, v1);
+  for (int r = 0; r < NR; r++) {
+    const uint8_t* g = u.bytes + (((uint64_t)r * n) << (u.c + u.log_split));
+    uint32_t y[3] = {0, 0, 0};
+    if (n_split == 1) {
+      y[0] = *reinterpret_cast<const uint32_t*>(g + 4 * o);
+      y[1] = *reinterpret_cast<const uint32_t*>(g + (4ull << u.c) + 4 * o);
+      const uint8_t* h = g + (8ull << u.c);
+      if (n == 9) y[2] = h[o];
+      else if (n == 12) y[2] = *reinterpret_cast<const uint32_t*>(h + 4 * o);
+      else y[2] = *reinterpret_cast<const uint16_t*>(h + 2 * o);
+      if (n == 11) y[2] |= (uint32_t)h[(2ull << u.c) + o] << 16;
+    } else {  // add the K slices and reduce again
 #pragma unroll
-      for (int j = 0; j < 16; j++)
-        lo[j] += (uint64_t)(f2u_small(v0[j]) + (f2u_small(v1[j]) << 8));
-    }
+      for (int q4 = 0; q4 < 3; q4++) {
+        uint32_t s[4] = {0, 0, 0, 0};
+        const uint32_t m = q4 < 2 ? 4u : n - 8u;  // small primes of this word
+        for (uint32_t k = 0; k < n_split; k++) {
+          const uint64_t e = ((uint64_t)k << u.c) + o;
+          uint32_t v;
+          if (m == 4) {
+            v = *reinterpret_cast<const uint32_t*>(g + 4 * e);
+          } else {
+            v = m == 1 ? (uint32_t)g[e] : (uint32_t)*reinterpret_cast<const uint16_t*>(g + 2 * e);
+            if (m == 3) v |= (uint32_t)g[((2ull << u.c) << u.log_split) + e] << 16;
+          }
+          s[0] += v & 0xFFu;
+          s[1] += (v >> 8) & 0xFFu;
+          s[2] += (v >> 16) & 0xFFu;
+          s[3] += v >> 24;
+        }
+        g += ((uint64_t)m << u.c) << u.log_split;
 #pragma unroll
-    for (int ss = 2; ss < 5; ss++) {
-      uint32_t v[16];
-      tmem_ld16(tl + (uint32_t)ss * kTileN, v);
-#pragma unroll
-      for (int j = 0; j < 16; j++) lo[j] += (uint64_t)__float2uint_rn(__uint_as_float(v[j])) << (8 * ss);
-    }
-    {
-      uint32_t v5[16], v6[16];
-      tmem_ld16(tl + 5 * kTileN, v5);
-      tmem_ld16(tl + 6 * kTileN, v6);
-#pragma unroll
-      for (int j = 0; j < 16; j++) hi[j] += f2u_small(v5[j]) + (f2u_small(v6[j]) << 8);
-    }
-    if ((c & 63u) == 63u) {
-#pragma unroll
-      for (int j = 0; j < 16; j++) {
-        lo[j] = tnc_dev::mod_reduce(lo[j], p, mu);
-        hi[j] = tnc_dev::mod_reduce(hi[j], p, mu);
+        for (int j = 0; j < 4; j++) {
+          const uint32_t q = small_prime(4 * q4 + j);
+          uint32_t v = s[j] - (__umulhi(s[j], small_magic(4 * q4 + j)) >> 7) * q;
+          if (v >= q) v -= q;
+          y[q4] |= v << (8 * j);
+        }
       }
     }
-    // the columns this warp just read of accumulators 4..6 start the chunk
-    // after next at zero
+    const auto& cc = jc.by_p[n - 9u][u.r0 + r];
+    uint32_t f = 1u << 12, b[4] = {0, 0, 0, 0};
 #pragma unroll
-    for (uint32_t ss = 4; ss < 7; ss++) tmem_zero16(tl + ss * kTileN);
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  }
-  if (!ok && tid == 0) atomicExch(err, 1u);
-
-  uint32_t res[16];
-  {
-    const uint32_t w40 = g->w256[5];  // 2^40 mod p
+    for (int q4 = 0; q4 < 3; q4++) {
+      f = __dp4a(y[q4], inv_word(q4), f);
 #pragma unroll
-    for (int j = 0; j < 16; j++)
-      res[j] = tnc_dev::mod_reduce(tnc_dev::mod_reduce(lo[j], p, mu) +
-                                       (uint64_t)tnc_dev::mod_reduce(hi[j], p, mu) * w40,
-                                   p, mu);
-  }
-  if (ok) {
-    // C[o(m, n)]: o = sum of the output weights of m's and n's bits
-    const uint32_t m = m0 + quarter * 32u + lane;
-    uint64_t om = 0;
-    for (uint32_t j = 0; j < g->fa; j++)
-      if ((m >> j) & 1u) om += g->wm[j];
-    uint32_t* C = g->log_split ? part + ((uint64_t)split << (g->fa + g->fb)) : arena + g->c_off;
-    const uint32_t nb = n0 + half * 16u;  // columns nb .. nb+15: bits 0..3 vary
-    uint64_t on0 = 0;
-    for (uint32_t j = 4; j < g->fb; j++)
-      if ((nb >> j) & 1u) on0 += g->wn[j];
-#pragma unroll
-    for (int jn = 0; jn < 16; jn++) {
-      uint64_t on = on0;
-#pragma unroll
-      for (int j = 0; j < 4; j++)
-        if ((jn >> j) & 1) on += g->wn[j];
-      C[om + on] = res[jn];
+      for (int i = 0; i < 4; i++) b[i] = __dp4a(y[q4], cc.c[q4][i], b[i]);
     }
+    const uint64_t acc = (uint64_t)(b[0] + (b[1] << 8)) + ((uint64_t)(b[2] + (b[3] << 8)) << 16) +
+                         (uint64_t)(f >> 15) * cc.neg;
+    res[r] = tnc_dev::mod_reduce(acc, jc.p[u.r0 + r], jc.mu[u.r0 + r]);
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
-#undef TC_SA
-#undef TC_SB
+  uint32_t* dst = u.out + o * stride;
+  if constexpr (NR == 4) *reinterpret_cast<uint4*>(dst) = make_uint4(res[0], res[1], res[2], res[3]);
+  else if constexpr (NR == 2) *reinterpret_cast<uint2*>(dst) = make_uint2(res[0], res[1]);
+  else *dst = res[0];
 }
 
-// Sum of the K-split partials of a dense step: C[o] = sum_j part[j][o] mod p.
-__global__ void tc_split_final_kernel(const TcStep* __restrict__ g, uint32_t* arena, const uint32_t* __restrict__ part) {
-  const uint64_t n = 1ull << (g->fa + g->fb);
-  uint32_t* C = arena + g->c_off;
-  for (uint64_t o = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; o < n; o += (uint64_t)gridDim.x * blockDim.x) {
-    uint64_t s = 0;
-    for (uint32_t j = 0; j < (1u << g->log_split); j++) s += part[((uint64_t)j << (g->fa + g->fb)) + o];
-    C[o] = tnc_dev::mod_reduce(s, g->p, g->mu);
-  }
-}
-
-}  // namespace tnc_tc
+}  // namespace tnc_rns
 
 namespace tnc {
+
+using tnc_rns::group_size;
+using tnc_rns::kMaxSmall;
+using tnc_rns::small_prime;
 
 // Can this step run on the tensor cores (possibly with A and B exchanged)?
 bool tc_eligible(const StepDesc& d) {
@@ -406,93 +295,188 @@ bool tc_eligible(const StepDesc& d) {
   return d.k >= 6 && ((fa >= 7 && fb >= 5) || (fb >= 7 && fa >= 5));
 }
 
-size_t tc_step_bytes() { return sizeof(tnc_tc::TcStep); }
-
-// K split of a dense step: double it while the tiles x splits stay below two
-// CTAs per SM of a 152-SM GPU, each split keeps >= 2 chunks of 64, and the
-// partials (2^c entries per split) stay within tc_part_entries().
-uint64_t tc_part_entries() { return 1ull << 24; }
-uint32_t tc_split_log(const StepDesc& d) {
-  const bool swap = !(d.ka >= 7 && d.kb >= 5);
-  const uint32_t fa = swap ? d.kb : d.ka, fb = swap ? d.ka : d.kb;
-  const uint64_t tiles = (1ull << (fa - 7)) << (fb - 5);
-  uint32_t ls = 0;
-  while ((tiles << ls) < 304 && d.k - ls > 7 && (1ull << (d.c + ls + 1)) <= tc_part_entries()) ls++;
-  return ls;
+// S < 2^(62 + k) (2^(60 + k) for the default primes, which then need one prime
+// less for two values of k in eight: not worth a second rule); Q >= 4/3 S.
+uint32_t tc_small_primes(uint32_t k) {
+  double bits = 0;
+  for (uint32_t n = 0; n < kMaxSmall; n++) {
+    bits += std::log2((double)small_prime(n));
+    if (n >= 8 && bits >= 62.0 + k + 0.4151) return n + 1;
+  }
+  return 0;
 }
 
-// Host-side descriptor for one dense step and residue prime p.
-void tc_make_step(const StepDesc& d, uint32_t p, void* out) {
-  using tnc_tc::TcStep;
-  TcStep t;
-  std::memset(&t, 0, sizeof(t));
-  int op[64] = {0}, dst[64] = {0};
-  if (d.nra != TNC_BITMAP) {
-    for (int i = 0; i < d.nra; i++)
-      for (int q = 0; q < d.map.runs.ra[i].len; q++) {
-        op[d.map.runs.ra[i].src + q] = 0;
-        dst[d.map.runs.ra[i].src + q] = d.map.runs.ra[i].dst + q;
+uint64_t tc_plane_bytes(const StepDesc& d) {
+  return 2ull * tc_small_primes(d.k) * ((1ull << (d.ka + d.k)) + (1ull << (d.kb + d.k)));
+}
+
+uint64_t tc_byte_bytes(const StepDesc& d) { return (uint64_t)tc_small_primes(d.k) << (d.c + p8_split_log(d)); }
+
+size_t tc_unit_bytes() { return sizeof(tnc_rns::PackUnit) + sizeof(tnc_rns::JoinUnit) + 4 * p8_prob_bytes(); }
+uint32_t tc_max_units(uint32_t nr) { return tnc_rns::kMaxUnits / 3 / nr; }  // (up to three groups of four primes a residue)
+
+int tc_batch(const TcUnit* units, int n, uint32_t nr, uint32_t rg, uint32_t* arena, uint64_t arena_bytes,
+             uint8_t* planes, uint8_t* bytes, std::vector<char>& host, TcBatch& b) {
+  using namespace tnc_rns;
+  b = TcBatch{};
+  b.nr = nr;
+  if (n > (int)tc_max_units(nr)) return set_error(TNC_ERR_INVALID, "internal: too many dense steps in a launch");
+  std::vector<PackUnit> packs;
+  std::vector<JoinUnit> joins;
+  P8Probs probs[3];  // residues per item 4, 2, 1
+  uint64_t tiles = 0, blocks = 0;
+  for (int i = 0; i < n; i++) {
+    const StepDesc& d = units[i].d;
+    const uint32_t nq = tc_small_primes(d.k), ls = p8_split_log(d);
+    if (!nq) return set_error(TNC_ERR_TOO_LARGE, "dense step with too many shared values");
+    if (units[i].r + nr > rg || (nr != 1 && nr != rg)) return set_error(TNC_ERR_INVALID, "internal: residues outside their pass");
+    {
+      const uint64_t ea = 1ull << (d.ka + d.k), eb = 1ull << (d.kb + d.k), ec = 1ull << d.c, w = 4ull * rg;
+      if ((d.a_off + ea) * w > arena_bytes || (d.b_off + eb) * w > arena_bytes || (d.c_off + ec) * w > arena_bytes)
+        return set_error(TNC_ERR_INVALID, "internal: dense step range outside the arena");
+    }
+    PackUnit pk;
+    std::memset(&pk, 0, sizeof(pk));
+    pk.a = arena + d.a_off * rg + units[i].r;
+    pk.b = arena + d.b_off * rg + units[i].r;
+    pk.y = reinterpret_cast<__half*>(planes);
+    pk.fa = d.ka;
+    pk.fb = d.kb;
+    pk.k = d.k;
+    pk.n = nq;
+    pk.mn_a = p8_operand_mn(d, 0);
+    pk.mn_b = p8_operand_mn(d, 1);
+    pk.scaled = d.ka <= d.kb ? 0u : 1u;  // (the smaller operand)
+    pk.tile_lo = (uint32_t)tiles;
+    pk.tiles_a = 1u << (d.ka + d.k - 10);  // (k >= 6, at least 32 rows: whole tiles of 1024 entries)
+    tiles += pk.tiles_a + (1ull << (d.kb + d.k - 10));
+    packs.push_back(pk);
+    JoinUnit ju;
+    std::memset(&ju, 0, sizeof(ju));
+    ju.bytes = bytes;
+    ju.out = arena + d.c_off * rg + units[i].r;
+    ju.c = d.c;
+    ju.log_split = ls;
+    ju.n = nq;
+    ju.r0 = units[i].r;
+    ju.block_lo = (uint32_t)blocks;
+    blocks += ((1ull << d.c) + 255) / 256;
+    joins.push_back(ju);
+    for (uint32_t r = 0; r < nr; r++) {
+      __half *ya = reinterpret_cast<__half*>(planes), *yb = ya + ((uint64_t)nq << (d.ka + d.k));
+      uint8_t* out = bytes;
+      for (uint32_t at = 0; at < nq; at += group_size(nq, at)) {
+        const uint32_t gs = group_size(nq, at);
+        const int rc = p8_gemm_desc(d, gs, ya + ((uint64_t)at << (d.ka + d.k)), yb + ((uint64_t)at << (d.kb + d.k)), out,
+                                    at, probs[gs == 4 ? 0 : (gs == 2 ? 1 : 2)]);
+        if (rc) return rc;
+        out += ((uint64_t)gs << d.c) << ls;
       }
-    for (int i = 0; i < d.nrb; i++)
-      for (int q = 0; q < d.map.runs.rb[i].len; q++) {
-        op[d.map.runs.rb[i].src + q] = 1;
-        dst[d.map.runs.rb[i].src + q] = d.map.runs.rb[i].dst + q;
-      }
-  } else {
-    for (int j = 0; j < d.c; j++) {
-      op[j] = d.map.bit[j] >> 7;
-      dst[j] = d.map.bit[j] & 63;
+      planes += tc_plane_bytes(d);
+      bytes += tc_byte_bytes(d);
+    }
+    if (units[i].r == 0) {
+      b.steps++;
+      b.splits += ls > 0;
     }
   }
-  // row operand = the one with >= 7 free bits (A unless only B qualifies)
-  const bool swap = !(d.ka >= 7 && d.kb >= 5);
-  const int row_op = swap ? 1 : 0;
-  t.a_off = swap ? d.b_off : d.a_off;
-  t.b_off = swap ? d.a_off : d.b_off;
-  t.c_off = d.c_off;
-  t.fa = swap ? d.kb : d.ka;
-  t.fb = swap ? d.ka : d.kb;
-  t.k = d.k;
-  t.log_split = tc_split_log(d);
-  for (int j = 0; j < d.c; j++) {
-    if (op[j] == row_op) t.wm[dst[j]] = 1ull << j;
-    else t.wn[dst[j]] = 1ull << j;
-  }
-  t.p = p;
-  t.mu = ~0ull / p;
-  uint64_t w = 1;
-  for (int s = 0; s < 7; s++) {
-    t.w256[s] = (uint32_t)w;
-    w = w * 256 % p;
-  }
-  std::memcpy(out, &t, sizeof(t));
+  if (std::max(tiles, blocks) >= (1ull << 31)) return set_error(TNC_ERR_TOO_LARGE, "dense steps of a level have too many tiles");
+  auto put = [&](const void* src, size_t size) {
+    const size_t at = host.size();
+    host.resize(at + size);
+    if (size) std::memcpy(host.data() + at, src, size);
+    return at;
+  };
+  b.n_units = (uint32_t)n;
+  b.pack_tiles = (uint32_t)tiles;
+  b.blocks = (uint32_t)blocks;
+  b.pack_off = put(packs.data(), packs.size() * sizeof(PackUnit));
+  b.join_off = put(joins.data(), joins.size() * sizeof(JoinUnit));
+  for (int g = 0; g < 3; g++)
+    for (int v = 0; v < 6; v++) {
+      b.gemm[g][v].n = probs[g].n[v];
+      b.gemm[g][v].items = (uint32_t)probs[g].items[v];
+      b.gemm[g][v].off = put(probs[g].descs[v].data(), probs[g].descs[v].size());
+    }
+  return TNC_OK;
 }
 
-int tc_launch(const void* dev_step, const StepDesc& d, uint32_t* arena, uint32_t* part, uint32_t* dev_err,
-              void* stream) {
+namespace {
+
+uint32_t pow_mod(uint64_t a, uint32_t e, uint32_t p) {
+  uint64_t r = 1;
+  for (a %= p; e; e >>= 1) {
+    if (e & 1) r = r * a % p;
+    a = a * a % p;
+  }
+  return (uint32_t)r;
+}
+
+// Product of the first n small primes without the j-th (all of them: j = n), mod p.
+uint32_t cofactor(uint32_t n, uint32_t j, uint32_t p) {
+  uint64_t x = 1 % p;
+  for (uint32_t i = 0; i < n; i++)
+    if (i != j) x = x * small_prime(i) % p;
+  return (uint32_t)x;
+}
+
+const tnc_rns::PackConsts& pack_consts() {
+  static const tnc_rns::PackConsts pc = [] {
+    tnc_rns::PackConsts c{};
+    for (uint32_t n = 9; n <= kMaxSmall; n++)
+      for (uint32_t j = 0; j < n; j++)
+        c.w[n - 9][j] = pow_mod(cofactor(n, j, small_prime(j)), small_prime(j) - 2, small_prime(j));
+    return c;
+  }();
+  return pc;
+}
+
+}  // namespace
+
+std::vector<char> tc_consts(const uint32_t* primes, uint32_t rg) {
+  tnc_rns::JoinConsts jc;
+  std::memset(&jc, 0, sizeof(jc));
+  for (uint32_t r = 0; r < rg; r++) {
+    jc.p[r] = primes[r];
+    jc.mu[r] = ~0ull / primes[r];
+    for (uint32_t n = 9; n <= kMaxSmall; n++) {
+      for (uint32_t j = 0; j < n; j++) {
+        const uint32_t c = cofactor(n, j, primes[r]);
+        for (uint32_t i = 0; i < 4; i++) jc.by_p[n - 9][r].c[j / 4][i] |= ((c >> (8 * i)) & 0xFFu) << (8 * (j % 4));
+      }
+      jc.by_p[n - 9][r].neg = primes[r] - cofactor(n, n, primes[r]);
+    }
+  }
+  const char* p = reinterpret_cast<const char*>(&jc);
+  return std::vector<char>(p, p + sizeof(jc));
+}
+
+int tc_run(const TcBatch& b, const char* dev, const std::vector<char>& consts, uint32_t rg, uint32_t* dev_err, int sms,
+           void* stream) {
+  using namespace tnc_rns;
   cudaStream_t st = (cudaStream_t)stream;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(tnc_tc::tc_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)tnc_tc::kSmemBytes);
-    if (e != cudaSuccess) return set_error(TNC_ERR_CUDA, std::string("tc attribute: ") + cudaGetErrorString(e));
-    attr_set = true;
-  }
-  const bool swap = !(d.ka >= 7 && d.kb >= 5);
-  const uint32_t fa = swap ? d.kb : d.ka, fb = swap ? d.ka : d.kb;
-  const uint32_t ls = tc_split_log(d);
-  const uint64_t tiles = ((1ull << (fa - 7)) * (1ull << (fb - 5))) << ls;
-  if (tiles >= (1ull << 31)) return set_error(TNC_ERR_TOO_LARGE, "dense step has too many tiles");
-  tnc_tc::tc_step_kernel<<<(unsigned)tiles, tnc_tc::kThreads, tnc_tc::kSmemBytes, st>>>(
-      (const tnc_tc::TcStep*)dev_step, arena, part, dev_err);
-  launch_counts().tc_gemm++;
-  if (ls) launch_counts().tc_split++;
-  if (ls) {
-    const uint64_t n = 1ull << (fa + fb);
-    tnc_tc::tc_split_final_kernel<<<(unsigned)std::min<uint64_t>((n + 255) / 256, 8192), 256, 0, st>>>(
-        (const tnc_tc::TcStep*)dev_step, arena, part);
-  }
-  cudaError_t e = cudaGetLastError();
+  uint32_t small[kMaxSmall];
+  for (uint32_t i = 0; i < kMaxSmall; i++) small[i] = small_prime(i);
+  const unsigned pack_blocks = (unsigned)std::min<uint64_t>(b.pack_tiles, (uint64_t)sms * 16);
+  const PackUnit* pu = reinterpret_cast<const PackUnit*>(dev + b.pack_off);
+  if (b.nr == 4) rns_pack_kernel<4><<<pack_blocks, 256, 0, st>>>(pu, b.n_units, b.pack_tiles, rg, pack_consts());
+  else if (b.nr == 2) rns_pack_kernel<2><<<pack_blocks, 256, 0, st>>>(pu, b.n_units, b.pack_tiles, rg, pack_consts());
+  else rns_pack_kernel<1><<<pack_blocks, 256, 0, st>>>(pu, b.n_units, b.pack_tiles, rg, pack_consts());
+  for (int v = 6; v-- > 0;)
+    for (int g = 0; g < 3; g++)
+      if (b.gemm[g][v].n)
+        if (int rc = p8_gemm_launch(4u >> g, v, dev + b.gemm[g][v].off, b.gemm[g][v].n, b.gemm[g][v].items, small,
+                                    kMaxSmall, dev_err, sms, stream))
+          return rc;
+  JoinConsts jc;
+  std::memcpy(&jc, consts.data(), sizeof(jc));
+  const JoinUnit* ju = reinterpret_cast<const JoinUnit*>(dev + b.join_off);
+  if (b.nr == 4) rns_join_kernel<4><<<b.blocks, 256, 0, st>>>(ju, b.n_units, rg, jc);
+  else if (b.nr == 2) rns_join_kernel<2><<<b.blocks, 256, 0, st>>>(ju, b.n_units, rg, jc);
+  else rns_join_kernel<1><<<b.blocks, 256, 0, st>>>(ju, b.n_units, rg, jc);
+  launch_counts().tc_gemm += (int32_t)b.steps;
+  launch_counts().tc_split += (int32_t)b.splits;
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return set_error(TNC_ERR_CUDA, std::string("tc launch: ") + cudaGetErrorString(e));
   return TNC_OK;
 }

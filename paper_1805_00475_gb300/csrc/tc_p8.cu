@@ -116,13 +116,15 @@ struct alignas(64) P8Prob {
   uint32_t a_mn, b_mn;      // operand planes row-contiguous (MN-major) instead of K-contiguous
   uint32_t direct;          // output as rg balanced fp16 planes, plane i at out + i 2^(fa+fb) halves
   uint32_t pairs;           // row bit 0 has output weight 1: entries written two at a time (TN >= 32)
+  uint32_t prime_at;        // the first of the launch's primes that the step's residues belong to
   uint8_t* out;             // C (entry o at out[o * rg]), or the split partials [split][2^(fa+fb) * rg]
 };
 constexpr uint32_t kMaxProbs = 256;  // steps of one launch (their first items are searched in shared memory)
 
-// What a launch needs of its pass: the residues' primes.
+// The primes of a launch: the pass's (from 0), or several steps' own.
+constexpr uint32_t kLaunchPrimes = 16;
 struct P8Primes {
-  float pf[4], invp[4];
+  float pf[kLaunchPrimes], invp[kLaunchPrimes];
 };
 
 // Index of the last of n ascending values lo[0..n) that is <= x (lo[0] <= x).
@@ -924,7 +926,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // the two entries o, o + 1, adjacent in the staging and in C, and the
     // lane and table bits start one higher.
     // (all of this per step: set up again when an item belongs to another one)
-    uint32_t pv = 0, lane_off = 0, lane_sid = 0, cur = ~0u, fa = 0, fb = 0, log_split = 0;
+    uint32_t pv = 0, lane_off = 0, lane_sid = 0, cur = ~0u, fa = 0, fb = 0, log_split = 0, pset = 0;
     bool direct = false;
     uint8_t* out = nullptr;
     Step st;
@@ -938,6 +940,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         fa = g.fa;
         fb = g.fb;
         log_split = g.log_split;
+        pset = g.prime_at;
         direct = g.direct != 0;
         out = g.out;
         if (cur != ~0u) epi_bar();  // the previous step's entries are out: the tables are free
@@ -995,7 +998,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_fence_after();
             const uint32_t tb = tmem + ((quarter * 32u) << 16) + ra * TN + cbeg;
             if (ok && !idle) {
-              const float pf = pr.pf[r], invp = pr.invp[r], pm = kMagic + pf;
+              const float pf = pr.pf[pset + r], invp = pr.invp[pset + r], pm = kMagic + pf;
 #pragma unroll 1
               for (uint32_t col = 0; col < kHalf; col += kBatch) {
                 uint32_t v[kBatch / 16][16];
@@ -1388,48 +1391,16 @@ uint32_t p8_max_steps() { return tnc_p8::kMaxProbs; }
 
 namespace {
 
-// One dense step's descriptors: operands and output in the arena, packed
-// planes at `scratch`, K-split partials at `part`.
-int fill_step(const P8Step& step, uint32_t rg, uint8_t* arena, uint64_t arena_bytes, uint8_t* scratch, uint8_t* part,
-              tnc_p8::P8Prob& g, tnc_p8::PackProb& pk, tnc_p8::SplitProb& sp, uint32_t& variant,
-              tnc_launch_counts& lc) {
-  const StepDesc& d = step.d;
-  const Shape s = shape_of(d);
+// The GEMM's descriptor of a dense step: rg operand planes of the row side at
+// pa and of the column side at pb (laid out as p8_operand_mn says), output (or
+// K-split partials) at out.
+int fill_gemm(const StepDesc& d, const Shape& s, uint32_t rg, __half* pa, __half* pb, bool direct, uint8_t* out,
+              uint32_t prime_at, tnc_p8::P8Prob& g) {
   const uint32_t ls = p8_split_log(d);
-  variant = variant_of(s);
-  const uint64_t a_off = s.swap ? d.b_off : d.a_off, b_off = s.swap ? d.a_off : d.b_off;
-  // operands by tile side (row side = A unless swapped): read row-contiguous
-  // (mn), and taken straight from the planes their producing dense step
-  // wrote (direct), which occupy twice the entries' bytes
   const int side_a = s.swap ? 1 : 0, side_b = 1 - side_a;
   const bool mn_a = p8_operand_mn(d, side_a), mn_b = p8_operand_mn(d, side_b);
-  const bool dir_a = (step.flags & (side_a ? kP8DirectB : kP8DirectA)) != 0;
-  const bool dir_b = (step.flags & (side_b ? kP8DirectB : kP8DirectA)) != 0;
-  const bool dir_out = (step.flags & kP8DirectOut) != 0;
-  if ((dir_a && !mn_a) || (dir_b && !mn_b) || (dir_out && ls))
-    return set_error(TNC_ERR_INVALID, "internal: direct fp16 planes for an operand read K-contiguous");
-  {  // every range the launch touches lies inside the arena
-    const uint64_t ea = (1ull << (s.fa + s.k)) * rg * (dir_a ? 2 : 1), eb = (1ull << (s.fb + s.k)) * rg * (dir_b ? 2 : 1);
-    const uint64_t ec = (1ull << d.c) * rg * (dir_out ? 2 : 1);
-    if (a_off * rg + ea > arena_bytes || b_off * rg + eb > arena_bytes || d.c_off * rg + ec > arena_bytes)
-      return set_error(TNC_ERR_INVALID, "internal: dense step range outside the arena");
-  }
-  __half* a16 = reinterpret_cast<__half*>(scratch);  // rg planes of 2^(fa + kp)
-  __half* b16 = a16 + (dir_a ? 0 : (uint64_t)rg << (s.fa + s.kp));
-  __half* pa = dir_a ? reinterpret_cast<__half*>(arena + a_off * rg) : a16;
-  __half* pb = dir_b ? reinterpret_cast<__half*>(arena + b_off * rg) : b16;
   if (((uintptr_t)pa | (uintptr_t)pb) & 15u)
     return set_error(TNC_ERR_INVALID, "internal: fp16 operand planes not 16-byte aligned");
-  std::memset(&pk, 0, sizeof(pk));
-  pk.a = tnc_p8::PackOperand{arena + a_off * rg, a16, s.fa, dir_a ? 0u : (mn_a ? 2u : 1u)};
-  pk.b = tnc_p8::PackOperand{arena + b_off * rg, b16, s.fb, dir_b ? 0u : (mn_b ? 2u : 1u)};
-  pk.k = s.k;
-  pk.kp = s.kp;
-  const uint64_t tiles = ((dir_a ? 0 : (uint64_t)((1u << s.fa) + 63u) / 64u) +
-                          (dir_b ? 0 : (uint64_t)((1u << s.fb) + 63u) / 64u))
-                         << (s.kp - 6);
-  if (tiles >= (1ull << 31)) return set_error(TNC_ERR_TOO_LARGE, "dense step has too many operand tiles");
-  pk.n_tiles = (uint32_t)tiles;
   std::memset(&g, 0, sizeof(g));
   int rc = mn_a ? make_map_mn(&g.map_a, pa, 1ull << s.fa, 1ull << s.k, rg)
                 : make_map(&g.map_a, pa, 1ull << s.fa, 1ull << s.kp, rg, tnc_p8::kTileM);
@@ -1448,11 +1419,12 @@ int fill_step(const P8Step& step, uint32_t rg, uint8_t* arena, uint64_t arena_by
     while ((2u << gm) <= g.tiles_m && (uint64_t)(2u << gm) * tile_rows * (2ull << s.kp) * rg <= kP8GroupBytes) gm++;
     g.gm_log = gm;
   }
+  g.prime_at = prime_at;
   if ((s.tiles << ls) >= (1ull << 31)) return set_error(TNC_ERR_TOO_LARGE, "dense step has too many tiles");
   g.n_items = (uint32_t)((s.pair ? s.tiles / 2 : s.tiles) << ls);
   g.a_mn = mn_a ? 1u : 0u;
   g.b_mn = mn_b ? 1u : 0u;
-  g.direct = dir_out ? 1u : 0u;
+  g.direct = direct ? 1u : 0u;
   // output address weights (the output bit j comes from one operand's free bit)
   int op[64] = {0}, dst[64] = {0};
   if (d.nra != TNC_BITMAP) {
@@ -1487,8 +1459,52 @@ int fill_step(const P8Step& step, uint32_t rg, uint8_t* arena, uint64_t arena_by
     for (size_t i = 0; i < bits.size(); i++) g.ebit[i] = bits[i].second;
   }
   g.pairs = (s.tn >= 32 && g.wm[0] == 1) ? 1u : 0u;  // output bit 0 is row bit 0
-  uint8_t* out = arena + d.c_off * rg;               // direct: the planes, same place (twice the bytes)
-  g.out = ls ? part : out;
+  g.out = out;
+  return TNC_OK;
+}
+
+// One dense step's descriptors: operands and output in the arena, packed
+// planes at `scratch`, K-split partials at `part`.
+int fill_step(const P8Step& step, uint32_t rg, uint8_t* arena, uint64_t arena_bytes, uint8_t* scratch, uint8_t* part,
+              tnc_p8::P8Prob& g, tnc_p8::PackProb& pk, tnc_p8::SplitProb& sp, uint32_t& variant,
+              tnc_launch_counts& lc) {
+  const StepDesc& d = step.d;
+  const Shape s = shape_of(d);
+  const uint32_t ls = p8_split_log(d);
+  variant = variant_of(s);
+  const uint64_t a_off = s.swap ? d.b_off : d.a_off, b_off = s.swap ? d.a_off : d.b_off;
+  // operands by tile side (row side = A unless swapped): read row-contiguous
+  // (mn), and taken straight from the planes their producing dense step
+  // wrote (direct), which occupy twice the entries' bytes
+  const int side_a = s.swap ? 1 : 0, side_b = 1 - side_a;
+  const bool mn_a = p8_operand_mn(d, side_a), mn_b = p8_operand_mn(d, side_b);
+  const bool dir_a = (step.flags & (side_a ? kP8DirectB : kP8DirectA)) != 0;
+  const bool dir_b = (step.flags & (side_b ? kP8DirectB : kP8DirectA)) != 0;
+  const bool dir_out = (step.flags & kP8DirectOut) != 0;
+  if ((dir_a && !mn_a) || (dir_b && !mn_b) || (dir_out && ls))
+    return set_error(TNC_ERR_INVALID, "internal: direct fp16 planes for an operand read K-contiguous");
+  {  // every range the launch touches lies inside the arena
+    const uint64_t ea = (1ull << (s.fa + s.k)) * rg * (dir_a ? 2 : 1), eb = (1ull << (s.fb + s.k)) * rg * (dir_b ? 2 : 1);
+    const uint64_t ec = (1ull << d.c) * rg * (dir_out ? 2 : 1);
+    if (a_off * rg + ea > arena_bytes || b_off * rg + eb > arena_bytes || d.c_off * rg + ec > arena_bytes)
+      return set_error(TNC_ERR_INVALID, "internal: dense step range outside the arena");
+  }
+  __half* a16 = reinterpret_cast<__half*>(scratch);  // rg planes of 2^(fa + kp)
+  __half* b16 = a16 + (dir_a ? 0 : (uint64_t)rg << (s.fa + s.kp));
+  __half* pa = dir_a ? reinterpret_cast<__half*>(arena + a_off * rg) : a16;
+  __half* pb = dir_b ? reinterpret_cast<__half*>(arena + b_off * rg) : b16;
+  std::memset(&pk, 0, sizeof(pk));
+  pk.a = tnc_p8::PackOperand{arena + a_off * rg, a16, s.fa, dir_a ? 0u : (mn_a ? 2u : 1u)};
+  pk.b = tnc_p8::PackOperand{arena + b_off * rg, b16, s.fb, dir_b ? 0u : (mn_b ? 2u : 1u)};
+  pk.k = s.k;
+  pk.kp = s.kp;
+  const uint64_t tiles = ((dir_a ? 0 : (uint64_t)((1u << s.fa) + 63u) / 64u) +
+                          (dir_b ? 0 : (uint64_t)((1u << s.fb) + 63u) / 64u))
+                         << (s.kp - 6);
+  if (tiles >= (1ull << 31)) return set_error(TNC_ERR_TOO_LARGE, "dense step has too many operand tiles");
+  pk.n_tiles = (uint32_t)tiles;
+  uint8_t* out = arena + d.c_off * rg;  // direct: the planes, same place (twice the bytes)
+  if (int rc = fill_gemm(d, s, rg, pa, pb, dir_out, ls ? part : out, 0, g)) return rc;
   std::memset(&sp, 0, sizeof(sp));
   sp.part = part;
   sp.out = out;
@@ -1611,5 +1627,41 @@ int p8_run(const P8Batch& b, const char* dev, const uint32_t* primes, uint32_t r
   if (e != cudaSuccess) return set_error(TNC_ERR_CUDA, std::string("p8 launch: ") + cudaGetErrorString(e));
   return TNC_OK;
 }
+
+int p8_gemm_desc(const StepDesc& d, uint32_t rg, void* planes_a, void* planes_b, uint8_t* out, uint32_t prime_at,
+                 P8Probs& probs) {
+  const Shape s = shape_of(d);
+  const uint32_t v = variant_of(s);
+  tnc_p8::P8Prob g;
+  if (int rc = fill_gemm(d, s, rg, (__half*)(s.swap ? planes_b : planes_a), (__half*)(s.swap ? planes_a : planes_b),
+                         false, out, prime_at, g))
+    return rc;
+  if (probs.items[v] + g.n_items >= (1ull << 31) || prime_at + rg > tnc_p8::kLaunchPrimes)
+    return set_error(TNC_ERR_TOO_LARGE, "dense steps of a level have too many tiles");
+  g.item_lo = (uint32_t)probs.items[v];
+  probs.items[v] += g.n_items;
+  const char* p = reinterpret_cast<const char*>(&g);
+  probs.descs[v].insert(probs.descs[v].end(), p, p + sizeof(g));
+  probs.n[v]++;
+  return TNC_OK;
+}
+
+int p8_gemm_launch(uint32_t rg, int variant, const char* dev, uint32_t n, uint32_t items, const uint32_t* primes,
+                   uint32_t n_primes, uint32_t* dev_err, int sms, void* stream) {
+  using namespace tnc_p8;
+  if (n > kMaxProbs || n_primes > kLaunchPrimes) return set_error(TNC_ERR_INVALID, "internal: too many dense steps in a launch");
+  P8Primes pr{};
+  for (uint32_t i = 0; i < n_primes; i++) {
+    pr.pf[i] = (float)primes[i];
+    pr.invp[i] = 1.0f / (float)primes[i];
+  }
+  const P8Prob* p = reinterpret_cast<const P8Prob*>(dev);
+  cudaStream_t st = (cudaStream_t)stream;
+  if (rg == 4) return launch_variant<4>((uint32_t)variant, p, n, items, pr, sms, dev_err, st);
+  if (rg == 2) return launch_variant<2>((uint32_t)variant, p, n, items, pr, sms, dev_err, st);
+  return launch_variant<1>((uint32_t)variant, p, n, items, pr, sms, dev_err, st);
+}
+
+size_t p8_prob_bytes() { return sizeof(tnc_p8::P8Prob); }
 
 }  // namespace tnc

@@ -156,7 +156,7 @@ constexpr int kP8MaxResidues = 53;  // odd primes in [3, 251]
 std::vector<uint32_t> default_primes_p8(int n);
 bool is_prime_u32(uint32_t n);
 
-// tc.cu: dense steps on the tensor cores (exact 8-bit-limb GEMMs)
+// tc.cu: dense steps of TNC_PATH_TC (u32 residues) on the tensor cores
 bool tc_eligible(const StepDesc& d);
 // TNC_PATH_TC_P8 dense steps (tc_p8.cu).
 bool p8_eligible(const StepDesc& d);
@@ -200,11 +200,46 @@ int p8_batch(const P8Step* steps, int n, uint32_t rg, uint8_t* arena, uint64_t a
              uint8_t* part, std::vector<char>& host, P8Batch& b);
 int p8_run(const P8Batch& b, const char* dev, const uint32_t* primes, uint32_t rg, uint32_t* dev_err, int sms,
            void* stream);
-size_t tc_step_bytes();
-void tc_make_step(const StepDesc& d, uint32_t p, void* out);
-uint32_t tc_split_log(const StepDesc& d);
-uint64_t tc_part_entries();
-int tc_launch(const void* dev_step, const StepDesc& d, uint32_t* arena, uint32_t* part, uint32_t* dev_err,
-              void* stream);
+// GEMM descriptors for operand planes that the caller packs (tc.cu): one step
+// appended to the variant's list; and the launch of a list.
+struct P8Probs {
+  std::vector<char> descs[6];
+  uint64_t items[6] = {0, 0, 0, 0, 0, 0};
+  uint32_t n[6] = {0, 0, 0, 0, 0, 0};
+};
+int p8_gemm_desc(const StepDesc& d, uint32_t rg, void* planes_a, void* planes_b, uint8_t* out, uint32_t prime_at,
+                 P8Probs& probs);
+int p8_gemm_launch(uint32_t rg, int variant, const char* dev, uint32_t n, uint32_t items, const uint32_t* primes,
+                   uint32_t n_primes, uint32_t* dev_err, int sms, void* stream);
+size_t p8_prob_bytes();
+
+// One dense step of TNC_PATH_TC for residues r .. of the pass's entries.
+struct TcUnit {
+  StepDesc d;
+  uint32_t r;
+};
+// Small primes that a step of 2^k products of residues below 2^31 needs, and
+// per residue the bytes of its operands' fp16 planes and of its output's small
+// residues.
+uint32_t tc_small_primes(uint32_t k);
+uint64_t tc_plane_bytes(const StepDesc& d);
+uint64_t tc_byte_bytes(const StepDesc& d);
+// Units of nr residues (all rg of the pass, or one) launched together (as
+// P8Batch), and their descriptors (at most n nr tc_unit_bytes()).
+struct TcBatch {
+  struct Gemm {
+    uint32_t n, items;
+    size_t off;
+  } gemm[3][6];  // residues per item 4, 2, 1; tile widths as P8Batch
+  uint32_t nr, n_units, pack_tiles, blocks, steps, splits;
+  size_t pack_off, join_off;
+};
+size_t tc_unit_bytes();
+uint32_t tc_max_units(uint32_t nr);
+int tc_batch(const TcUnit* units, int n, uint32_t nr, uint32_t rg, uint32_t* arena, uint64_t arena_bytes, uint8_t* planes,
+             uint8_t* bytes, std::vector<char>& host, TcBatch& b);
+std::vector<char> tc_consts(const uint32_t* primes, uint32_t rg);  // a pass's, for tc_run
+int tc_run(const TcBatch& b, const char* dev, const std::vector<char>& consts, uint32_t rg, uint32_t* dev_err, int sms,
+           void* stream);
 
 }  // namespace tnc
