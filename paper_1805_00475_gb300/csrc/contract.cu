@@ -206,31 +206,126 @@ uint32_t splitk_log(const StepDesc& d) {
   return std::min<uint32_t>(ls, d.k - 8u);
 }
 
+// Output bit j of a step comes from bit dst[j] of operand op[j] (0: A, 1: B).
+struct BitMap {
+  int op[64] = {0}, dst[64] = {0};
+  explicit BitMap(const StepDesc& d) {
+    if (d.nra != TNC_BITMAP) {
+      for (int side = 0; side < 2; side++)
+        for (int i = 0; i < (side ? d.nrb : d.nra); i++) {
+          const TncRun& x = side ? d.map.runs.rb[i] : d.map.runs.ra[i];
+          for (int q = 0; q < x.len; q++) {
+            op[x.src + q] = side;
+            dst[x.src + q] = x.dst + q;
+          }
+        }
+    } else {
+      for (int j = 0; j < d.c; j++) {
+        op[j] = d.map.bit[j] >> 7;
+        dst[j] = d.map.bit[j] & 63;
+      }
+    }
+  }
+};
+
+// Grid-wide steps of u32 residues with at least 16 shared values run in
+// shared-memory tiles (block_kernel); the tile shape, -1 if none.
+int block_shape(const StepDesc& d) {
+  const int shape = d.c >= 19 ? 0 : d.c >= 17 ? 1 : d.c >= 16 ? 2 : -1;
+  const int la = std::max(d.ka, d.kb), lb = std::min(d.ka, d.kb);
+  if (shape < 0 || d.k < 4) return -1;
+  if (la >= (shape == 0 ? 6 : 5) && lb >= (shape == 2 ? 4 : 5)) return shape;
+  return -1;
+}
+
+template <int SHAPE>
+tnc_dev::BlockStep make_block_step(const StepDesc& d) {
+  using B = tnc_dev::Blk<SHAPE>;
+  tnc_dev::BlockStep g;
+  std::memset(&g, 0, sizeof(g));
+  // rows from the operand with more free bits (LA >= LB)
+  const int rows = d.ka >= d.kb ? 0 : 1;
+  g.a_off = rows ? d.b_off : d.a_off;
+  g.b_off = rows ? d.a_off : d.b_off;
+  g.c_off = d.c_off;
+  g.k = d.k;
+  g.ka = rows ? d.kb : d.ka;
+  g.kb = rows ? d.ka : d.kb;
+  const BitMap m(d);
+  for (int j = 0; j < d.c; j++) (m.op[j] == rows ? g.wA : g.wB)[m.dst[j]] = 1u << j;
+  int n = 0;
+  for (int j = 0; j < d.c; j++) {  // ascending output weight
+    const bool row = m.op[j] == rows;
+    if (m.dst[j] < (row ? B::LA - B::RA : B::LB - B::RB)) g.bit[n++] = (uint8_t)(m.dst[j] | (row ? 0 : 0x80));
+  }
+  return g;
+}
+static_assert(sizeof(tnc_dev::BlockStep) <= sizeof(GridStep), "either fits the step's part of the workspace");
+
+// Register tiles (tile_kernel) for grid-wide steps that leave enough threads.
+constexpr int kTileMinC = 18, kTileMinCBytes = 16;
+bool tile_eligible(const StepDesc& d, bool bytes) {
+  return d.c >= (bytes ? kTileMinCBytes : kTileMinC) && d.ka >= tnc_dev::kTileA && d.kb >= tnc_dev::kTileB;
+}
+
+tnc_dev::TileStep make_tile_step(const StepDesc& d) {
+  using tnc_dev::kTileA;
+  using tnc_dev::kTileB;
+  tnc_dev::TileStep t;
+  std::memset(&t, 0, sizeof(t));
+  t.a_off = d.a_off;
+  t.b_off = d.b_off;
+  t.c_off = d.c_off;
+  t.k = d.k;
+  t.ka = d.ka;
+  t.kb = d.kb;
+  const BitMap m(d);
+  uint32_t out_a[kTileA], out_b[kTileB];  // output bits of the operands' highest free bits
+  for (int j = 0; j < d.c; j++) {
+    const int top = m.op[j] ? m.dst[j] - (d.kb - kTileB) : m.dst[j] - (d.ka - kTileA);
+    if (top >= 0) {
+      (m.op[j] ? out_b : out_a)[top] = (uint32_t)j;
+    } else {
+      t.wA[t.n_bits] = m.op[j] ? 0u : 1u << m.dst[j];
+      t.wB[t.n_bits] = m.op[j] ? 1u << m.dst[j] : 0u;
+      t.wC[t.n_bits++] = 1u << j;
+    }
+  }
+  for (uint32_t i = 0; i < (1u << kTileA); i++) {
+    t.tA[i] = i << (d.ka - kTileA);
+    for (int b = 0; b < kTileA; b++)
+      if ((i >> b) & 1u) t.cA[i] += 1u << out_a[b];
+  }
+  for (uint32_t i = 0; i < (1u << kTileB); i++) {
+    t.tB[i] = i << (d.kb - kTileB);
+    for (int b = 0; b < kTileB; b++)
+      if ((i >> b) & 1u) t.cB[i] += 1u << out_b[b];
+  }
+  int threads, blocks, sh;
+  grid_shape((int)t.n_bits, &threads, &blocks, &sh);
+  t.s = (uint8_t)sh;
+  for (uint32_t b = (uint32_t)sh; b < t.n_bits; b++) {
+    t.dA[b] = t.wA[b];
+    t.dB[b] = t.wB[b];
+    t.dC[b] = t.wC[b];
+    for (uint32_t j = (uint32_t)sh; j < b; j++) {  // (modulo 2^32)
+      t.dA[b] -= t.wA[j];
+      t.dB[b] -= t.wB[j];
+      t.dC[b] -= t.wC[j];
+    }
+  }
+  return t;
+}
+static_assert(sizeof(tnc_dev::TileStep) <= sizeof(GridStep), "either fits the step's part of the workspace");
+
 GridStep make_grid_step(const StepDesc& d) {
   GridStep g;
   std::memset(&g, 0, sizeof(g));
   g.d = d;
-  int op[64] = {0}, dst[64] = {0};
-  if (d.nra != TNC_BITMAP) {
-    for (int i = 0; i < d.nra; i++)
-      for (int q = 0; q < d.map.runs.ra[i].len; q++) {
-        op[d.map.runs.ra[i].src + q] = 0;
-        dst[d.map.runs.ra[i].src + q] = d.map.runs.ra[i].dst + q;
-      }
-    for (int i = 0; i < d.nrb; i++)
-      for (int q = 0; q < d.map.runs.rb[i].len; q++) {
-        op[d.map.runs.rb[i].src + q] = 1;
-        dst[d.map.runs.rb[i].src + q] = d.map.runs.rb[i].dst + q;
-      }
-  } else {
-    for (int j = 0; j < d.c; j++) {
-      op[j] = d.map.bit[j] >> 7;
-      dst[j] = d.map.bit[j] & 63;
-    }
-  }
+  const BitMap m(d);
   for (int j = 0; j < d.c; j++) {
-    g.wA[j] = op[j] == 0 ? 1ull << dst[j] : 0ull;
-    g.wB[j] = op[j] == 1 ? 1ull << dst[j] : 0ull;
+    g.wA[j] = m.op[j] == 0 ? 1ull << m.dst[j] : 0ull;
+    g.wB[j] = m.op[j] == 1 ? 1ull << m.dst[j] : 0ull;
   }
   int threads, blocks, sh;
   grid_shape(d.c, &threads, &blocks, &sh);
@@ -266,28 +361,11 @@ tnc_dev::OuterStep make_outer_step(const StepDesc& d) {
   o.l_off = s_side ? d.a_off : d.b_off;
   o.c_off = d.c_off;
   o.blocks = (uint32_t)std::min<uint64_t>(((1ull << o.fl) + 255) / 256, (uint64_t)sm_count() * 8);
-  int op[64] = {0}, dst[64] = {0};
-  if (d.nra != TNC_BITMAP) {
-    for (int i = 0; i < d.nra; i++)
-      for (int q = 0; q < d.map.runs.ra[i].len; q++) {
-        op[d.map.runs.ra[i].src + q] = 0;
-        dst[d.map.runs.ra[i].src + q] = d.map.runs.ra[i].dst + q;
-      }
-    for (int i = 0; i < d.nrb; i++)
-      for (int q = 0; q < d.map.runs.rb[i].len; q++) {
-        op[d.map.runs.rb[i].src + q] = 1;
-        dst[d.map.runs.rb[i].src + q] = d.map.runs.rb[i].dst + q;
-      }
-  } else {
-    for (int j = 0; j < d.c; j++) {
-      op[j] = d.map.bit[j] >> 7;
-      dst[j] = d.map.bit[j] & 63;
-    }
-  }
+  const BitMap m(d);
   uint64_t wS[4] = {0, 0, 0, 0};
   for (int j = 0; j < d.c; j++) {
-    if (op[j] == s_side) wS[dst[j]] = 1ull << j;
-    else o.oL[dst[j]] = 1ull << j;
+    if (m.op[j] == s_side) wS[m.dst[j]] = 1ull << j;
+    else o.oL[m.dst[j]] = 1ull << j;
   }
   for (uint32_t x = 0; x < (1u << o.fs); x++)
     for (uint32_t i = 0; i < o.fs; i++)
@@ -967,7 +1045,7 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
   };
   struct Level {
     uint32_t small_lo = 0, small_n = 0, small_work = 0;
-    Range grid{}, outer{};
+    Range grid{}, tile{}, block[3] = {}, outer{};
     std::vector<Range> split;
     std::vector<std::pair<uint32_t, uint32_t>> p8;   // ranges of p8 steps launched together
     std::vector<StepDesc> dense;                     // TNC_PATH_TC dense steps
@@ -975,6 +1053,8 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
   std::vector<Level> lev(n_lev);
   std::vector<GridStep> gsteps;
   std::vector<tnc_dev::OuterStep> outers;
+  std::vector<tnc_dev::TileStep> tiles;
+  std::vector<tnc_dev::BlockStep> blocked[3];  // by tile shape
   std::vector<StepDesc> small;
   std::vector<P8Step> p8steps;
   const int rg_max = groups.rg[0];
@@ -985,6 +1065,9 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
     std::vector<GridStep> split;
     lv.grid.lo = (uint32_t)gsteps.size();
     lv.outer.lo = (uint32_t)outers.size();
+    lv.tile.lo = (uint32_t)tiles.size();
+    for (int q = 0; q < 3; q++) lv.block[q].lo = (uint32_t)blocked[q].size();
+    uint64_t block_tiles[3] = {0, 0, 0};
     const uint32_t p8_lo = (uint32_t)p8steps.size();
     for (int w = 0; w < nw; w++) {
       const Lowered& lw = work[w]->low;
@@ -1008,6 +1091,14 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
           lv.outer.blocks += outers.back().blocks;
         } else if (splitk_log(d) > 0) {
           split.push_back(make_grid_step(d));
+        } else if (const int q = p8 ? -1 : block_shape(d); q >= 0) {
+          blocked[q].push_back(q == 0 ? make_block_step<0>(d) : q == 1 ? make_block_step<1>(d) : make_block_step<2>(d));
+          blocked[q].back().tile_lo = (uint32_t)block_tiles[q];
+          block_tiles[q] += 1ull << (d.c - 11 + q);  // (2^11, 2^10 or 2^9 outputs a tile)
+        } else if (tile_eligible(d, p8)) {
+          tiles.push_back(make_tile_step(d));
+          tiles.back().block_lo = lv.tile.blocks;
+          lv.tile.blocks += 1u << (tiles.back().s - 8);  // 256 threads per block
         } else if (d.c >= 16) {
           gsteps.push_back(make_grid_step(d));
           gsteps.back().block_lo = lv.grid.blocks;
@@ -1024,6 +1115,12 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
     lv.small_work = (uint32_t)wk;
     lv.grid.n = (uint32_t)gsteps.size() - lv.grid.lo;
     lv.outer.n = (uint32_t)outers.size() - lv.outer.lo;
+    lv.tile.n = (uint32_t)tiles.size() - lv.tile.lo;
+    for (int q = 0; q < 3; q++) {
+      if (block_tiles[q] >= (1ull << 31)) return set_error(TNC_ERR_TOO_LARGE, "a merged level has too many tiles");
+      lv.block[q].n = (uint32_t)blocked[q].size() - lv.block[q].lo;
+      lv.block[q].blocks = (uint32_t)block_tiles[q];
+    }
     // split-K steps: as many per launch as the partials' section holds
     const uint64_t part_cap = L.part_bytes / ((uint64_t)rg_max * sizeof(uint32_t));
     for (GridStep& g : split) {
@@ -1058,6 +1155,9 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
   const size_t at_small = put(small.data(), small.size() * sizeof(StepDesc));
   const size_t at_grid = put(gsteps.data(), gsteps.size() * sizeof(GridStep));
   const size_t at_outer = put(outers.data(), outers.size() * sizeof(tnc_dev::OuterStep));
+  size_t at_block[3];
+  for (int q = 0; q < 3; q++) at_block[q] = put(blocked[q].data(), blocked[q].size() * sizeof(tnc_dev::BlockStep));
+  const size_t at_tile = put(tiles.data(), tiles.size() * sizeof(tnc_dev::TileStep));
   // dense descriptors, for each number of residues per entry that a pass has
   uint32_t* part = (uint32_t*)(ws + L.off_part);
   std::vector<P8Batch> p8batches[5];
@@ -1133,6 +1233,7 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
   }
   const GridStep* d_steps = (const GridStep*)(ws + at_grid);
   const StepDesc* d_small = (const StepDesc*)(ws + at_small);
+  const tnc_dev::TileStep* d_tile = (const tnc_dev::TileStep*)(ws + at_tile);
   const tnc_dev::OuterStep* d_outer = (const tnc_dev::OuterStep*)(ws + at_outer);
   uint32_t* results = (uint32_t*)(ws + L.off_results);
   std::vector<tnc_dev::Roots> roots;
@@ -1202,6 +1303,30 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
         if (lv.outer.n) {
           tnc_dev::outer_kernel<RG, W, N30><<<lv.outer.blocks, 256, 0, st>>>(d_outer + lv.outer.lo, lv.outer.n, arena, mg);
           g_launches.outer++;
+        }
+        if constexpr (sizeof(W) == 4) {
+          auto blocks = [&](auto shape) -> int {
+            constexpr int Q = decltype(shape)::value;
+            const Range& r = lv.block[Q];
+            if (!r.n) return TNC_OK;
+            using B = tnc_dev::Blk<Q>;
+            constexpr size_t smem =
+                (size_t)tnc_dev::kBlkStages * ((1 << B::LA) + (1 << B::LB)) * tnc_dev::kBlkK * RG * sizeof(uint32_t);
+            auto k = tnc_dev::block_kernel<RG, Q, N30>;
+            if (smem > 48 * 1024) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            k<<<std::min(r.blocks, 2u * (unsigned)sms), 256, smem, st>>>(
+                (const tnc_dev::BlockStep*)(ws + at_block[Q]) + r.lo, r.n, r.blocks, arena, mg);
+            g_launches.grid_step++;
+            return TNC_OK;
+          };
+          int rc2 = blocks(std::integral_constant<int, 0>());
+          if (!rc2) rc2 = blocks(std::integral_constant<int, 1>());
+          if (!rc2) rc2 = blocks(std::integral_constant<int, 2>());
+          if (rc2) return rc2;
+        }
+        if (lv.tile.n) {
+          tnc_dev::tile_kernel<RG, W, N30><<<lv.tile.blocks, 256, 0, st>>>(d_tile + lv.tile.lo, lv.tile.n, arena, mg);
+          g_launches.grid_step++;
         }
         if (lv.grid.n) {
           tnc_dev::step_kernel<RG, W, N30><<<lv.grid.blocks, 256, 0, st>>>(d_steps + lv.grid.lo, lv.grid.n, arena, mg);

@@ -67,6 +67,299 @@ __global__ void __launch_bounds__(256) step_kernel(const GridStep* __restrict__ 
   }
 }
 
+// The bigger of these steps in register tiles: a thread computes 2^kTileA rows
+// x 2^kTileB columns of outputs (the operands' highest free bits), so each
+// operand entry it loads serves several products.  The other output bits are
+// walked as in step_kernel, with the output's address by deltas too.  (Byte
+// residues, 10 launches of a cubic VC formula with n = 180: 111 -> 78 us; u32
+// residues, 2^20 outputs: 9.6 -> 7.4 us.  4 x 4 outputs: no faster on these, and the dense
+// steps it would help run in shared-memory tiles.)
+constexpr int kTileA = 1, kTileB = 1;
+struct TileStep {
+  uint64_t a_off, b_off, c_off;
+  uint32_t wA[32], wB[32], wC[32];  // address weights of the bits walked
+  uint32_t dA[32], dB[32], dC[32];  // address deltas when the counter sets bit t
+  uint32_t tA[1 << kTileA], cA[1 << kTileA];  // operand and output offsets of the tile's rows
+  uint32_t tB[1 << kTileB], cB[1 << kTileB];  // and columns
+  uint32_t n_bits, block_lo;        // bits walked; first block in the launch
+  uint8_t k, ka, kb, s;             // 2^s threads
+  uint32_t pad;
+};
+
+template <int RG, typename W = uint32_t, bool N30 = false>
+__global__ void __launch_bounds__(256) tile_kernel(const TileStep* __restrict__ steps, uint32_t n_steps,
+                                                   W* __restrict__ arena, ModGroup mg) {
+  uint32_t lo = 0, hi = n_steps - 1;
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi + 1) >> 1;
+    if (steps[mid].block_lo <= blockIdx.x) lo = mid;
+    else hi = mid - 1;
+  }
+  const TileStep* __restrict__ g = steps + lo;
+  constexpr int NA = 1 << kTileA, NB = 1 << kTileB;
+  using Acc = std::conditional_t<sizeof(W) == 1, uint32_t, uint64_t>;
+  const uint32_t s = g->s, K = 1u << g->k;
+  const uint64_t n = 1ull << g->n_bits;
+  const uint64_t sa = (uint64_t)RG << g->ka, sb = (uint64_t)RG << g->kb;
+  uint64_t t = (uint64_t)(blockIdx.x - g->block_lo) * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  uint32_t ia = 0, ib = 0, ic = 0;
+  for (uint32_t j = 0; j < g->n_bits; j++)
+    if ((t >> j) & 1ull) {
+      ia += g->wA[j];
+      ib += g->wB[j];
+      ic += g->wC[j];
+    }
+  uint64_t oa[NA], ob[NB];
+#pragma unroll
+  for (int i = 0; i < NA; i++) oa[i] = (uint64_t)g->tA[i] * RG;
+#pragma unroll
+  for (int i = 0; i < NB; i++) ob[i] = (uint64_t)g->tB[i] * RG;
+  for (;;) {
+    const W* A = arena + (g->a_off + ia) * RG;
+    const W* B = arena + (g->b_off + ib) * RG;
+    Acc acc[NA][NB][RG];
+#pragma unroll
+    for (int i = 0; i < NA; i++)
+#pragma unroll
+      for (int j = 0; j < NB; j++)
+#pragma unroll
+        for (int r = 0; r < RG; r++) acc[i][j][r] = 0;
+    auto product = [&] {
+      uint32_t va[NA][RG], vb[NB][RG];
+#pragma unroll
+      for (int i = 0; i < NA; i++) load_entry<RG, W>(A + oa[i], va[i]);
+#pragma unroll
+      for (int j = 0; j < NB; j++) load_entry<RG, W>(B + ob[j], vb[j]);
+      A += sa;
+      B += sb;
+#pragma unroll
+      for (int i = 0; i < NA; i++)
+#pragma unroll
+        for (int j = 0; j < NB; j++)
+#pragma unroll
+          for (int r = 0; r < RG; r++) acc[i][j][r] += (Acc)va[i][r] * vb[j][r];
+    };
+    uint32_t q = 0;
+#pragma unroll 1
+    for (; q + 4 <= K; q += 4) {
+#pragma unroll
+      for (int u = 0; u < 4; u++) product();
+      if (((q + 4) & mg.red_mask) == 0) {
+#pragma unroll
+        for (int i = 0; i < NA; i++)
+#pragma unroll
+          for (int j = 0; j < NB; j++)
+#pragma unroll
+            for (int r = 0; r < RG; r++) acc[i][j][r] = reduce_acc<N30>(acc[i][j][r], mg, r);
+      }
+    }
+    for (; q < K; q++) product();  // K < 4
+    W* C = arena + (g->c_off + ic) * RG;
+#pragma unroll
+    for (int i = 0; i < NA; i++)
+#pragma unroll
+      for (int j = 0; j < NB; j++) {
+        uint32_t out[RG];
+#pragma unroll
+        for (int r = 0; r < RG; r++) out[r] = reduce_acc<N30>(acc[i][j][r], mg, r);
+        store_entry<RG, W>(C + (uint64_t)(g->cA[i] + g->cB[j]) * RG, out);
+      }
+    const uint64_t u = t >> s;
+    t += 1ull << s;
+    if (t >= n) break;
+    const uint32_t b = s + (uint32_t)(__ffsll((long long)~u) - 1);
+    ia += g->dA[b];
+    ib += g->dB[b];
+    ic += g->dC[b];
+  }
+}
+
+// The densest of these steps (u32 residues) in shared-memory tiles, as a
+// modular matrix product: a CTA computes 2^LA rows x 2^LB columns, staging 16
+// shared values of its rows and columns at a time (cp.async, three stages,
+// running on across its tiles), a thread 2^RA x 2^RB of the outputs.  Without
+// the staging every warp reads its operands from L2 (about 7 TB/s at 2^21
+// outputs of 512 products, which is what bounds step_kernel there), and with
+// 2^16 outputs a thread per output leaves most of each SM idle.  A tile's
+// output bits other than the thread's own (the rows' RA highest, the columns'
+// RB highest) go to lanes and warps by output weight, lightest first, so that a
+// warp's stores are as close together as the step's bit map allows.
+// Bound by the 64-bit multiply-adds: 2^21 outputs of 512 products, 4 residues,
+// 1190 -> 724 us = 5.9e12 products/s, the rate of the bare primitive
+// (tnc_probe_modmac 5.8e12); the 16 shared values of a stage fully unrolled (by 4:
+// 908 us, by 8: 823) at two CTAs per SM.  2^24 outputs of 16 products: 474 ->
+// 216 us; 2^16 outputs of 256 products, 2 residues of wide primes: 34 -> 17 us.
+constexpr int kBlkK = 16, kBlkStages = 3;
+// Shapes by the step's outputs: 64 x 32 (4 x 2 a thread) from 2^19 on, 32 x 32
+// (2 x 2) from 2^17 on, 32 x 16 (2 x 1) at 2^16: at least 128 tiles.
+template <int SHAPE>
+struct Blk {
+  static constexpr int LA = SHAPE == 0 ? 6 : 5, LB = SHAPE == 2 ? 4 : 5, RA = SHAPE == 0 ? 2 : 1, RB = SHAPE == 2 ? 0 : 1;
+};
+struct BlockStep {
+  uint64_t a_off, b_off, c_off;
+  uint32_t wA[32], wB[32];  // output weight of row bit j / column bit j
+  uint8_t bit[8];           // thread bit i: column bit j (0x80 | j) or row bit j
+  uint32_t k, ka, kb, tile_lo;
+};
+
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void* dst, const void* src) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  if constexpr (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES) : "memory");
+}
+
+template <int RG, int SHAPE, bool N30 = false>
+__global__ void __launch_bounds__(256, 2) block_kernel(const BlockStep* __restrict__ steps, uint32_t n_steps,
+                                                       uint32_t n_tiles, uint32_t* __restrict__ arena, ModGroup mg) {
+  constexpr int kBlkA = Blk<SHAPE>::LA, kBlkB = Blk<SHAPE>::LB, RA = Blk<SHAPE>::RA, RB = Blk<SHAPE>::RB;
+  constexpr int TA = 1 << RA, TB = 1 << RB;
+  constexpr uint32_t NA = 1u << kBlkA, NB = 1u << kBlkB, kStage = (NA + NB) * kBlkK * RG;  // words
+  extern __shared__ __align__(16) uint32_t sm[];
+  const uint32_t tid = threadIdx.x;
+  auto step_of = [&](uint32_t tile) {
+    uint32_t lo = 0, hi = n_steps - 1;
+    while (lo < hi) {
+      const uint32_t mid = (lo + hi + 1) >> 1;
+      if (steps[mid].tile_lo <= tile) lo = mid;
+      else hi = mid - 1;
+    }
+    return steps + lo;
+  };
+  // the loader runs kBlkStages - 1 chunks ahead of the products
+  uint32_t l_tile = blockIdx.x, l_chunk = 0, l_n = 0, l_slot = 0;
+  const uint32_t *l_a = nullptr, *l_b = nullptr;
+  uint64_t l_sa = 0, l_sb = 0;
+  auto load_next = [&] {
+    if (l_tile < n_tiles) {
+      if (l_chunk == 0) {
+        const BlockStep* g = step_of(l_tile);
+        const uint32_t t = l_tile - g->tile_lo, ta = t & ((1u << (g->ka - kBlkA)) - 1u), tb = t >> (g->ka - kBlkA);
+        l_n = 1u << (g->k - 4);
+        l_sa = (uint64_t)RG << g->ka;
+        l_sb = (uint64_t)RG << g->kb;
+        l_a = arena + (g->a_off + ((uint64_t)ta << kBlkA)) * RG;
+        l_b = arena + (g->b_off + ((uint64_t)tb << kBlkB)) * RG;
+      }
+      uint32_t* dst = sm + l_slot * kStage;
+#pragma unroll
+      for (uint32_t i = 0; i < NA * kBlkK / 256; i++) {
+        const uint32_t e = tid + 256 * i, q = e >> kBlkA, row = e & (NA - 1);
+        cp_async<4 * RG>(dst + e * RG, l_a + q * l_sa + row * RG);
+      }
+#pragma unroll
+      for (uint32_t i = 0; i < NB * kBlkK / 256; i++) {  // (at least one)
+        const uint32_t e = tid + 256 * i, q = e >> kBlkB, col = e & (NB - 1);
+        cp_async<4 * RG>(dst + (NA * kBlkK + e) * RG, l_b + q * l_sb + col * RG);
+      }
+      l_a += kBlkK * l_sa;
+      l_b += kBlkK * l_sb;
+      if (++l_slot == kBlkStages) l_slot = 0;
+      if (++l_chunk == l_n) {
+        l_chunk = 0;
+        l_tile += gridDim.x;
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int i = 0; i < kBlkStages - 1; i++) load_next();
+  uint32_t slot = 0;
+  const BlockStep* cur = nullptr;
+  uint32_t row = 0, col = 0, off = 0;
+  for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    const BlockStep* g = step_of(tile);
+    if (g != cur) {  // this thread's place in a tile of the step
+      cur = g;
+      row = col = off = 0;
+#pragma unroll
+      for (int i = 0; i < 8; i++)
+        if ((tid >> i) & 1u) {
+          const uint32_t b = g->bit[i];
+          if (b & 0x80u) {
+            col |= 1u << (b & 31u);
+            off += g->wB[b & 31u];
+          } else {
+            row |= 1u << b;
+            off += g->wA[b];
+          }
+        }
+    }
+    uint64_t acc[TA][TB][RG];
+#pragma unroll
+    for (int i = 0; i < TA; i++)
+#pragma unroll
+      for (int j = 0; j < TB; j++)
+#pragma unroll
+        for (int r = 0; r < RG; r++) acc[i][j][r] = 0;
+    const uint32_t chunks = 1u << (g->k - 4);
+    for (uint32_t c = 0; c < chunks; c++) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(kBlkStages - 2) : "memory");
+      __syncthreads();  // the chunk has landed for every thread, and the slot that is loaded next is free
+      load_next();
+      const uint32_t* sa = sm + slot * kStage + row * RG;
+      const uint32_t* sb = sm + slot * kStage + (NA * kBlkK + col) * RG;
+      if (++slot == kBlkStages) slot = 0;
+#pragma unroll 16
+      for (uint32_t q = 0; q < kBlkK; q++) {
+        uint32_t va[TA][RG], vb[TB][RG];
+#pragma unroll
+        for (int i = 0; i < 4; i++) load_entry<RG>(sa + (q * NA + i * (NA / TA)) * RG, va[i]);
+#pragma unroll
+        for (int j = 0; j < TB; j++) load_entry<RG>(sb + (q * NB + j * (NB / TB)) * RG, vb[j]);
+#pragma unroll
+        for (int i = 0; i < TA; i++)
+#pragma unroll
+          for (int j = 0; j < TB; j++)
+#pragma unroll
+            for (int r = 0; r < RG; r++) acc[i][j][r] += (uint64_t)va[i][r] * vb[j][r];
+        if (!N30 && ((q + 1) & mg.red_mask) == 0) {  // (16 products fit for the default primes)
+#pragma unroll
+          for (int i = 0; i < TA; i++)
+#pragma unroll
+            for (int j = 0; j < TB; j++)
+#pragma unroll
+              for (int r = 0; r < RG; r++) acc[i][j][r] = reduce64<N30>(acc[i][j][r], mg, r);
+        }
+      }
+      if (N30) {
+#pragma unroll
+        for (int i = 0; i < TA; i++)
+#pragma unroll
+          for (int j = 0; j < TB; j++)
+#pragma unroll
+            for (int r = 0; r < RG; r++) acc[i][j][r] = reduce64<N30>(acc[i][j][r], mg, r);
+      }
+    }
+    const uint32_t t = tile - g->tile_lo, ta = t & ((1u << (g->ka - kBlkA)) - 1u), tb = t >> (g->ka - kBlkA);
+    uint32_t o = off;
+    for (uint32_t j = kBlkA; j < g->ka; j++)
+      if ((ta >> (j - kBlkA)) & 1u) o += g->wA[j];
+    for (uint32_t j = kBlkB; j < g->kb; j++)
+      if ((tb >> (j - kBlkB)) & 1u) o += g->wB[j];
+    uint32_t* C = arena + g->c_off * RG;
+#pragma unroll
+    for (int i = 0; i < TA; i++)
+#pragma unroll
+      for (int j = 0; j < TB; j++) {
+        uint32_t out[RG];
+#pragma unroll
+        for (int r = 0; r < RG; r++) out[r] = (uint32_t)acc[i][j][r];  // (reduced after every chunk)
+        uint32_t e = o;
+#pragma unroll
+        for (int b = 0; b < RA; b++)
+          if ((i >> b) & 1) e += g->wA[kBlkA - RA + b];
+#pragma unroll
+        for (int b = 0; b < RB; b++)
+          if ((j >> b) & 1) e += g->wB[kBlkB - RB + b];
+        store_entry<RG>(C + (uint64_t)e * RG, out);
+      }
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 // A big step with one small operand (Sec. 2.1 with a skinny matrix): S has
 // 2^fs <= 16 rows, the shared dimension 2^k <= 8, the large operand L 2^fl
 // rows.  S's 2^(fs+k) entries are staged in shared memory; a thread takes a
