@@ -167,6 +167,13 @@ int dispatch_rg(int rg, F&& f) {
 
 // ---------------------------------------------------------------- single formula
 
+// One pass over the steps: `groups` residue groups of rg residues each, side
+// by side in one launch per kind of step, from residue `col` on (the last group
+// of a filled-up pass has fewer).
+struct PassShape {
+  int rg, groups, col;
+};
+
 // Workspace of a group of plans contracted together (one plan: the
 // single-formula layout).  Descriptors of all plans side by side; every plan's
 // tensors in its own part of one arena (arena_base, in entries, a multiple of
@@ -177,6 +184,8 @@ struct SeqLayout {
       off_arena, total;
   uint64_t n_out;  // result entries of the whole group
   uint64_t part_bytes, p8_bytes;  // the sections' sizes
+  std::vector<PassShape> passes;
+  uint64_t arena_entries;  // of one residue group's arena
   size_t n_dense;
   std::vector<uint64_t> arena_base, res_base, leaf_base, table_base;
 };
@@ -381,10 +390,13 @@ tnc_dev::OuterStep make_outer_step(const StepDesc& d) {
 // group's maximum).
 struct Foot {
   size_t leaves = 0, tables = 0, nseq = 0, nlvl = 0, n_dense = 0;
-  uint64_t n_out = 0, arena = 0, part = 0, p8 = 0;
-  // dense steps of a tree level on the tensor-core paths: planes, and partials
-  // or small residues
-  std::vector<uint64_t> lvl_p8, lvl_part;
+  uint64_t n_out = 0, arena = 0;
+  double cost = 0;  // multiply-adds and entries per residue
+  // bytes per residue of the largest step: split-K partials; on the
+  // tensor-core paths a dense step's planes, and its partials or small residues
+  uint64_t split = 0, planes = 0, parts = 0;
+  uint64_t kept = 0;  // (kept_split_bytes)
+  std::vector<uint64_t> lvl_planes, lvl_parts;  // of all dense steps of a tree level
   void add(const Foot& f) {
     leaves += f.leaves;
     tables += f.tables;
@@ -393,16 +405,38 @@ struct Foot {
     n_dense += f.n_dense;
     n_out += f.n_out;
     arena += f.arena;
-    part = std::max(part, f.part);
-    p8 = std::max(p8, f.p8);
-    lvl_p8.resize(std::max(lvl_p8.size(), f.lvl_p8.size()));
-    lvl_part.resize(std::max(lvl_part.size(), f.lvl_part.size()));
-    for (size_t l = 0; l < f.lvl_p8.size(); l++) {
-      lvl_p8[l] += f.lvl_p8[l];
-      lvl_part[l] += f.lvl_part[l];
+    cost += f.cost;
+    split = std::max(split, f.split);
+    planes = std::max(planes, f.planes);
+    parts = std::max(parts, f.parts);
+    kept = std::max(kept, f.kept);
+    lvl_planes.resize(std::max(lvl_planes.size(), f.lvl_planes.size()));
+    lvl_parts.resize(std::max(lvl_parts.size(), f.lvl_parts.size()));
+    for (size_t l = 0; l < f.lvl_planes.size(); l++) {
+      lvl_planes[l] += f.lvl_planes[l];
+      lvl_parts[l] += f.lvl_parts[l];
     }
   }
 };
+
+// Residue groups run side by side while their arenas together stay within
+// kMergeArena: 16 to 20 residues of cubic VC formulas with 100 to 160 vertices
+// on TNC_PATH_TC_P8 took 1.4 to 2.4 times as long in one pass per group. (512
+// MiB, 2 GiB, 8 GiB: 48 1-in-3 formulas 5.98, 5.87, 5.49 ms; 4 slices of a
+// formula with n = 160 1.82, 1.49, 1.48 ms; n = 180, 20 residues 11.0, 11.1,
+// 10.5 ms.)
+constexpr uint64_t kMergeArena = 8192ull << 20;
+
+// The last group is filled up to four residues, instead of passes of two and of
+// one, where the residues that nobody asked for cost less than the launches
+// saved: a pass is 15 to 25 launches (50 to 100 us), a residue `cost`
+// multiply-adds at about 5e12 per second on the CUDA cores, 5e14 on
+// TNC_PATH_TC_P8 and a tenth of that on TNC_PATH_TC.
+bool fill_up(int R, double cost, int path) {
+  const int rest = R % 4, saved = rest == 3 ? (R > 4 ? 2 : 1) : (R > 4 ? 1 : 0);
+  const double rate = path == TNC_PATH_TC_P8 ? 5e14 : path == TNC_PATH_TC ? 5e13 : 5e12;
+  return rest && (4 - rest) * cost / rate < saved * 50e-6;
+}
 
 // The dense steps of a level are launched together as far as their planes and
 // partials fit; up to these sizes the sections grow beyond the largest single
@@ -435,43 +469,42 @@ uint64_t kept_split_bytes(const StepDesc& d) {
 }
 constexpr size_t kKeptDenseBytes = 600;
 
-Foot foot_of(const tnc_plan_t* p, int R, int path) {
-  const int rg_max = R >= 4 ? 4 : (R >= 2 ? 2 : 1);
+Foot foot_of(const tnc_plan_t* p, int path) {
   Foot f;
   f.leaves = p->low.leaves.size();
   f.tables = p->low.leaf_tables.size();
   f.nseq = p->low.seq_steps.size();
   f.nlvl = p->low.lvl_steps.size();
   f.n_out = 1ull << p->net.open_vars.size();
+  f.cost = p->cost.macs + p->cost.entries;
   const bool p8 = path == TNC_PATH_TC_P8, tc = path == TNC_PATH_TC;
   for (size_t l = 0; l + 1 < p->low.lvl_start.size(); l++) {
-    uint64_t sum_p8 = 0, sum_part = 0;
+    uint64_t sum_planes = 0, sum_parts = 0;
     for (uint32_t i = p->low.lvl_start[l]; i < p->low.lvl_start[l + 1]; i++) {
       const StepDesc& d = p->low.lvl_steps[i];
       if (splitk_log(d) > 0)
-        f.part = std::max<uint64_t>(f.part, (1ull << (d.c + splitk_log(d))) * rg_max * sizeof(uint32_t));
-      uint64_t planes = 0, parts = 0, units = 1;
+        f.split = std::max<uint64_t>(f.split, (1ull << (d.c + splitk_log(d))) * sizeof(uint32_t));
+      uint64_t planes = 0, parts = 0;
       if (p8 && p8_eligible(d)) {
-        planes = p8_scratch_bytes(P8Step{d, p8_flags(p->low, i)}, rg_max);
-        parts = p8_part_bytes(d, rg_max);
+        planes = p8_scratch_bytes(P8Step{d, p8_flags(p->low, i)}, 1);
+        parts = p8_part_bytes(d, 1);
         f.n_dense++;
       } else if (!p8 && tc_eligible(d)) {
         f.n_dense++;
         if (tc) {
           planes = tc_plane_bytes(d);
           parts = tc_byte_bytes(d);
-          units = rg_max;
         } else {
-          f.part = std::max<uint64_t>(f.part, kept_split_bytes(d));
+          f.kept = std::max<uint64_t>(f.kept, kept_split_bytes(d));
         }
       }
-      f.part = std::max<uint64_t>(f.part, parts);
-      f.p8 = std::max<uint64_t>(f.p8, planes);
-      sum_p8 += planes * units;
-      sum_part += parts * units;
+      f.planes = std::max<uint64_t>(f.planes, planes);
+      f.parts = std::max<uint64_t>(f.parts, parts);
+      sum_planes += planes;
+      sum_parts += parts;
     }
-    f.lvl_p8.push_back(sum_p8);
-    f.lvl_part.push_back(sum_part);
+    f.lvl_planes.push_back(sum_planes);
+    f.lvl_parts.push_back(sum_parts);
   }
   uint64_t arena = std::max(p->low.seq_arena_entries, p->low.lvl_arena_entries);
   if (p8) arena = std::max(arena, p->low.p8_arena_entries);
@@ -479,10 +512,36 @@ Foot foot_of(const tnc_plan_t* p, int R, int path) {
   return f;
 }
 
-// Offsets of the workspace sections for the group footprint f.
-SeqLayout layout_of(const Foot& f, int R, int path) {
+// Offsets of the workspace sections for the group footprint f.  wide: with the
+// residue groups side by side as far as kMergeArena allows; else one group at a
+// time (the least that works).
+SeqLayout layout_of(const Foot& f, int R, int path, bool wide) {
   SeqLayout s{};
-  const int rg_max = R >= 4 ? 4 : (R >= 2 ? 2 : 1);
+  const bool p8 = path == TNC_PATH_TC_P8, tc = path == TNC_PATH_TC;
+  const size_t word = p8 ? 1 : sizeof(uint32_t);  // bytes per residue
+  // the passes
+  int quads = R / 4, rest = R % 4;
+  if (wide && fill_up(R, f.cost, path)) {
+    quads++;
+    rest = 0;
+  }
+  int most = 1;
+  if (wide && quads > 1) {
+    most = (int)std::max<uint64_t>(1, std::min<uint64_t>(quads, kMergeArena / std::max<uint64_t>(1, f.arena * 4 * word)));
+    const int n = (quads + most - 1) / most;
+    most = (quads + n - 1) / n;  // evenly
+  }
+  for (int q = 0; q < quads; q += most) s.passes.push_back(PassShape{4, std::min(most, quads - q), 4 * q});
+  if (rest & 2) s.passes.push_back(PassShape{2, 1, 4 * quads});
+  if (rest & 1) s.passes.push_back(PassShape{1, 1, 4 * quads + (rest & 2)});
+  const uint64_t res = (uint64_t)s.passes[0].rg * s.passes[0].groups;  // residues of the widest pass
+  uint64_t kinds = 0;  // residues and groups of the different passes (their dense descriptors)
+  uint64_t kind_groups = 0;
+  for (size_t i = 0; i < s.passes.size(); i++) {
+    if (i && s.passes[i].rg == s.passes[i - 1].rg && s.passes[i].groups == s.passes[i - 1].groups) continue;
+    kinds += (uint64_t)s.passes[i].rg * s.passes[i].groups;
+    kind_groups += s.passes[i].groups;
+  }
   size_t o = 0;
   auto sect = [&](size_t& off, size_t bytes) {
     off = o;
@@ -492,41 +551,42 @@ SeqLayout layout_of(const Foot& f, int R, int path) {
   sect(s.off_tables, f.tables * sizeof(uint32_t));
   sect(s.off_steps, std::max(f.nseq, f.nlvl) * sizeof(GridStep));
   sect(s.off_small, f.nlvl * sizeof(StepDesc));
-  uint64_t part = f.part, p8 = f.p8;
-  const bool tc = path == TNC_PATH_TC;
-  for (uint64_t v : f.lvl_part) part = std::max(part, std::min(v, tc ? kTcBytes : kGroupParts));
-  for (uint64_t v : f.lvl_p8) p8 = std::max(p8, std::min(v, tc ? kTcPlanes : kGroupPlanes));
+  // planes and partials: of the largest step (one residue of it on TNC_PATH_TC),
+  // or of a level's steps together as far as the limits allow
+  uint64_t part = std::max(std::max(f.split, p8 ? f.parts : 0) * res, std::max(f.kept, tc ? f.parts : 0));
+  uint64_t planes = p8 ? f.planes * res : f.planes;
+  for (uint64_t v : f.lvl_parts) part = std::max(part, std::min(v * res, tc ? kTcBytes : kGroupParts));
+  for (uint64_t v : f.lvl_planes) planes = std::max(planes, std::min(v * res, tc ? kTcPlanes : kGroupPlanes));
   s.part_bytes = part;
-  s.p8_bytes = p8;
-  // (dense descriptors hold addresses for a pass's residues per entry: 4, 2 and 1)
-  sect(s.off_tc, path == TNC_PATH_TC_P8 ? f.n_dense * 3 * p8_step_bytes()
-                 : path == TNC_PATH_TC ? f.n_dense * 7 * tc_unit_bytes()
-                                       : f.n_dense * R * kKeptDenseBytes);
+  s.p8_bytes = planes;
+  sect(s.off_tc, p8   ? f.n_dense * kind_groups * p8_step_bytes()
+                 : tc ? f.n_dense * kinds * tc_unit_bytes()
+                      : f.n_dense * R * kKeptDenseBytes);
   sect(s.off_part, part);
   sect(s.off_err, 64);
   sect(s.off_results, f.n_out * R * sizeof(uint32_t));
   sect(s.off_limbs, f.n_out * ((31 * R + 31) / 32) * sizeof(uint32_t));
-  sect(s.off_p8, p8);
-  const size_t word = path == TNC_PATH_TC_P8 ? 1 : sizeof(uint32_t);  // bytes per residue
-  sect(s.off_arena, f.arena * rg_max * word);
+  sect(s.off_p8, planes);
+  sect(s.off_arena, f.arena * res * word);
   s.total = o;
   s.n_out = f.n_out;
   s.n_dense = f.n_dense;
+  s.arena_entries = f.arena;
   return s;
 }
 
-SeqLayout group_layout(const tnc_plan_t* const* plans, int n, int R, int path = TNC_PATH_INT64) {
+SeqLayout group_layout(const tnc_plan_t* const* plans, int n, int R, int path, bool wide) {
   Foot sum;
   std::vector<uint64_t> arena_base, res_base, leaf_base, table_base;
   for (int i = 0; i < n; i++) {
-    const Foot f = foot_of(plans[i], R, path);
+    const Foot f = foot_of(plans[i], path);
     leaf_base.push_back(sum.leaves);
     table_base.push_back(sum.tables);
     res_base.push_back(sum.n_out);
     arena_base.push_back(sum.arena);
     sum.add(f);
   }
-  SeqLayout s = layout_of(sum, R, path);
+  SeqLayout s = layout_of(sum, R, path, wide);
   s.arena_base = std::move(arena_base);
   s.res_base = std::move(res_base);
   s.leaf_base = std::move(leaf_base);
@@ -542,25 +602,31 @@ int plan_groups(const tnc_plan_t* const* plans, int n, int R, int path, size_t b
   int b = 0;
   Foot sum;
   for (int i = 0; i < n; i++) {
-    Foot f = foot_of(plans[i], R, path);
+    Foot f = foot_of(plans[i], path);
     Foot t = sum;
     t.add(f);
-    if (i > b && layout_of(t, R, path).total > budget) {
+    if (i > b && layout_of(t, R, path, false).total > budget) {
       out.push_back({b, i});
       b = i;
       sum = Foot();
       t = f;
     }
-    if (layout_of(t, R, path).total > budget)
+    if (layout_of(t, R, path, false).total > budget)
       return set_error(TNC_ERR_BUFFER, "plan " + std::to_string(i) + " alone needs " +
-                                           std::to_string(layout_of(t, R, path).total) + " bytes of workspace");
+                                           std::to_string(layout_of(t, R, path, false).total) + " bytes of workspace");
     sum = t;
   }
   if (b < n) out.push_back({b, n});
   return TNC_OK;
 }
 
-SeqLayout seq_layout(const tnc_plan_t* p, int R, int path = TNC_PATH_INT64) { return group_layout(&p, 1, R, path); }
+// What a single plan is given, and the least it needs.
+size_t plan_bytes(const tnc_plan_t* p, int R, int path) {
+  return std::max(group_layout(&p, 1, R, path, true).total, group_layout(&p, 1, R, path, false).total);
+}
+
+// One residue group at a time on the CUDA cores (tnc_contract_noalloc).
+SeqLayout seq_layout(const tnc_plan_t* p, int R) { return group_layout(&p, 1, R, TNC_PATH_INT64, false); }
 
 int fill_count(tnc_count* out, uint64_t n_out, const Arith& a, const uint32_t* res, const uint32_t* limbs,
                uint32_t flags) {
@@ -888,7 +954,7 @@ int solo_enqueue(const SoloPack& s, const SeqLayout& L, const Arith& a, char* ws
 
 extern "C" size_t tnc_workspace_bytes(const tnc_plan_t* plan, int32_t n_residues) {
   if (!plan || n_residues < 1 || n_residues > 16) return 0;
-  return std::max(seq_layout(plan, n_residues).total, seq_layout(plan, n_residues, TNC_PATH_TC).total);
+  return std::max(plan_bytes(plan, n_residues, TNC_PATH_INT64), plan_bytes(plan, n_residues, TNC_PATH_TC));
 }
 
 extern "C" void tnc_set_step_timing(int32_t on) { g_time_dense = on != 0; }
@@ -931,7 +997,7 @@ extern "C" size_t tnc_workspace_bytes_opts(const tnc_plan_t* plan, const tnc_con
   clear_error();
   Arith a;
   if (!plan || make_arith(opts, a)) return 0;
-  return seq_layout(plan, a.R, opts->path).total;
+  return plan_bytes(plan, a.R, opts->path);
 }
 
 // Residues r of a sum of contractions: acc[e R + r] = (acc + sum_w src_w) mod
@@ -985,7 +1051,8 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
   }
   if (work.empty()) return TNC_OK;
   const int nw = (int)work.size();
-  const SeqLayout L = group_layout(work.data(), nw, a.R, opts->path);
+  SeqLayout L = group_layout(work.data(), nw, a.R, opts->path, true);
+  if (ws_bytes < L.total) L = group_layout(work.data(), nw, a.R, opts->path, false);
   if (!dev_ws || ws_bytes < L.total) return set_error(TNC_ERR_BUFFER, "workspace smaller than tnc_workspace_bytes");
   if (((uintptr_t)dev_ws) % kAlign) return set_error(TNC_ERR_INVALID, "workspace must be 256-byte aligned");
   if (inject_hit(TNC_INJECT_LAUNCH)) return set_error(TNC_ERR_CUDA, "injected failure (TNC_INJECT_LAUNCH)");
@@ -1036,7 +1103,6 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
     tables.insert(tables.end(), lw.leaf_tables.begin(), lw.leaf_tables.end());
     n_lev = std::max(n_lev, lw.lvl_start.empty() ? (size_t)0 : lw.lvl_start.size() - 1);
   }
-  const Groups& groups = a.groups;
   // the group's steps by level: small ones (one index space per level across
   // the plans), big, one-small-operand, split-K and dense ones: each kind one
   // launch per level (split-K and dense steps as many as their scratch holds)
@@ -1057,7 +1123,7 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
   std::vector<tnc_dev::BlockStep> blocked[3];  // by tile shape
   std::vector<StepDesc> small;
   std::vector<P8Step> p8steps;
-  const int rg_max = groups.rg[0];
+  const int res_max = L.passes[0].rg * L.passes[0].groups;  // residues of the widest pass
   for (size_t l = 0; l < n_lev; l++) {
     Level& lv = lev[l];
     lv.small_lo = (uint32_t)small.size();
@@ -1122,7 +1188,7 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
       lv.block[q].blocks = (uint32_t)block_tiles[q];
     }
     // split-K steps: as many per launch as the partials' section holds
-    const uint64_t part_cap = L.part_bytes / ((uint64_t)rg_max * sizeof(uint32_t));
+    const uint64_t part_cap = L.part_bytes / ((uint64_t)res_max * sizeof(uint32_t));
     for (GridStep& g : split) {
       const uint32_t parts = 1u << (g.d.c + g.log_split);
       if (lv.split.empty() || (uint64_t)lv.split.back().blocks + parts > part_cap)
@@ -1139,9 +1205,9 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
     // are timed)
     uint64_t planes = 0, parts = 0;
     for (uint32_t i = p8_lo; i < (uint32_t)p8steps.size(); i++) {
-      const uint64_t pl = p8_scratch_bytes(p8steps[i], rg_max), pt = p8_part_bytes(p8steps[i].d, rg_max);
+      const uint64_t pl = p8_scratch_bytes(p8steps[i], res_max), pt = p8_part_bytes(p8steps[i].d, res_max);
       if (lv.p8.empty() || g_time_dense || planes + pl > L.p8_bytes || parts + pt > L.part_bytes ||
-          i - lv.p8.back().first >= p8_max_steps()) {
+          (i - lv.p8.back().first + 1) * L.passes[0].groups > p8_max_steps()) {
         lv.p8.push_back({i, i});
         planes = parts = 0;
       }
@@ -1158,56 +1224,64 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
   size_t at_block[3];
   for (int q = 0; q < 3; q++) at_block[q] = put(blocked[q].data(), blocked[q].size() * sizeof(tnc_dev::BlockStep));
   const size_t at_tile = put(tiles.data(), tiles.size() * sizeof(tnc_dev::TileStep));
-  // dense descriptors, for each number of residues per entry that a pass has
+  // dense descriptors, for each shape of a pass
   uint32_t* part = (uint32_t*)(ws + L.off_part);
-  std::vector<P8Batch> p8batches[5];
   struct TcLaunch {
     TcBatch b;
     StepDesc first;
   };
-  std::vector<std::vector<TcLaunch>> tcbatches[5];  // by level
-  size_t at_dense[5] = {0};
-  for (int rg : {4, 2, 1}) {
-    if (!tc || std::find(groups.rg.begin(), groups.rg.end(), rg) == groups.rg.end()) continue;
+  struct Dense {
+    int rg, groups;
+    std::vector<P8Batch> p8;
+    std::vector<std::vector<TcLaunch>> tc;  // by level
+    size_t at;
+  };
+  std::vector<Dense> dense;
+  const size_t word = p8 ? 1 : sizeof(uint32_t);
+  for (const PassShape& ps : L.passes) {
+    if (!tc || (!dense.empty() && dense.back().rg == ps.rg && dense.back().groups == ps.groups)) continue;
+    dense.push_back(Dense{ps.rg, ps.groups, {}, {}, 0});
+    Dense& dn = dense.back();
+    const uint32_t rg = (uint32_t)ps.rg;
     std::vector<char> host;
-    const uint64_t arena_bytes = (uint64_t)(L.total - L.off_arena);
+    const uint64_t group_bytes = L.arena_entries * rg * word;
     for (const Level& lv : lev) {
       for (const auto& r : lv.p8) {
-        p8batches[rg].emplace_back();
-        rc = p8_batch(p8steps.data() + r.first, (int)(r.second - r.first), (uint32_t)rg, (uint8_t*)(ws + L.off_arena),
-                      arena_bytes, (uint8_t*)(ws + L.off_p8), (uint8_t*)part, host, p8batches[rg].back());
+        dn.p8.emplace_back();
+        rc = p8_batch(p8steps.data() + r.first, (int)(r.second - r.first), rg, ps.groups, group_bytes,
+                      (uint8_t*)(ws + L.off_arena), group_bytes, (uint8_t*)(ws + L.off_p8), (uint8_t*)part, host,
+                      dn.p8.back());
         if (rc) return rc;
       }
-      tcbatches[rg].emplace_back();
-      std::vector<TcUnit> units;  // steps with all residues of the pass, or a residue of a step each
+      dn.tc.emplace_back();
+      std::vector<TcUnit> units;  // steps with all residues of a group, or a residue of a step each
       uint64_t planes = 0, bytes = 0;
       uint32_t nr = 0;
       auto flush = [&]() -> int {
         if (units.empty()) return TNC_OK;
-        tcbatches[rg].back().push_back(TcLaunch{TcBatch{}, units[0].d});
-        const int rc2 = tc_batch(units.data(), (int)units.size(), nr, (uint32_t)rg, (uint32_t*)(ws + L.off_arena),
-                                 arena_bytes, (uint8_t*)(ws + L.off_p8), (uint8_t*)part, host,
-                                 tcbatches[rg].back().back().b);
+        dn.tc.back().push_back(TcLaunch{TcBatch{}, units[0].d});
+        const int rc2 = tc_batch(units.data(), (int)units.size(), nr, rg, (uint32_t*)(ws + L.off_arena), group_bytes / 4,
+                                 group_bytes, (uint8_t*)(ws + L.off_p8), (uint8_t*)part, host, dn.tc.back().back().b);
         units.clear();
         planes = bytes = 0;
         return rc2;
       };
       for (const StepDesc& d : lv.dense) {
         const uint64_t pl = tc_plane_bytes(d), by = tc_byte_bytes(d);
-        const uint32_t m = rg * pl <= L.p8_bytes && rg * by <= L.part_bytes ? (uint32_t)rg : 1u;
-        for (uint32_t r = 0; r < (uint32_t)rg; r += m) {
+        const uint32_t m = rg * pl <= L.p8_bytes && rg * by <= L.part_bytes ? rg : 1u;
+        for (uint32_t gr = 0; gr < (uint32_t)ps.groups * rg; gr += m) {
           if (m != nr || planes + m * pl > L.p8_bytes || bytes + m * by > L.part_bytes ||
-              units.size() >= tc_max_units(m) || (g_time_dense && r == 0))
+              units.size() >= tc_max_units(m) || (g_time_dense && gr == 0))
             if ((rc = flush())) return rc;
           nr = m;
-          units.push_back(TcUnit{d, r});
+          units.push_back(TcUnit{d, gr / rg, gr % rg});
           planes += m * pl;
           bytes += m * by;
         }
       }
       if ((rc = flush())) return rc;
     }
-    at_dense[rg] = put(host.data(), host.size());
+    dn.at = put(host.data(), host.size());
   }
   if (stage.size() > L.off_part) return set_error(TNC_ERR_INVALID, "internal: descriptors beyond their section");
   CUDA_TRY(cudaMemcpyAsync(ws, stage.data(), stage.size(), cudaMemcpyHostToDevice, st));
@@ -1249,11 +1323,27 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
     rt.res_lo = L.res_base[w];
     rs.n_entries += 1ull << rt.map.n_open;
   }
-  for (size_t gi = 0; gi < groups.rg.size(); gi++) {
-    uint32_t gp[4];
-    for (int r = 0; r < 4; r++) gp[r] = r < groups.rg[gi] ? a.primes[groups.col[gi] + r] : a.primes[groups.col[gi]];
-    const ModGroup mg = tnc_dev::make_mod_group(gp);
-    // one pass over the residue group; the 8-bit-prime path stores a residue
+  for (const PassShape& shape : L.passes) {
+    const unsigned ng = (unsigned)shape.groups;
+    tnc_dev::Pass ps{};
+    std::vector<uint32_t> primes;  // of the pass; a filled-up group repeats its first
+    bool near30 = true;
+    for (unsigned g = 0; g < ng; g++) {
+      uint32_t gp[4];
+      for (int r = 0; r < 4; r++) {
+        const int i = shape.col + (int)g * shape.rg + r;
+        gp[r] = a.primes[r < shape.rg && i < a.R ? i : shape.col + (int)g * shape.rg];
+        if (r < shape.rg) primes.push_back(gp[r]);
+      }
+      ps.mg[g] = tnc_dev::make_mod_group(gp);
+      near30 = near30 && ps.mg[g].near30;
+    }
+    ps.arena_stride = L.arena_entries * shape.rg;
+    ps.part_stride = L.part_bytes / ((uint64_t)res_max * sizeof(uint32_t)) * shape.rg;
+    const Dense* dn = nullptr;
+    for (const Dense& x : dense)
+      if (x.rg == shape.rg && x.groups == shape.groups) dn = &x;
+    // one pass over its residue groups; the 8-bit-prime path stores a residue
     // per byte
     auto pass = [&](auto rgc, auto wtag, auto n30tag) -> int {
       constexpr int RG = decltype(rgc)::value;
@@ -1263,10 +1353,11 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
       const int nl = (int)leaves.size();
       size_t next_p8 = 0;
       const std::vector<char> dense_consts =
-          tc && !p8 ? tc_consts(a.primes.data() + groups.col[gi], RG) : std::vector<char>();
-      tnc_dev::leaf_fill_kernel<RG, W><<<std::min(nl, sms * 8), 64, 0, st>>>(
-          (const LeafDesc*)(ws + at_leaves), nl, (const uint32_t*)(ws + at_tables), arena, mg);
-      g_launches.leaf_fill += tc && !p8 ? RG : 1;  // (recorded per residue on TNC_PATH_TC)
+          tc && !p8 ? tc_consts(primes.data(), (uint32_t)primes.size()) : std::vector<char>();
+      tnc_dev::leaf_fill_kernel<RG, W><<<dim3(std::min(nl, sms * 8), ng), 64, 0, st>>>(
+          (const LeafDesc*)(ws + at_leaves), nl, (const uint32_t*)(ws + at_tables), arena, ps);
+      // (recorded per residue group, on TNC_PATH_TC per residue)
+      g_launches.leaf_fill += tc && !p8 ? std::min((int)ng * RG, a.R - shape.col) : (int)ng;
       // a timed dense launch: events around it and its shape
       auto timed = [&](const StepDesc& d, uint32_t residues, auto&& launch) -> int {
         cudaEvent_t ev[2] = {nullptr, nullptr};
@@ -1296,12 +1387,13 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
         NvtxRange level_range("tnc level");
         if (lv.small_n) {
           const unsigned blocks = (unsigned)std::min<uint64_t>((lv.small_work + 255) / 256, (uint64_t)sms * 8);
-          tnc_dev::level_kernel<RG, W, N30><<<blocks, 256, 0, st>>>(d_small + lv.small_lo, lv.small_n, lv.small_work, arena,
-                                                                   mg);
+          tnc_dev::level_kernel<RG, W, N30><<<dim3(blocks, ng), 256, 0, st>>>(d_small + lv.small_lo, lv.small_n,
+                                                                             lv.small_work, arena, ps);
           g_launches.level++;
         }
         if (lv.outer.n) {
-          tnc_dev::outer_kernel<RG, W, N30><<<lv.outer.blocks, 256, 0, st>>>(d_outer + lv.outer.lo, lv.outer.n, arena, mg);
+          tnc_dev::outer_kernel<RG, W, N30><<<dim3(lv.outer.blocks, ng), 256, 0, st>>>(d_outer + lv.outer.lo, lv.outer.n,
+                                                                                       arena, ps);
           g_launches.outer++;
         }
         if constexpr (sizeof(W) == 4) {
@@ -1314,8 +1406,8 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
                 (size_t)tnc_dev::kBlkStages * ((1 << B::LA) + (1 << B::LB)) * tnc_dev::kBlkK * RG * sizeof(uint32_t);
             auto k = tnc_dev::block_kernel<RG, Q, N30>;
             if (smem > 48 * 1024) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            k<<<std::min(r.blocks, 2u * (unsigned)sms), 256, smem, st>>>(
-                (const tnc_dev::BlockStep*)(ws + at_block[Q]) + r.lo, r.n, r.blocks, arena, mg);
+            k<<<dim3(std::min(r.blocks, (2u * (unsigned)sms + ng - 1) / ng), ng), 256, smem, st>>>(
+                (const tnc_dev::BlockStep*)(ws + at_block[Q]) + r.lo, r.n, r.blocks, arena, ps);
             g_launches.grid_step++;
             return TNC_OK;
           };
@@ -1325,46 +1417,50 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
           if (rc2) return rc2;
         }
         if (lv.tile.n) {
-          tnc_dev::tile_kernel<RG, W, N30><<<lv.tile.blocks, 256, 0, st>>>(d_tile + lv.tile.lo, lv.tile.n, arena, mg);
+          tnc_dev::tile_kernel<RG, W, N30><<<dim3(lv.tile.blocks, ng), 256, 0, st>>>(d_tile + lv.tile.lo, lv.tile.n, arena,
+                                                                                     ps);
           g_launches.grid_step++;
         }
         if (lv.grid.n) {
-          tnc_dev::step_kernel<RG, W, N30><<<lv.grid.blocks, 256, 0, st>>>(d_steps + lv.grid.lo, lv.grid.n, arena, mg);
+          tnc_dev::step_kernel<RG, W, N30><<<dim3(lv.grid.blocks, ng), 256, 0, st>>>(d_steps + lv.grid.lo, lv.grid.n, arena,
+                                                                                     ps);
           g_launches.grid_step++;
         }
         for (const Range& r : lv.split) {
-          tnc_dev::splitk_partial_kernel<RG, W, N30><<<r.blocks, 256, 0, st>>>(d_steps + r.lo, r.n, arena, part, mg);
-          tnc_dev::splitk_final_kernel<RG, W, N30><<<r.finals, 256, 0, st>>>(d_steps + r.lo, r.n, arena, part, mg);
+          tnc_dev::splitk_partial_kernel<RG, W, N30><<<dim3(r.blocks, ng), 256, 0, st>>>(d_steps + r.lo, r.n, arena, part,
+                                                                                         ps);
+          tnc_dev::splitk_final_kernel<RG, W, N30><<<dim3(r.finals, ng), 256, 0, st>>>(d_steps + r.lo, r.n, arena, part, ps);
           g_launches.splitk++;
         }
         if (tc && !p8)
-          for (const TcLaunch& x : tcbatches[RG][&lv - lev.data()]) {
+          for (const TcLaunch& x : dn->tc[&lv - lev.data()]) {
             NvtxRange dense_range("tnc dense steps");
             if (int rc2 = timed(x.first, x.b.n_units * x.b.nr, [&] {
-                  return tc_run(x.b, ws + at_dense[RG], dense_consts, RG, d_err, sms, st);
+                  return tc_run(x.b, ws + dn->at, dense_consts, RG, d_err, sms, st);
                 }))
               return rc2;
           }
         for (const auto& r : lv.p8) {
           NvtxRange dense_range("tnc dense steps");
-          const P8Batch& b = p8batches[RG][next_p8++];
-          if (int rc2 = timed(p8steps[r.first].d, RG, [&] {
-                return p8_run(b, ws + at_dense[RG], a.primes.data() + groups.col[gi], RG, d_err, sms, st);
+          const P8Batch& b = dn->p8[next_p8++];
+          if (int rc2 = timed(p8steps[r.first].d, RG * ng, [&] {
+                return p8_run(b, ws + dn->at, primes.data(), (uint32_t)primes.size(), RG, d_err, sms, st);
               }))
             return rc2;
         }
       }
       for (const tnc_dev::Roots& rs : roots) {
-        tnc_dev::extract_kernel<RG, W><<<(unsigned)std::min<uint64_t>((rs.n_entries + 255) / 256, 1024), 256, 0, st>>>(
-            arena, rs, results, a.R, groups.col[gi]);
+        const unsigned blocks = (unsigned)std::min<uint64_t>((rs.n_entries + 255) / 256, 1024);
+        tnc_dev::extract_kernel<RG, W><<<dim3(blocks, ng), 256, 0, st>>>(arena, ps.arena_stride, rs, results, a.R,
+                                                                        shape.col);
         g_launches.extract++;
       }
       CUDA_TRY(cudaGetLastError());
       return TNC_OK;
     };
-    rc = dispatch_rg(groups.rg[gi], [&](auto rgc) -> int {
+    rc = dispatch_rg(shape.rg, [&](auto rgc) -> int {
       if (p8) return pass(rgc, WordTag<uint8_t>(), std::false_type());
-      return mg.near30 ? pass(rgc, WordTag<uint32_t>(), std::true_type())
+      return near30 ? pass(rgc, WordTag<uint32_t>(), std::true_type())
                        : pass(rgc, WordTag<uint32_t>(), std::false_type());
     });
     if (rc) return rc;
@@ -1454,7 +1550,7 @@ extern "C" size_t tnc_workspace_bytes_sliced(const tnc_plan_t* const* plans, int
   size_t body = 256;
   for (int i = 0; i < n; i++) {
     if (!plans[i]) return 0;
-    body = std::max(body, seq_layout(plans[i], a.R, opts->path).total);
+    body = std::max(body, plan_bytes(plans[i], a.R, opts->path));
   }
   return sliced_head_bytes(1ull << plans[0]->net.open_vars.size(), a) + body;
 }
@@ -1516,7 +1612,7 @@ extern "C" size_t tnc_workspace_bytes_many(const tnc_plan_t* const* plans, int32
     const int m = std::min<int>(group, n - i);
     for (int j = i; j < i + m; j++)
       if (!plans[j]) return 0;
-    need = std::max(need, group_layout(plans + i, m, a.R, opts->path).total);
+    for (bool wide : {true, false}) need = std::max(need, group_layout(plans + i, m, a.R, opts->path, wide).total);
   }
   return need;
 }
@@ -1803,11 +1899,11 @@ int batch_enqueue(tnc_batch_t* b, void* dev_ws, cudaStream_t st) {
             &cl.cfg,
             mg.near30 ? tnc_dev::batch_kernel<RG, true, tnc_dev::kBatchClusters>
                       : tnc_dev::batch_kernel<RG, false, tnc_dev::kBatchClusters>,
-            args, mg, b->a.crt));
+            args, mg, 0));
         return TNC_OK;
       }
-      if (mg.near30) tnc_dev::batch_kernel<RG, true><<<grid, threads, smem, st>>>(args, mg, b->a.crt);
-      else tnc_dev::batch_kernel<RG, false><<<grid, threads, smem, st>>>(args, mg, b->a.crt);
+      if (mg.near30) tnc_dev::batch_kernel<RG, true><<<grid, threads, smem, st>>>(args, mg, 0);
+      else tnc_dev::batch_kernel<RG, false><<<grid, threads, smem, st>>>(args, mg, 0);
       CUDA_TRY(cudaGetLastError());
       return TNC_OK;
     });
@@ -2233,29 +2329,30 @@ extern "C" int tnc_contract_noalloc(const tnc_plan_t* plan, const tnc_contract_o
   for (int gi = 0; gi < n_groups; gi++) {
     uint32_t gp[4];
     for (int r = 0; r < 4; r++) gp[r] = r < grp_rg[gi] ? primes[grp_col[gi] + r] : primes[grp_col[gi]];
-    const ModGroup mg = tnc_dev::make_mod_group(gp);
+    tnc_dev::Pass ps{};
+    ps.mg[0] = tnc_dev::make_mod_group(gp);
     rc = dispatch_rg(grp_rg[gi], [&](auto rgc) -> int {
       constexpr int RG = decltype(rgc)::value;
       tnc_dev::leaf_fill_kernel<RG><<<std::min(nl, sms * 8), 64, 0, st>>>(
-          (const LeafDesc*)(ws + L.off_leaves), nl, (const uint32_t*)(ws + L.off_tables), arena, mg);
+          (const LeafDesc*)(ws + L.off_leaves), nl, (const uint32_t*)(ws + L.off_tables), arena, ps);
       g_launches.leaf_fill++;
       for (size_t i = 0; i < plan->low.seq_steps.size(); i++) {
         const StepDesc& d = plan->low.seq_steps[i];
         const uint32_t ls = splitk_log(d);
         if (ls > 0) {  // few outputs, long shared sum: K split over blocks, as in tnc_contract
           tnc_dev::splitk_partial_kernel<RG><<<(unsigned)(1ull << (d.c + ls)), 256, 0, st>>>(d_steps + i, 1, arena, part,
-                                                                                           mg);
-          tnc_dev::splitk_final_kernel<RG><<<(unsigned)(1ull << d.c), 256, 0, st>>>(d_steps + i, 1, arena, part, mg);
+                                                                                           ps);
+          tnc_dev::splitk_final_kernel<RG><<<(unsigned)(1ull << d.c), 256, 0, st>>>(d_steps + i, 1, arena, part, ps);
           g_launches.splitk++;
           continue;
         }
         int threads, blocks, sh;
         grid_shape(d.c, &threads, &blocks, &sh);
-        tnc_dev::step_kernel<RG><<<blocks, threads, 0, st>>>(d_steps + i, 1, arena, mg);
+        tnc_dev::step_kernel<RG><<<blocks, threads, 0, st>>>(d_steps + i, 1, arena, ps);
         g_launches.grid_step++;
       }
       tnc_dev::extract_kernel<RG><<<(unsigned)std::min<uint64_t>((n_out + 255) / 256, 1024), 256, 0, st>>>(
-          arena, roots, results, R, grp_col[gi]);
+          arena, 0, roots, results, R, grp_col[gi]);
       g_launches.extract++;
       CUDA_TRY(cudaGetLastError());
       return TNC_OK;

@@ -194,43 +194,6 @@ __device__ __forceinline__ void step_entry(const StepDesc& d, uint64_t o, const 
   step_entry_at<RG, W, N30>(d.k, d.ka, d.kb, o, ia, ib, A0, B0, C0, mg);
 }
 
-// ------------------------------------------------------------------ kernels
-
-template <int RG, typename W = uint32_t>
-__global__ void __launch_bounds__(256) leaf_fill_kernel(const LeafDesc* __restrict__ leaves, int n_leaves,
-                                                        const uint32_t* __restrict__ tables,
-                                                        W* __restrict__ arena, ModGroup mg) {
-  for (int l = blockIdx.x; l < n_leaves; l += gridDim.x) {
-    const LeafDesc ld = leaves[l];
-    const uint64_t n = 1ull << ld.rank;
-    W* dst = arena + ld.off * RG;
-    for (uint64_t idx = threadIdx.x; idx < n; idx += blockDim.x) {
-      uint32_t v[RG];
-#pragma unroll
-      for (int r = 0; r < RG; r++) v[r] = leaf_value(ld.kind, ld.rank, (uint32_t)idx, tables, ld.table_off, mg.p[r]);
-      store_entry<RG, W>(dst + idx * RG, v);
-    }
-  }
-}
-
-// All the small steps of one tree level in one launch: they are independent,
-// so their output entries form one index space (step i owns [work_lo,
-// work_lo + 2^c)); each thread finds its step by binary search.
-template <int RG, typename W = uint32_t, bool N30 = false>
-__global__ void __launch_bounds__(256) level_kernel(const StepDesc* __restrict__ steps, uint32_t n_steps,
-                                                    uint32_t total, W* arena, ModGroup mg) {
-  for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < total; w += gridDim.x * blockDim.x) {
-    uint32_t lo = 0, hi = n_steps - 1;
-    while (lo < hi) {
-      const uint32_t mid = (lo + hi + 1) >> 1;
-      if (steps[mid].work_lo <= w) lo = mid;
-      else hi = mid - 1;
-    }
-    const StepDesc& d = steps[lo];
-    step_entry<RG, W, N30>(d, w - d.work_lo, arena + d.a_off * RG, arena + d.b_off * RG, arena + d.c_off * RG, mg);
-  }
-}
-
 // Chinese remaindering by Garner's mixed radix:
 //   v0 = r0,  v_i = (r_i - (v0 + v1 p0 + ... + v_{i-1} p0..p_{i-2})) * inv_i  mod p_i,
 //   X = v0 + p0 (v1 + p1 (v2 + ...)),  0 <= X < p0 p1 ... p_{R-1}.
@@ -245,7 +208,7 @@ struct CrtConsts {
 };
 
 // Residues r[0..R) of one entry to its n_limbs limbs.
-__device__ __noinline__ void crt_entry(const uint32_t* r, const CrtConsts& cc, uint32_t* limbs) {
+__device__ __forceinline__ void crt_entry(const uint32_t* r, const CrtConsts& cc, uint32_t* limbs) {
   uint32_t v[kCrtMaxResidues];
   for (int i = 0; i < cc.R; i++) {
     const uint32_t p = cc.p[i];
@@ -466,10 +429,12 @@ __device__ __forceinline__ uint32_t map_runs(uint32_t o, const uint16_t* runs, i
 // formula that takes longer alone than the batch's average CTA would
 // otherwise be what the launch ends with.  Then every CTA takes formulas from
 // the queue as above.
+template <int MODE>
+using BatchCrt = std::conditional_t<MODE == 2, CrtConsts, int>;  // (only kBatchSolo has a use for the constants)
 enum BatchMode { kBatchCtas, kBatchClusters, kBatchSolo };  // kBatchSolo: one formula, one cluster, and its CRT
 template <int RG, bool N30 = false, int MODE = kBatchCtas>
 __global__ void __launch_bounds__(256, MODE == kBatchCtas ? 0 : (MODE == kBatchSolo ? 1 : (RG == 4 && !N30 ? 3 : 4)))
-    batch_kernel(BatchArgs a, ModGroup mg, const __grid_constant__ CrtConsts cc) {
+    batch_kernel(BatchArgs a, ModGroup mg, const __grid_constant__ BatchCrt<MODE> cc) {
   constexpr bool CLUSTER = MODE != kBatchCtas;
   extern __shared__ uint4 smem_raw[];
   __shared__ uint32_t task;
@@ -610,7 +575,8 @@ __global__ void __launch_bounds__(256, MODE == kBatchCtas ? 0 : (MODE == kBatchS
         a.results[((uint64_t)f.res_off + J) * a.R + a.col + r] = arena[((uint64_t)f.root_off + ad) * RG + r];
     }
     barrier();
-    if (MODE == kBatchSolo && a.limbs)
+    if constexpr (MODE == kBatchSolo)
+      if (a.limbs)
       for (uint32_t J = tid; J < f.n_out; J += nthreads)
         crt_entry(a.results + (uint64_t)J * a.R, cc, a.limbs + (uint64_t)J * cc.n_limbs);
   }

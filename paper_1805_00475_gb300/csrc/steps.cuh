@@ -6,6 +6,56 @@
 
 namespace tnc_dev {
 
+// The residue groups of a pass run side by side: blockIdx.y is the group, with
+// its own primes, its own copy of the arena (arena_stride words further) and
+// its own split-K partials.  (A formula with 2^24 products or fewer spends most of
+// its time between launches; 20 residues in five passes took five times the
+// launches.)
+constexpr int kMaxGroups = 14;
+struct Pass {
+  ModGroup mg[kMaxGroups];
+  uint64_t arena_stride, part_stride;  // words
+};
+
+template <int RG, typename W = uint32_t>
+__global__ void __launch_bounds__(256) leaf_fill_kernel(const LeafDesc* __restrict__ leaves, int n_leaves,
+                                                        const uint32_t* __restrict__ tables,
+                                                        W* __restrict__ arena0, const __grid_constant__ Pass ps) {
+  W* __restrict__ arena = arena0 + blockIdx.y * ps.arena_stride;
+  const ModGroup& mg = ps.mg[blockIdx.y];
+  for (int l = blockIdx.x; l < n_leaves; l += gridDim.x) {
+    const LeafDesc ld = leaves[l];
+    const uint64_t n = 1ull << ld.rank;
+    W* dst = arena + ld.off * RG;
+    for (uint64_t idx = threadIdx.x; idx < n; idx += blockDim.x) {
+      uint32_t v[RG];
+#pragma unroll
+      for (int r = 0; r < RG; r++) v[r] = leaf_value(ld.kind, ld.rank, (uint32_t)idx, tables, ld.table_off, mg.p[r]);
+      store_entry<RG, W>(dst + idx * RG, v);
+    }
+  }
+}
+
+// All the small steps of one tree level in one launch: they are independent,
+// so their output entries form one index space (step i owns [work_lo,
+// work_lo + 2^c)); each thread finds its step by binary search.
+template <int RG, typename W = uint32_t, bool N30 = false>
+__global__ void __launch_bounds__(256) level_kernel(const StepDesc* __restrict__ steps, uint32_t n_steps,
+                                                    uint32_t total, W* arena0, const __grid_constant__ Pass ps) {
+  W* arena = arena0 + blockIdx.y * ps.arena_stride;
+  const ModGroup& mg = ps.mg[blockIdx.y];
+  for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < total; w += gridDim.x * blockDim.x) {
+    uint32_t lo = 0, hi = n_steps - 1;
+    while (lo < hi) {
+      const uint32_t mid = (lo + hi + 1) >> 1;
+      if (steps[mid].work_lo <= w) lo = mid;
+      else hi = mid - 1;
+    }
+    const StepDesc& d = steps[lo];
+    step_entry<RG, W, N30>(d, w - d.work_lo, arena + d.a_off * RG, arena + d.b_off * RG, arena + d.c_off * RG, mg);
+  }
+}
+
 // A step launched over the whole GPU.  With S = 2^s threads in the grid, a
 // thread visits o, o + S, o + 2S, ...: from one to the next the counter o >> s
 // gains one, which clears its trailing ones and sets bit t, so each operand
@@ -41,7 +91,9 @@ __device__ __forceinline__ const GridStep* step_of_block(const GridStep* steps, 
 
 template <int RG, typename W = uint32_t, bool N30 = false>
 __global__ void __launch_bounds__(256) step_kernel(const GridStep* __restrict__ steps, uint32_t n_steps,
-                                                   W* __restrict__ arena, ModGroup mg) {
+                                                   W* __restrict__ arena0, const __grid_constant__ Pass ps) {
+  W* __restrict__ arena = arena0 + blockIdx.y * ps.arena_stride;
+  const ModGroup& mg = ps.mg[blockIdx.y];
   const GridStep* __restrict__ g = step_of_block<&GridStep::block_lo>(steps, n_steps);
   const uint32_t c = g->d.c, k = g->d.k, ka = g->d.ka, kb = g->d.kb, s = g->s;
   const uint64_t n = 1ull << c;
@@ -88,7 +140,9 @@ struct TileStep {
 
 template <int RG, typename W = uint32_t, bool N30 = false>
 __global__ void __launch_bounds__(256) tile_kernel(const TileStep* __restrict__ steps, uint32_t n_steps,
-                                                   W* __restrict__ arena, ModGroup mg) {
+                                                   W* __restrict__ arena0, const __grid_constant__ Pass ps) {
+  W* __restrict__ arena = arena0 + blockIdx.y * ps.arena_stride;
+  const ModGroup& mg = ps.mg[blockIdx.y];
   uint32_t lo = 0, hi = n_steps - 1;
   while (lo < hi) {
     const uint32_t mid = (lo + hi + 1) >> 1;
@@ -213,7 +267,10 @@ __device__ __forceinline__ void cp_async(void* dst, const void* src) {
 
 template <int RG, int SHAPE, bool N30 = false>
 __global__ void __launch_bounds__(256, 2) block_kernel(const BlockStep* __restrict__ steps, uint32_t n_steps,
-                                                       uint32_t n_tiles, uint32_t* __restrict__ arena, ModGroup mg) {
+                                                       uint32_t n_tiles, uint32_t* __restrict__ arena0,
+                                                       const __grid_constant__ Pass ps) {
+  uint32_t* __restrict__ arena = arena0 + blockIdx.y * ps.arena_stride;
+  const ModGroup& mg = ps.mg[blockIdx.y];
   constexpr int kBlkA = Blk<SHAPE>::LA, kBlkB = Blk<SHAPE>::LB, RA = Blk<SHAPE>::RA, RB = Blk<SHAPE>::RB;
   constexpr int TA = 1 << RA, TB = 1 << RB;
   constexpr uint32_t NA = 1u << kBlkA, NB = 1u << kBlkB, kStage = (NA + NB) * kBlkK * RG;  // words
@@ -377,7 +434,9 @@ struct OuterStep {
 
 template <int RG, typename W = uint32_t, bool N30 = false>
 __global__ void __launch_bounds__(256) outer_kernel(const OuterStep* __restrict__ steps, uint32_t n_steps,
-                                                    W* __restrict__ arena, ModGroup mg) {
+                                                    W* __restrict__ arena0, const __grid_constant__ Pass ps) {
+  W* __restrict__ arena = arena0 + blockIdx.y * ps.arena_stride;
+  const ModGroup& mg = ps.mg[blockIdx.y];
   __shared__ uint32_t sm[256 * RG];  // S entry (s, q) at (s + (q << fs)) * RG + r
   __shared__ OuterStep os;
   {
@@ -469,7 +528,11 @@ __global__ void __launch_bounds__(256) outer_kernel(const OuterStep* __restrict_
 // adds the parts of each output.  part[o * n_split + j] holds RG residues.
 template <int RG, typename W = uint32_t, bool N30 = false>
 __global__ void __launch_bounds__(256) splitk_partial_kernel(const GridStep* __restrict__ steps, uint32_t n_steps,
-                                                             const W* arena, uint32_t* __restrict__ part, ModGroup mg) {
+                                                             const W* arena0, uint32_t* __restrict__ part0,
+                                                             const __grid_constant__ Pass ps) {
+  const W* arena = arena0 + blockIdx.y * ps.arena_stride;
+  uint32_t* __restrict__ part = part0 + blockIdx.y * ps.part_stride;
+  const ModGroup& mg = ps.mg[blockIdx.y];
   __shared__ uint32_t red[256 * RG];
   const GridStep* __restrict__ g = step_of_block<&GridStep::block_lo>(steps, n_steps);
   const uint32_t log_split = g->log_split, blk = blockIdx.x - g->block_lo;
@@ -550,7 +613,11 @@ __global__ void __launch_bounds__(256) splitk_partial_kernel(const GridStep* __r
 // One block per output entry: its threads add the parts, then combine.
 template <int RG, typename W = uint32_t, bool N30 = false>
 __global__ void __launch_bounds__(256) splitk_final_kernel(const GridStep* __restrict__ steps, uint32_t n_steps,
-                                                           W* arena, const uint32_t* __restrict__ part, ModGroup mg) {
+                                                           W* arena0, const uint32_t* __restrict__ part0,
+                                                           const __grid_constant__ Pass ps) {
+  W* arena = arena0 + blockIdx.y * ps.arena_stride;
+  const ModGroup& mg = ps.mg[blockIdx.y];
+  const uint32_t* __restrict__ part = part0 + blockIdx.y * ps.part_stride;
   __shared__ uint32_t red[256 * RG];
   const GridStep* __restrict__ g = step_of_block<&GridStep::final_lo>(steps, n_steps);
   const uint32_t log_split = g->log_split;
@@ -598,8 +665,11 @@ struct Roots {
 };
 
 template <int RG, typename W = uint32_t>
-__global__ void __launch_bounds__(256) extract_kernel(const W* __restrict__ arena, const __grid_constant__ Roots rs,
-                                                      uint32_t* __restrict__ results, int R, int col) {
+__global__ void __launch_bounds__(256) extract_kernel(const W* __restrict__ arena0, uint64_t arena_stride,
+                                                      const __grid_constant__ Roots rs, uint32_t* __restrict__ results,
+                                                      int R, int col0) {
+  const W* __restrict__ arena = arena0 + blockIdx.y * arena_stride;
+  const int col = col0 + RG * (int)blockIdx.y;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < rs.n_entries;
        i += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t e = rs.r[0].res_lo + i;
@@ -614,7 +684,8 @@ __global__ void __launch_bounds__(256) extract_kernel(const W* __restrict__ aren
     uint64_t a = 0;
     for (int j = 0; j < rt.map.n_open; j++) a |= (uint64_t)((J >> rt.map.perm[j]) & 1u) << j;
 #pragma unroll
-    for (int r = 0; r < RG; r++) results[e * R + col + r] = arena[(rt.root_off + a) * RG + r];
+    for (int r = 0; r < RG; r++)
+      if (col + r < R) results[e * R + col + r] = arena[(rt.root_off + a) * RG + r];  // (a group may be filled up)
   }
 }
 

@@ -69,9 +69,10 @@ struct alignas(64) PackUnit {
 struct alignas(64) JoinUnit {
   const uint8_t* bytes;
   uint32_t* out;
-  uint32_t c, log_split, n, r0;  // r0: the first residue's place in the entries
+  uint32_t c, log_split, n, r0;  // r0: the first residue's place among the launch's primes
   uint32_t block_lo;
 };
+constexpr uint32_t kTcPrimes = 16;
 
 constexpr uint32_t kMaxUnits = 256;
 
@@ -194,9 +195,9 @@ __global__ void __launch_bounds__(256) rns_pack_kernel(const PackUnit* __restric
 struct JoinConsts {
   struct {
     uint32_t c[3][4], neg;
-  } by_p[4][4];
-  uint32_t p[4];
-  uint64_t mu[4];
+  } by_p[4][kTcPrimes];
+  uint32_t p[kTcPrimes];
+  uint64_t mu[kTcPrimes];
 };
 
 // round(2^15 / q_j), four a word (131 .. 172; 0 beyond n: those bytes are 0)
@@ -315,8 +316,8 @@ uint64_t tc_byte_bytes(const StepDesc& d) { return (uint64_t)tc_small_primes(d.k
 size_t tc_unit_bytes() { return sizeof(tnc_rns::PackUnit) + sizeof(tnc_rns::JoinUnit) + 4 * p8_prob_bytes(); }
 uint32_t tc_max_units(uint32_t nr) { return tnc_rns::kMaxUnits / 3 / nr; }  // (up to three groups of four primes a residue)
 
-int tc_batch(const TcUnit* units, int n, uint32_t nr, uint32_t rg, uint32_t* arena, uint64_t arena_bytes,
-             uint8_t* planes, uint8_t* bytes, std::vector<char>& host, TcBatch& b) {
+int tc_batch(const TcUnit* units, int n, uint32_t nr, uint32_t rg, uint32_t* arena0, uint64_t arena_stride,
+             uint64_t arena_bytes, uint8_t* planes, uint8_t* bytes, std::vector<char>& host, TcBatch& b) {
   using namespace tnc_rns;
   b = TcBatch{};
   b.nr = nr;
@@ -329,7 +330,8 @@ int tc_batch(const TcUnit* units, int n, uint32_t nr, uint32_t rg, uint32_t* are
     const StepDesc& d = units[i].d;
     const uint32_t nq = tc_small_primes(d.k), ls = p8_split_log(d);
     if (!nq) return set_error(TNC_ERR_TOO_LARGE, "dense step with too many shared values");
-    if (units[i].r + nr > rg || (nr != 1 && nr != rg)) return set_error(TNC_ERR_INVALID, "internal: residues outside their pass");
+    uint32_t* const arena = arena0 + units[i].group * arena_stride;
+    if (units[i].r + nr > rg || (nr != 1 && nr != rg) || (units[i].group + 1) * rg > kTcPrimes) return set_error(TNC_ERR_INVALID, "internal: residues outside their pass");
     {
       const uint64_t ea = 1ull << (d.ka + d.k), eb = 1ull << (d.kb + d.k), ec = 1ull << d.c, w = 4ull * rg;
       if ((d.a_off + ea) * w > arena_bytes || (d.b_off + eb) * w > arena_bytes || (d.c_off + ec) * w > arena_bytes)
@@ -358,7 +360,7 @@ int tc_batch(const TcUnit* units, int n, uint32_t nr, uint32_t rg, uint32_t* are
     ju.c = d.c;
     ju.log_split = ls;
     ju.n = nq;
-    ju.r0 = units[i].r;
+    ju.r0 = units[i].group * rg + units[i].r;
     ju.block_lo = (uint32_t)blocks;
     blocks += ((1ull << d.c) + 255) / 256;
     joins.push_back(ju);
@@ -375,7 +377,7 @@ int tc_batch(const TcUnit* units, int n, uint32_t nr, uint32_t rg, uint32_t* are
       planes += tc_plane_bytes(d);
       bytes += tc_byte_bytes(d);
     }
-    if (units[i].r == 0) {
+    if (units[i].r == 0 && units[i].group == 0) {
       b.steps++;
       b.splits += ls > 0;
     }
@@ -433,10 +435,10 @@ const tnc_rns::PackConsts& pack_consts() {
 
 }  // namespace
 
-std::vector<char> tc_consts(const uint32_t* primes, uint32_t rg) {
+std::vector<char> tc_consts(const uint32_t* primes, uint32_t n_primes) {
   tnc_rns::JoinConsts jc;
   std::memset(&jc, 0, sizeof(jc));
-  for (uint32_t r = 0; r < rg; r++) {
+  for (uint32_t r = 0; r < std::min(n_primes, tnc_rns::kTcPrimes); r++) {
     jc.p[r] = primes[r];
     jc.mu[r] = ~0ull / primes[r];
     for (uint32_t n = 9; n <= kMaxSmall; n++) {

@@ -122,7 +122,7 @@ struct alignas(64) P8Prob {
 constexpr uint32_t kMaxProbs = 256;  // steps of one launch (their first items are searched in shared memory)
 
 // The primes of a launch: the pass's (from 0), or several steps' own.
-constexpr uint32_t kLaunchPrimes = 16;
+constexpr uint32_t kLaunchPrimes = 56;  // (14 residue groups of four)
 struct P8Primes {
   float pf[kLaunchPrimes], invp[kLaunchPrimes];
 };
@@ -471,7 +471,7 @@ __device__ __forceinline__ uint32_t staged_half2_res(uint32_t w, uint32_t ra) {
 // Row-contiguous planes (mode 2, K >= 64): Y_i[q * R + r], the entries' own
 // order, converted in place of the transpose (8-byte writes along r).
 struct PackPrimes {
-  uint32_t p[4];
+  uint32_t p[kLaunchPrimes];
 };
 
 // half2 of the balanced residues (a, b) given as bytes ia of wa and ib of wb:
@@ -502,12 +502,12 @@ struct PackOperand {
 // first tile in the launch, which takes up to kMaxProbs steps of a level.
 struct alignas(64) PackProb {
   PackOperand a, b;
-  uint32_t k, kp, tile_lo, n_tiles;
+  uint32_t k, kp, tile_lo, n_tiles, prime_at;
 };
 
 template <int RG>
 __global__ void __launch_bounds__(256) p8_pack_kernel(const PackProb* __restrict__ probs, uint32_t n_probs,
-                                                      uint32_t n_tiles, PackPrimes pp) {
+                                                      uint32_t n_tiles, const __grid_constant__ PackPrimes pp) {
   // [residue][row][pair of shared values] half2 words; a row is 32 words + 1
   // of padding, so both phases are free of bank conflicts (phase 1: lanes =
   // 8 row quads x 4 pairs; phase 2: lanes = 8 chunks x 4 rows)
@@ -517,14 +517,18 @@ __global__ void __launch_bounds__(256) p8_pack_kernel(const PackProb* __restrict
   if (t < n_probs) tile_lo[t] = probs[t].tile_lo;
   __syncthreads();
   __half2 hp2[RG], np2[RG];
-#pragma unroll
-  for (int i = 0; i < RG; i++) {
-    hp2[i] = __float2half2_rn((float)((pp.p[i] - 1) / 2));
-    np2[i] = __float2half2_rn(-(float)pp.p[i]);
-  }
+  uint32_t prime_at = ~0u;
   for (uint32_t gt = blockIdx.x; gt < n_tiles; gt += gridDim.x) {
     const PackProb& pb = probs[find_last(tile_lo, n_probs, gt)];
     const PackOperand opA = pb.a, opB = pb.b;
+    if (pb.prime_at != prime_at) {
+      prime_at = pb.prime_at;
+#pragma unroll
+      for (int i = 0; i < RG; i++) {
+        hp2[i] = __float2half2_rn((float)((pp.p[prime_at + i] - 1) / 2));
+        np2[i] = __float2half2_rn(-(float)pp.p[prime_at + i]);
+      }
+    }
     const uint32_t K = 1u << pb.k, Kp = 1u << pb.kp, bt = gt - pb.tile_lo;
     const uint32_t tiles_a = opA.mode ? (((1u << opA.f) + 63u) / 64u) << (pb.kp - 6) : 0;
     const bool isA = bt < tiles_a;  // uniform over the block
@@ -625,11 +629,11 @@ __global__ void __launch_bounds__(256) p8_pack_kernel(const PackProb* __restrict
 struct alignas(64) SplitProb {
   const uint8_t* part;
   uint8_t* out;
-  uint32_t log_n, log_split, block_lo, pad;  // n = 2^log_n residues; its first block of 1024 in the launch
+  uint32_t log_n, log_split, block_lo, prime_at;  // n = 2^log_n residues; its first block of 1024 in the launch
 };
 
 __global__ void __launch_bounds__(256) p8_split_final_kernel(const SplitProb* __restrict__ probs, uint32_t n_probs,
-                                                             uint32_t rg, uint4 primes) {
+                                                             uint32_t rg, const __grid_constant__ PackPrimes pp) {
   __shared__ uint32_t block_lo[kMaxProbs];
   if (threadIdx.x < n_probs) block_lo[threadIdx.x] = probs[threadIdx.x].block_lo;
   __syncthreads();
@@ -637,7 +641,6 @@ __global__ void __launch_bounds__(256) p8_split_final_kernel(const SplitProb* __
   const uint64_t n = 1ull << sp.log_n;
   const uint64_t i = ((uint64_t)(blockIdx.x - sp.block_lo) * 256u + threadIdx.x) * 4u;
   if (i >= n) return;
-  const uint32_t pr[4] = {primes.x, primes.y, primes.z, primes.w};
   uint32_t s[4] = {0, 0, 0, 0};
   for (uint32_t j0 = 0; j0 < (1u << sp.log_split); j0 += 256) {
     uint32_t even = 0, odd = 0;
@@ -655,7 +658,7 @@ __global__ void __launch_bounds__(256) p8_split_final_kernel(const SplitProb* __
   }
   uint32_t w = 0;
 #pragma unroll
-  for (uint32_t q = 0; q < 4; q++) w |= (s[q] % pr[q % rg]) << (8 * q);
+  for (uint32_t q = 0; q < 4; q++) w |= (s[q] % pp.p[sp.prime_at + q % rg]) << (8 * q);
   *reinterpret_cast<uint32_t*>(sp.out + i) = w;
 }
 
@@ -1465,7 +1468,8 @@ int fill_gemm(const StepDesc& d, const Shape& s, uint32_t rg, __half* pa, __half
 
 // One dense step's descriptors: operands and output in the arena, packed
 // planes at `scratch`, K-split partials at `part`.
-int fill_step(const P8Step& step, uint32_t rg, uint8_t* arena, uint64_t arena_bytes, uint8_t* scratch, uint8_t* part,
+int fill_step(const P8Step& step, uint32_t rg, uint32_t prime_at, uint8_t* arena, uint64_t arena_bytes,
+              uint8_t* scratch, uint8_t* part,
               tnc_p8::P8Prob& g, tnc_p8::PackProb& pk, tnc_p8::SplitProb& sp, uint32_t& variant,
               tnc_launch_counts& lc) {
   const StepDesc& d = step.d;
@@ -1504,12 +1508,14 @@ int fill_step(const P8Step& step, uint32_t rg, uint8_t* arena, uint64_t arena_by
   if (tiles >= (1ull << 31)) return set_error(TNC_ERR_TOO_LARGE, "dense step has too many operand tiles");
   pk.n_tiles = (uint32_t)tiles;
   uint8_t* out = arena + d.c_off * rg;  // direct: the planes, same place (twice the bytes)
-  if (int rc = fill_gemm(d, s, rg, pa, pb, dir_out, ls ? part : out, 0, g)) return rc;
+  if (int rc = fill_gemm(d, s, rg, pa, pb, dir_out, ls ? part : out, prime_at, g)) return rc;
+  pk.prime_at = prime_at;
   std::memset(&sp, 0, sizeof(sp));
   sp.part = part;
   sp.out = out;
   sp.log_n = d.c + (rg == 4 ? 2u : rg == 2 ? 1u : 0u);
   sp.log_split = ls;
+  sp.prime_at = prime_at;
   if (tiles) lc.p8_pack++;
   lc.p8_gemm++;
   if (ls) lc.p8_split++;
@@ -1539,22 +1545,26 @@ size_t put_descs(std::vector<char>& host, const std::vector<T>& v) {
 
 }  // namespace
 
-int p8_batch(const P8Step* steps, int n, uint32_t rg, uint8_t* arena, uint64_t arena_bytes, uint8_t* scratch,
-             uint8_t* part, std::vector<char>& host, P8Batch& b) {
+int p8_batch(const P8Step* steps, int n, uint32_t rg, int groups, uint64_t arena_stride, uint8_t* arena0,
+             uint64_t arena_bytes, uint8_t* scratch, uint8_t* part, std::vector<char>& host, P8Batch& b) {
   using namespace tnc_p8;
   if (rg != 1 && rg != 2 && rg != 4) return set_error(TNC_ERR_INVALID, "internal: residues per pass must be 1, 2 or 4");
-  if (n > (int)kMaxProbs) return set_error(TNC_ERR_INVALID, "internal: too many dense steps in a launch");
+  if (n * groups > (int)kMaxProbs || rg * groups > kLaunchPrimes)
+    return set_error(TNC_ERR_INVALID, "internal: too many dense steps in a launch");
   b = P8Batch{};
   std::vector<P8Prob> probs[6];
   std::vector<PackProb> packs;
   std::vector<SplitProb> splits;
   uint64_t tiles = 0, blocks = 0, items[6] = {0};
-  for (int i = 0; i < n; i++) {
+  for (int ig = 0; ig < n * groups; ig++) {
+    const int i = ig / groups, grp = ig % groups;
     P8Prob g;
     PackProb pk;
     SplitProb sp;
     uint32_t v = 0;
-    if (int rc = fill_step(steps[i], rg, arena, arena_bytes, scratch, part, g, pk, sp, v, b.counts)) return rc;
+    if (int rc = fill_step(steps[i], rg, rg * (uint32_t)grp, arena0 + (uint64_t)grp * arena_stride, arena_bytes, scratch,
+                           part, g, pk, sp, v, b.counts))
+      return rc;
     scratch += p8_scratch_bytes(steps[i], (int)rg);
     if (sp.log_split) {
       part += p8_part_bytes(steps[i].d, (int)rg);
@@ -1587,14 +1597,15 @@ int p8_batch(const P8Step* steps, int n, uint32_t rg, uint8_t* arena, uint64_t a
   return TNC_OK;
 }
 
-int p8_run(const P8Batch& b, const char* dev, const uint32_t* primes, uint32_t rg, uint32_t* dev_err, int sms,
-           void* stream) {
+int p8_run(const P8Batch& b, const char* dev, const uint32_t* primes, uint32_t n_primes, uint32_t rg,
+           uint32_t* dev_err, int sms, void* stream) {
   using namespace tnc_p8;
   cudaStream_t st = (cudaStream_t)stream;
   PackPrimes pp{};
   P8Primes pr{};
-  for (uint32_t i = 0; i < 4; i++) {
-    pp.p[i] = primes[i < rg ? i : 0];
+  if (n_primes > kLaunchPrimes) return set_error(TNC_ERR_INVALID, "internal: too many primes in a launch");
+  for (uint32_t i = 0; i < kLaunchPrimes; i++) {
+    pp.p[i] = primes[i < n_primes ? i : 0];
     pr.pf[i] = (float)pp.p[i];
     pr.invp[i] = 1.0f / (float)pp.p[i];
     if (pp.p[i] < 3 || pp.p[i] > 251) return set_error(TNC_ERR_INVALID, "tensor-core p8 steps need primes in [3, 251]");
@@ -1617,7 +1628,7 @@ int p8_run(const P8Batch& b, const char* dev, const uint32_t* primes, uint32_t r
   }
   if (b.split_n)
     p8_split_final_kernel<<<b.split_blocks, 256, 0, st>>>(reinterpret_cast<const SplitProb*>(dev + b.split_off),
-                                                          b.split_n, rg, make_uint4(pp.p[0], pp.p[1], pp.p[2], pp.p[3]));
+                                                          b.split_n, rg, pp);
   tnc_launch_counts& lc = launch_counts();
   const int32_t chunks = std::max(lc.p8_max_chunks, b.counts.p8_max_chunks);
   for (size_t i = 0; i < sizeof(lc) / sizeof(int32_t); i++)

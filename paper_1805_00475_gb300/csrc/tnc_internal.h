@@ -176,12 +176,14 @@ struct P8Step {
 };
 uint64_t p8_scratch_bytes(const P8Step& s, int rg);  // fp16 planes of the operands to pack
 // Dense steps launched together (independent ones: of one tree level), for
-// all rg residues of a pass whose entries hold rg residues of one byte each:
+// all groups of rg residues of a pass (group g's arena arena_stride bytes after
+// the one before) whose entries hold rg residues of one byte each:
 // one launch packs the operands not already in fp16 planes, one GEMM launch
 // per tile width computes every residue of each output tile and writes whole
 // entries (or planes), one launch adds the K-split partials.  p8_batch appends
 // the launches' descriptors (at most n p8_step_bytes()) to `host`, which the
-// caller copies to 64-byte aligned device memory, and lays the steps' planes
+// caller copies to 64-byte aligned device memory (n groups p8_step_bytes()
+// bytes), and lays the steps' planes
 // and partials out side by side from `scratch` and `part`; arena_bytes bounds
 // every range the steps touch.  p8_run launches them for the primes of a pass;
 // dev: the device copy of `host`.
@@ -196,10 +198,10 @@ struct P8Batch {
 };
 size_t p8_step_bytes();
 uint32_t p8_max_steps();
-int p8_batch(const P8Step* steps, int n, uint32_t rg, uint8_t* arena, uint64_t arena_bytes, uint8_t* scratch,
-             uint8_t* part, std::vector<char>& host, P8Batch& b);
-int p8_run(const P8Batch& b, const char* dev, const uint32_t* primes, uint32_t rg, uint32_t* dev_err, int sms,
-           void* stream);
+int p8_batch(const P8Step* steps, int n, uint32_t rg, int groups, uint64_t arena_stride, uint8_t* arena0,
+             uint64_t arena_bytes, uint8_t* scratch, uint8_t* part, std::vector<char>& host, P8Batch& b);
+int p8_run(const P8Batch& b, const char* dev, const uint32_t* primes, uint32_t n_primes, uint32_t rg,
+           uint32_t* dev_err, int sms, void* stream);
 // GEMM descriptors for operand planes that the caller packs (tc.cu): one step
 // appended to the variant's list; and the launch of a list.
 struct P8Probs {
@@ -216,7 +218,7 @@ size_t p8_prob_bytes();
 // One dense step of TNC_PATH_TC for residues r .. of the pass's entries.
 struct TcUnit {
   StepDesc d;
-  uint32_t r;
+  uint32_t group, r;  // the pass's residue group, the first residue in its entries
 };
 // Small primes that a step of 2^k products of residues below 2^31 needs, and
 // per residue the bytes of its operands' fp16 planes and of its output's small
@@ -236,9 +238,9 @@ struct TcBatch {
 };
 size_t tc_unit_bytes();
 uint32_t tc_max_units(uint32_t nr);
-int tc_batch(const TcUnit* units, int n, uint32_t nr, uint32_t rg, uint32_t* arena, uint64_t arena_bytes, uint8_t* planes,
-             uint8_t* bytes, std::vector<char>& host, TcBatch& b);
-std::vector<char> tc_consts(const uint32_t* primes, uint32_t rg);  // a pass's, for tc_run
+int tc_batch(const TcUnit* units, int n, uint32_t nr, uint32_t rg, uint32_t* arena0, uint64_t arena_stride,
+             uint64_t arena_bytes, uint8_t* planes, uint8_t* bytes, std::vector<char>& host, TcBatch& b);
+std::vector<char> tc_consts(const uint32_t* primes, uint32_t n_primes);  // a pass's, for tc_run
 int tc_run(const TcBatch& b, const char* dev, const std::vector<char>& consts, uint32_t rg, uint32_t* dev_err, int sms,
            void* stream);
 

@@ -26,7 +26,7 @@ def test_group_equals_one_by_one(path, R, copies):
     want = [tnc.contract_many([p, plans[2]], n_residues=R, path=path)[0] for p in plans]
     got = tnc.contract_many(plans * copies, n_residues=R, path=path, group=3 * copies)
     lc = tnc.last_launch_counts()
-    assert lc["crt"] == 1 and lc["extract"] >= (R // 4 + bin(R % 4).count("1")) * ((3 * copies + 63) // 64)
+    assert lc["crt"] == 1 and lc["extract"] >= (3 * copies + 63) // 64
     if path == "tc_p8":
         assert lc["p8_gemm"] >= 3 * copies
     for i, r in enumerate(got):
