@@ -44,56 +44,56 @@ __device__ __forceinline__ float ld<__nv_bfloat16>(const __nv_bfloat16* p, int i
   return __bfloat162float(p[i]);
 }
 
-// Eight consecutive weights from a 16-byte aligned position.
-__device__ __forceinline__ void ld8(const float* p, float (&v)[8]) {
-  const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
-  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-}
-__device__ __forceinline__ void ld8(const __nv_bfloat16* p, float (&v)[8]) {
-  const uint4 a = *reinterpret_cast<const uint4*>(p);
-  const uint32_t w[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-  for (int i = 0; i < 4; i++) {  // a bf16 is the upper half of a float
-    v[2 * i] = __uint_as_float(w[i] << 16);
-    v[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
-  }
+// Eight consecutive weights from a 16-byte aligned position; four from shared memory.
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 ld4(const __nv_bfloat16* p) {  // (a bf16 is the upper half of a float)
+  const uint2 w = *reinterpret_cast<const uint2*>(p);
+  return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u), __uint_as_float(w.y << 16),
+                     __uint_as_float(w.y & 0xFFFF0000u));
 }
 
-// W2 as fp32 in shared memory, S[j * kPitch + t] = W2[j][t].  vec: P is
-// 16-byte aligned (the caller's pointer may be any float's).
+// W2 in shared memory as it is, S[j * kPitch + t] = W2[j][t].  vec: P is
+// 16-byte aligned (the caller's pointer may be any element's).
 template <typename WT>
-__device__ __forceinline__ void stage_w2(const WT* __restrict__ P, float* S, bool vec) {
+__device__ __forceinline__ void stage_w2(const WT* __restrict__ P, WT* S, bool vec) {
+  constexpr int N = 16 / sizeof(WT);  // weights of a 16-byte copy
   if (vec) {
 #pragma unroll 8
-    for (int i = threadIdx.x * 8; i < H * H; i += H * 8) {
-      float v[8];
-      ld8(P + OFF_W2 + i, v);
-      float* d = S + (i / H) * kPitch + i % H;
-      *reinterpret_cast<float4*>(d) = make_float4(v[0], v[1], v[2], v[3]);
-      *reinterpret_cast<float4*>(d + 4) = make_float4(v[4], v[5], v[6], v[7]);
+    for (int i = threadIdx.x * N; i < H * H; i += H * N) {
+      const uint4 v = *reinterpret_cast<const uint4*>(P + OFF_W2 + i);
+      WT* d = S + (i / H) * kPitch + i % H;
+      if constexpr (sizeof(WT) == 4) {
+        *reinterpret_cast<uint4*>(d) = v;
+      } else {  // (rows of kPitch bf16 are 8-byte aligned)
+        reinterpret_cast<uint2*>(d)[0] = make_uint2(v.x, v.y);
+        reinterpret_cast<uint2*>(d)[1] = make_uint2(v.z, v.w);
+      }
     }
   } else {
 #pragma unroll 8
-    for (int i = threadIdx.x; i < H * H; i += H) S[(i / H) * kPitch + i % H] = ld(P, OFF_W2 + i);
+    for (int i = threadIdx.x; i < H * H; i += H) S[(i / H) * kPitch + i % H] = P[OFF_W2 + i];
   }
 }
 
-constexpr int kSmemFloats = H * kPitch + H * kRows + kRows * F;  // W2, a tile of activations, its inputs
-constexpr size_t kSmemBytes = kSmemFloats * sizeof(float);       // 75.0 KiB: three CTAs per SM
+// W2, a tile of activations, its inputs: 75.0 KiB, or 42.0 KiB with bf16
+// weights (below the 48 KiB that need no opt-in, which costs 1 us per call)
+template <typename WT>
+constexpr size_t kSmemBytes = H * kPitch * sizeof(WT) + (H * kRows + kRows * F) * sizeof(float);
 
 // y[r] = w3 . relu(W2^T relu(W1^T x_r + b1) + b2) + b3; optionally saves h1, h2.
 // H threads; in the H x H layer a warp owns 4 rows of the tile and a lane 4
 // consecutive hidden units.  The sums run over the units in ascending order.
-// 2048 rows: 23.6 us -> 8.0 us (fp32 weights), 20.9 -> 7.6 us (bf16): the
-// latency of one tile (staging W2, 128 steps of the inner loop); 70000 rows:
-// 96 -> 86 us, bound by the shared-memory reads of the inner loop.
+// 2048 rows: 23.6 us -> 8.0 us (fp32 weights): the latency of one tile (staging
+// W2, 128 steps of the inner loop); 70000 rows 96 -> 84 us, bound by the
+// shared-memory reads of the inner loop.  bf16 weights: 22.6 -> 8.3 us a call
+// among others (its launch), 70000 rows 98 -> 75 us.
 template <typename WT>
 __global__ void __launch_bounds__(H) mlp_forward_kernel(const WT* __restrict__ P, const float* __restrict__ X,
                                                         int64_t rows, float* __restrict__ Y, float* __restrict__ h1s,
                                                         float* __restrict__ h2s, int vec) {
   extern __shared__ __align__(16) float sm[];
-  float* w2 = sm;
-  float* h1 = w2 + H * kPitch;  // h1[j * kRows + r]
+  WT* w2 = reinterpret_cast<WT*>(sm);
+  float* h1 = reinterpret_cast<float*>(w2 + H * kPitch);  // h1[j * kRows + r]
   float* xs = h1 + H * kRows;   // xs[r * F + f]
   const int t = threadIdx.x, lane = t & 31, r4 = 4 * (t >> 5), c4 = 4 * lane;
   stage_w2(P, w2, vec != 0);
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(H) mlp_forward_kernel(const WT* __restrict__ P
 #pragma unroll 8
     for (int j = 0; j < H; j++) {
       const float4 h = *reinterpret_cast<const float4*>(h1 + j * kRows + r4);
-      const float4 w = *reinterpret_cast<const float4*>(w2 + j * kPitch + c4);
+      const float4 w = ld4(w2 + j * kPitch + c4);
       const float hv[4] = {h.x, h.y, h.z, h.w}, wv[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
       for (int i = 0; i < 4; i++)
@@ -418,11 +418,12 @@ unsigned blocks_for(int64_t rows) {
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
-// The forward and row kernels' dynamic shared memory limit (a property of the
-// kernel on the current device; setting it again is harmless).
+// The fp32 kernels' dynamic shared memory limit (a property of the kernel on
+// the current device; setting it again is harmless).
 template <typename K>
 int allow_smem(K kernel) {
-  MLP_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tnc_mlp::kSmemBytes));
+  MLP_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)tnc_mlp::kSmemBytes<float>));
   return TNC_OK;
 }
 }  // namespace
@@ -442,7 +443,7 @@ int mlp_forward_dev(const float* P, const float* X, int64_t rows, float* Y, floa
   if (rows <= 0) return TNC_OK;
   if (int rc = allow_smem(tnc_mlp::mlp_forward_kernel<float>)) return rc;
   const int vec = aligned16(P) && aligned16(h2);
-  tnc_mlp::mlp_forward_kernel<float><<<blocks_for(rows), tnc_mlp::H, tnc_mlp::kSmemBytes, (cudaStream_t)stream>>>(
+  tnc_mlp::mlp_forward_kernel<float><<<blocks_for(rows), tnc_mlp::H, tnc_mlp::kSmemBytes<float>, (cudaStream_t)stream>>>(
       P, X, rows, Y, h1, h2, vec);
   MLP_TRY(cudaGetLastError());
   return TNC_OK;
@@ -450,9 +451,8 @@ int mlp_forward_dev(const float* P, const float* X, int64_t rows, float* Y, floa
 
 int mlp_forward_bf16_dev(const void* Pb, const float* X, int64_t rows, float* Y, void* stream) {
   if (rows <= 0) return TNC_OK;
-  if (int rc = allow_smem(tnc_mlp::mlp_forward_kernel<__nv_bfloat16>)) return rc;
   tnc_mlp::mlp_forward_kernel<__nv_bfloat16>
-      <<<blocks_for(rows), tnc_mlp::H, tnc_mlp::kSmemBytes, (cudaStream_t)stream>>>(
+      <<<blocks_for(rows), tnc_mlp::H, tnc_mlp::kSmemBytes<__nv_bfloat16>, (cudaStream_t)stream>>>(
           (const __nv_bfloat16*)Pb, X, rows, Y, nullptr, nullptr, aligned16(Pb));
   MLP_TRY(cudaGetLastError());
   return TNC_OK;
@@ -484,7 +484,7 @@ int tnc_mlp_backward(const float* d_params, const float* d_x, const float* d_h1,
   float* dh2 = dh1 + rows * TNC_MLP_HIDDEN;
   float* part = dh2 + rows * TNC_MLP_HIDDEN;
   if (int rc = allow_smem(tnc_mlp::mlp_backward_rows_kernel)) return rc;
-  tnc_mlp::mlp_backward_rows_kernel<<<blocks_for(rows), tnc_mlp::H, tnc_mlp::kSmemBytes, st>>>(
+  tnc_mlp::mlp_backward_rows_kernel<<<blocks_for(rows), tnc_mlp::H, tnc_mlp::kSmemBytes<float>, st>>>(
       d_params, d_h1, d_h2, d_y, d_t, rows, dy, dh1, dh2);
   const int64_t slice = (rows + tnc_mlp::splits_for(rows) - 1) / tnc_mlp::splits_for(rows);
   const int n = (int)((rows + slice - 1) / slice);
