@@ -82,11 +82,14 @@ struct Groups {
   std::vector<int> rg, col;
 };
 
+// Three residues left over are a group of four with one that nobody asked for:
+// a batch launch with four residues takes less than one with two and one with one
+// (217 cubic VC formulas with n = 48, 3 residues: 85 -> 63 us).
 Groups split_groups(int R) {
   Groups g;
   int c = 0;
   for (int s : {4, 2, 1})
-    while (R - c >= s) {
+    while (R - c >= s || (s == 4 && R - c == 3)) {
       g.rg.push_back(s);
       g.col.push_back(c);
       c += s;
@@ -102,7 +105,10 @@ struct Arith {
   Groups groups;
   ModGroup group(int gi) const {
     uint32_t p[4];
-    for (int r = 0; r < 4; r++) p[r] = r < groups.rg[gi] ? primes[groups.col[gi] + r] : primes[groups.col[gi]];
+    for (int r = 0; r < 4; r++) {  // (a filled-up group repeats its first prime)
+      const int i = groups.col[gi] + r;
+      p[r] = primes[r < groups.rg[gi] && i < R ? i : groups.col[gi]];
+    }
     return tnc_dev::make_mod_group(p);
   }
 };
@@ -907,12 +913,22 @@ void make_solo(const tnc_plan_t* p, SoloPack& s) {
   s.ok = blob.size() <= 160 * 1024;
 }
 
+// The CRT of n entries: a warp each while that is at most four warps per
+// scheduler of the GPU, else a thread each.
+void launch_crt(const uint32_t* residues, uint64_t n, const CrtConsts& cc, uint32_t* limbs, cudaStream_t st) {
+  if (n <= 2048)
+    tnc_dev::crt_warp_kernel<<<(unsigned)((n + 3) / 4), 128, 0, st>>>(residues, n, cc, limbs);
+  else
+    tnc_dev::crt_kernel<<<(unsigned)std::min<uint64_t>((n + 127) / 128, 1024), 128, 0, st>>>(residues, n, cc, limbs);
+  g_launches.crt++;
+}
+
 // Enqueues the one-launch contraction (descriptors up, a launch per residue
 // group); results and limbs are left in their workspace sections.
 int solo_enqueue(const SoloPack& s, const SeqLayout& L, const Arith& a, char* ws, cudaStream_t st) {
   CUDA_TRY(cudaMemcpyAsync(ws, s.bytes.data(), s.bytes.size(), cudaMemcpyHostToDevice, st));
   g_h2d_bytes += s.bytes.size();
-  for (size_t gi = 0; gi < a.groups.rg.size(); gi++) {
+  for (const PassShape& shape : L.passes) {
     tnc_dev::BatchArgs args{};
     args.forms = (const BForm*)ws;
     args.blobs = (const uint4*)(ws + s.off_blob);
@@ -923,20 +939,33 @@ int solo_enqueue(const SoloPack& s, const SeqLayout& L, const Arith& a, char* ws
     args.n_forms = args.n_heavy = args.cluster_slots = 1;
     args.results = (uint32_t*)(ws + L.off_results);
     args.garena = (uint32_t*)(ws + L.off_arena);
+    args.slot_entries = L.arena_entries;
     args.blob_cap = (uint32_t)s.blob_bytes;
     args.R = a.R;
-    args.col = a.groups.col[gi];
-    args.limbs = gi + 1 == a.groups.rg.size() ? (uint32_t*)(ws + L.off_limbs) : nullptr;
-    const ModGroup mg = a.group((int)gi);
-    int rc = dispatch_rg(a.groups.rg[gi], [&](auto rgc) -> int {
+    args.col = shape.col;
+    const bool alone = L.passes.size() == 1 && shape.groups == 1;
+    args.limbs = alone ? (uint32_t*)(ws + L.off_limbs) : nullptr;
+    tnc_dev::SoloConsts sc{};
+    if (alone) sc.crt = a.crt;
+    bool near30 = true;
+    for (int g = 0; g < shape.groups; g++) {
+      uint32_t gp[4];
+      for (int r = 0; r < 4; r++) {
+        const int i = shape.col + g * shape.rg + r;
+        gp[r] = a.primes[r < shape.rg && i < a.R ? i : shape.col + g * shape.rg];
+      }
+      sc.mg[g] = tnc_dev::make_mod_group(gp);
+      near30 = near30 && sc.mg[g].near30;
+    }
+    int rc = dispatch_rg(shape.rg, [&](auto rgc) -> int {
       constexpr int RG = decltype(rgc)::value;
-      auto k = mg.near30 ? tnc_dev::batch_kernel<RG, true, tnc_dev::kBatchSolo>
-                         : tnc_dev::batch_kernel<RG, false, tnc_dev::kBatchSolo>;
+      auto k = near30 ? tnc_dev::batch_kernel<RG, true, tnc_dev::kBatchSolo>
+                      : tnc_dev::batch_kernel<RG, false, tnc_dev::kBatchSolo>;
       if (s.blob_bytes > 48 * 1024 - 64)
         CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
       if (s.ctas > 8) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-      const ClusterLaunch cl(s.ctas, 256, s.blob_bytes, st, s.ctas);
-      CUDA_TRY(cudaLaunchKernelEx(&cl.cfg, k, args, mg, a.crt));
+      const ClusterLaunch cl(s.ctas * (unsigned)shape.groups, 256, s.blob_bytes, st, s.ctas);
+      CUDA_TRY(cudaLaunchKernelEx(&cl.cfg, k, args, sc.mg[0], sc));
       return TNC_OK;
     });
     if (rc) return rc;
@@ -946,7 +975,9 @@ int solo_enqueue(const SoloPack& s, const SeqLayout& L, const Arith& a, char* ws
     g_launches.extract++;
     g_launches.splitk += s.long_sums;
   }
-  g_launches.crt++;
+  if (L.passes.size() == 1 && L.passes[0].groups == 1) g_launches.crt++;
+  else launch_crt((const uint32_t*)(ws + L.off_results), L.n_out, a.crt, (uint32_t*)(ws + L.off_limbs), st);
+  CUDA_TRY(cudaGetLastError());
   return TNC_OK;
 }
 
@@ -1481,9 +1512,7 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
     return TNC_OK;
   }
   uint32_t* limbs = (uint32_t*)(ws + L.off_limbs);
-  tnc_dev::crt_kernel<<<(unsigned)std::min<uint64_t>((L.n_out + 127) / 128, 1024), 128, 0, st>>>(results, L.n_out, a.crt,
-                                                                                                  limbs);
-  g_launches.crt++;
+  launch_crt(results, L.n_out, a.crt, limbs, st);
   CUDA_TRY(cudaGetLastError());
   if (g_time_dense) CUDA_TRY(cudaEventRecord(whole[1], st));
   // status, residues and limbs: consecutive sections, one copy
@@ -1591,15 +1620,13 @@ extern "C" int tnc_contract_sliced(const tnc_plan_t* const* plans, int32_t n, co
                         acc);
     if (rc) return rc;
   }
-  tnc_dev::crt_kernel<<<(unsigned)std::min<uint64_t>((n_out + 127) / 128, 1024), 128, 0, st>>>(acc, n_out, a.crt, limbs);
-  g_launches.crt++;
+  launch_crt(acc, n_out, a.crt, limbs, st);
   CUDA_TRY(cudaGetLastError());
-  std::vector<uint32_t> h_res(n_out * a.R), h_limbs(n_out * a.crt.n_limbs);
-  CUDA_TRY(cudaMemcpyAsync(h_res.data(), acc, h_res.size() * 4, cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaMemcpyAsync(h_limbs.data(), limbs, h_limbs.size() * 4, cudaMemcpyDeviceToHost, st));
-  g_d2h_bytes += (h_res.size() + h_limbs.size()) * 4;
+  std::vector<uint32_t> down((limbs - acc) + n_out * a.crt.n_limbs);  // residues and limbs: one copy
+  CUDA_TRY(cudaMemcpyAsync(down.data(), acc, down.size() * 4, cudaMemcpyDeviceToHost, st));
+  g_d2h_bytes += down.size() * 4;
   CUDA_TRY(cudaStreamSynchronize(st));
-  return fill_count(out, n_out, a, h_res.data(), h_limbs.data(), bound >= a.log2_prod - 1e-9 ? TNC_MAYBE_WRAPPED : 0u);
+  return fill_count(out, n_out, a, down.data(), down.data() + (limbs - acc), bound >= a.log2_prod - 1e-9 ? TNC_MAYBE_WRAPPED : 0u);
 }
 
 extern "C" size_t tnc_workspace_bytes_many(const tnc_plan_t* const* plans, int32_t n, const tnc_contract_opts* opts,

@@ -429,25 +429,35 @@ __device__ __forceinline__ uint32_t map_runs(uint32_t o, const uint16_t* runs, i
 // formula that takes longer alone than the batch's average CTA would
 // otherwise be what the launch ends with.  Then every CTA takes formulas from
 // the queue as above.
+// kBatchSolo: one formula; cluster g contracts it for residue group g (its
+// primes in mg[g], its arena in slot g), a single group's cluster also runs the CRT.
+enum BatchMode { kBatchCtas, kBatchClusters, kBatchSolo };
+struct SoloConsts {
+  CrtConsts crt;
+  ModGroup mg[4];
+};
 template <int MODE>
-using BatchCrt = std::conditional_t<MODE == 2, CrtConsts, int>;  // (only kBatchSolo has a use for the constants)
-enum BatchMode { kBatchCtas, kBatchClusters, kBatchSolo };  // kBatchSolo: one formula, one cluster, and its CRT
+using BatchConsts = std::conditional_t<MODE == kBatchSolo, SoloConsts, int>;
 template <int RG, bool N30 = false, int MODE = kBatchCtas>
 __global__ void __launch_bounds__(256, MODE == kBatchCtas ? 0 : (MODE == kBatchSolo ? 1 : (RG == 4 && !N30 ? 3 : 4)))
-    batch_kernel(BatchArgs a, ModGroup mg, const __grid_constant__ BatchCrt<MODE> cc) {
+    batch_kernel(BatchArgs a, ModGroup mg, const __grid_constant__ BatchConsts<MODE> sc) {
   constexpr bool CLUSTER = MODE != kBatchCtas;
   extern __shared__ uint4 smem_raw[];
   __shared__ uint32_t task;
   const int lane = threadIdx.x & 31;
   uint4* blob = smem_raw;
   uint32_t* sarena = reinterpret_cast<uint32_t*>(smem_raw + (a.blob_cap >> 4));
+  if constexpr (MODE == kBatchSolo) {
+    mg = sc.mg[blockIdx.x / cluster_ctas()];
+    a.col += RG * (int)(blockIdx.x / cluster_ctas());
+  }
   bool coop = CLUSTER;       // contracting the heavy formulas, cluster by cluster
   uint32_t round = 0;
   for (;;) {
     uint32_t t;
     if (CLUSTER && coop) {
       const uint32_t nc = gridDim.x / cluster_ctas(), c = blockIdx.x / cluster_ctas();
-      t = round * nc + ((round & 1u) ? nc - 1u - c : c);
+      t = MODE == kBatchSolo ? round : round * nc + ((round & 1u) ? nc - 1u - c : c);
       round++;
       if (t >= a.n_heavy) {
         if (a.n_heavy == a.n_forms) break;
@@ -572,13 +582,14 @@ __global__ void __launch_bounds__(256, MODE == kBatchCtas ? 0 : (MODE == kBatchS
       for (uint32_t j = 0; j < f.n_open; j++) ad |= ((J >> a.perms[f.perm_off + j]) & 1u) << j;
 #pragma unroll
       for (int r = 0; r < RG; r++)
-        a.results[((uint64_t)f.res_off + J) * a.R + a.col + r] = arena[((uint64_t)f.root_off + ad) * RG + r];
+        if (RG != 4 || a.col + r < a.R)  // (a group of four may be filled up)
+          a.results[((uint64_t)f.res_off + J) * a.R + a.col + r] = arena[((uint64_t)f.root_off + ad) * RG + r];
     }
     barrier();
     if constexpr (MODE == kBatchSolo)
       if (a.limbs)
       for (uint32_t J = tid; J < f.n_out; J += nthreads)
-        crt_entry(a.results + (uint64_t)J * a.R, cc, a.limbs + (uint64_t)J * cc.n_limbs);
+        crt_entry(a.results + (uint64_t)J * a.R, sc.crt, a.limbs + (uint64_t)J * sc.crt.n_limbs);
   }
 }
 
