@@ -171,9 +171,10 @@ __global__ void __launch_bounds__(256) rns_pack_kernel(const PackUnit* __restric
     if (isA ? u.mn_a : u.mn_b) {
       e0 = at = (uint64_t)tile * 1024u + threadIdx.x * 4u;
       step = 1;
-    } else {  // row r, shared values q .. q + 3 (lanes along the rows)
-      const uint64_t i = (uint64_t)tile * 256u + threadIdx.x;
-      const uint64_t r = i & ((1u << f) - 1u), q = (i >> f) * 4u;
+    } else {  // row r, shared values q .. q + 3; a warp takes 8 rows x 16 shared values: a row's 4 lanes write a
+              // whole 32-byte sector (lanes along 32 rows: 552 us instead of 132 for 2^22 entries, 4 residues)
+      const uint64_t i = (uint64_t)tile * 256u + threadIdx.x, hi = i >> 5;
+      const uint64_t r = (hi & ((1u << (f - 3)) - 1u)) * 8u + (i & 7u), q = ((hi >> (f - 3)) * 4u + ((i >> 3) & 3u)) * 4u;
       e0 = (q << f) + r;
       step = 1ull << f;
       at = (r << u.k) + q;
@@ -298,20 +299,25 @@ bool tc_eligible(const StepDesc& d) {
 
 // S < 2^(62 + k) (2^(60 + k) for the default primes, which then need one prime
 // less for two values of k in eight: not worth a second rule); Q >= 4/3 S.
-uint32_t tc_small_primes(uint32_t k) {
+// Small steps take all 12: three groups of four are one GEMM launch (6 to 8 us)
+// where 9 to 11 are two or three, and up to 2^kFewMacs products the extra ones
+// take less (2^25 products, one residue: launches of 15 + 10 us -> one of 15).
+constexpr uint32_t kFewMacs = 27;
+uint32_t tc_small_primes(const StepDesc& d) {
+  if (d.ka + d.kb + d.k <= kFewMacs) return kMaxSmall;  // (k <= 15: Q is large enough)
   double bits = 0;
   for (uint32_t n = 0; n < kMaxSmall; n++) {
     bits += std::log2((double)small_prime(n));
-    if (n >= 8 && bits >= 62.0 + k + 0.4151) return n + 1;
+    if (n >= 8 && bits >= 62.0 + d.k + 0.4151) return n + 1;
   }
   return 0;
 }
 
 uint64_t tc_plane_bytes(const StepDesc& d) {
-  return 2ull * tc_small_primes(d.k) * ((1ull << (d.ka + d.k)) + (1ull << (d.kb + d.k)));
+  return 2ull * tc_small_primes(d) * ((1ull << (d.ka + d.k)) + (1ull << (d.kb + d.k)));
 }
 
-uint64_t tc_byte_bytes(const StepDesc& d) { return (uint64_t)tc_small_primes(d.k) << (d.c + p8_split_log(d)); }
+uint64_t tc_byte_bytes(const StepDesc& d) { return (uint64_t)tc_small_primes(d) << (d.c + p8_split_log(d)); }
 
 size_t tc_unit_bytes() { return sizeof(tnc_rns::PackUnit) + sizeof(tnc_rns::JoinUnit) + 4 * p8_prob_bytes(); }
 uint32_t tc_max_units(uint32_t nr) { return tnc_rns::kMaxUnits / 3 / nr; }  // (up to three groups of four primes a residue)
@@ -328,7 +334,7 @@ int tc_batch(const TcUnit* units, int n, uint32_t nr, uint32_t rg, uint32_t* are
   uint64_t tiles = 0, blocks = 0;
   for (int i = 0; i < n; i++) {
     const StepDesc& d = units[i].d;
-    const uint32_t nq = tc_small_primes(d.k), ls = p8_split_log(d);
+    const uint32_t nq = tc_small_primes(d), ls = p8_split_log(d);
     if (!nq) return set_error(TNC_ERR_TOO_LARGE, "dense step with too many shared values");
     uint32_t* const arena = arena0 + units[i].group * arena_stride;
     if (units[i].r + nr > rg || (nr != 1 && nr != rg) || (units[i].group + 1) * rg > kTcPrimes) return set_error(TNC_ERR_INVALID, "internal: residues outside their pass");

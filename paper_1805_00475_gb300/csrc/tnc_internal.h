@@ -220,10 +220,10 @@ struct TcUnit {
   StepDesc d;
   uint32_t group, r;  // the pass's residue group, the first residue in its entries
 };
-// Small primes that a step of 2^k products of residues below 2^31 needs, and
+// Small primes that a step takes (residues below 2^31), and
 // per residue the bytes of its operands' fp16 planes and of its output's small
 // residues.
-uint32_t tc_small_primes(uint32_t k);
+uint32_t tc_small_primes(const StepDesc& d);
 uint64_t tc_plane_bytes(const StepDesc& d);
 uint64_t tc_byte_bytes(const StepDesc& d);
 // Units of nr residues (all rg of the pass, or one) launched together (as
