@@ -256,7 +256,8 @@ void tnc_free_plan(tnc_plan_t* plan);
 size_t tnc_workspace_bytes(const tnc_plan_t* plan, int32_t n_residues);
 /* Device workspace needed by tnc_contract with these options (any path; adds
  * TNC_PATH_TC_P8's packed fp16 operands and K-split partials); 0 if the options
- * are invalid. */
+ * are invalid.  It holds the residue groups side by side as far as that is
+ * faster; the calls also run in a workspace that only holds them one at a time. */
 size_t tnc_workspace_bytes_opts(const tnc_plan_t* plan, const tnc_contract_opts* opts);
 /* Sliced contraction (bond slicing: fixing s variables of a formula splits its
  * count into 2^s counts of smaller networks, each with at most the original

@@ -626,10 +626,18 @@ int plan_groups(const tnc_plan_t* const* plans, int n, int R, int path, size_t b
   return TNC_OK;
 }
 
-// What a single plan is given, and the least it needs.
-size_t plan_bytes(const tnc_plan_t* p, int R, int path) {
-  return std::max(group_layout(&p, 1, R, path, true).total, group_layout(&p, 1, R, path, false).total);
+// What a group of plans is given: the wide layout (contract_group takes the
+// other where the workspace holds only that); on the u32 paths the larger of
+// both, so that one workspace serves either.
+size_t group_bytes(const tnc_plan_t* const* plans, int n, int R, int path) {
+  size_t b = 0;
+  for (int other : {TNC_PATH_INT64, TNC_PATH_TC, TNC_PATH_TC_P8}) {
+    if ((other == TNC_PATH_TC_P8) != (path == TNC_PATH_TC_P8)) continue;
+    for (bool wide : {true, false}) b = std::max(b, group_layout(plans, n, R, other, wide).total);
+  }
+  return b;
 }
+size_t plan_bytes(const tnc_plan_t* p, int R, int path) { return group_bytes(&p, 1, R, path); }
 
 // One residue group at a time on the CUDA cores (tnc_contract_noalloc).
 SeqLayout seq_layout(const tnc_plan_t* p, int R) { return group_layout(&p, 1, R, TNC_PATH_INT64, false); }
@@ -985,7 +993,7 @@ int solo_enqueue(const SoloPack& s, const SeqLayout& L, const Arith& a, char* ws
 
 extern "C" size_t tnc_workspace_bytes(const tnc_plan_t* plan, int32_t n_residues) {
   if (!plan || n_residues < 1 || n_residues > 16) return 0;
-  return std::max(plan_bytes(plan, n_residues, TNC_PATH_INT64), plan_bytes(plan, n_residues, TNC_PATH_TC));
+  return plan_bytes(plan, n_residues, TNC_PATH_INT64);
 }
 
 extern "C" void tnc_set_step_timing(int32_t on) { g_time_dense = on != 0; }
@@ -1601,7 +1609,9 @@ extern "C" int tnc_contract_sliced(const tnc_plan_t* const* plans, int32_t n, co
     const double b = plans[i]->net.log2_bound;
     bound = i == 0 ? b : std::max(bound, b) + std::log2(1.0 + std::exp2(-std::fabs(bound - b)));
   }
-  const size_t need = tnc_workspace_bytes_sliced(plans, n, opts);
+  size_t need = 256;  // (one residue group at a time)
+  for (int i = 0; i < n; i++) need = std::max(need, group_layout(plans + i, 1, a.R, opts->path, false).total);
+  need += sliced_head_bytes(1ull << n_open, a);
   if (!dev_ws || ws_bytes < need) return set_error(TNC_ERR_BUFFER, "workspace smaller than tnc_workspace_bytes_sliced");
   if (((uintptr_t)dev_ws) % kAlign) return set_error(TNC_ERR_INVALID, "workspace must be 256-byte aligned");
   cudaStream_t st = (cudaStream_t)cuda_stream;
@@ -1639,7 +1649,7 @@ extern "C" size_t tnc_workspace_bytes_many(const tnc_plan_t* const* plans, int32
     const int m = std::min<int>(group, n - i);
     for (int j = i; j < i + m; j++)
       if (!plans[j]) return 0;
-    for (bool wide : {true, false}) need = std::max(need, group_layout(plans + i, m, a.R, opts->path, wide).total);
+    need = std::max(need, group_bytes(plans + i, m, a.R, opts->path));
   }
   return need;
 }

@@ -692,7 +692,8 @@ __global__ void __launch_bounds__(256) extract_kernel(const W* __restrict__ aren
 // The CRT of few entries, a warp each: Garner's digits one after the other, but
 // every prime's running value v0 + v1 p0 + .. (mod p_i) and its next weight
 // p0 .. p_k (mod p_i) kept by a lane of its own (two primes a lane).  One
-// thread alone does R^2 / 2 dependent steps: 20 us for 20 residues; this way 2 R: 6 us.
+// thread alone does R^2 / 2 dependent steps: 20 us for 20 residues; this way 2 R,
+// and the limbs: 12 us.
 __global__ void __launch_bounds__(128) crt_warp_kernel(const uint32_t* __restrict__ residues, uint64_t n_entries,
                                                        const __grid_constant__ CrtConsts cc,
                                                        uint32_t* __restrict__ limbs) {

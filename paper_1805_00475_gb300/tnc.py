@@ -475,6 +475,13 @@ def _workspace(nbytes: int, ws=None):
     return torch.empty(max(nbytes, 256), dtype=torch.uint8, device="cuda")
 
 
+def _check_ws(rc: int):
+    """_check for calls whose only buffer that can be too small is the workspace."""
+    if rc == -4:
+        raise ValueError("workspace too small")
+    _check(rc)
+
+
 def workspace_bytes(p: Plan, n_residues: int, path: str = "int64", primes=None) -> int:
     """tnc_workspace_bytes_opts for the path (tnc_workspace_bytes on int64 / tc)."""
     return _plan_bytes(p, _opts(n_residues, primes, path)[0])
@@ -491,10 +498,12 @@ def contract(p: Plan, n_residues: int = 4, primes=None, workspace=None, stream=N
     """Contract one plan on the GPU (tnc_contract); returns exact counts."""
     o, pr = _opts(n_residues, primes, path)
     nb = _plan_bytes(p, o)
+    if workspace is not None:  # (less than the library would use may still do)
+        nb = min(nb, workspace.numel() * workspace.element_size())
     ws = _workspace(nb, workspace)
     c, res, limbs = _count_buffers(1 << p.n_open, n_residues)
-    _check(lib().tnc_contract(p.h, ctypes.byref(o), ctypes.c_void_p(ws.data_ptr()), nb, _stream_ptr(stream),
-                              ctypes.byref(c)))
+    _check_ws(lib().tnc_contract(p.h, ctypes.byref(o), ctypes.c_void_p(ws.data_ptr()), nb, _stream_ptr(stream),
+                                 ctypes.byref(c)))
     return _to_count(c, res, limbs, pr)
 
 
@@ -584,11 +593,11 @@ def contract_sliced(plans: Sequence[Plan], n_residues: int = 4, primes=None, wor
     nb = int(lib().tnc_workspace_bytes_sliced(arr, len(plans), ctypes.byref(o)))
     if nb == 0:
         raise TncError(-1, lib().tnc_last_error().decode() or "invalid slices")
-    ws = _workspace(nb, workspace)
+    ws = workspace if workspace is not None else _workspace(nb)
     nb = ws.numel() * ws.element_size()  # a larger workspace lets slices run merged
     c, res, limbs = _count_buffers(1 << plans[0].n_open, n_residues)
-    _check(lib().tnc_contract_sliced(arr, len(plans), ctypes.byref(o), ctypes.c_void_p(ws.data_ptr()), nb,
-                                     _stream_ptr(stream), ctypes.byref(c)))
+    _check_ws(lib().tnc_contract_sliced(arr, len(plans), ctypes.byref(o), ctypes.c_void_p(ws.data_ptr()), nb,
+                                        _stream_ptr(stream), ctypes.byref(c)))
     return _to_count(c, res, limbs, pr)
 
 

@@ -33,3 +33,26 @@ def test_group_equals_one_by_one(path, R, copies):
         assert r.residues.tolist() == want[i % 3].residues.tolist() and r.counts == want[i % 3].counts, i
     for f, w in zip(forms[::2], want[::2]):
         assert w.residues.tolist() == oracle.residues(oracle.count(f, max_rank=28), w.primes)
+
+
+@pytest.mark.parametrize("path,R", [("int64", 7), ("tc", 7), ("tc_p8", 11)])
+def test_workspaces(path, R):
+    """One workspace serves both u32 paths; less than the library would use, down to
+    one residue group at a time, gives the same counts; too little is refused."""
+    import torch
+    f = I.cubic_vertex_cover(90, 4)
+    p = tnc.plan_formula(f, heuristic="bisect", rank_cap=24)
+    nb = tnc.workspace_bytes(p, R, "tc_p8" if path == "tc_p8" else "int64")
+    want = tnc.contract(p, n_residues=R, path=path, workspace=torch.empty(nb, dtype=torch.uint8, device="cuda"))
+    assert want.residues.tolist() == oracle.residues(oracle.count(f, max_rank=24), want.primes)
+    ran = 0
+    for k in range(1, 8):
+        try:
+            r = tnc.contract(p, n_residues=R, path=path, workspace=torch.empty(nb * k // 8, dtype=torch.uint8, device="cuda"))
+        except ValueError:
+            continue
+        ran += 1
+        assert r.residues.tolist() == want.residues.tolist() and r.counts == want.counts
+    assert ran >= 1
+    with pytest.raises(ValueError):
+        tnc.contract(p, n_residues=R, path=path, workspace=torch.empty(4096, dtype=torch.uint8, device="cuda"))
