@@ -295,7 +295,7 @@ tnc_dev::TileStep make_tile_step(const StepDesc& d) {
   t.ka = d.ka;
   t.kb = d.kb;
   const BitMap m(d);
-  uint32_t out_a[kTileA], out_b[kTileB];  // output bits of the operands' highest free bits
+  uint32_t out_a[kTileA] = {}, out_b[kTileB] = {};  // output bits of the operands' highest free bits
   for (int j = 0; j < d.c; j++) {
     const int top = m.op[j] ? m.dst[j] - (d.kb - kTileB) : m.dst[j] - (d.ka - kTileA);
     if (top >= 0) {
@@ -1122,8 +1122,8 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
   const bool tc = opts->path == TNC_PATH_TC || p8;
   const int sms = sm_count();
   std::vector<char> stage;
-  auto put = [&](const void* src, size_t bytes) {  // 64-byte aligned; returns the offset
-    const size_t at = (stage.size() + 63) / 64 * 64;
+  auto put = [&](const void* src, size_t bytes) {  // 128-byte aligned; returns the offset
+    const size_t at = (stage.size() + 127) / 128 * 128;
     stage.resize(at + bytes);
     if (bytes) std::memcpy(stage.data() + at, src, bytes);
     return at;

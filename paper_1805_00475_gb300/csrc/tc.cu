@@ -319,7 +319,7 @@ uint64_t tc_plane_bytes(const StepDesc& d) {
 
 uint64_t tc_byte_bytes(const StepDesc& d) { return (uint64_t)tc_small_primes(d) << (d.c + p8_split_log(d)); }
 
-size_t tc_unit_bytes() { return sizeof(tnc_rns::PackUnit) + sizeof(tnc_rns::JoinUnit) + 4 * p8_prob_bytes(); }
+size_t tc_unit_bytes() { return sizeof(tnc_rns::PackUnit) + sizeof(tnc_rns::JoinUnit) + 4 * p8_prob_bytes() + 256; }
 uint32_t tc_max_units(uint32_t nr) { return tnc_rns::kMaxUnits / 3 / nr; }  // (up to three groups of four primes a residue)
 
 int tc_batch(const TcUnit* units, int n, uint32_t nr, uint32_t rg, uint32_t* arena0, uint64_t arena_stride,
@@ -390,7 +390,7 @@ int tc_batch(const TcUnit* units, int n, uint32_t nr, uint32_t rg, uint32_t* are
   }
   if (std::max(tiles, blocks) >= (1ull << 31)) return set_error(TNC_ERR_TOO_LARGE, "dense steps of a level have too many tiles");
   auto put = [&](const void* src, size_t size) {
-    const size_t at = host.size();
+    const size_t at = size ? (host.size() + 127) / 128 * 128 : host.size();  // (the tensor maps' alignment)
     host.resize(at + size);
     if (size) std::memcpy(host.data() + at, src, size);
     return at;

@@ -103,7 +103,7 @@ constexpr uint64_t kWaitNs = 2000000000ull;
 // One dense step as the GEMM launch sees it, in device memory: a launch takes
 // the work items of up to kMaxProbs steps (of one tree level, with one tile
 // width) one after another.
-struct alignas(64) P8Prob {
+struct alignas(128) P8Prob {
   CUtensorMap map_a, map_b;  // operand planes of the row side and of the column side
   uint32_t fa, fb, k, log_split;  // rows 2^fa, columns 2^fb, shared 2^k, K split 2^log_split
   uint32_t n_items, tiles_m;      // work items (tiles x splits); row tiles
@@ -1389,7 +1389,8 @@ uint64_t p8_scratch_bytes(const P8Step& s, int rg) {
   return b;
 }
 
-size_t p8_step_bytes() { return sizeof(tnc_p8::P8Prob) + sizeof(tnc_p8::PackProb) + sizeof(tnc_p8::SplitProb); }
+// (with the padding between the arrays of a launch)
+size_t p8_step_bytes() { return sizeof(tnc_p8::P8Prob) + sizeof(tnc_p8::PackProb) + sizeof(tnc_p8::SplitProb) + 256; }
 uint32_t p8_max_steps() { return tnc_p8::kMaxProbs; }
 
 namespace {
@@ -1532,12 +1533,12 @@ int fill_step(const P8Step& step, uint32_t rg, uint32_t prime_at, uint8_t* arena
   return TNC_OK;
 }
 
-// Appends the descriptors `v` to the staging buffer; returns their offset
-// (every descriptor is a multiple of 64 bytes, the buffer 64-byte aligned).
+// Appends the descriptors `v` to the staging buffer at a multiple of 128 bytes
+// (the tensor maps' alignment); returns their offset.
 template <typename T>
 size_t put_descs(std::vector<char>& host, const std::vector<T>& v) {
   static_assert(sizeof(T) % 64 == 0, "descriptors keep 64-byte alignment");
-  const size_t at = host.size();
+  const size_t at = v.empty() ? host.size() : (host.size() + 127) / 128 * 128;
   host.resize(at + v.size() * sizeof(T));
   if (!v.empty()) std::memcpy(host.data() + at, v.data(), v.size() * sizeof(T));
   return at;

@@ -182,7 +182,7 @@ uint64_t p8_scratch_bytes(const P8Step& s, int rg);  // fp16 planes of the opera
 // per tile width computes every residue of each output tile and writes whole
 // entries (or planes), one launch adds the K-split partials.  p8_batch appends
 // the launches' descriptors (at most n p8_step_bytes()) to `host`, which the
-// caller copies to 64-byte aligned device memory (n groups p8_step_bytes()
+// caller copies to 128-byte aligned device memory (n groups p8_step_bytes()
 // bytes), and lays the steps' planes
 // and partials out side by side from `scratch` and `part`; arena_bytes bounds
 // every range the steps touch.  p8_run launches them for the primes of a pass;
