@@ -1537,7 +1537,7 @@ int fill_step(const P8Step& step, uint32_t rg, uint32_t prime_at, uint8_t* arena
 // (the tensor maps' alignment); returns their offset.
 template <typename T>
 size_t put_descs(std::vector<char>& host, const std::vector<T>& v) {
-  static_assert(sizeof(T) % 64 == 0, "descriptors keep 64-byte alignment");
+  static_assert(sizeof(T) % 64 == 0, "at most 64 bytes of padding before each array");
   const size_t at = v.empty() ? host.size() : (host.size() + 127) / 128 * 128;
   host.resize(at + v.size() * sizeof(T));
   if (!v.empty()) std::memcpy(host.data() + at, v.data(), v.size() * sizeof(T));
