@@ -251,6 +251,14 @@ template <int SHAPE>
 struct Blk {
   static constexpr int LA = SHAPE == 0 ? 6 : 5, LB = SHAPE == 2 ? 4 : 5, RA = SHAPE == 0 ? 2 : 1, RB = SHAPE == 2 ? 0 : 1;
 };
+// A thread's operand entries of one shared value: its N rows (or columns) of the
+// staged ones at s, `apart` entries from one to the next.
+template <int N, int RG>
+__host__ __device__ __forceinline__ void load_rows(const uint32_t* s, uint32_t apart, uint32_t (&v)[N][RG]) {
+#pragma unroll
+  for (int i = 0; i < N; i++) load_entry<RG>(s + i * apart * RG, v[i]);
+}
+
 struct BlockStep {
   uint64_t a_off, b_off, c_off;
   uint32_t wA[32], wB[32];  // output weight of row bit j / column bit j
@@ -362,10 +370,8 @@ __global__ void __launch_bounds__(256, 2) block_kernel(const BlockStep* __restri
 #pragma unroll 16
       for (uint32_t q = 0; q < kBlkK; q++) {
         uint32_t va[TA][RG], vb[TB][RG];
-#pragma unroll
-        for (int i = 0; i < 4; i++) load_entry<RG>(sa + (q * NA + i * (NA / TA)) * RG, va[i]);
-#pragma unroll
-        for (int j = 0; j < TB; j++) load_entry<RG>(sb + (q * NB + j * (NB / TB)) * RG, vb[j]);
+        load_rows(sa + q * NA * RG, NA / TA, va);
+        load_rows(sb + q * NB * RG, NB / TB, vb);
 #pragma unroll
         for (int i = 0; i < TA; i++)
 #pragma unroll
