@@ -14,7 +14,7 @@ namespace tnc_dev {
 // residue: u32 words for primes below 2^31, bytes for the 8-bit primes of the
 // TNC_PATH_TC_P8 arithmetic (four residues in one 32-bit word).
 template <int RG, typename W = uint32_t>
-__host__ __device__ __forceinline__ void load_entry(const W* src, uint32_t (&v)[RG]) {
+__device__ __forceinline__ void load_entry(const W* src, uint32_t (&v)[RG]) {
   if constexpr (sizeof(W) == 1) {
     if constexpr (RG == 4) {
       const uint32_t t = *reinterpret_cast<const uint32_t*>(src);

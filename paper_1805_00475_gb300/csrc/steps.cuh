@@ -252,11 +252,23 @@ struct Blk {
   static constexpr int LA = SHAPE == 0 ? 6 : 5, LB = SHAPE == 2 ? 4 : 5, RA = SHAPE == 0 ? 2 : 1, RB = SHAPE == 2 ? 0 : 1;
 };
 // A thread's operand entries of one shared value: its N rows (or columns) of the
-// staged ones at s, `apart` entries from one to the next.
+// staged ones at s, `apart` entries from one to the next.  (A host function too:
+// its bounds are checked there.)
 template <int N, int RG>
 __host__ __device__ __forceinline__ void load_rows(const uint32_t* s, uint32_t apart, uint32_t (&v)[N][RG]) {
 #pragma unroll
-  for (int i = 0; i < N; i++) load_entry<RG>(s + i * apart * RG, v[i]);
+  for (int i = 0; i < N; i++) {
+    const uint32_t* e = s + i * apart * RG;
+    if constexpr (RG == 4) {
+      const uint4 t = *reinterpret_cast<const uint4*>(e);
+      v[i][0] = t.x; v[i][1] = t.y; v[i][2] = t.z; v[i][3] = t.w;
+    } else if constexpr (RG == 2) {
+      const uint2 t = *reinterpret_cast<const uint2*>(e);
+      v[i][0] = t.x; v[i][1] = t.y;
+    } else {
+      v[i][0] = *e;
+    }
+  }
 }
 
 struct BlockStep {
