@@ -944,16 +944,16 @@ int solo_enqueue(const SoloPack& s, const SeqLayout& L, const Arith& a, char* ws
     args.tables = (const uint32_t*)(ws + s.off_tables);
     args.perms = (const uint8_t*)(ws + s.off_perms);
     args.order = (const uint32_t*)(ws + s.off_order);
-    args.n_forms = args.n_heavy = args.cluster_slots = 1;
+    args.n_forms = args.n_heavy = 1;
     args.results = (uint32_t*)(ws + L.off_results);
     args.garena = (uint32_t*)(ws + L.off_arena);
-    args.slot_entries = L.arena_entries;
     args.blob_cap = (uint32_t)s.blob_bytes;
     args.R = a.R;
     args.col = shape.col;
     const bool alone = L.passes.size() == 1 && shape.groups == 1;
     args.limbs = alone ? (uint32_t*)(ws + L.off_limbs) : nullptr;
     tnc_dev::SoloConsts sc{};
+    sc.heavy_entries = L.arena_entries;
     if (alone) sc.crt = a.crt;
     bool near30 = true;
     for (int g = 0; g < shape.groups; g++) {
@@ -1691,10 +1691,12 @@ struct tnc_batch_s {
   uint32_t n_heavy = 0;      // formulas contracted by whole clusters (the first of the order)
   uint64_t total_out = 0;
   std::vector<uint64_t> res_off;
-  uint64_t max_arena = 0;    // entries
+  uint64_t max_arena = 0;    // entries (of the light formulas, where clusters take the heavy ones)
   uint64_t max_blob = 0;     // bytes of the largest descriptor blob
   uint64_t slot_entries = 0;  // global arena slot of one CTA (entries)
-  uint32_t slots = 0;         // arena slots: CTAs (clusters, if every formula is heavy) any launch shape can have
+  uint32_t slots = 0;         // arena slots: CTAs any launch shape can have
+  uint64_t heavy_entries = 0;  // the same of a cluster, for the heavy formulas
+  uint32_t heavy_slots = 0, max_clusters = 0;
   // launch configuration (autotuned)
   int threads = 128;
   int cta_cap = 0;           // CTAs per SM cap (0: as many as fit)
@@ -1792,7 +1794,7 @@ int batch_configure(tnc_batch_t* b, int threads, size_t smem, int cap) {
       const int n_light = (int)(b->n_forms - b->n_heavy), cs = (int)kClusterCtas;
       int nc = std::min(clusters, std::max(1, sms * occ / cs));
       nc = std::min(nc, std::max((int)b->n_heavy, (n_light + cs - 1) / cs));
-      nc = std::min(nc, (int)b->slots / (n_light ? cs : 1));
+      nc = std::min(nc, (int)b->max_clusters);
       if (clusters <= 0 || nc <= 0) return set_error(TNC_ERR_TOO_LARGE, "no cluster of the batch kernel fits");
       grid.push_back(nc * cs);
       continue;
@@ -1819,6 +1821,7 @@ int batch_pack(tnc_batch_t* b) {
   std::vector<uint8_t> perms;
   b->res_off.assign(n, 0);
   uint64_t out = 0;
+  uint64_t heavy_arena = 0;
   b->max_arena = 8;
   b->max_blob = 16;
   // largest formulas first (longest-processing-time order)
@@ -1853,17 +1856,21 @@ int batch_pack(tnc_batch_t* b) {
     pack_leaves(lw, (uint32_t)tables.size(), leaves);
     tables.insert(tables.end(), lw.leaf_tables.begin(), lw.leaf_tables.end());
     perms.insert(perms.end(), lw.root_perm.begin(), lw.root_perm.end());
-    b->max_arena = std::max<uint64_t>(b->max_arena, lw.lvl_arena_entries);
+    uint64_t& most = threads[i] > 256 ? heavy_arena : b->max_arena;
+    most = std::max<uint64_t>(most, lw.lvl_arena_entries);
   }
   if (blobs.size() / 16 >= (1ull << 32)) return set_error(TNC_ERR_TOO_LARGE, "batch descriptors above 64 GiB");
   b->total_out = out;
   // global arena slots: one per CTA, at most 32 CTAs per SM in any launch
-  // shape (one per cluster where all formulas are heavy)
+  // shape, of the largest (light) formula's arena; before them one of the
+  // largest heavy formula's arena for each cluster that takes heavy formulas.
+  // All slots together are no more than formulas, or than CTAs.
+  const uint32_t max_ctas = (uint32_t)sm_count() * 32u;
   b->slot_entries = (b->max_arena + 7) / 8 * 8;
-  const uint32_t n_light = n - b->n_heavy;
-  uint64_t units = n;
-  if (b->n_heavy && n_light) units = (uint64_t)kClusterCtas * std::max(b->n_heavy, (n_light + kClusterCtas - 1) / kClusterCtas);
-  b->slots = (uint32_t)std::min<uint64_t>(units, (uint64_t)sm_count() * 32u);
+  b->heavy_entries = (heavy_arena + 7) / 8 * 8;
+  b->max_clusters = max_ctas / kClusterCtas;
+  b->heavy_slots = std::min(b->n_heavy, b->max_clusters);
+  b->slots = std::min(n - b->n_heavy, max_ctas - b->heavy_slots);
   const int rg_max = b->a.groups.rg.empty() ? 1 : b->a.groups.rg[0];
   // workspace layout
   size_t o = 0;
@@ -1871,6 +1878,7 @@ int batch_pack(tnc_batch_t* b) {
     off = o;
     o = align_up(o + bytes);
   };
+  static_assert(tnc_dev::kSlotCounter >= 16, "at most 16 residue groups, a counter each");
   sect(b->off_queue, 64 * sizeof(uint32_t));
   sect(b->off_forms, forms.size() * sizeof(BForm));
   sect(b->off_blobs, blobs.size());
@@ -1881,7 +1889,8 @@ int batch_pack(tnc_batch_t* b) {
   b->desc_bytes = o - b->off_forms;
   sect(b->off_results, out * b->a.R * sizeof(uint32_t));
   sect(b->off_limbs, out * b->a.crt.n_limbs * sizeof(uint32_t));
-  sect(b->off_arena, (size_t)b->slots * b->slot_entries * rg_max * sizeof(uint32_t));
+  sect(b->off_arena, ((size_t)b->slots * b->slot_entries + (size_t)b->heavy_slots * b->heavy_entries) * rg_max *
+                         sizeof(uint32_t));
   b->total = o;
   CUDA_TRY(cudaMallocHost((void**)&b->staging, std::max<size_t>(b->desc_bytes, 1)));
   std::memset(b->staging, 0, b->desc_bytes);
@@ -1923,7 +1932,7 @@ int batch_enqueue(tnc_batch_t* b, void* dev_ws, cudaStream_t st) {
     args.R = b->a.R;
     args.col = b->a.groups.col[gi];
     args.n_heavy = b->n_heavy;
-    args.cluster_slots = b->n_heavy == b->n_forms;
+    const tnc_dev::ClusterConsts cc{b->heavy_entries, b->heavy_slots * b->heavy_entries, b->slots};
     const ModGroup mg = b->a.group((int)gi);
     const int grid = b->grid[gi];
     const size_t smem = b->max_blob + b->smem_bytes;
@@ -1936,7 +1945,7 @@ int batch_enqueue(tnc_batch_t* b, void* dev_ws, cudaStream_t st) {
             &cl.cfg,
             mg.near30 ? tnc_dev::batch_kernel<RG, true, tnc_dev::kBatchClusters>
                       : tnc_dev::batch_kernel<RG, false, tnc_dev::kBatchClusters>,
-            args, mg, 0));
+            args, mg, cc));
         return TNC_OK;
       }
       if (mg.near30) tnc_dev::batch_kernel<RG, true><<<grid, threads, smem, st>>>(args, mg, 0);

@@ -364,6 +364,8 @@ struct BForm {
   uint32_t n_open, root_off, arena, dl_at;  // arena: entries this formula needs; dl_at: deltas
 };
 
+constexpr uint32_t kSlotCounter = 32;  // a launch's slot counter lies this far behind its work counter
+
 struct BatchArgs {
   const BForm* forms;
   const uint4* blobs;
@@ -372,17 +374,16 @@ struct BatchArgs {
   const uint8_t* perms;
   const uint32_t* order;  // queue slot -> formula (largest first)
   uint32_t n_forms;
-  uint32_t* queue;        // work counter, zeroed before the launch
+  uint32_t* queue;        // work counter, zeroed before the launch (with the slot counter)
   uint32_t* results;      // [entry][R]
   uint32_t* garena;       // global arenas, one slot per CTA, reused by every formula the CTA takes
-  uint64_t slot_entries;  // entries of a slot (the largest formula's arena)
+  uint64_t slot_entries;  // entries of a slot (the largest formula's arena; cluster launches: the largest light one's)
   uint32_t blob_cap;      // bytes of dynamic shared memory reserved for a blob
   uint32_t smem_cap;      // entries of dynamic shared memory available for an arena
   int R;
   int col;                // first residue column of this group
   // cluster launches only
   uint32_t n_heavy;       // the first n_heavy formulas of `order` are contracted by whole clusters
-  uint32_t cluster_slots; // arena slots are per cluster (there are no other formulas), not per CTA
   uint32_t* limbs;        // not NULL: this launch also runs the CRT (one formula, the last residue group)
 };
 
@@ -425,19 +426,27 @@ __device__ __forceinline__ uint32_t map_runs(uint32_t o, const uint16_t* runs, i
 // first n_heavy) are contracted first, each by all CTAs of one cluster: the
 // segments of a level are shared out over the warps of the cluster, the
 // barrier between levels is the cluster's, the tensors live in the slot of the
-// cluster's first CTA (formula t goes to cluster t, then back and forth).  A
+// cluster (formula t goes to cluster t, then back and forth).  A
 // formula that takes longer alone than the batch's average CTA would
 // otherwise be what the launch ends with.  Then every CTA takes formulas from
-// the queue as above.
+// the queue as above, into the next free one of the slots for light formulas
+// (no more of them than light formulas: a CTA that finds none is not needed).
 // kBatchSolo: one formula; cluster g contracts it for residue group g (its
 // primes in mg[g], its arena in slot g), a single group's cluster also runs the CRT.
 enum BatchMode { kBatchCtas, kBatchClusters, kBatchSolo };
-struct SoloConsts {
+// (Beside BatchArgs, not in it: the plain kernel's registers depend on the
+// layout of its parameters, 62 or, with spills, 48 for two residues.)
+struct ClusterConsts {
+  uint64_t heavy_entries;  // entries of a cluster's slot (the largest heavy formula's arena)
+  uint64_t light_off;      // entries of all clusters' slots; behind them
+  uint32_t light_slots;    // the slots for CTAs with a light formula
+};
+struct SoloConsts : ClusterConsts {
   CrtConsts crt;
   ModGroup mg[4];
 };
 template <int MODE>
-using BatchConsts = std::conditional_t<MODE == kBatchSolo, SoloConsts, int>;
+using BatchConsts = std::conditional_t<MODE == kBatchSolo, SoloConsts, std::conditional_t<MODE == kBatchClusters, ClusterConsts, int>>;
 template <int RG, bool N30 = false, int MODE = kBatchCtas>
 __global__ void __launch_bounds__(256, MODE == kBatchCtas ? 0 : (MODE == kBatchSolo ? 1 : (RG == 4 && !N30 ? 3 : 4)))
     batch_kernel(BatchArgs a, ModGroup mg, const __grid_constant__ BatchConsts<MODE> sc) {
@@ -452,7 +461,7 @@ __global__ void __launch_bounds__(256, MODE == kBatchCtas ? 0 : (MODE == kBatchS
     a.col += RG * (int)(blockIdx.x / cluster_ctas());
   }
   bool coop = CLUSTER;       // contracting the heavy formulas, cluster by cluster
-  uint32_t round = 0;
+  uint32_t round = 0, slot = 0;
   for (;;) {
     uint32_t t;
     if (CLUSTER && coop) {
@@ -462,6 +471,13 @@ __global__ void __launch_bounds__(256, MODE == kBatchCtas ? 0 : (MODE == kBatchS
       if (t >= a.n_heavy) {
         if (a.n_heavy == a.n_forms) break;
         coop = false;
+        if constexpr (MODE == kBatchClusters) {
+          if (threadIdx.x == 0) task = atomicAdd(a.queue + kSlotCounter, 1u);
+          __syncthreads();
+          slot = task;
+          __syncthreads();  // (the queue's next value goes to the same place)
+          if (slot >= sc.light_slots) break;
+        }
         continue;
       }
     } else {
@@ -481,10 +497,12 @@ __global__ void __launch_bounds__(256, MODE == kBatchCtas ? 0 : (MODE == kBatchS
     const BForm f = a.forms[a.order[t]];
     for (uint32_t i = threadIdx.x; i < f.blob_n; i += blockDim.x) blob[i] = a.blobs[f.blob + i];
     uint32_t* arena = a.garena;
-    if (CLUSTER && coop)
-      arena += (uint64_t)(a.cluster_slots ? blockIdx.x / cluster_ctas() : blockIdx.x - cluster_cta()) * a.slot_entries * RG;
-    else
+    if constexpr (CLUSTER) {
+      if (coop) arena += (uint64_t)(blockIdx.x / cluster_ctas()) * sc.heavy_entries * RG;
+      else arena = f.arena <= a.smem_cap ? sarena : arena + (sc.light_off + slot * a.slot_entries) * RG;
+    } else {
       arena = f.arena <= a.smem_cap ? sarena : arena + (uint64_t)blockIdx.x * a.slot_entries * RG;
+    }
     auto barrier = [&] {
       if (CLUSTER && coop) cluster_barrier();
       else __syncthreads();

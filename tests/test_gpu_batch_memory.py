@@ -1,0 +1,41 @@
+"""Device memory of a batch: no more arena slots than formulas (or resident
+CTAs), also where clusters of CTAs contract the heavy formulas, and the light
+ones share what slots there are."""
+import pytest
+
+from paper_1805_00475_gb300 import build as tnc_build
+from paper_1805_00475_gb300 import instances as I
+from paper_1805_00475_gb300 import tnc
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    tnc_build.build()
+
+
+@pytest.mark.parametrize("R", [1, 4])
+@pytest.mark.parametrize("sizes", [
+    (76,) * 19 + (30,),        # fewer light formulas than CTAs: most CTAs find no slot
+    (76,) * 3 + (30,) * 5,
+    (76, 30),
+    (72,) + (24,) * 700,       # more light formulas than CTAs
+    (70,) * 90 + (30,) * 90,   # more heavy formulas than clusters
+])
+def test_batch_memory_is_a_slot_per_formula(sizes, R):
+    import torch
+    plans = {n: tnc.plan_formula(I.cubic_vertex_cover(n, n), heuristic="gn") for n in set(sizes)}
+    want = {n: tnc.contract_noalloc(p, n_residues=R) for n, p in plans.items()}
+    b = tnc.Batch([plans[n] for n in sizes], n_residues=R)
+    largest = max(p.stats.batch_arena_entries for p in plans.values()) + 7
+    limbs = (31 * R + 31) // 32
+    rest = b.info()[0] + len(sizes) * 4 * (R + limbs) + 4096  # descriptors, results; sections aligned
+    assert b.workspace_bytes() <= rest + len(sizes) * largest * 4 * R
+    ws = torch.empty(b.workspace_bytes(), dtype=torch.uint8, device="cuda")
+    b.upload(ws)
+    for shape in ((256, 0, 0), (64, 0, 0), (128, 16384, 1)):
+        b.set_launch(*shape)
+        b.launch(ws)
+        for n, r in zip(sizes, b.download(ws)):
+            assert r.residues.tolist() == want[n].residues.tolist() and r.counts == want[n].counts, (n, shape)
