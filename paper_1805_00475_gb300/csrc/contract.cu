@@ -1843,7 +1843,14 @@ int batch_pack(tnc_batch_t* b) {
     const tnc_plan_t* p = b->plans[i];
     const Lowered& lw = p->low;
     BForm& f = forms[i];
-    const int rc = pack_form(p, threads[i], blob, f);
+    int rc = pack_form(p, threads[i], blob, f);
+    if (threads[i] > 256 && (rc || blob.size() > kSmemMax - 256)) {
+      // (a cluster's finer segments take up to a few KiB more of descriptors: with
+      // one CTA's, which a cluster shares out just as well, the formula fits as a
+      // light one does; 256: a CTA's static shared memory and more)
+      clear_error();
+      rc = pack_form(p, 256, blob, f);
+    }
     if (rc) return rc;
     f.blob = (uint32_t)(blobs.size() / 16);
     blobs.insert(blobs.end(), blob.begin(), blob.end());
