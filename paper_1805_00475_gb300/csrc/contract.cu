@@ -1718,16 +1718,18 @@ constexpr size_t kSmemMax = 227 * 1024;
 
 // Batch formulas contracted by whole clusters: those with more than
 // kHeavyShare of the batch's work (multiply-adds and entries) per resident CTA
-// (four per SM; per formula where there are fewer), and more than kHeavyMin;
-// none unless the largest exceeds kHeavyTop, below which a cluster's barriers
-// cost what its CTAs gain.  Measured on 2048 cubic VC formulas with n = 60
-// (4 residues; three seeds): no clusters 498-709 us, shares of 0.5 / 0.7 / 1 /
-// 1.4 / 2: 430 / 365 / 328 / 370 / 520 us; on 700 with n = 64: 850, 416, 331,
-// 280 us for none / 0.7 / 1 / 1.4; on 777 uneven 1-in-3 formulas (2 residues):
-// 1330-3130 us without, 226-545 us with.  20 formulas with n = 48, all below
-// kHeavyTop: 28-41 us without, 40-48 us with.
+// (four per SM; per formula where there are fewer), and more than kHeavyLevel
+// per tree level; none unless the largest exceeds kHeavyTop.  Measured on 2048
+// cubic VC formulas with n = 60 (4 residues; three seeds): no clusters 498-709
+// us, shares of 0.5 / 0.7 / 1 / 1.4 / 2: 430 / 365 / 328 / 370 / 520 us; on 700
+// with n = 64: 850, 416, 331, 280 us for none / 0.7 / 1 / 1.4; on 777 uneven
+// 1-in-3 formulas (2 residues): 1330-3130 us without, 226-545 us with.
+// kHeavyLevel: a cluster's barrier per level costs about 0.7 us more than a
+// CTA's.  Formulas alone, on a cluster against on one CTA (70 of them, 4
+// residues): 0.7-0.9 of the speed below 4000 per level, 0.9-1.0 up to 5500,
+// 1.0-1.2 up to 10000, 1.3-1.6 at 20000, 2-3 at 50000.
 constexpr uint32_t kClusterCtas = 8;
-constexpr double kHeavyShare = 1.2, kHeavyMin = 16384.0, kHeavyTop = 131072.0;
+constexpr double kHeavyShare = 1.2, kHeavyLevel = 5500.0, kHeavyTop = 131072.0;
 
 // CTAs of batch_kernel<RG, N30, MODE> per SM for (threads, dynamic shared memory),
 // capped at `cap` (0: no cap).  The L1 / shared-memory split is then set to
@@ -1793,7 +1795,7 @@ int batch_configure(tnc_batch_t* b, int threads, size_t smem, int cap) {
     if (b->n_heavy) {  // clusters resident at once, as many as there is work for
       const int n_light = (int)(b->n_forms - b->n_heavy), cs = (int)kClusterCtas;
       int nc = std::min(clusters, std::max(1, sms * occ / cs));
-      nc = std::min(nc, std::max((int)b->n_heavy, (n_light + cs - 1) / cs));
+      nc = std::min(nc, (int)b->n_heavy + (n_light + cs - 1) / cs);  // (the light ones wait for no heavy one)
       nc = std::min(nc, (int)b->max_clusters);
       if (clusters <= 0 || nc <= 0) return set_error(TNC_ERR_TOO_LARGE, "no cluster of the batch kernel fits");
       grid.push_back(nc * cs);
@@ -1834,9 +1836,12 @@ int batch_pack(tnc_batch_t* b) {
   // heavy formulas, contracted by whole clusters (batch_kernel)
   const uint32_t ctas = 4u * (uint32_t)sm_count();  // resident at once
   const double share = n <= ctas / kClusterCtas / 2 ? 0.0 : total / std::min(n, ctas);
-  while (cost(order[0]) > kHeavyTop && b->n_heavy < n &&
-         cost(order[b->n_heavy]) > std::max(kHeavyShare * share, kHeavyMin))
-    b->n_heavy++;
+  if (cost(order[0]) > kHeavyTop) {
+    const auto light = std::stable_partition(order.begin(), order.end(), [&](uint32_t i) {
+      return cost(i) > std::max(kHeavyShare * share, kHeavyLevel * (double)(b->plans[i]->low.lvl_start.size() - 1));
+    });
+    b->n_heavy = (uint32_t)(light - order.begin());
+  }
   std::vector<uint32_t> threads(n, 256);
   for (uint32_t i = 0; i < b->n_heavy; i++) threads[order[i]] = 256 * kClusterCtas;
   for (uint32_t i = 0; i < n; i++) {

@@ -39,3 +39,19 @@ def test_batch_memory_is_a_slot_per_formula(sizes, R):
         b.launch(ws)
         for n, r in zip(sizes, b.download(ws)):
             assert r.residues.tolist() == want[n].residues.tolist() and r.counts == want[n].counts, (n, shape)
+
+
+def test_deep_formulas_beside_heavy_ones():
+    """Formulas of many levels are light even where smaller, flatter ones are heavy."""
+    import torch
+    forms = [I.cubic_vertex_cover(72, 72), I.one_in_three(70, 43, 25), I.cubic_vertex_cover(50, 14), I.cubic_vertex_cover(24, 0)]
+    plans = [tnc.plan_formula(f, heuristic="gn", rank_cap=24) for f in forms]
+    work = [p.stats.total_macs + p.stats.total_entries for p in plans]
+    per_level = [w / p.stats.depth for w, p in zip(work, plans)]
+    assert work[1] > work[2] and per_level[1] < 5500 < per_level[2]
+    b = tnc.Batch(plans, n_residues=2)
+    ws = torch.empty(b.workspace_bytes(), dtype=torch.uint8, device="cuda")
+    b.upload(ws)
+    b.launch(ws)
+    for p, r in zip(plans, b.download(ws)):
+        assert r.residues.tolist() == tnc.contract_noalloc(p, n_residues=2).residues.tolist()
