@@ -17,9 +17,9 @@ def built():
 
 @pytest.mark.parametrize("R", [1, 4])
 @pytest.mark.parametrize("sizes", [
-    (76,) * 19 + (30,),        # fewer light formulas than CTAs: most CTAs find no slot
-    (76,) * 3 + (30,) * 5,
-    (76, 30),
+    (72,) * 19 + (30,),        # fewer light formulas than CTAs: most CTAs find no slot
+    (72,) * 3 + (30,) * 5,
+    (72, 30),
     (72,) + (24,) * 700,       # more light formulas than CTAs
     (70,) * 90 + (30,) * 90,   # more heavy formulas than clusters
 ])
