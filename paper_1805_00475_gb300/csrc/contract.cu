@@ -82,14 +82,12 @@ struct Groups {
   std::vector<int> rg, col;
 };
 
-// Three residues left over are a group of four with one that nobody asked for:
-// a batch launch with four residues takes less than one with two and one with one
-// (217 cubic VC formulas with n = 48, 3 residues: 85 -> 63 us).
-Groups split_groups(int R) {
+// fill: three residues left over are a group of four with one that nobody asked for.
+Groups split_groups(int R, bool fill) {
   Groups g;
   int c = 0;
   for (int s : {4, 2, 1})
-    while (R - c >= s || (s == 4 && R - c == 3)) {
+    while (R - c >= s || (fill && s == 4 && R - c == 3)) {
       g.rg.push_back(s);
       g.col.push_back(c);
       c += s;
@@ -148,7 +146,7 @@ int make_arith(const tnc_contract_opts* o, Arith& a) {
   }
   // limbs of the CRT value: enough for prod p < 2^(32 n_limbs)
   a.crt.n_limbs = p8 ? (int)std::floor(a.log2_prod / 32.0) + 1 : (31 * a.R + 31) / 32;
-  a.groups = split_groups(a.R);
+  a.groups = split_groups(a.R, false);
   return TNC_OK;
 }
 
@@ -1731,6 +1729,15 @@ constexpr size_t kSmemMax = 227 * 1024;
 constexpr uint32_t kClusterCtas = 8;
 constexpr double kHeavyShare = 1.2, kHeavyLevel = 5500.0, kHeavyTop = 131072.0;
 
+// Three residues left over are filled up to four where the largest formula has at
+// most kFillTop multiply-adds and entries: one launch takes less than one with
+// two residues and one with one (3 residues, cubic VC and uneven 1-in-3 formulas,
+// 5 to 1500 of them: 1.04-1.5 times the speed with the largest at 3.8e6 or less;
+// with 1e7, where its cluster's products count, 0.82-0.97).  With 3 residues
+// the arenas double: only up to kFillArena bytes of them.
+constexpr double kFillTop = 5e6;
+constexpr uint64_t kFillArena = 1ull << 30;
+
 // CTAs of batch_kernel<RG, N30, MODE> per SM for (threads, dynamic shared memory),
 // capped at `cap` (0: no cap).  The L1 / shared-memory split is then set to
 // the smallest shared-memory share that holds those CTAs, so that the rest of
@@ -1883,6 +1890,8 @@ int batch_pack(tnc_batch_t* b) {
   b->max_clusters = max_ctas / kClusterCtas;
   b->heavy_slots = std::min(b->n_heavy, b->max_clusters);
   b->slots = std::min(n - b->n_heavy, max_ctas - b->heavy_slots);
+  const uint64_t arena = (uint64_t)b->slots * b->slot_entries + (uint64_t)b->heavy_slots * b->heavy_entries;
+  b->a.groups = split_groups(b->a.R, cost(order[0]) <= kFillTop && (b->a.R > 4 || arena * 16 <= kFillArena));
   const int rg_max = b->a.groups.rg.empty() ? 1 : b->a.groups.rg[0];
   // workspace layout
   size_t o = 0;
@@ -1901,8 +1910,7 @@ int batch_pack(tnc_batch_t* b) {
   b->desc_bytes = o - b->off_forms;
   sect(b->off_results, out * b->a.R * sizeof(uint32_t));
   sect(b->off_limbs, out * b->a.crt.n_limbs * sizeof(uint32_t));
-  sect(b->off_arena, ((size_t)b->slots * b->slot_entries + (size_t)b->heavy_slots * b->heavy_entries) * rg_max *
-                         sizeof(uint32_t));
+  sect(b->off_arena, (size_t)arena * rg_max * sizeof(uint32_t));
   b->total = o;
   CUDA_TRY(cudaMallocHost((void**)&b->staging, std::max<size_t>(b->desc_bytes, 1)));
   std::memset(b->staging, 0, b->desc_bytes);

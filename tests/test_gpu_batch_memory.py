@@ -55,3 +55,15 @@ def test_deep_formulas_beside_heavy_ones():
     b.launch(ws)
     for p, r in zip(plans, b.download(ws)):
         assert r.residues.tolist() == tnc.contract_noalloc(p, n_residues=2).residues.tolist()
+
+
+def test_three_residues_take_four_only_where_that_is_small():
+    """Launches (residue groups and the CRT) and device memory of 3 residues."""
+    small = tnc.plan_formula(I.cubic_vertex_cover(72, 72), heuristic="gn")
+    large = tnc.plan_formula(I.cubic_vertex_cover(110, 0), heuristic="best", rank_cap=24)
+    assert tnc.Batch([small], n_residues=3).info()[3] == 2       # one group of four
+    assert tnc.Batch([small, large], n_residues=3).info()[3] == 3  # two and one
+    b = tnc.Batch([small] * 6000, n_residues=3)  # arenas beyond 1 GiB with four
+    assert b.info()[3] == 3
+    rest = b.info()[0] + 6000 * 4 * (3 + 3) + 4096
+    assert b.workspace_bytes() <= rest + 6000 * (small.stats.batch_arena_entries + 7) * 4 * 2
