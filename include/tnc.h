@@ -559,6 +559,8 @@ int tnc_probe_modmac(void* cuda_stream, int32_t iters, double* macs_per_s);
                                 -> TNC_ERR_CUDA, nothing enqueued                  */
 #define TNC_INJECT_TIMEOUT 4 /* tnc_contract / _sliced: the device status reads as a
                                 timed-out wait -> TNC_ERR_TIMEOUT                  */
+#define TNC_INJECT_CLUSTER 5 /* tnc_contract / tnc_batch_create: no thread-block cluster of
+                                the size asked for can be resident -> smaller ones or none */
 int tnc_inject_failure(int32_t kind, int32_t after);
 
 /* ---- allocation-free variant (the paper has no counterpart) --------------

@@ -13,6 +13,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -879,6 +880,7 @@ void pack_leaves(const Lowered& lw, uint32_t table0, std::vector<BLeaf>& leaves)
 // 328 -> 522), on clusters of 16 CTAs from kSoloWide on (2^19.7: 158 us
 // against 180 on 8; 2^15: no difference).
 constexpr double kSoloMax = 4e6, kSoloWide = 3e4;
+constexpr int kSoloSmem = 160 * 1024;  // most descriptor bytes
 
 }  // namespace
 
@@ -916,7 +918,7 @@ void make_solo(const tnc_plan_t* p, SoloPack& s) {
   s.off_perms = blob_put(s.bytes, p->low.root_perm.data(), p->low.root_perm.size());
   s.off_order = blob_put(s.bytes, &first, sizeof(first));
   for (const StepDesc& d : p->low.lvl_steps) s.long_sums += splitk_log(d) > 0;
-  s.ok = blob.size() <= 160 * 1024;
+  s.ok = blob.size() <= (size_t)kSoloSmem;
 }
 
 // The CRT of n entries: a warp each while that is at most four warps per
@@ -929,12 +931,87 @@ void launch_crt(const uint32_t* residues, uint64_t n, const CrtConsts& cc, uint3
   g_launches.crt++;
 }
 
+// The kernel's limits for clusters of `ctas` CTAs with `smem` bytes of dynamic shared memory each.
+template <typename K>
+int cluster_limits(K kernel, uint32_t ctas, size_t smem) {
+  if (smem > 48 * 1024 - 64) CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSoloSmem));
+  if (ctas > 8) CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  return TNC_OK;
+}
+
+// Can a cluster of `ctas` CTAs of this kernel be resident?  Asked once per kernel,
+// cluster size and device, for the most shared memory.
+template <int RG, bool N30>
+int solo_fits(uint32_t ctas, bool* fits) {
+  static std::atomic<int> known[2][64];  // 0: not asked yet, 1: yes, -1: no
+  const auto kernel = tnc_dev::batch_kernel<RG, N30, tnc_dev::kBatchSolo>;
+  int dev = 0;
+  CUDA_TRY(cudaGetDevice(&dev));
+  std::atomic<int>* at = dev >= 0 && dev < 64 ? &known[ctas > 8][dev] : nullptr;
+  int k = at ? at->load(std::memory_order_relaxed) : 0;
+  if (!k) {
+    if (int rc = cluster_limits(kernel, ctas, kSoloSmem)) return rc;
+    const ClusterLaunch cl(ctas, 256, kSoloSmem, nullptr, ctas);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cl.cfg) != cudaSuccess) {
+      cudaGetLastError();  // (a size that the device does not have)
+      n = 0;
+    }
+    k = n > 0 ? 1 : -1;
+    if (at) at->store(k, std::memory_order_relaxed);
+  }
+  *fits = k > 0;
+  return TNC_OK;
+}
+
+// A pass of the one-launch contraction: its primes by residue group.
+struct SoloPass {
+  tnc_dev::SoloConsts sc{};
+  bool near30 = true;
+  SoloPass(const PassShape& shape, const Arith& a) {
+    for (int g = 0; g < shape.groups; g++) {
+      uint32_t gp[4];
+      for (int r = 0; r < 4; r++) {
+        const int i = shape.col + g * shape.rg + r;
+        gp[r] = a.primes[r < shape.rg && i < a.R ? i : shape.col + g * shape.rg];
+      }
+      sc.mg[g] = tnc_dev::make_mod_group(gp);
+      near30 = near30 && sc.mg[g].near30;
+    }
+  }
+};
+
+// CTAs of the clusters that contract the formula: as many as it was packed for, 8 where
+// no such cluster can be resident (a partition of the GPU, other work on it),
+// 0 where none of 8 can either: the formula then goes level by level.
+int solo_ctas(const SoloPack& s, const SeqLayout& L, const std::vector<SoloPass>& passes, uint32_t* ctas) {
+  *ctas = 0;
+  for (uint32_t c = s.ctas; c >= 8; c -= 8) {  // (16, 8)
+    bool all = !inject_hit(TNC_INJECT_CLUSTER);
+    for (size_t i = 0; i < passes.size() && all; i++) {
+      const int rc = dispatch_rg(L.passes[i].rg, [&](auto rgc) -> int {
+        constexpr int RG = decltype(rgc)::value;
+        return passes[i].near30 ? solo_fits<RG, true>(c, &all) : solo_fits<RG, false>(c, &all);
+      });
+      if (rc) return rc;
+    }
+    if (all) {
+      *ctas = c;
+      return TNC_OK;
+    }
+  }
+  return TNC_OK;
+}
+
 // Enqueues the one-launch contraction (descriptors up, a launch per residue
 // group); results and limbs are left in their workspace sections.
-int solo_enqueue(const SoloPack& s, const SeqLayout& L, const Arith& a, char* ws, cudaStream_t st) {
+int solo_enqueue(const SoloPack& s, uint32_t ctas, std::vector<SoloPass>& passes, const SeqLayout& L, const Arith& a,
+                 char* ws, cudaStream_t st) {
   CUDA_TRY(cudaMemcpyAsync(ws, s.bytes.data(), s.bytes.size(), cudaMemcpyHostToDevice, st));
   g_h2d_bytes += s.bytes.size();
-  for (const PassShape& shape : L.passes) {
+  for (size_t i = 0; i < passes.size(); i++) {
+    const PassShape& shape = L.passes[i];
+    tnc_dev::SoloConsts& sc = passes[i].sc;
     tnc_dev::BatchArgs args{};
     args.forms = (const BForm*)ws;
     args.blobs = (const uint4*)(ws + s.off_blob);
@@ -950,27 +1027,14 @@ int solo_enqueue(const SoloPack& s, const SeqLayout& L, const Arith& a, char* ws
     args.col = shape.col;
     const bool alone = L.passes.size() == 1 && shape.groups == 1;
     args.limbs = alone ? (uint32_t*)(ws + L.off_limbs) : nullptr;
-    tnc_dev::SoloConsts sc{};
     sc.heavy_entries = L.arena_entries;
     if (alone) sc.crt = a.crt;
-    bool near30 = true;
-    for (int g = 0; g < shape.groups; g++) {
-      uint32_t gp[4];
-      for (int r = 0; r < 4; r++) {
-        const int i = shape.col + g * shape.rg + r;
-        gp[r] = a.primes[r < shape.rg && i < a.R ? i : shape.col + g * shape.rg];
-      }
-      sc.mg[g] = tnc_dev::make_mod_group(gp);
-      near30 = near30 && sc.mg[g].near30;
-    }
     int rc = dispatch_rg(shape.rg, [&](auto rgc) -> int {
       constexpr int RG = decltype(rgc)::value;
-      auto k = near30 ? tnc_dev::batch_kernel<RG, true, tnc_dev::kBatchSolo>
-                      : tnc_dev::batch_kernel<RG, false, tnc_dev::kBatchSolo>;
-      if (s.blob_bytes > 48 * 1024 - 64)
-        CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
-      if (s.ctas > 8) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-      const ClusterLaunch cl(s.ctas * (unsigned)shape.groups, 256, s.blob_bytes, st, s.ctas);
+      const auto k = passes[i].near30 ? tnc_dev::batch_kernel<RG, true, tnc_dev::kBatchSolo>
+                                      : tnc_dev::batch_kernel<RG, false, tnc_dev::kBatchSolo>;
+      if (int rc2 = cluster_limits(k, ctas, s.blob_bytes)) return rc2;
+      const ClusterLaunch cl(ctas * (unsigned)shape.groups, 256, s.blob_bytes, st, ctas);
       CUDA_TRY(cudaLaunchKernelEx(&cl.cfg, k, args, sc.mg[0], sc));
       return TNC_OK;
     });
@@ -1101,8 +1165,15 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
       work[0]->solo = std::move(s);
     });
     const SoloPack& s = *work[0]->solo;
+    uint32_t ctas = 0;
+    std::vector<SoloPass> passes;
     if (s.ok && s.bytes.size() <= L.off_results) {  // (the descriptor sections and scratch before the results)
-      rc = solo_enqueue(s, L, a, ws, st);
+      passes.reserve(L.passes.size());
+      for (const PassShape& shape : L.passes) passes.emplace_back(shape, a);
+      if ((rc = solo_ctas(s, L, passes, &ctas))) return rc;
+    }
+    if (ctas) {
+      rc = solo_enqueue(s, ctas, passes, L, a, ws, st);
       if (rc) return rc;
       std::vector<uint32_t> h((L.off_limbs - L.off_results) / 4 + L.n_out * a.crt.n_limbs);
       CUDA_TRY(cudaMemcpyAsync(h.data(), ws + L.off_results, h.size() * 4, cudaMemcpyDeviceToHost, st));
@@ -1821,6 +1892,27 @@ int batch_configure(tnc_batch_t* b, int threads, size_t smem, int cap) {
   return TNC_OK;
 }
 
+// Can clusters be resident on the device at all, for every residue group's kernel and
+// any launch shape (one CTA per SM)?  Otherwise every formula is a light one.
+bool clusters_fit(tnc_batch_t* b) {
+  if (inject_hit(TNC_INJECT_CLUSTER)) return false;
+  for (size_t gi = 0; gi < b->a.groups.rg.size(); gi++) {
+    int occ = 0, clusters = 0;
+    const bool n30 = b->a.group((int)gi).near30 != 0;
+    const int rc = dispatch_rg(b->a.groups.rg[gi], [&](auto rgc) -> int {
+      constexpr int RG = decltype(rgc)::value;
+      return n30 ? occupancy<RG, true, tnc_dev::kBatchClusters>(256, kSmemMax - 256, 0, &occ, &clusters)
+                 : occupancy<RG, false, tnc_dev::kBatchClusters>(256, kSmemMax - 256, 0, &occ, &clusters);
+    });
+    if (rc || clusters <= 0) {
+      clear_error();
+      cudaGetLastError();
+      return false;
+    }
+  }
+  return true;
+}
+
 int batch_pack(tnc_batch_t* b) {
   const uint32_t n = b->n_forms;
   std::vector<BForm> forms(n);
@@ -1843,7 +1935,7 @@ int batch_pack(tnc_batch_t* b) {
   // heavy formulas, contracted by whole clusters (batch_kernel)
   const uint32_t ctas = 4u * (uint32_t)sm_count();  // resident at once
   const double share = n <= ctas / kClusterCtas / 2 ? 0.0 : total / std::min(n, ctas);
-  if (cost(order[0]) > kHeavyTop) {
+  if (cost(order[0]) > kHeavyTop && clusters_fit(b)) {
     const auto light = std::stable_partition(order.begin(), order.end(), [&](uint32_t i) {
       return cost(i) > std::max(kHeavyShare * share, kHeavyLevel * (double)(b->plans[i]->low.lvl_start.size() - 1));
     });

@@ -33,7 +33,7 @@ bool inject_hit(int kind) {
 
 extern "C" int tnc_inject_failure(int32_t kind, int32_t after) {
   tnc::clear_error();
-  if (kind < TNC_INJECT_NONE || kind > TNC_INJECT_TIMEOUT || after < 0)
+  if (kind < TNC_INJECT_NONE || kind > TNC_INJECT_CLUSTER || after < 0)
     return tnc::set_error(TNC_ERR_INVALID, "unknown injection kind or negative count");
   std::lock_guard<std::mutex> lock(g_mu);
   g_kind = kind;

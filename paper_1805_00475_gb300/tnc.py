@@ -27,7 +27,7 @@ ERRORS = {-1: "TNC_ERR_INVALID", -2: "TNC_ERR_TOO_LARGE", -3: "TNC_ERR_CUDA", -4
 HEURISTICS = {"greedy": 0, "bisect": 1, "gn": 2, "explicit": 3, "best": 4, "portfolio": 5, "coarsen": 6}
 PATHS = {"int64": 0, "tc": 1, "tc_p8": 2}
 TNC_MAYBE_WRAPPED = 1
-INJECT = {"none": 0, "nomem": 1, "plan": 2, "launch": 3, "timeout": 4}
+INJECT = {"none": 0, "nomem": 1, "plan": 2, "launch": 3, "timeout": 4, "cluster": 5}
 
 # every symbol include/tnc.h declares
 EXPORTS = [
@@ -783,7 +783,7 @@ def _dp(x):
 
 def inject_failure(kind: str, after: int = 0):
     """tnc_inject_failure: arm one host-side failure ("nomem", "plan",
-    "launch", "timeout"; "none" disarms)."""
+    "launch", "timeout", "cluster"; "none" disarms)."""
     _check(lib().tnc_inject_failure(INJECT[kind], after))
 
 
