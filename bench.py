@@ -582,7 +582,7 @@ def c4_block(args, dev, steps, warmup, compare):
     R8 = len(p8_primes)
     ws_bytes = max(tnc.workspace_bytes(p, R8, "tc_p8") for p in plans)
     if compare:
-        ws_bytes = max(ws_bytes, max(tnc.workspace_bytes(p, Rc) for p in plans))
+        ws_bytes = max(ws_bytes, max(tnc.workspace_bytes(p, Rc, c) for p in plans for c in ("int64", "tc")))
     ws = torch.empty(ws_bytes, dtype=torch.uint8, device=dev)
     stream = torch.cuda.Stream(device=dev)
     macs = sum(p.stats.total_macs for p in plans)

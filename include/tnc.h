@@ -251,22 +251,33 @@ int tnc_plan_steps(const tnc_plan_t* plan, int32_t* left, int32_t* right, int32_
 void tnc_free_plan(tnc_plan_t* plan);
 
 /* ---- single formula (Sec. 2.1 contraction; one launch per step) --------- */
-/* Device workspace needed by tnc_contract for R residues on TNC_PATH_INT64 or
- * TNC_PATH_TC. */
+/* Device workspace for tnc_contract with R residues, whether on TNC_PATH_INT64 or
+ * on TNC_PATH_TC (tnc_workspace_bytes_opts: one path's). */
 size_t tnc_workspace_bytes(const tnc_plan_t* plan, int32_t n_residues);
 /* Device workspace needed by tnc_contract with these options (any path; adds
  * TNC_PATH_TC_P8's packed fp16 operands and K-split partials); 0 if the options
  * are invalid.  It holds the residue groups side by side as far as that is
- * faster; the calls also run in a workspace that only holds them one at a time. */
+ * faster (up to 12 GiB more than the least that works); the calls also run in
+ * smaller workspaces, one residue group or one residue at a time, and TNC_PATH_TC
+ * in any that TNC_PATH_INT64 runs in (dense steps on the CUDA cores where their
+ * operands do not fit otherwise). */
 size_t tnc_workspace_bytes_opts(const tnc_plan_t* plan, const tnc_contract_opts* opts);
+/* For callers short of device memory: the largest workspace of less than `below`
+ * bytes that a call with these options uses in full, 0 if none that small works.
+ * sliced: for tnc_contract_sliced; else for tnc_contract (n = 1) and
+ * tnc_contract_many, whose groups are then single plans.  Calling it with its own
+ * result until that is 0 gives the least that works. */
+size_t tnc_workspace_bytes_below(const tnc_plan_t* const* plans, int32_t n, const tnc_contract_opts* opts,
+                                 int32_t sliced, size_t below);
 /* Sliced contraction (bond slicing: fixing s variables of a formula splits its
  * count into 2^s counts of smaller networks, each with at most the original
  * ranks; the paper leaves memory as the bottleneck of its method, Sec. 4).
  * plans[i] are the networks of the slices (same open variables); the result
  * is the sum of their counts, exact: each slice's residues are added on the
- * device modulo the primes, then one CRT.  As many slices at a time as the
- * workspace holds beyond tnc_workspace_bytes_sliced's minimum run with their
- * tree levels merged (as tnc_contract_many).  `flags` certifies the sum (the sum
+ * device modulo the primes, then one CRT.  tnc_workspace_bytes_sliced holds the
+ * largest slice (tnc_workspace_bytes_below: smaller ones that work); as many
+ * slices at a time as the workspace holds run with their tree levels merged (as
+ * tnc_contract_many).  `flags` certifies the sum (the sum
  * of the slices' bounds).  dev_ws: tnc_workspace_bytes_sliced bytes, 256-byte
  * aligned.  Synchronises `cuda_stream`. */
 size_t tnc_workspace_bytes_sliced(const tnc_plan_t* const* plans, int32_t n, const tnc_contract_opts* opts);
@@ -279,7 +290,7 @@ int tnc_contract_sliced(const tnc_plan_t* const* plans, int32_t n, const tnc_con
  * the workspace holds (each plan alone must fit: TNC_ERR_BUFFER otherwise).
  * Any path; outs: n counts, as tnc_contract would give them one by one.
  * tnc_workspace_bytes_many gives the bytes that hold groups of `group`
- * consecutive plans (group = 1: the least that works).  dev_ws 256-byte
+ * consecutive plans (less works too: tnc_workspace_bytes_below).  dev_ws 256-byte
  * aligned; synchronises `cuda_stream`. */
 size_t tnc_workspace_bytes_many(const tnc_plan_t* const* plans, int32_t n, const tnc_contract_opts* opts,
                                 int32_t group);
@@ -583,8 +594,10 @@ int tnc_inject_failure(int32_t kind, int32_t after);
  *     streams, other host threads, same device) race and corrupt each other's
  *     results.  Serialise them.  Nothing in the array needs to start zeroed,
  *     so the previous call's contents do no harm.
- *   - A plan whose scratch (tnc_workspace_bytes for the same R) exceeds the
- *     array fails with TNC_ERR_TOO_LARGE and a message giving both sizes.
+ *   - A plan whose scratch exceeds the array fails with TNC_ERR_TOO_LARGE and a
+ *     message giving both sizes.  That scratch holds one residue group at a time
+ *     (4 residues of every entry of the plan's arena, and the descriptors); it is
+ *     never more than tnc_workspace_bytes for the same R, and may be less.
  *   - Synchronises `cuda_stream` before returning. */
 #define TNC_NOALLOC_SCRATCH_BYTES (32u << 20)
 int tnc_contract_noalloc(const tnc_plan_t* plan, const tnc_contract_opts* opts, void* cuda_stream,

@@ -187,6 +187,7 @@ struct PassShape {
 struct SeqLayout {
   size_t off_leaves, off_tables, off_steps, off_small, off_tc, off_err, off_part, off_results, off_limbs, off_p8,
       off_arena, total;
+  int path;        // of the choice laid out
   uint64_t n_out;  // result entries of the whole group
   uint64_t part_bytes, p8_bytes;  // the sections' sizes
   std::vector<PassShape> passes;
@@ -517,11 +518,33 @@ Foot foot_of(const tnc_plan_t* p, int path) {
   return f;
 }
 
-// Offsets of the workspace sections for the group footprint f.  wide: with the
-// residue groups side by side as far as kMergeArena allows; else one group at a
-// time (the least that works).
-SeqLayout layout_of(const Foot& f, int R, int path, bool wide) {
+// How a call may lay its workspace out, from the fastest to the smallest.
+enum Fit {
+  kWide,    // residue groups side by side as far as kMergeArena allows, scratch for the dense steps of a level together
+  kNarrow,  // one residue group at a time
+  kLeast,   // and scratch for one dense step at a time (TNC_PATH_TC: one residue of it)
+  kSingle   // and one residue at a time
+};
+struct Choice {
+  int path;  // TNC_PATH_TC runs on the CUDA cores alone where its planes do not fit
+  Fit fit;
+};
+// A path's choices; the last is the least that works, no more than the path
+// needed before tensor-core steps had planes (TNC_PATH_TC: TNC_PATH_INT64's).
+const std::vector<Choice>& choices(int path) {
+  static const std::vector<Choice> int64{{TNC_PATH_INT64, kWide}, {TNC_PATH_INT64, kNarrow}};
+  static const std::vector<Choice> p8{{TNC_PATH_TC_P8, kWide}, {TNC_PATH_TC_P8, kNarrow}, {TNC_PATH_TC_P8, kLeast},
+                                      {TNC_PATH_TC_P8, kSingle}};
+  static const std::vector<Choice> tc{{TNC_PATH_TC, kWide}, {TNC_PATH_TC, kNarrow}, {TNC_PATH_TC, kLeast},
+                                      {TNC_PATH_TC, kSingle}, {TNC_PATH_INT64, kNarrow}};
+  return path == TNC_PATH_TC_P8 ? p8 : path == TNC_PATH_TC ? tc : int64;
+}
+
+// Offsets of the workspace sections for the group footprint f (of the choice's path).
+SeqLayout layout_of(const Foot& f, int R, Choice ch) {
   SeqLayout s{};
+  const int path = s.path = ch.path;
+  const bool wide = ch.fit == kWide, together = ch.fit <= kNarrow;
   const bool p8 = path == TNC_PATH_TC_P8, tc = path == TNC_PATH_TC;
   const size_t word = p8 ? 1 : sizeof(uint32_t);  // bytes per residue
   // the passes
@@ -529,6 +552,10 @@ SeqLayout layout_of(const Foot& f, int R, int path, bool wide) {
   if (wide && fill_up(R, f.cost, path)) {
     quads++;
     rest = 0;
+  }
+  if (ch.fit == kSingle) {
+    quads = rest = 0;
+    for (int r = 0; r < R; r++) s.passes.push_back(PassShape{1, 1, r});
   }
   int most = 1;
   if (wide && quads > 1) {
@@ -554,14 +581,23 @@ SeqLayout layout_of(const Foot& f, int R, int path, bool wide) {
   };
   sect(s.off_leaves, f.leaves * sizeof(LeafDesc));
   sect(s.off_tables, f.tables * sizeof(uint32_t));
-  sect(s.off_steps, std::max(f.nseq, f.nlvl) * sizeof(GridStep));
-  sect(s.off_small, f.nlvl * sizeof(StepDesc));
+  if ((p8 || tc) && f.n_dense) {
+    // contract_group stages its descriptors without gaps: a step on the CUDA cores has
+    // one, of at most sizeof(GridStep), a dense one only that of section off_tc
+    sect(s.off_steps, (f.nlvl - f.n_dense) * sizeof(GridStep));
+    sect(s.off_small, 2048);  // (each array at a multiple of 128 bytes)
+  } else {
+    sect(s.off_steps, std::max(f.nseq, f.nlvl) * sizeof(GridStep));
+    sect(s.off_small, f.nlvl * sizeof(StepDesc));
+  }
   // planes and partials: of the largest step (one residue of it on TNC_PATH_TC),
   // or of a level's steps together as far as the limits allow
   uint64_t part = std::max(std::max(f.split, p8 ? f.parts : 0) * res, std::max(f.kept, tc ? f.parts : 0));
   uint64_t planes = p8 ? f.planes * res : f.planes;
-  for (uint64_t v : f.lvl_parts) part = std::max(part, std::min(v * res, tc ? kTcBytes : kGroupParts));
-  for (uint64_t v : f.lvl_planes) planes = std::max(planes, std::min(v * res, tc ? kTcPlanes : kGroupPlanes));
+  if (together) {
+    for (uint64_t v : f.lvl_parts) part = std::max(part, std::min(v * res, tc ? kTcBytes : kGroupParts));
+    for (uint64_t v : f.lvl_planes) planes = std::max(planes, std::min(v * res, tc ? kTcPlanes : kGroupPlanes));
+  }
   s.part_bytes = part;
   s.p8_bytes = planes;
   sect(s.off_tc, p8   ? f.n_dense * kind_groups * p8_step_bytes()
@@ -580,18 +616,18 @@ SeqLayout layout_of(const Foot& f, int R, int path, bool wide) {
   return s;
 }
 
-SeqLayout group_layout(const tnc_plan_t* const* plans, int n, int R, int path, bool wide) {
+SeqLayout group_layout(const tnc_plan_t* const* plans, int n, int R, Choice ch) {
   Foot sum;
   std::vector<uint64_t> arena_base, res_base, leaf_base, table_base;
   for (int i = 0; i < n; i++) {
-    const Foot f = foot_of(plans[i], path);
+    const Foot f = foot_of(plans[i], ch.path);
     leaf_base.push_back(sum.leaves);
     table_base.push_back(sum.tables);
     res_base.push_back(sum.n_out);
     arena_base.push_back(sum.arena);
     sum.add(f);
   }
-  SeqLayout s = layout_of(sum, R, path, wide);
+  SeqLayout s = layout_of(sum, R, ch);
   s.arena_base = std::move(arena_base);
   s.res_base = std::move(res_base);
   s.leaf_base = std::move(leaf_base);
@@ -599,8 +635,18 @@ SeqLayout group_layout(const tnc_plan_t* const* plans, int n, int R, int path, b
   return s;
 }
 
-// Consecutive groups of the plans whose workspace each fits `budget` bytes
-// (every plan alone must fit): [begin, end) ranges.
+// The first of the path's choices that fits `budget` bytes (the last one if none does).
+SeqLayout fitting_layout(const tnc_plan_t* const* plans, int n, int R, int path, size_t budget) {
+  SeqLayout s;
+  for (const Choice& ch : choices(path)) {
+    s = group_layout(plans, n, R, ch);
+    if (s.total <= budget) break;
+  }
+  return s;
+}
+
+// Consecutive groups of the plans, [begin, end) ranges: as many plans as fit
+// `budget` bytes one residue group at a time, or one plan that fits in any way.
 int plan_groups(const tnc_plan_t* const* plans, int n, int R, int path, size_t budget,
                 std::vector<std::pair<int, int>>& out) {
   out.clear();
@@ -610,36 +656,41 @@ int plan_groups(const tnc_plan_t* const* plans, int n, int R, int path, size_t b
     Foot f = foot_of(plans[i], path);
     Foot t = sum;
     t.add(f);
-    if (i > b && layout_of(t, R, path, false).total > budget) {
+    if (i > b && layout_of(t, R, {path, kNarrow}).total > budget) {
       out.push_back({b, i});
       b = i;
-      sum = Foot();
       t = f;
     }
-    if (layout_of(t, R, path, false).total > budget)
-      return set_error(TNC_ERR_BUFFER, "plan " + std::to_string(i) + " alone needs " +
-                                           std::to_string(layout_of(t, R, path, false).total) + " bytes of workspace");
+    if (i == b && layout_of(f, R, {path, kNarrow}).total > budget) {
+      const size_t least = fitting_layout(plans + i, 1, R, path, budget).total;
+      if (least > budget)
+        return set_error(TNC_ERR_BUFFER, "plan " + std::to_string(i) + " alone needs " + std::to_string(least) +
+                                             " bytes of workspace");
+    }
     sum = t;
   }
   if (b < n) out.push_back({b, n});
   return TNC_OK;
 }
 
-// What a group of plans is given: the wide layout (contract_group takes the
-// other where the workspace holds only that); on the u32 paths the larger of
-// both, so that one workspace serves either.
+// What a call is given for a group of plans on a path: its first choice, unless
+// scratch of very large steps makes that more than kMostExtra above the least.
+constexpr uint64_t kMostExtra = 12ull << 30;
 size_t group_bytes(const tnc_plan_t* const* plans, int n, int R, int path) {
-  size_t b = 0;
-  for (int other : {TNC_PATH_INT64, TNC_PATH_TC, TNC_PATH_TC_P8}) {
-    if ((other == TNC_PATH_TC_P8) != (path == TNC_PATH_TC_P8)) continue;
-    for (bool wide : {true, false}) b = std::max(b, group_layout(plans, n, R, other, wide).total);
-  }
-  return b;
+  const size_t least = group_layout(plans, n, R, choices(path).back()).total;
+  return fitting_layout(plans, n, R, path, least + kMostExtra).total;
 }
 size_t plan_bytes(const tnc_plan_t* p, int R, int path) { return group_bytes(&p, 1, R, path); }
 
+// The least that a path works with.
+size_t least_bytes(const tnc_plan_t* p, int R, int path) {
+  size_t least = SIZE_MAX;
+  for (const Choice& ch : choices(path)) least = std::min(least, group_layout(&p, 1, R, ch).total);
+  return least;
+}
+
 // One residue group at a time on the CUDA cores (tnc_contract_noalloc).
-SeqLayout seq_layout(const tnc_plan_t* p, int R) { return group_layout(&p, 1, R, TNC_PATH_INT64, false); }
+SeqLayout seq_layout(const tnc_plan_t* p, int R) { return group_layout(&p, 1, R, {TNC_PATH_INT64, kNarrow}); }
 
 int fill_count(tnc_count* out, uint64_t n_out, const Arith& a, const uint32_t* res, const uint32_t* limbs,
                uint32_t flags) {
@@ -1055,7 +1106,7 @@ int solo_enqueue(const SoloPack& s, uint32_t ctas, std::vector<SoloPass>& passes
 
 extern "C" size_t tnc_workspace_bytes(const tnc_plan_t* plan, int32_t n_residues) {
   if (!plan || n_residues < 1 || n_residues > 16) return 0;
-  return plan_bytes(plan, n_residues, TNC_PATH_INT64);
+  return std::max(plan_bytes(plan, n_residues, TNC_PATH_INT64), plan_bytes(plan, n_residues, TNC_PATH_TC));
 }
 
 extern "C" void tnc_set_step_timing(int32_t on) { g_time_dense = on != 0; }
@@ -1152,8 +1203,7 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
   }
   if (work.empty()) return TNC_OK;
   const int nw = (int)work.size();
-  SeqLayout L = group_layout(work.data(), nw, a.R, opts->path, true);
-  if (ws_bytes < L.total) L = group_layout(work.data(), nw, a.R, opts->path, false);
+  const SeqLayout L = fitting_layout(work.data(), nw, a.R, opts->path, ws_bytes);
   if (!dev_ws || ws_bytes < L.total) return set_error(TNC_ERR_BUFFER, "workspace smaller than tnc_workspace_bytes");
   if (((uintptr_t)dev_ws) % kAlign) return set_error(TNC_ERR_INVALID, "workspace must be 256-byte aligned");
   if (inject_hit(TNC_INJECT_LAUNCH)) return set_error(TNC_ERR_CUDA, "injected failure (TNC_INJECT_LAUNCH)");
@@ -1187,8 +1237,8 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
   // Every plan runs level by level (the tree-level schedule of the lowering);
   // offsets are shifted to the plan's part of the group's arena, tables and
   // results.  All descriptors are staged in one buffer and copied at once.
-  const bool p8 = opts->path == TNC_PATH_TC_P8;
-  const bool tc = opts->path == TNC_PATH_TC || p8;
+  const bool p8 = L.path == TNC_PATH_TC_P8;
+  const bool tc = L.path == TNC_PATH_TC || p8;
   const int sms = sm_count();
   std::vector<char> stage;
   auto put = [&](const void* src, size_t bytes) {  // 128-byte aligned; returns the offset
@@ -1678,8 +1728,8 @@ extern "C" int tnc_contract_sliced(const tnc_plan_t* const* plans, int32_t n, co
     const double b = plans[i]->net.log2_bound;
     bound = i == 0 ? b : std::max(bound, b) + std::log2(1.0 + std::exp2(-std::fabs(bound - b)));
   }
-  size_t need = 256;  // (one residue group at a time)
-  for (int i = 0; i < n; i++) need = std::max(need, group_layout(plans + i, 1, a.R, opts->path, false).total);
+  size_t need = 256;
+  for (int i = 0; i < n; i++) need = std::max(need, least_bytes(plans[i], a.R, opts->path));
   need += sliced_head_bytes(1ull << n_open, a);
   if (!dev_ws || ws_bytes < need) return set_error(TNC_ERR_BUFFER, "workspace smaller than tnc_workspace_bytes_sliced");
   if (((uintptr_t)dev_ws) % kAlign) return set_error(TNC_ERR_INVALID, "workspace must be 256-byte aligned");
@@ -1721,6 +1771,31 @@ extern "C" size_t tnc_workspace_bytes_many(const tnc_plan_t* const* plans, int32
     need = std::max(need, group_bytes(plans + i, m, a.R, opts->path));
   }
   return need;
+}
+
+extern "C" size_t tnc_workspace_bytes_below(const tnc_plan_t* const* plans, int32_t n, const tnc_contract_opts* opts,
+                                            int32_t sliced, size_t below) {
+  clear_error();
+  Arith a;
+  if (!plans || n <= 0 || make_arith(opts, a)) return 0;
+  size_t least = 256;
+  std::vector<size_t> need(choices(opts->path).size(), 256);  // of every choice, for the largest plan
+  for (int i = 0; i < n; i++) {
+    if (!plans[i]) return 0;
+    size_t own = SIZE_MAX;
+    for (size_t c = 0; c < need.size(); c++) {
+      const size_t b = group_layout(plans + i, 1, a.R, choices(opts->path)[c]).total;
+      need[c] = std::max(need[c], b);
+      own = std::min(own, b);
+    }
+    least = std::max(least, own);
+  }
+  need.push_back(least);
+  const size_t head = sliced ? sliced_head_bytes(1ull << plans[0]->net.open_vars.size(), a) : 0;
+  size_t most = 0;
+  for (size_t b : need)
+    if (b + head < below) most = std::max(most, b + head);
+  return most;
 }
 
 extern "C" int tnc_contract_many(const tnc_plan_t* const* plans, int32_t n, const tnc_contract_opts* opts,

@@ -33,7 +33,7 @@ INJECT = {"none": 0, "nomem": 1, "plan": 2, "launch": 3, "timeout": 4, "cluster"
 EXPORTS = [
     "tnc_version", "tnc_last_error", "tnc_default_primes", "tnc_default_primes_p8", "tnc_build_network", "tnc_network_info",
     "tnc_free_network", "tnc_plan", "tnc_plan_many", "tnc_plan_sliced", "tnc_slice_network", "tnc_network_formula", "tnc_plan_steps", "tnc_free_plan", "tnc_workspace_bytes", "tnc_workspace_bytes_opts", "tnc_set_step_timing", "tnc_last_dense_time", "tnc_last_contract_time", "tnc_last_launch_counts", "tnc_last_io_bytes", "tnc_last_dense_steps", "tnc_workspace_bytes_sliced", "tnc_contract_sliced",
-    "tnc_workspace_bytes_many", "tnc_contract_many",
+    "tnc_workspace_bytes_many", "tnc_workspace_bytes_below", "tnc_contract_many",
     "tnc_contract", "tnc_crt_host", "tnc_residue_add_host", "tnc_batch_create", "tnc_batch_workspace_bytes", "tnc_batch_info", "tnc_batch_upload", "tnc_batch_autotune", "tnc_batch_set_launch", "tnc_batch_get_launch",
     "tnc_batch_launch", "tnc_batch_download", "tnc_batch_download_flat", "tnc_batch_status", "tnc_free_batch",
     "tnc_contract_batch", "tnc_contract_noalloc", "tnc_probe_modmac", "tnc_inject_failure", "tnc_learned_save",
@@ -158,6 +158,7 @@ def lib():
             "tnc_last_dense_steps": ([ctypes.POINTER(_DenseStepTime), i32, i32p], ctypes.c_int),
             "tnc_workspace_bytes_sliced": ([vp, i32, vp], sz),
             "tnc_contract_sliced": ([vp, i32, vp, vp, sz, vp, vp], ctypes.c_int),
+            "tnc_workspace_bytes_below": ([vp, i32, vp, i32, sz], sz),
             "tnc_workspace_bytes_many": ([vp, i32, vp, i32], sz),
             "tnc_contract_many": ([vp, i32, vp, vp, sz, vp, vp], ctypes.c_int),
             "tnc_contract": ([vp, ctypes.POINTER(_ContractOpts), vp, sz, vp, ctypes.POINTER(_Count)],
@@ -466,13 +467,30 @@ def _stream_ptr(stream):
     return ctypes.c_void_p(s.cuda_stream)
 
 
-def _workspace(nbytes: int, ws=None):
+def _workspace(nbytes: int, ws=None, smaller=None):
+    """The caller's workspace, or a new one of nbytes; where the device has less
+    memory left, of the next smaller size that works (smaller: size -> size or 0)."""
     import torch
     if ws is not None:
         if ws.numel() * ws.element_size() < nbytes:
             raise ValueError("workspace too small")
         return ws
-    return torch.empty(max(nbytes, 256), dtype=torch.uint8, device="cuda")
+    while True:
+        try:
+            return torch.empty(max(nbytes, 256), dtype=torch.uint8, device="cuda")
+        except torch.cuda.OutOfMemoryError:
+            nbytes = smaller(nbytes) if smaller else 0
+            if nbytes == 0:
+                raise
+
+
+def workspace_bytes_below(plans: Sequence[Plan], n_residues: int, below: int, path: str = "int64", primes=None,
+                          sliced: bool = False) -> int:
+    """tnc_workspace_bytes_below: the largest workspace of less than `below` bytes
+    that contract / contract_many (or contract_sliced) uses; 0 if none works."""
+    o, _ = _opts(n_residues, primes, path)
+    arr = (ctypes.c_void_p * len(plans))(*[pp.h.value for pp in plans])
+    return int(lib().tnc_workspace_bytes_below(arr, len(plans), ctypes.byref(o), int(sliced), below))
 
 
 def _check_ws(rc: int):
@@ -483,7 +501,7 @@ def _check_ws(rc: int):
 
 
 def workspace_bytes(p: Plan, n_residues: int, path: str = "int64", primes=None) -> int:
-    """tnc_workspace_bytes_opts for the path (tnc_workspace_bytes on int64 / tc)."""
+    """tnc_workspace_bytes_opts for the path."""
     return _plan_bytes(p, _opts(n_residues, primes, path)[0])
 
 
@@ -500,7 +518,8 @@ def contract(p: Plan, n_residues: int = 4, primes=None, workspace=None, stream=N
     nb = _plan_bytes(p, o)
     if workspace is not None:  # (less than the library would use may still do)
         nb = min(nb, workspace.numel() * workspace.element_size())
-    ws = _workspace(nb, workspace)
+    ws = _workspace(nb, workspace, lambda b: workspace_bytes_below([p], n_residues, b, path, primes))
+    nb = min(nb, ws.numel() * ws.element_size())
     c, res, limbs = _count_buffers(1 << p.n_open, n_residues)
     _check_ws(lib().tnc_contract(p.h, ctypes.byref(o), ctypes.c_void_p(ws.data_ptr()), nb, _stream_ptr(stream),
                                  ctypes.byref(c)))
@@ -526,7 +545,8 @@ def contract_many(plans: Sequence[Plan], n_residues: int = 4, primes=None, works
     arr = (ctypes.c_void_p * len(plans))(*[pp.h.value for pp in plans])
     nb = workspace_bytes_many(plans, n_residues, path, group, primes) if workspace is None else \
         workspace.numel() * workspace.element_size()
-    ws = _workspace(nb, workspace)
+    ws = _workspace(nb, workspace, lambda b: workspace_bytes_below(plans, n_residues, b, path, primes))
+    nb = ws.numel() * ws.element_size()
     bufs = [_count_buffers(1 << pp.n_open, n_residues) for pp in plans]
     outs = (_Count * len(plans))(*[b[0] for b in bufs])
     _check(lib().tnc_contract_many(arr, len(plans), ctypes.byref(o), ctypes.c_void_p(ws.data_ptr()), nb,
@@ -593,7 +613,8 @@ def contract_sliced(plans: Sequence[Plan], n_residues: int = 4, primes=None, wor
     nb = int(lib().tnc_workspace_bytes_sliced(arr, len(plans), ctypes.byref(o)))
     if nb == 0:
         raise TncError(-1, lib().tnc_last_error().decode() or "invalid slices")
-    ws = workspace if workspace is not None else _workspace(nb)
+    ws = workspace if workspace is not None else \
+        _workspace(nb, None, lambda b: workspace_bytes_below(plans, n_residues, b, path, primes, sliced=True))
     nb = ws.numel() * ws.element_size()  # a larger workspace lets slices run merged
     c, res, limbs = _count_buffers(1 << plans[0].n_open, n_residues)
     _check_ws(lib().tnc_contract_sliced(arr, len(plans), ctypes.byref(o), ctypes.c_void_p(ws.data_ptr()), nb,
