@@ -319,18 +319,21 @@ int tnc_last_dense_steps(tnc_dense_step_time* out, int32_t cap, int32_t* n);
 /* Same mode: device time (ms) of the last tnc_contract's kernels, from its
  * first launch to its CRT (host work and the final copies excluded). */
 int tnc_last_contract_time(double* device_ms);
-/* The device kernels the calling thread's last tnc_contract,
- * tnc_contract_sliced or tnc_contract_noalloc enqueued, by kind: a record of
- * which branches of the pairwise step (Sec. 2.1) actually ran.  Always
- * recorded (host counters, no device work); a sliced call sums its slices.
- * A small formula's one launch (TNC_PATH_INT64) counts as a leaf fill, a level,
- * an extraction and the CRT, and its long shared sums under splitk.  p8_*
- * counts dense steps: one launch may serve several of a tree level. */
+/* What the calling thread's last tnc_contract, tnc_contract_sliced or
+ * tnc_contract_noalloc did, by kind: a record of which branches of the pairwise
+ * step (Sec. 2.1) it took, whichever kernel ran them (tnc_last_kernel_launches:
+ * the kernels).  Always recorded (host counters, no device work); a sliced call
+ * sums its slices.  A small formula's one launch (TNC_PATH_INT64) fills the leaves,
+ * contracts the levels (one under level), extracts the result and, for up to
+ * four residues, runs the CRT; its shared sums of the split-K shapes that are
+ * split over lanes count under splitk.  p8_* and tc_* count dense steps: one
+ * launch may serve several of a tree level. */
 typedef struct {
   int32_t leaf_fill;      /* leaf tensors (Eq. var, ...); TNC_PATH_TC: per residue    */
   int32_t level;          /* one launch for all small steps of a tree level           */
   int32_t grid_step;      /* large steps of a tree level over the whole GPU          */
-  int32_t splitk;         /* split-K steps on CUDA cores (a partial + final pair)    */
+  int32_t splitk;         /* split-K on CUDA cores: launches over blocks (a partial +
+                             final pair), or a small formula's steps over lanes      */
   int32_t tc_gemm;        /* TNC_PATH_TC dense steps (tcgen05 GEMMs)                  */
   int32_t tc_split;       /*   of which split over K (partials summed after)          */
   int32_t p8_pack;        /* TNC_PATH_TC_P8 dense steps with operands to pack          */
@@ -354,6 +357,16 @@ typedef struct {
   int32_t p8_cta_pair;    /* TNC_PATH_TC_P8 dense steps on CTA pairs: 256 x 256 tiles,
                              one cta_group::2 MMA over two SMs' shared memory         */
 } tnc_launch_counts;
+/* The kernels that the same call launched, by name (block_*: block_kernel by tile;
+ * one_launch: batch_kernel on one formula), and all of them together. */
+typedef struct {
+  int32_t total;
+  int32_t leaf_fill, level, outer, block_64x32, block_32x32, block_32x16, tile, step, splitk_partial, splitk_final;
+  int32_t one_launch, extract, crt, crt_warp, residue_add;
+  int32_t rns_pack, rns_join;                 /* TNC_PATH_TC */
+  int32_t p8_pack, p8_gemm, p8_split_final;   /* p8_gemm: both tensor-core paths */
+} tnc_kernel_launches;
+int tnc_last_kernel_launches(tnc_kernel_launches* out);
 int tnc_last_launch_counts(tnc_launch_counts* out);
 /* Bytes the calling thread's last tnc_contract or tnc_contract_sliced copied
  * host -> device (descriptors, weight tables) and device -> host (residues,

@@ -56,6 +56,7 @@ thread_local double g_dense_ms = 0.0;
 thread_local int g_dense_launches = 0;
 thread_local double g_total_ms = 0.0;
 thread_local tnc_launch_counts g_launches{};
+thread_local tnc_kernel_launches g_kernels{};
 thread_local std::vector<tnc_dense_step_time> g_dense_steps;  // timing mode: per dense launch
 thread_local uint64_t g_h2d_bytes = 0, g_d2h_bytes = 0;  // host <-> device copies of the last contraction
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
@@ -942,7 +943,7 @@ struct SoloPack {
   std::vector<char> bytes;  // forms, blob, leaves, tables, perms, order: copied to the workspace as they are
   size_t off_blob = 0, off_leaves = 0, off_tables = 0, off_perms = 0, off_order = 0;
   size_t blob_bytes = 0;
-  int long_sums = 0;  // steps of the split-K shapes (their sums are split over lanes)
+  int long_sums = 0;  // steps of the split-K shapes with their sums split over lanes
 };
 }  // namespace tnc
 
@@ -968,7 +969,8 @@ void make_solo(const tnc_plan_t* p, SoloPack& s) {
   s.off_tables = blob_put(s.bytes, p->low.leaf_tables.data(), p->low.leaf_tables.size() * sizeof(uint32_t));
   s.off_perms = blob_put(s.bytes, p->low.root_perm.data(), p->low.root_perm.size());
   s.off_order = blob_put(s.bytes, &first, sizeof(first));
-  for (const StepDesc& d : p->low.lvl_steps) s.long_sums += splitk_log(d) > 0;
+  const BStep* steps = reinterpret_cast<const BStep*>(blob.data());
+  for (size_t i = 0; i < p->low.lvl_steps.size(); i++) s.long_sums += splitk_log(p->low.lvl_steps[i]) > 0 && steps[i].g < 5;
   s.ok = blob.size() <= (size_t)kSoloSmem;
 }
 
@@ -979,6 +981,7 @@ void launch_crt(const uint32_t* residues, uint64_t n, const CrtConsts& cc, uint3
     tnc_dev::crt_warp_kernel<<<(unsigned)((n + 3) / 4), 128, 0, st>>>(residues, n, cc, limbs);
   else
     tnc_dev::crt_kernel<<<(unsigned)std::min<uint64_t>((n + 127) / 128, 1024), 128, 0, st>>>(residues, n, cc, limbs);
+  launched(n <= 2048 ? &tnc_kernel_launches::crt_warp : &tnc_kernel_launches::crt);
   g_launches.crt++;
 }
 
@@ -1090,7 +1093,8 @@ int solo_enqueue(const SoloPack& s, uint32_t ctas, std::vector<SoloPass>& passes
       return TNC_OK;
     });
     if (rc) return rc;
-    // the record: the one launch does the work of these
+    launched(&tnc_kernel_launches::one_launch);
+    // the record of the work: the one launch does all of it
     g_launches.leaf_fill++;
     g_launches.level++;
     g_launches.extract++;
@@ -1132,6 +1136,16 @@ extern "C" int tnc_last_contract_time(double* device_ms) {
 }
 
 tnc_launch_counts& tnc::launch_counts() { return g_launches; }
+void tnc::launched(int32_t tnc_kernel_launches::*kernel) {
+  g_kernels.*kernel += 1;
+  g_kernels.total += 1;
+}
+
+extern "C" int tnc_last_kernel_launches(tnc_kernel_launches* out) {
+  if (!out) return set_error(TNC_ERR_INVALID, "NULL argument");
+  *out = g_kernels;
+  return TNC_OK;
+}
 
 extern "C" int tnc_last_launch_counts(tnc_launch_counts* out) {
   if (!out) return set_error(TNC_ERR_INVALID, "NULL argument");
@@ -1194,6 +1208,7 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
       if (!dev_ws || ws_bytes < (size_t)a.R * 4) return set_error(TNC_ERR_BUFFER, "workspace too small");
       CUDA_TRY(cudaMemcpyAsync(dev_ws, res.data(), a.R * sizeof(uint32_t), cudaMemcpyHostToDevice, st));
       residue_add_kernel<<<1, 64, 0, st>>>(sum_into, (const uint32_t*)dev_ws, (uint64_t)a.R, 1, a.R, a.crt);
+      launched(&tnc_kernel_launches::residue_add);
       CUDA_TRY(cudaGetLastError());
       CUDA_TRY(cudaStreamSynchronize(st));
     } else {
@@ -1514,6 +1529,7 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
           tc && !p8 ? tc_consts(primes.data(), (uint32_t)primes.size()) : std::vector<char>();
       tnc_dev::leaf_fill_kernel<RG, W><<<dim3(std::min(nl, sms * 8), ng), 64, 0, st>>>(
           (const LeafDesc*)(ws + at_leaves), nl, (const uint32_t*)(ws + at_tables), arena, ps);
+      launched(&tnc_kernel_launches::leaf_fill);
       // (recorded per residue group, on TNC_PATH_TC per residue)
       g_launches.leaf_fill += tc && !p8 ? std::min((int)ng * RG, a.R - shape.col) : (int)ng;
       // a timed dense launch: events around it and its shape
@@ -1548,11 +1564,13 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
           tnc_dev::level_kernel<RG, W, N30><<<dim3(blocks, ng), 256, 0, st>>>(d_small + lv.small_lo, lv.small_n,
                                                                              lv.small_work, arena, ps);
           g_launches.level++;
+          launched(&tnc_kernel_launches::level);
         }
         if (lv.outer.n) {
           tnc_dev::outer_kernel<RG, W, N30><<<dim3(lv.outer.blocks, ng), 256, 0, st>>>(d_outer + lv.outer.lo, lv.outer.n,
                                                                                        arena, ps);
           g_launches.outer++;
+          launched(&tnc_kernel_launches::outer);
         }
         if constexpr (sizeof(W) == 4) {
           auto blocks = [&](auto shape) -> int {
@@ -1567,6 +1585,8 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
             k<<<dim3(std::min(r.blocks, (2u * (unsigned)sms + ng - 1) / ng), ng), 256, smem, st>>>(
                 (const tnc_dev::BlockStep*)(ws + at_block[Q]) + r.lo, r.n, r.blocks, arena, ps);
             g_launches.grid_step++;
+            launched(Q == 0 ? &tnc_kernel_launches::block_64x32
+                            : Q == 1 ? &tnc_kernel_launches::block_32x32 : &tnc_kernel_launches::block_32x16);
             return TNC_OK;
           };
           int rc2 = blocks(std::integral_constant<int, 0>());
@@ -1578,17 +1598,21 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
           tnc_dev::tile_kernel<RG, W, N30><<<dim3(lv.tile.blocks, ng), 256, 0, st>>>(d_tile + lv.tile.lo, lv.tile.n, arena,
                                                                                      ps);
           g_launches.grid_step++;
+          launched(&tnc_kernel_launches::tile);
         }
         if (lv.grid.n) {
           tnc_dev::step_kernel<RG, W, N30><<<dim3(lv.grid.blocks, ng), 256, 0, st>>>(d_steps + lv.grid.lo, lv.grid.n, arena,
                                                                                      ps);
           g_launches.grid_step++;
+          launched(&tnc_kernel_launches::step);
         }
         for (const Range& r : lv.split) {
           tnc_dev::splitk_partial_kernel<RG, W, N30><<<dim3(r.blocks, ng), 256, 0, st>>>(d_steps + r.lo, r.n, arena, part,
                                                                                          ps);
           tnc_dev::splitk_final_kernel<RG, W, N30><<<dim3(r.finals, ng), 256, 0, st>>>(d_steps + r.lo, r.n, arena, part, ps);
           g_launches.splitk++;
+          launched(&tnc_kernel_launches::splitk_partial);
+          launched(&tnc_kernel_launches::splitk_final);
         }
         if (tc && !p8)
           for (const TcLaunch& x : dn->tc[&lv - lev.data()]) {
@@ -1612,6 +1636,7 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
         tnc_dev::extract_kernel<RG, W><<<dim3(blocks, ng), 256, 0, st>>>(arena, ps.arena_stride, rs, results, a.R,
                                                                         shape.col);
         g_launches.extract++;
+        launched(&tnc_kernel_launches::extract);
       }
       CUDA_TRY(cudaGetLastError());
       return TNC_OK;
@@ -1628,6 +1653,7 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
     const uint64_t m = (1ull << roots[0].r[0].map.n_open) * (uint64_t)a.R;  // (the same for every plan)
     residue_add_kernel<<<(unsigned)std::min<uint64_t>((m + 255) / 256, 1024), 256, 0, st>>>(sum_into, results, m,
                                                                                            (uint32_t)nw, a.R, a.crt);
+    launched(&tnc_kernel_launches::residue_add);
     CUDA_TRY(cudaGetLastError());
     if (tc) {
       CUDA_TRY(cudaMemcpyAsync(&h_err, d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
@@ -1677,6 +1703,7 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
 // thread.
 static void reset_records() {
   g_launches = tnc_launch_counts{};
+  g_kernels = tnc_kernel_launches{};
   g_h2d_bytes = g_d2h_bytes = 0;
   g_dense_ms = 0.0;
   g_dense_launches = 0;
@@ -2446,6 +2473,7 @@ extern "C" int tnc_contract_noalloc(const tnc_plan_t* plan, const tnc_contract_o
                                     tnc_count* out) {
   clear_error();
   g_launches = tnc_launch_counts{};
+  g_kernels = tnc_kernel_launches{};
   NvtxRange range("tnc_contract_noalloc");
   if (!plan || !opts || !out) return set_error(TNC_ERR_INVALID, "NULL argument");
   if (opts->path != TNC_PATH_INT64)
@@ -2569,6 +2597,7 @@ extern "C" int tnc_contract_noalloc(const tnc_plan_t* plan, const tnc_contract_o
       tnc_dev::leaf_fill_kernel<RG><<<std::min(nl, sms * 8), 64, 0, st>>>(
           (const LeafDesc*)(ws + L.off_leaves), nl, (const uint32_t*)(ws + L.off_tables), arena, ps);
       g_launches.leaf_fill++;
+      launched(&tnc_kernel_launches::leaf_fill);
       for (size_t i = 0; i < plan->low.seq_steps.size(); i++) {
         const StepDesc& d = plan->low.seq_steps[i];
         const uint32_t ls = splitk_log(d);
@@ -2577,16 +2606,20 @@ extern "C" int tnc_contract_noalloc(const tnc_plan_t* plan, const tnc_contract_o
                                                                                            ps);
           tnc_dev::splitk_final_kernel<RG><<<(unsigned)(1ull << d.c), 256, 0, st>>>(d_steps + i, 1, arena, part, ps);
           g_launches.splitk++;
+          launched(&tnc_kernel_launches::splitk_partial);
+          launched(&tnc_kernel_launches::splitk_final);
           continue;
         }
         int threads, blocks, sh;
         grid_shape(d.c, &threads, &blocks, &sh);
         tnc_dev::step_kernel<RG><<<blocks, threads, 0, st>>>(d_steps + i, 1, arena, ps);
         g_launches.grid_step++;
+        launched(&tnc_kernel_launches::step);
       }
       tnc_dev::extract_kernel<RG><<<(unsigned)std::min<uint64_t>((n_out + 255) / 256, 1024), 256, 0, st>>>(
           arena, 0, roots, results, R, grp_col[gi]);
       g_launches.extract++;
+      launched(&tnc_kernel_launches::extract);
       CUDA_TRY(cudaGetLastError());
       return TNC_OK;
     });
@@ -2595,6 +2628,7 @@ extern "C" int tnc_contract_noalloc(const tnc_plan_t* plan, const tnc_contract_o
   tnc_dev::crt_kernel<<<(unsigned)std::min<uint64_t>((n_out + 127) / 128, 1024), 128, 0, st>>>(results, n_out, cc,
                                                                                                 limbs);
   g_launches.crt++;
+  launched(&tnc_kernel_launches::crt);
   CUDA_TRY(cudaGetLastError());
   if (out->residues)
     CUDA_TRY(cudaMemcpyAsync(out->residues, results, n_out * R * sizeof(uint32_t), cudaMemcpyDeviceToHost, st));

@@ -470,6 +470,7 @@ int tc_run(const TcBatch& b, const char* dev, const std::vector<char>& consts, u
   if (b.nr == 4) rns_pack_kernel<4><<<pack_blocks, 256, 0, st>>>(pu, b.n_units, b.pack_tiles, rg, pack_consts());
   else if (b.nr == 2) rns_pack_kernel<2><<<pack_blocks, 256, 0, st>>>(pu, b.n_units, b.pack_tiles, rg, pack_consts());
   else rns_pack_kernel<1><<<pack_blocks, 256, 0, st>>>(pu, b.n_units, b.pack_tiles, rg, pack_consts());
+  launched(&tnc_kernel_launches::rns_pack);
   for (int v = 6; v-- > 0;)
     for (int g = 0; g < 3; g++)
       if (b.gemm[g][v].n)
@@ -482,6 +483,7 @@ int tc_run(const TcBatch& b, const char* dev, const std::vector<char>& consts, u
   if (b.nr == 4) rns_join_kernel<4><<<b.blocks, 256, 0, st>>>(ju, b.n_units, rg, jc);
   else if (b.nr == 2) rns_join_kernel<2><<<b.blocks, 256, 0, st>>>(ju, b.n_units, rg, jc);
   else rns_join_kernel<1><<<b.blocks, 256, 0, st>>>(ju, b.n_units, rg, jc);
+  launched(&tnc_kernel_launches::rns_join);
   launch_counts().tc_gemm += (int32_t)b.steps;
   launch_counts().tc_split += (int32_t)b.splits;
   const cudaError_t e = cudaGetLastError();

@@ -1315,6 +1315,7 @@ uint32_t variant_of(const Shape& s) {
 template <uint32_t RG>
 int launch_variant(uint32_t v, const tnc_p8::P8Prob* probs, uint32_t n, uint32_t n_items, const tnc_p8::P8Primes& pr,
                    int sms, uint32_t* err, cudaStream_t st) {
+  launched(&tnc_kernel_launches::p8_gemm);
   switch (v) {
     case 0: return launch_gemm<16, RG, false>(probs, n, n_items, pr, sms, err, st);
     case 1: return launch_gemm<32, RG, false>(probs, n, n_items, pr, sms, err, st);
@@ -1617,6 +1618,7 @@ int p8_run(const P8Batch& b, const char* dev, const uint32_t* primes, uint32_t n
     if (rg == 4) p8_pack_kernel<4><<<blocks, 256, 0, st>>>(p, b.pack_n, b.pack_tiles, pp);
     else if (rg == 2) p8_pack_kernel<2><<<blocks, 256, 0, st>>>(p, b.pack_n, b.pack_tiles, pp);
     else p8_pack_kernel<1><<<blocks, 256, 0, st>>>(p, b.pack_n, b.pack_tiles, pp);
+    launched(&tnc_kernel_launches::p8_pack);
   }
   for (uint32_t v = 6; v-- > 0;) {  // wide tiles (the long steps) first
     if (!b.gemm[v].n) continue;
@@ -1627,9 +1629,11 @@ int p8_run(const P8Batch& b, const char* dev, const uint32_t* primes, uint32_t n
     else rc = launch_variant<1>(v, p, b.gemm[v].n, b.gemm[v].items, pr, sms, dev_err, st);
     if (rc) return rc;
   }
-  if (b.split_n)
+  if (b.split_n) {
     p8_split_final_kernel<<<b.split_blocks, 256, 0, st>>>(reinterpret_cast<const SplitProb*>(dev + b.split_off),
                                                           b.split_n, rg, pp);
+    launched(&tnc_kernel_launches::p8_split_final);
+  }
   tnc_launch_counts& lc = launch_counts();
   const int32_t chunks = std::max(lc.p8_max_chunks, b.counts.p8_max_chunks);
   for (size_t i = 0; i < sizeof(lc) / sizeof(int32_t); i++)

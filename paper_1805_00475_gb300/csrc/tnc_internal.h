@@ -118,9 +118,11 @@ namespace tnc {
 int set_error(int code, const std::string& msg);
 void clear_error();
 
-// Kernel launches of the calling thread's current (or last) contraction
+// The work of the calling thread's current (or last) contraction by kind
 // (tnc_last_launch_counts); contract.cu resets it per call.
 tnc_launch_counts& launch_counts();
+// One more launch of a kernel in it (tnc_last_kernel_launches).
+void launched(int32_t tnc_kernel_launches::*kernel);
 
 // Fault injection (inject.cpp): true if an armed failure of this kind fires
 // at this call site (tnc_inject_failure).

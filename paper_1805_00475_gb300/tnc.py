@@ -32,7 +32,7 @@ INJECT = {"none": 0, "nomem": 1, "plan": 2, "launch": 3, "timeout": 4, "cluster"
 # every symbol include/tnc.h declares
 EXPORTS = [
     "tnc_version", "tnc_last_error", "tnc_default_primes", "tnc_default_primes_p8", "tnc_build_network", "tnc_network_info",
-    "tnc_free_network", "tnc_plan", "tnc_plan_many", "tnc_plan_sliced", "tnc_slice_network", "tnc_network_formula", "tnc_plan_steps", "tnc_free_plan", "tnc_workspace_bytes", "tnc_workspace_bytes_opts", "tnc_set_step_timing", "tnc_last_dense_time", "tnc_last_contract_time", "tnc_last_launch_counts", "tnc_last_io_bytes", "tnc_last_dense_steps", "tnc_workspace_bytes_sliced", "tnc_contract_sliced",
+    "tnc_free_network", "tnc_plan", "tnc_plan_many", "tnc_plan_sliced", "tnc_slice_network", "tnc_network_formula", "tnc_plan_steps", "tnc_free_plan", "tnc_workspace_bytes", "tnc_workspace_bytes_opts", "tnc_set_step_timing", "tnc_last_dense_time", "tnc_last_contract_time", "tnc_last_launch_counts", "tnc_last_kernel_launches", "tnc_last_io_bytes", "tnc_last_dense_steps", "tnc_workspace_bytes_sliced", "tnc_contract_sliced",
     "tnc_workspace_bytes_many", "tnc_workspace_bytes_below", "tnc_contract_many",
     "tnc_contract", "tnc_crt_host", "tnc_residue_add_host", "tnc_batch_create", "tnc_batch_workspace_bytes", "tnc_batch_info", "tnc_batch_upload", "tnc_batch_autotune", "tnc_batch_set_launch", "tnc_batch_get_launch",
     "tnc_batch_launch", "tnc_batch_download", "tnc_batch_download_flat", "tnc_batch_status", "tnc_free_batch",
@@ -86,6 +86,13 @@ class _LaunchCounts(ctypes.Structure):
                [(n, ctypes.c_int32) for n in ("p8_max_chunks", "p8_swapped", "p8_padded", "extract", "crt",
                                               "p8_direct_out", "p8_direct_in", "p8_mn", "p8_pairs", "outer",
                                               "p8_cta_pair")]
+
+
+class _KernelLaunches(ctypes.Structure):
+    _fields_ = [(n, ctypes.c_int32) for n in ("total", "leaf_fill", "level", "outer", "block_64x32", "block_32x32",
+                                              "block_32x16", "tile", "step", "splitk_partial", "splitk_final",
+                                              "one_launch", "extract", "crt", "crt_warp", "residue_add", "rns_pack",
+                                              "rns_join", "p8_pack", "p8_gemm", "p8_split_final")]
 
 
 class _LearnedOpts(ctypes.Structure):
@@ -153,6 +160,7 @@ def lib():
             "tnc_set_step_timing": ([i32], None),
             "tnc_last_dense_time": ([ctypes.POINTER(ctypes.c_double), i32p], ctypes.c_int),
             "tnc_last_contract_time": ([ctypes.POINTER(ctypes.c_double)], ctypes.c_int),
+            "tnc_last_kernel_launches": ([ctypes.POINTER(_KernelLaunches)], ctypes.c_int),
             "tnc_last_launch_counts": ([ctypes.POINTER(_LaunchCounts)], ctypes.c_int),
             "tnc_last_io_bytes": ([ctypes.POINTER(ctypes.c_uint64), ctypes.POINTER(ctypes.c_uint64)], ctypes.c_int),
             "tnc_last_dense_steps": ([ctypes.POINTER(_DenseStepTime), i32, i32p], ctypes.c_int),
@@ -576,9 +584,17 @@ def last_contract_time() -> float:
 P8_TILE_WIDTHS = (16, 32, 64, 128, 256)
 
 
+def last_kernel_launches() -> dict:
+    """tnc_last_kernel_launches: the kernels that the calling thread's last
+    contraction launched, by name, and their "total"."""
+    c = _KernelLaunches()
+    _check(lib().tnc_last_kernel_launches(ctypes.byref(c)))
+    return {n: int(getattr(c, n)) for n, _ in _KernelLaunches._fields_}
+
+
 def last_launch_counts() -> dict:
-    """tnc_last_launch_counts: kernels the calling thread's last contraction
-    enqueued, by kind; "p8_tile_n" maps tile width -> GEMM launches."""
+    """tnc_last_launch_counts: the work of the calling thread's last contraction
+    by kind; "p8_tile_n" maps tile width -> dense steps."""
     c = _LaunchCounts()
     _check(lib().tnc_last_launch_counts(ctypes.byref(c)))
     d = {n: int(getattr(c, n)) for n, _ in _LaunchCounts._fields_ if n != "p8_tile_n"}
