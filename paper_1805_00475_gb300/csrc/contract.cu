@@ -683,13 +683,6 @@ size_t group_bytes(const tnc_plan_t* const* plans, int n, int R, int path) {
 }
 size_t plan_bytes(const tnc_plan_t* p, int R, int path) { return group_bytes(&p, 1, R, path); }
 
-// The least that a path works with.
-size_t least_bytes(const tnc_plan_t* p, int R, int path) {
-  size_t least = SIZE_MAX;
-  for (const Choice& ch : choices(path)) least = std::min(least, group_layout(&p, 1, R, ch).total);
-  return least;
-}
-
 // One residue group at a time on the CUDA cores (tnc_contract_noalloc).
 SeqLayout seq_layout(const tnc_plan_t* p, int R) { return group_layout(&p, 1, R, {TNC_PATH_INT64, kNarrow}); }
 
@@ -1755,22 +1748,19 @@ extern "C" int tnc_contract_sliced(const tnc_plan_t* const* plans, int32_t n, co
     const double b = plans[i]->net.log2_bound;
     bound = i == 0 ? b : std::max(bound, b) + std::log2(1.0 + std::exp2(-std::fabs(bound - b)));
   }
-  size_t need = 256;
-  for (int i = 0; i < n; i++) need = std::max(need, least_bytes(plans[i], a.R, opts->path));
-  need += sliced_head_bytes(1ull << n_open, a);
-  if (!dev_ws || ws_bytes < need) return set_error(TNC_ERR_BUFFER, "workspace smaller than tnc_workspace_bytes_sliced");
+  const size_t head = sliced_head_bytes(1ull << n_open, a);
+  if (!dev_ws || ws_bytes < head + 256)
+    return set_error(TNC_ERR_BUFFER, "workspace smaller than tnc_workspace_bytes_sliced");
+  // as many slices at a time as the workspace holds, their levels merged
+  std::vector<std::pair<int, int>> grp;
+  if ((rc = plan_groups(plans, n, a.R, opts->path, ws_bytes - head, grp))) return rc;
   if (((uintptr_t)dev_ws) % kAlign) return set_error(TNC_ERR_INVALID, "workspace must be 256-byte aligned");
   cudaStream_t st = (cudaStream_t)cuda_stream;
   const uint64_t n_out = 1ull << n_open;
   char* ws = (char*)dev_ws;
   uint32_t* acc = (uint32_t*)ws;
   uint32_t* limbs = (uint32_t*)(ws + align_up(n_out * a.R * sizeof(uint32_t)));
-  const size_t head = sliced_head_bytes(n_out, a);
   CUDA_TRY(cudaMemsetAsync(acc, 0, n_out * a.R * sizeof(uint32_t), st));
-  // as many slices at a time as the workspace holds, their levels merged
-  std::vector<std::pair<int, int>> grp;
-  rc = plan_groups(plans, n, a.R, opts->path, ws_bytes - head, grp);
-  if (rc) return rc;
   for (const auto& g : grp) {
     rc = contract_group(plans + g.first, g.second - g.first, opts, ws + head, ws_bytes - head, cuda_stream, nullptr,
                         acc);
