@@ -257,7 +257,7 @@ size_t tnc_workspace_bytes(const tnc_plan_t* plan, int32_t n_residues);
 /* Device workspace needed by tnc_contract with these options (any path; adds
  * TNC_PATH_TC_P8's packed fp16 operands and K-split partials); 0 if the options
  * are invalid.  It holds the residue groups side by side as far as that is
- * faster (up to 12 GiB more than the least that works); the calls also run in
+ * faster (up to 16 GiB more than the least that works, or twice that); the calls also run in
  * smaller workspaces, one residue group or one residue at a time, and TNC_PATH_TC
  * in any that TNC_PATH_INT64 runs in (dense steps on the CUDA cores where their
  * operands do not fit otherwise). */

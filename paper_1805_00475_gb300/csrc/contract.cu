@@ -675,11 +675,14 @@ int plan_groups(const tnc_plan_t* const* plans, int n, int R, int path, size_t b
 }
 
 // What a call is given for a group of plans on a path: its first choice, unless
-// scratch of very large steps makes that more than kMostExtra above the least.
-constexpr uint64_t kMostExtra = 12ull << 30;
+// scratch of very large steps makes that more than twice the least and more than
+// kMostExtra above it.  (TNC_PATH_TC, cubic VC with 180 vertices, rank 29: 15 GiB of
+// planes above 11 to 17; with 12 GiB as the limit 16 such formulas took 1041 ms
+// instead of 930.)
+constexpr uint64_t kMostExtra = 16ull << 30;
 size_t group_bytes(const tnc_plan_t* const* plans, int n, int R, int path) {
   const size_t least = group_layout(plans, n, R, choices(path).back()).total;
-  return fitting_layout(plans, n, R, path, least + kMostExtra).total;
+  return fitting_layout(plans, n, R, path, least + std::max<uint64_t>(least, kMostExtra)).total;
 }
 size_t plan_bytes(const tnc_plan_t* p, int R, int path) { return group_bytes(&p, 1, R, path); }
 
