@@ -44,7 +44,7 @@ __device__ __forceinline__ float ld<__nv_bfloat16>(const __nv_bfloat16* p, int i
   return __bfloat162float(p[i]);
 }
 
-// Eight consecutive weights from a 16-byte aligned position; four from shared memory.
+// Four consecutive weights from shared memory, from a position aligned to their size.
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ float4 ld4(const __nv_bfloat16* p) {  // (a bf16 is the upper half of a float)
   const uint2 w = *reinterpret_cast<const uint2*>(p);

@@ -7,15 +7,15 @@
 // mod p at the end.  S is computed modulo small primes q_1..q_n (the largest
 // below 2^8) whose product exceeds it, each product with exact fp16 operands
 // on the GEMM of the 8-bit-prime path (tc_p8.cu), and rebuilt modulo p by the
-// Chinese remainder theorem.  For primes below 2^30 and k <= 10 that is 9
-// products; splitting the residues into 8-bit limbs (fp16 exact, but at most 64
+// Chinese remainder theorem.  That is 9 products up to k = 8 and 10 up to k = 15
+// (12 for small steps, tc_small_primes); splitting the residues into 8-bit limbs (fp16 exact, but at most 64
 // shared values to an exact fp32 sum) takes 16 products, and 7 accumulators
 // folded into integers every 64 shared values.  The dense steps of a cubic VC
 // formula with n = 160 (2^34.4 products per residue, 4 residues): 7.09 ms with
 // limbs (operands staged by all threads, tensor pipe 15 % active), 3.58 ms
 // this way: GEMMs 2.17 (1.37 PFLOP/s on the largest step, 2^13 x 2^10 x 2^11),
-// packing 0.75 (its writes: 2^24 entries 374 us against 236 at HBM rate),
-// joining 0.66.
+// packing 0.75 (2^24 entries 376 us: the integer multiply pipe is 92 % busy, 4.7
+// TB/s of HBM), joining 0.66 (its loads' latency; 3.0 TB/s).
 //
 //   rns_pack_kernel   entries -> one fp16 plane per small prime (balanced)
 //   p8_gemm_kernel    four, two or one small primes at a time -> bytes
@@ -149,7 +149,8 @@ __device__ __forceinline__ void load_words(const uint32_t* p, uint32_t (&v)[NR])
 // Four entries per thread, so that a plane's writes are 8 bytes per lane; per
 // value and small prime a high product, a shift and a multiply-add, half an
 // add and half a packed subtraction.  Writes 2 bytes per small prime and
-// residue: 18 to 20 bytes where it reads 4.
+// residue: 18 to 20 bytes where it reads 4 (HBM at 0.69 of the measured copy
+// rate: the multiplies bound it).
 template <int NR>
 __global__ void __launch_bounds__(256) rns_pack_kernel(const PackUnit* __restrict__ units, uint32_t n_units,
                                                        uint32_t n_tiles, uint32_t stride,
