@@ -67,3 +67,19 @@ def test_three_residues_take_four_only_where_that_is_small():
     assert b.info()[3] == 3
     rest = b.info()[0] + 6000 * 4 * (3 + 3) + 4096
     assert b.workspace_bytes() <= rest + 6000 * (small.stats.batch_arena_entries + 7) * 4 * 2
+
+
+def test_graph_replays_with_heavy_formulas():
+    """On a stream of its own the launch is a captured graph: its counters start anew each time."""
+    import torch
+    sizes = (72, 72, 30, 24, 24)
+    plans = {n: tnc.plan_formula(I.cubic_vertex_cover(n, n), heuristic="gn") for n in sizes}
+    want = [tnc.contract_noalloc(plans[n], n_residues=4).residues.tolist() for n in sizes]
+    b = tnc.Batch([plans[n] for n in sizes], n_residues=4)
+    ws = torch.empty(b.workspace_bytes(), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    st = torch.cuda.Stream()
+    b.upload(ws, st)
+    for _ in range(3):
+        b.launch(ws, st)
+        assert [r.residues.tolist() for r in b.download(ws, st)] == want
