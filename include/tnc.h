@@ -259,8 +259,8 @@ size_t tnc_workspace_bytes(const tnc_plan_t* plan, int32_t n_residues);
  * are invalid.  It holds the residue groups side by side as far as that is
  * faster (up to 16 GiB more than the least that works, or twice that); the calls also run in
  * smaller workspaces, one residue group or one residue at a time, and TNC_PATH_TC
- * in any that TNC_PATH_INT64 runs in (dense steps on the CUDA cores where their
- * operands do not fit otherwise). */
+ * in any that TNC_PATH_INT64 runs in (with what it leaves as the dense steps' scratch,
+ * those that do not fit on the CUDA cores). */
 size_t tnc_workspace_bytes_opts(const tnc_plan_t* plan, const tnc_contract_opts* opts);
 /* For callers short of device memory: the largest workspace of less than `below`
  * bytes that a call with these options uses in full, 0 if none that small works.

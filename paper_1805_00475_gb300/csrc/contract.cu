@@ -463,6 +463,25 @@ uint32_t p8_flags(const Lowered& lw, uint32_t i) {
          (sb >= 0 && lw.p8_direct[sb] ? kP8DirectB : 0u);
 }
 
+// TNC_PATH_TC dense steps whose planes do not fit are summed in 2^chunks parts of
+// their shared values, up to 2^kMaxChunkLog.
+constexpr uint32_t kMaxChunkLog = 3;
+StepDesc tc_part(const StepDesc& d, uint32_t chunks, uint64_t part) {
+  StepDesc x = d;
+  x.k = (uint8_t)(d.k - chunks);
+  x.a_off += part << (x.k + d.ka);  // (shared values are the operands' highest bits)
+  x.b_off += part << (x.k + d.kb);
+  return x;
+}
+bool tc_chunks(const StepDesc& d, uint64_t planes, uint64_t bytes, uint32_t* chunks) {
+  for (*chunks = 0; *chunks <= kMaxChunkLog; ++*chunks) {
+    const StepDesc x = tc_part(d, *chunks, 0);
+    if (!tc_eligible(x)) return false;
+    if (tc_plane_bytes(x) <= planes && tc_byte_bytes(x) <= bytes) return true;
+  }
+  return false;
+}
+
 // Bytes that the CUDA-core layout sets aside for a dense step's K split and
 // (per residue) descriptor.  No kernel uses them any more; they stay because
 // tnc_contract_noalloc takes or refuses a plan by this layout's size.
@@ -524,10 +543,11 @@ enum Fit {
   kWide,    // residue groups side by side as far as kMergeArena allows, scratch for the dense steps of a level together
   kNarrow,  // one residue group at a time
   kLeast,   // and scratch for one dense step at a time (TNC_PATH_TC: one residue of it)
-  kSingle   // and one residue at a time
+  kSingle,  // and one residue at a time
+  kSpare    // TNC_PATH_TC: one residue at a time, its scratch what the workspace leaves
 };
 struct Choice {
-  int path;  // TNC_PATH_TC runs on the CUDA cores alone where its planes do not fit
+  int path;  // TNC_PATH_TC runs on the CUDA cores alone where too few of its planes fit
   Fit fit;
 };
 // A path's choices; the last is the least that works, no more than the path
@@ -537,7 +557,7 @@ const std::vector<Choice>& choices(int path) {
   static const std::vector<Choice> p8{{TNC_PATH_TC_P8, kWide}, {TNC_PATH_TC_P8, kNarrow}, {TNC_PATH_TC_P8, kLeast},
                                       {TNC_PATH_TC_P8, kSingle}};
   static const std::vector<Choice> tc{{TNC_PATH_TC, kWide}, {TNC_PATH_TC, kNarrow}, {TNC_PATH_TC, kLeast},
-                                      {TNC_PATH_TC, kSingle}, {TNC_PATH_INT64, kNarrow}};
+                                      {TNC_PATH_TC, kSingle}, {TNC_PATH_TC, kSpare}, {TNC_PATH_INT64, kNarrow}};
   return path == TNC_PATH_TC_P8 ? p8 : path == TNC_PATH_TC ? tc : int64;
 }
 
@@ -545,7 +565,7 @@ const std::vector<Choice>& choices(int path) {
 SeqLayout layout_of(const Foot& f, int R, Choice ch) {
   SeqLayout s{};
   const int path = s.path = ch.path;
-  const bool wide = ch.fit == kWide, together = ch.fit <= kNarrow;
+  const bool wide = ch.fit == kWide, together = ch.fit <= kNarrow, spare = ch.fit == kSpare;
   const bool p8 = path == TNC_PATH_TC_P8, tc = path == TNC_PATH_TC;
   const size_t word = p8 ? 1 : sizeof(uint32_t);  // bytes per residue
   // the passes
@@ -554,7 +574,7 @@ SeqLayout layout_of(const Foot& f, int R, Choice ch) {
     quads++;
     rest = 0;
   }
-  if (ch.fit == kSingle) {
+  if (ch.fit >= kSingle) {
     quads = rest = 0;
     for (int r = 0; r < R; r++) s.passes.push_back(PassShape{1, 1, r});
   }
@@ -582,7 +602,7 @@ SeqLayout layout_of(const Foot& f, int R, Choice ch) {
   };
   sect(s.off_leaves, f.leaves * sizeof(LeafDesc));
   sect(s.off_tables, f.tables * sizeof(uint32_t));
-  if ((p8 || tc) && f.n_dense) {
+  if ((p8 || tc) && f.n_dense && !spare) {
     // contract_group stages its descriptors without gaps: a step on the CUDA cores has
     // one, of at most sizeof(GridStep), a dense one only that of section off_tc
     sect(s.off_steps, (f.nlvl - f.n_dense) * sizeof(GridStep));
@@ -593,8 +613,9 @@ SeqLayout layout_of(const Foot& f, int R, Choice ch) {
   }
   // planes and partials: of the largest step (one residue of it on TNC_PATH_TC),
   // or of a level's steps together as far as the limits allow
-  uint64_t part = std::max(std::max(f.split, p8 ? f.parts : 0) * res, std::max(f.kept, tc ? f.parts : 0));
-  uint64_t planes = p8 ? f.planes * res : f.planes;
+  // (kSpare: none yet)
+  uint64_t part = std::max(std::max(f.split, p8 ? f.parts : 0) * res, std::max(f.kept, tc && !spare ? f.parts : 0));
+  uint64_t planes = p8 ? f.planes * res : spare ? 0 : f.planes;
   if (together) {
     for (uint64_t v : f.lvl_parts) part = std::max(part, std::min(v * res, tc ? kTcBytes : kGroupParts));
     for (uint64_t v : f.lvl_planes) planes = std::max(planes, std::min(v * res, tc ? kTcPlanes : kGroupPlanes));
@@ -602,7 +623,7 @@ SeqLayout layout_of(const Foot& f, int R, Choice ch) {
   s.part_bytes = part;
   s.p8_bytes = planes;
   sect(s.off_tc, p8   ? f.n_dense * kind_groups * p8_step_bytes()
-                 : tc ? f.n_dense * kinds * tc_unit_bytes()
+                 : tc ? f.n_dense * (spare ? 1 << kMaxChunkLog : kinds) * tc_unit_bytes()
                       : f.n_dense * R * kKeptDenseBytes);
   sect(s.off_part, part);
   sect(s.off_err, 64);
@@ -636,11 +657,59 @@ SeqLayout group_layout(const tnc_plan_t* const* plans, int n, int R, Choice ch) 
   return s;
 }
 
+// kSpare: the dense steps' scratch is what `budget` leaves beside one residue's
+// arena.  Of the sizes of the small residues' section those that a dense step
+// needs are tried, the rest is for planes (of a part of the shared values where that is
+// all that fits); the one is taken with which most of the multiply-adds run on the tensor
+// cores, if that is at least half of them (else one residue at a time costs more
+// than it gains).  In workspaces of TNC_PATH_INT64's least, on the CUDA cores
+// alone -> this way: cubic VC, n = 180, 8 residues 104.5 -> 27.5 ms and 722 -> 517, 3
+// residues 147.8 -> 65.6; n = 160, 3 residues 12.6 -> 8.3; n = 130, 3 residues 1.79 -> 1.90.
+SeqLayout spare_layout(const tnc_plan_t* const* plans, int n, int R, size_t budget) {
+  SeqLayout s = group_layout(plans, n, R, {TNC_PATH_TC, kSpare});
+  std::vector<StepDesc> dense;
+  double all = 0, most = 0;
+  for (int i = 0; i < n; i++) {
+    all += plans[i]->cost.macs;
+    for (const StepDesc& d : plans[i]->low.lvl_steps)
+      if (tc_eligible(d)) dense.push_back(d);
+  }
+  uint64_t left = budget > s.total ? (budget - s.total) / kAlign * kAlign : 0, part = 0;
+  // (not below the least that needs no such choice: that stays the least)
+  if (budget < group_layout(plans, n, R, choices(TNC_PATH_TC).back()).total) left = 0;
+  for (const StepDesc& x : dense)
+    for (uint32_t c = 0; c <= kMaxChunkLog && tc_eligible(tc_part(x, c, 0)); c++) {
+      const uint64_t bytes = align_up(tc_byte_bytes(tc_part(x, c, 0)));
+      if (bytes >= left) continue;
+      double covered = 0;
+      for (const StepDesc& d : dense) {
+        uint32_t chunks;
+        if (tc_chunks(d, left - bytes, bytes, &chunks)) covered += std::ldexp(1.0, d.ka + d.kb + d.k);
+      }
+      if (covered > most) {
+        most = covered;
+        part = bytes;
+      }
+    }
+  if (most < 0.5 * all) {
+    s.total = SIZE_MAX;
+    return s;
+  }
+  // (the small residues in place of the section of the K splits, if larger)
+  const uint64_t more = part > s.part_bytes ? part - align_up(s.part_bytes) : 0;
+  s.part_bytes = std::max(s.part_bytes, part);
+  s.p8_bytes = left - more;
+  for (size_t* at : {&s.off_err, &s.off_results, &s.off_limbs, &s.off_p8}) *at += more;
+  s.off_arena += left;
+  s.total += left;
+  return s;
+}
+
 // The first of the path's choices that fits `budget` bytes (the last one if none does).
 SeqLayout fitting_layout(const tnc_plan_t* const* plans, int n, int R, int path, size_t budget) {
   SeqLayout s;
   for (const Choice& ch : choices(path)) {
-    s = group_layout(plans, n, R, ch);
+    s = ch.fit == kSpare ? spare_layout(plans, n, R, budget) : group_layout(plans, n, R, ch);
     if (s.total <= budget) break;
   }
   return s;
@@ -682,7 +751,13 @@ int plan_groups(const tnc_plan_t* const* plans, int n, int R, int path, size_t b
 constexpr uint64_t kMostExtra = 16ull << 30;
 size_t group_bytes(const tnc_plan_t* const* plans, int n, int R, int path) {
   const size_t least = group_layout(plans, n, R, choices(path).back()).total;
-  return fitting_layout(plans, n, R, path, least + std::max<uint64_t>(least, kMostExtra)).total;
+  size_t bytes = least;
+  for (const Choice& ch : choices(path)) {
+    if (ch.fit == kSpare) continue;  // (has no size of its own)
+    bytes = group_layout(plans, n, R, ch).total;
+    if (bytes <= least + std::max<uint64_t>(least, kMostExtra)) break;
+  }
+  return bytes;
 }
 size_t plan_bytes(const tnc_plan_t* p, int R, int path) { return group_bytes(&p, 1, R, path); }
 
@@ -1283,7 +1358,7 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
     Range grid{}, tile{}, block[3] = {}, outer{};
     std::vector<Range> split;
     std::vector<std::pair<uint32_t, uint32_t>> p8;   // ranges of p8 steps launched together
-    std::vector<StepDesc> dense;                     // TNC_PATH_TC dense steps
+    std::vector<std::pair<StepDesc, uint32_t>> dense;  // TNC_PATH_TC dense steps, their parts (log2)
   };
   std::vector<Level> lev(n_lev);
   std::vector<GridStep> gsteps;
@@ -1316,8 +1391,8 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
         const uint32_t flags = p8 ? p8_flags(lw, i) : 0u;
         if (p8 && p8_eligible(d)) {
           p8steps.push_back(P8Step{d, flags});
-        } else if (tc && !p8 && tc_eligible(d)) {
-          lv.dense.push_back(d);
+        } else if (uint32_t chunks; tc && !p8 && tc_eligible(d) && tc_chunks(d, L.p8_bytes, L.part_bytes, &chunks)) {
+          lv.dense.push_back({d, chunks});
         } else if (flags) {
           return set_error(TNC_ERR_INVALID, "internal: direct fp16 planes on a CUDA-core step");
         } else if (outer_eligible(d)) {
@@ -1435,7 +1510,17 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
         planes = bytes = 0;
         return rc2;
       };
-      for (const StepDesc& d : lv.dense) {
+      for (const auto& [d, chunks] : lv.dense) {
+        if (chunks) {  // part after part, a residue at a time; each adds to the ones before
+          for (uint32_t gr = 0; gr < (uint32_t)ps.groups * rg; gr++)
+            for (uint32_t j = 0; j < 1u << chunks; j++) {
+              if ((rc = flush())) return rc;
+              nr = 1;
+              units.push_back(TcUnit{tc_part(d, chunks, j), gr / rg, gr % rg, j > 0});
+            }
+          if ((rc = flush())) return rc;
+          continue;
+        }
         const uint64_t pl = tc_plane_bytes(d), by = tc_byte_bytes(d);
         const uint32_t m = rg * pl <= L.p8_bytes && rg * by <= L.part_bytes ? rg : 1u;
         for (uint32_t gr = 0; gr < (uint32_t)ps.groups * rg; gr += m) {
@@ -1443,7 +1528,7 @@ static int contract_group(const tnc_plan_t* const* plans, int n, const tnc_contr
               units.size() >= tc_max_units(m) || (g_time_dense && gr == 0))
             if ((rc = flush())) return rc;
           nr = m;
-          units.push_back(TcUnit{d, gr / rg, gr % rg});
+          units.push_back(TcUnit{d, gr / rg, gr % rg, false});
           planes += m * pl;
           bytes += m * by;
         }
@@ -1804,6 +1889,10 @@ extern "C" size_t tnc_workspace_bytes_below(const tnc_plan_t* const* plans, int3
     if (!plans[i]) return 0;
     size_t own = SIZE_MAX;
     for (size_t c = 0; c < need.size(); c++) {
+      if (choices(opts->path)[c].fit == kSpare) {  // (has no size of its own)
+        need[c] = 0;
+        continue;
+      }
       const size_t b = group_layout(plans + i, 1, a.R, choices(opts->path)[c]).total;
       need[c] = std::max(need[c], b);
       own = std::min(own, b);
@@ -1814,7 +1903,7 @@ extern "C" size_t tnc_workspace_bytes_below(const tnc_plan_t* const* plans, int3
   const size_t head = sliced ? sliced_head_bytes(1ull << plans[0]->net.open_vars.size(), a) : 0;
   size_t most = 0;
   for (size_t b : need)
-    if (b + head < below) most = std::max(most, b + head);
+    if (b && b + head < below) most = std::max(most, b + head);
   return most;
 }
 

@@ -70,7 +70,7 @@ struct alignas(64) JoinUnit {
   const uint8_t* bytes;
   uint32_t* out;
   uint32_t c, log_split, n, r0;  // r0: the first residue's place among the launch's primes
-  uint32_t block_lo;
+  uint32_t block_lo, add;        // add: to the residues there (of the shared values before)
 };
 constexpr uint32_t kTcPrimes = 16;
 
@@ -279,6 +279,15 @@ __global__ void __launch_bounds__(256) rns_join_kernel(const JoinUnit* __restric
     res[r] = tnc_dev::mod_reduce(acc, jc.p[u.r0 + r], jc.mu[u.r0 + r]);
   }
   uint32_t* dst = u.out + o * stride;
+  if (u.add) {
+    uint32_t old[NR];
+    load_words<NR>(dst, old);
+#pragma unroll
+    for (int r = 0; r < NR; r++) {  // (both below p < 2^31)
+      const uint32_t s = res[r] + old[r], p = jc.p[u.r0 + r];
+      res[r] = s >= p ? s - p : s;
+    }
+  }
   if constexpr (NR == 4) *reinterpret_cast<uint4*>(dst) = make_uint4(res[0], res[1], res[2], res[3]);
   else if constexpr (NR == 2) *reinterpret_cast<uint2*>(dst) = make_uint2(res[0], res[1]);
   else *dst = res[0];
@@ -369,6 +378,7 @@ int tc_batch(const TcUnit* units, int n, uint32_t nr, uint32_t rg, uint32_t* are
     ju.n = nq;
     ju.r0 = units[i].group * rg + units[i].r;
     ju.block_lo = (uint32_t)blocks;
+    ju.add = units[i].add;
     blocks += ((1ull << d.c) + 255) / 256;
     joins.push_back(ju);
     for (uint32_t r = 0; r < nr; r++) {
@@ -384,7 +394,7 @@ int tc_batch(const TcUnit* units, int n, uint32_t nr, uint32_t rg, uint32_t* are
       planes += tc_plane_bytes(d);
       bytes += tc_byte_bytes(d);
     }
-    if (units[i].r == 0 && units[i].group == 0) {
+    if (units[i].r == 0 && units[i].group == 0 && !units[i].add) {
       b.steps++;
       b.splits += ls > 0;
     }

@@ -221,6 +221,7 @@ size_t p8_prob_bytes();
 struct TcUnit {
   StepDesc d;
   uint32_t group, r;  // the pass's residue group, the first residue in its entries
+  bool add;           // to the output's residues: a later part of the step's shared values
 };
 // Small primes that a step takes (residues below 2^31), and
 // per residue the bytes of its operands' fp16 planes and of its output's small

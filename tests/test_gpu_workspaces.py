@@ -1,12 +1,14 @@
 """The same counts in every workspace that a call takes, from what it asks for down
 to the least: residue groups side by side, one at a time, one residue at a time,
 and TNC_PATH_TC without room for its operand planes (CUDA cores alone)."""
+import numpy as np
 import pytest
 
 import oracle
 from paper_1805_00475_gb300 import build as tnc_build
 from paper_1805_00475_gb300 import instances as I
 from paper_1805_00475_gb300 import tnc
+from test_gpu_dense_shapes import WIDE, _formula
 
 pytestmark = pytest.mark.gpu
 
@@ -47,6 +49,31 @@ def test_counts_in_every_workspace(path, R):
     ws = torch.empty(_sizes([p], "int64", R, False, tnc.workspace_bytes(p, R))[-1], dtype=torch.uint8, device="cuda")
     if path == "tc":
         assert tnc.contract(p, R, path=path, workspace=ws).residues.tolist() == want
+
+
+@pytest.mark.parametrize("R,wide", [(1, False), (3, True), (4, False)])
+@pytest.mark.parametrize("fa,fb,k", [(9, 7, 11), (7, 5, 13), (8, 6, 8), (7, 6, 16), (10, 9, 10)])
+def test_dense_steps_in_what_the_workspace_leaves(fa, fb, k, R, wide):
+    """TNC_PATH_TC between its smallest size of its own and what TNC_PATH_INT64 takes: one
+    residue at a time, a step's shared values in parts that are added (more joins than steps)."""
+    import torch
+    f, order, exact = _formula(fa, fb, k, 100 * fa + 10 * fb + k)
+    p = tnc.plan(tnc.build_network(f), order=order, n_open=fa + fb)
+    primes = WIDE[:R] if wide else None
+    want = tnc.contract(p, R, primes=primes, path="tc")
+    assert np.array_equal(want.residues, np.stack([exact(q) for q in want.primes], axis=1))
+    own, least = _sizes([p], "tc", R, False, tnc.workspace_bytes(p, R, "tc"))[-2:]
+    if least < _sizes([p], "int64", R, False, tnc.workspace_bytes(p, R))[-1]:
+        return  # one residue at a time takes less than all of them on the CUDA cores: nothing in between
+    parts = 0
+    for i in range(13):
+        size = least + (own - least) * i // 13 // 256 * 256
+        r = tnc.contract(p, R, primes=primes, path="tc", workspace=torch.empty(size, dtype=torch.uint8, device="cuda"))
+        parts += tnc.last_kernel_launches()["rns_join"] > tnc.last_launch_counts()["tc_gemm"]
+        assert r.residues.tolist() == want.residues.tolist(), size
+    assert parts >= 1
+    with pytest.raises(ValueError):
+        tnc.contract(p, R, primes=primes, path="tc", workspace=torch.empty(least - 256, dtype=torch.uint8, device="cuda"))
 
 
 @pytest.mark.parametrize("path,R", [("int64", 5), ("tc", 3), ("tc_p8", 6)])
